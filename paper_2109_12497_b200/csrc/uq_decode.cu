@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
     using Q = typename U::Q;
     const size_t row_bytes = LevelFmt<FMT>::row_bytes(p.stride);
 
+    const bool want_values = p.out != nullptr || UPDATE;           // else: the integer sums only
     U unit;
     uint32_t kw[WORDS];
     if (active) {
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
         }
         for (; m < p.M; ++m)
             unit.add(U::template load<ROWS>(ROWS ? (const char *)p.rows[m] : (const char *)p.lev + (size_t)m * row_bytes, i, p.stride));
-        if (MULTI && p.out != nullptr) {
+        if (MULTI && want_values) {
             // idx bits of coordinates i..i+C-1 start at byte i*IB/8 (a multiple of 4 bytes, of 2 for 16 bits)
             if (C * IB == 16) {
                 kw[0] = __ldg((const uint16_t *)(p.idx + (size_t)i * IB / 8));
@@ -305,7 +306,6 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
     // more CTAs per SM than 32 sums and 32 values held at once would allow.
     unit.prepare();
     const bool full = i + C <= p.d;
-    const bool want_values = p.out != nullptr || UPDATE;
     // every warp looks up the segment of its own row of 32*C coordinates; lane k holds the
     // reconstruction factor of scale k (single-scale: every lane holds the same factor)
     const int64_t row1 = min(row0 + 32 * C, p.d);

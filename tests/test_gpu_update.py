@@ -53,6 +53,20 @@ def _fused_update_case(w, lr, mu, wd, use_mom):
             assert np.array_equal(gm[pad: pad + w.d], mom0) and (gm[:pad] == 7).all() and (gm[pad + w.d:] == 7).all()
 
 
+@pytest.mark.parametrize("fmt,s", [("i8", 127), ("i4x2", 7), ("i2x4", 1), ("i6p", 31)])
+@pytest.mark.parametrize("N,idx_bits", [(2, 1), (4, 2), (8, 4), (3, 8)])
+def test_update_without_the_gradient_output(fmt, s, N, idx_bits):
+    """out = NULL (the update a training loop makes): the same parameters and momentum as with it."""
+    w = wl.scaled("c3", 33_001, M=8, fmt=fmt, s=s, scales=tuple(s * 8 ** k for k in range(N)), idx_bits=idx_bits)
+    q = run_gpu(w, wl.generate(w))["q"]
+    got = []
+    for out in (torch.empty(w.d, device="cuda"), None):
+        theta, mom = torch.ones(w.d, device="cuda"), torch.zeros(w.d, device="cuda")
+        B.uq_decode_update(q.layout, q.lev, q.fmt, q.W, q.s, q.scales, q.idx, q.idx_bits, theta, mom, 0.1, 0.9, 5e-4, out)
+        got.append((theta, mom))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 def test_update_rejects_bad_arguments():
     w = wl.scaled("c1", 1000)
     q = run_gpu(w, wl.generate(w))["q"]
