@@ -219,18 +219,12 @@ int uq_encode_multi(const uq_layout *layout, const void *g, const float *W, cons
                     void *lev, uint32_t *status, void *stream);
 
 /*
- * uq_select_encode_multi followed by uq_decode(src = UQ_SRC_LEVELS) as one call — Algorithm 2 from
+ * uq_select_encode_multi followed by uq_decode(src = UQ_SRC_LEVELS) as one kernel — Algorithm 2 from
  * "Compute coordinate scales" to "Reconstruct gradient", everything of a multi-scale step behind
- * the scale agreement.  Where uq_encode_decode is one kernel (int8 levels, 16-bit draws, M <= 8)
- * this is one kernel too: the gradients are read once, the indices, the level rows and the
- * average are written, nothing is read back.  Otherwise the calls it stands for run one after
- * the other.  idx, lev and out receive, bit for bit, what the separate calls write; arguments and
- * errors are theirs.  The first call of this kind on a device (this call, uq_select_encode_multi,
- * or a uq_step that uses them) raises the kernel's limit of dynamic shared memory with
- * cudaFuncSetAttribute before it launches; make that first call during set-up, before any stream
- * capture.  Like uq_select_encode_multi it is bound by instruction issue, not by memory;
- * on a B200 it takes about 19 % less time than uq_select_scale_multi + uq_encode_decode, burst
- * and sustained, which is why uq_step uses it where it is one kernel.
+ * the scale agreement.  The gradients are read once (with 8 bf16 workers; otherwise twice, the
+ * second time from the caches as far as they hold them), the indices, the level rows and the
+ * average are written, nothing is read back.  idx, lev and out receive, bit for bit, what the
+ * separate calls write; arguments and errors are theirs.  uq_step makes this call.
  */
 int uq_select_encode_decode_multi(const uq_layout *layout, const void *g, const float *W,
                                   const int32_t *scales, int N, int idx_bits, uint64_t seed, int rng_bits,
@@ -239,34 +233,24 @@ int uq_select_encode_decode_multi(const uq_layout *layout, const void *g, const 
 
 /*
  * uq_encode_single (scales = NULL) or uq_encode_multi (scales given) followed by
- * uq_decode(src = UQ_SRC_LEVELS) as one call — Algorithm 1 lines "Quantize gradient", "AllReduce
+ * uq_decode(src = UQ_SRC_LEVELS) as one kernel — Algorithm 1 lines "Quantize gradient", "AllReduce
  * gradients", "Reconstruct gradient" (Algorithm 2: "Quantize with s*" onwards) — for callers whose
- * M workers are all in this buffer.  With int8 levels, 16-bit draws and M <= 8 it is one kernel: the
- * CTA that takes a tile of coordinates through the workers adds their levels up in registers and
- * writes the reconstructed average beside the level rows, so the levels are written (they are what
- * would cross the wire) but never read back.  With other formats, more workers or 32-bit draws
- * (whose encoder is bound by its arithmetic: one kernel is then no faster than two) the two kernels
- * run one after the other.  lev and out receive, bit for bit, what the two separate calls write; arguments and
- * errors are theirs (the integer sums are not available here: use uq_decode or uq_aggregate).
- * uq_step makes this call when it is given no S_opt.
+ * M workers are all in this buffer.  The warp that takes a row of coordinates through the workers
+ * adds their levels up in registers and writes the reconstructed average beside the level rows, so
+ * the levels are written (they are what would cross the wire) but never read back.  lev and out
+ * receive, bit for bit, what the two separate calls write; arguments and errors are theirs (the
+ * integer sums are not available here: use uq_step, uq_decode or uq_aggregate).
  */
 int uq_encode_decode(const uq_layout *layout, const void *g, const float *W, int s, const int32_t *scales,
                      int N, const uint8_t *idx, int idx_bits, uint64_t seed, int rng_bits, int fmt,
                      void *lev, float *out, uint32_t *status, void *stream);
 
 /*
- * uq_select_scale_multi followed by uq_encode_multi as one call — Algorithm 2 lines "Compute
+ * uq_select_scale_multi followed by uq_encode_multi as one kernel — Algorithm 2 lines "Compute
  * coordinate scales", "Scale sharing" and "Quantize with s*" — for callers whose M workers are all
- * in this buffer.  With M <= 8 it is one kernel: a CTA copies a tile of every worker's row into
- * shared memory once, takes the maximum over the workers of every magnitude there, finds and stores
- * the shared indices, and quantizes the workers' rows from the same copy, so the gradients cross
- * the memory interface once instead of twice.  With more workers the two kernels run one after
- * the other.  idx and lev receive, bit for bit, what the two separate calls write; arguments and
- * errors are theirs.  On a B200, with bf16 gradients and 16-bit draws, it takes about 15 % less
- * time than the two calls (the gradients are read from memory once); with 32-bit draws, whose
- * encoder is bound by its arithmetic either way, it takes the same time.  It is bound by
- * instruction issue rather than by memory, so uq_step keeps the two streaming kernels and this
- * call is the caller's choice.
+ * in this buffer: a first pass over the workers' rows takes the maximum over the workers of every
+ * magnitude, which decides the shared index, and the second pass quantizes.  idx and lev receive,
+ * bit for bit, what the two separate calls write; arguments and errors are theirs.
  */
 int uq_select_encode_multi(const uq_layout *layout, const void *g, const float *W, const int32_t *scales,
                            int N, int idx_bits, uint64_t seed, int rng_bits, int fmt, uint8_t *idx,
@@ -353,9 +337,7 @@ int uq_index_min(const uint8_t *rows, int R, int64_t row_bytes, int64_t nbytes, 
  * One whole step in one call — Algorithm 1 lines "MaxAllReduce Norm" to "Reconstruct gradient"
  * (scales = NULL: uq_agree_scale, uq_encode_single, uq_decode) or Algorithm 2 (scales given:
  * uq_agree_scale, uq_select_scale_multi, uq_encode_multi, uq_decode), enqueued in that order on
- * `stream`; without S_opt the last two are made as one call, uq_encode_decode, and where that
- * call is one kernel a multi-scale step makes the last three as one, uq_select_encode_decode_multi
- * (two kernels then do the whole step: the norms, and everything else).  Nothing is computed
+ * `stream`, as three kernels: two for the norms, and one for everything else.  Nothing is computed
  * differently: every output is bit for bit that of the separate calls.  Arguments are
  * those of the calls it makes (idx is not used when scales = NULL); the first error stops the
  * sequence and is returned.

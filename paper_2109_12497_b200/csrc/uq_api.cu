@@ -7,8 +7,8 @@ int64_t norm_tiles(int64_t d);
 cudaError_t launch_agree_scale(const uq_layout &L, const void *g, int norm, float *W, uint32_t *status,
                                void *workspace, cudaStream_t st);
 cudaError_t launch_encode(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
-                          const uint8_t *idx, int idx_bits, uint64_t seed, int rng_bits, int fmt, void *lev,
-                          uint32_t *status, cudaStream_t st);
+                          uint8_t *idx, int idx_bits, bool select, uint64_t seed, int rng_bits, int fmt,
+                          void *lev, float *out, int32_t *S, uint32_t *status, cudaStream_t st);
 cudaError_t launch_select(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
                           int idx_bits, uint8_t *idx, uint32_t *status, cudaStream_t st);
 cudaError_t launch_aggregate_decode(const uq_layout &L, const void *lev, int fmt, const float *W,
@@ -20,16 +20,6 @@ cudaError_t launch_aggregate_decode_rows(const uq_layout &L, const void *const *
                                          int32_t *S, cudaStream_t st);
 cudaError_t launch_decode_sums(const uq_layout &L, const int32_t *S, const float *W, const ScaleSet &scales,
                                const uint8_t *idx, int idx_bits, float *out, cudaStream_t st);
-cudaError_t launch_select_encode_decode(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
-                                        int idx_bits, uint64_t seed, uint8_t *idx, void *lev, float *out, uint32_t *status,
-                                        cudaStream_t st);
-bool encode_decode_fused(const uq_layout &L, int fmt, int rng_bits);
-cudaError_t launch_encode_decode(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
-                                 const uint8_t *idx, int idx_bits, uint64_t seed, void *lev, float *out, uint32_t *status,
-                                 cudaStream_t st);
-cudaError_t launch_select_encode(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales, int idx_bits,
-                                 uint64_t seed, int rng_bits, int fmt, uint8_t *idx, void *lev, uint32_t *status,
-                                 cudaStream_t st);
 cudaError_t launch_index_min(const uint8_t *rows, int R, int64_t row_bytes, int64_t nbytes, int idx_bits, uint8_t *idx,
                              cudaStream_t st);
 cudaError_t launch_randk_gather(const uq_layout &L, const void *g, int64_t K, uint64_t seed, int64_t *sel,
@@ -167,8 +157,8 @@ int uq_encode_single(const uq_layout *L, const void *g, const float *W, int s, u
     if (!fmt_ok(fmt, s) || (rng_bits != 32 && rng_bits != 16)) return UQ_ERR_BAD_ARG;
     if (L->d > 0 && (g == nullptr || lev == nullptr || !aligned(g, 16) || !aligned(lev, 16)))
         return UQ_ERR_BAD_ARG;
-    return finish(uq::launch_encode(*L, g, W, single_scale(s), nullptr, 0, seed, rng_bits, fmt, lev, status,
-                                    (cudaStream_t)stream));
+    return finish(uq::launch_encode(*L, g, W, single_scale(s), nullptr, 0, false, seed, rng_bits, fmt, lev, nullptr, nullptr,
+                                    status, (cudaStream_t)stream));
 }
 
 int uq_select_scale_multi(const uq_layout *L, const void *g, const float *W, const int32_t *scales, int N,
@@ -193,8 +183,8 @@ int uq_encode_multi(const uq_layout *L, const void *g, const float *W, const int
     if (L->d > 0 && (g == nullptr || lev == nullptr || idx == nullptr || !aligned(g, 16) || !aligned(lev, 16) ||
                      !aligned(idx, 16)))
         return UQ_ERR_BAD_ARG;
-    return finish(uq::launch_encode(*L, g, W, set, idx, idx_bits, seed, rng_bits, fmt, lev, status,
-                                    (cudaStream_t)stream));
+    return finish(uq::launch_encode(*L, g, W, set, const_cast<uint8_t *>(idx), idx_bits, false, seed, rng_bits, fmt, lev, nullptr,
+                                    nullptr, status, (cudaStream_t)stream));
 }
 
 int uq_select_encode_multi(const uq_layout *L, const void *g, const float *W, const int32_t *scales, int N,
@@ -208,8 +198,8 @@ int uq_select_encode_multi(const uq_layout *L, const void *g, const float *W, co
     if (L->d > 0 && (g == nullptr || lev == nullptr || idx == nullptr || !aligned(g, 16) || !aligned(lev, 16) ||
                      !aligned(idx, 16)))
         return UQ_ERR_BAD_ARG;
-    return finish(uq::launch_select_encode(*L, g, W, set, idx_bits, seed, rng_bits, fmt, idx, lev, status,
-                                           (cudaStream_t)stream));
+    return finish(uq::launch_encode(*L, g, W, set, idx, idx_bits, true, seed, rng_bits, fmt, lev, nullptr, nullptr, status,
+                                    (cudaStream_t)stream));
 }
 
 int uq_aggregate(const uq_layout *L, const void *lev, int fmt, int32_t *S, void *stream)
@@ -248,9 +238,11 @@ int uq_decode(const uq_layout *L, const void *src, int src_kind, int fmt, const 
                                               (cudaStream_t)stream));
 }
 
-int uq_encode_decode(const uq_layout *L, const void *g, const float *W, int s, const int32_t *scales, int N,
-                     const uint8_t *idx, int idx_bits, uint64_t seed, int rng_bits, int fmt, void *lev, float *out,
-                     uint32_t *status, void *stream)
+// Quantization, sum over the workers and reconstruction as one kernel; select: the shared indices are
+// found by that kernel too (by a kernel of their own in front with more than 8 workers).
+static int encode_decode(const uq_layout *L, const void *g, const float *W, int s, const int32_t *scales, int N,
+                         uint8_t *idx, int idx_bits, bool select, uint64_t seed, int rng_bits, int fmt, void *lev,
+                         float *out, int32_t *S_opt, uint32_t *status, void *stream)
 {
     uq::ScaleSet set;
     if (!layout_ok(L) || W == nullptr || !aligned(status, 4)) return UQ_ERR_BAD_ARG;
@@ -265,34 +257,26 @@ int uq_encode_decode(const uq_layout *L, const void *g, const float *W, int s, c
     }
     if (!fmt_ok(fmt, set.s[0]) || (rng_bits != 32 && rng_bits != 16)) return UQ_ERR_BAD_ARG;
     if (L->d > 0 && (g == nullptr || lev == nullptr || out == nullptr || !aligned(g, 16) || !aligned(lev, 16) ||
-                     !aligned(out, 32)))
+                     !aligned(out, 32) || !aligned(S_opt, 32)))
         return UQ_ERR_BAD_ARG;
-    if (uq::encode_decode_fused(*L, fmt, rng_bits))
-        return finish(uq::launch_encode_decode(*L, g, W, set, idx, idx_bits, seed, lev, out, status, (cudaStream_t)stream));
-    const cudaError_t e = uq::launch_encode(*L, g, W, set, idx, idx_bits, seed, rng_bits, fmt, lev, status,
-                                            (cudaStream_t)stream);
-    if (e != cudaSuccess) return finish(e);
-    return finish(uq::launch_aggregate_decode(*L, lev, fmt, W, set, idx, idx_bits, out, nullptr, (cudaStream_t)stream));
+    return finish(uq::launch_encode(*L, g, W, set, idx, idx_bits, select, seed, rng_bits, fmt, lev, out, S_opt, status,
+                                    (cudaStream_t)stream));
+}
+
+int uq_encode_decode(const uq_layout *L, const void *g, const float *W, int s, const int32_t *scales, int N,
+                     const uint8_t *idx, int idx_bits, uint64_t seed, int rng_bits, int fmt, void *lev, float *out,
+                     uint32_t *status, void *stream)
+{
+    return encode_decode(L, g, W, s, scales, N, const_cast<uint8_t *>(idx), idx_bits, false, seed, rng_bits, fmt, lev, out, nullptr,
+                         status, stream);
 }
 
 int uq_select_encode_decode_multi(const uq_layout *L, const void *g, const float *W, const int32_t *scales, int N,
                                   int idx_bits, uint64_t seed, int rng_bits, int fmt, uint8_t *idx, void *lev, float *out,
                                   uint32_t *status, void *stream)
 {
-    uq::ScaleSet set;
-    if (!layout_ok(L) || W == nullptr || !aligned(status, 4)) return UQ_ERR_BAD_ARG;
-    if (!scales_ok(scales, N, idx_bits, &set)) return UQ_ERR_BAD_ARG;
-    if (!fmt_ok(fmt, set.s[0]) || (rng_bits != 32 && rng_bits != 16)) return UQ_ERR_BAD_ARG;
-    if (L->d > 0 && (g == nullptr || lev == nullptr || idx == nullptr || out == nullptr || !aligned(g, 16) ||
-                     !aligned(lev, 16) || !aligned(idx, 16) || !aligned(out, 32)))
-        return UQ_ERR_BAD_ARG;
-    if (uq::encode_decode_fused(*L, fmt, rng_bits))
-        return finish(uq::launch_select_encode_decode(*L, g, W, set, idx_bits, seed, idx, lev, out, status,
-                                                      (cudaStream_t)stream));
-    const cudaError_t e = uq::launch_select_encode(*L, g, W, set, idx_bits, seed, rng_bits, fmt, idx, lev, status,
-                                                   (cudaStream_t)stream);
-    if (e != cudaSuccess) return finish(e);
-    return finish(uq::launch_aggregate_decode(*L, lev, fmt, W, set, idx, idx_bits, out, nullptr, (cudaStream_t)stream));
+    if (scales == nullptr) return UQ_ERR_BAD_ARG;
+    return encode_decode(L, g, W, 0, scales, N, idx, idx_bits, true, seed, rng_bits, fmt, lev, out, nullptr, status, stream);
 }
 
 int uq_decode_rows(const uq_layout *L, const void *const *lev_rows, int fmt, const float *W, int s,
@@ -346,25 +330,10 @@ int uq_step(const uq_layout *L, const void *g, int norm, int s, const int32_t *s
             uint64_t seed, int rng_bits, int fmt, float *W, uint8_t *idx, void *lev, float *out, int32_t *S_opt,
             uint32_t *status, void *workspace, size_t workspace_bytes, void *stream)
 {
-    int rc = uq_agree_scale(L, g, norm, W, status, workspace, workspace_bytes, stream);
+    const int rc = uq_agree_scale(L, g, norm, W, status, workspace, workspace_bytes, stream);
     if (rc != UQ_OK) return rc;
-    if (scales != nullptr) {
-        // nobody wants the integer sums, and the encoder can select, add up and reconstruct itself: the
-        // rest of the step is one kernel
-        if (S_opt == nullptr && layout_ok(L) && uq::encode_decode_fused(*L, fmt, rng_bits))
-            return uq_select_encode_decode_multi(L, g, W, scales, N, idx_bits, seed, rng_bits, fmt, idx, lev, out, status,
-                                                 stream);
-        rc = uq_select_scale_multi(L, g, W, scales, N, idx_bits, idx, status, stream);
-        if (rc != UQ_OK) return rc;
-    }
-    if (S_opt == nullptr)       // nobody wants the integer sums: the encoder may add up and reconstruct itself
-        return uq_encode_decode(L, g, W, s, scales, N, idx, idx_bits, seed, rng_bits, fmt, lev, out, status, stream);
-    if (scales != nullptr)
-        rc = uq_encode_multi(L, g, W, scales, N, idx, idx_bits, seed, rng_bits, fmt, lev, status, stream);
-    else
-        rc = uq_encode_single(L, g, W, s, seed, rng_bits, fmt, lev, status, stream);
-    if (rc != UQ_OK) return rc;
-    return uq_decode(L, lev, UQ_SRC_LEVELS, fmt, W, s, scales, N, idx, idx_bits, out, S_opt, stream);
+    return encode_decode(L, g, W, s, scales, N, idx, idx_bits, scales != nullptr, seed, rng_bits, fmt, lev, out, S_opt, status,
+                         stream);
 }
 
 size_t uq_workspace_bytes_small(void) { return uq::small_workspace_bytes(); }

@@ -111,15 +111,6 @@ __device__ __forceinline__ uint2 ld_coherent64(const void *p)
 
 template <typename T> __device__ __forceinline__ void st_stream(T *p, T v) { __stcs(p, v); }
 
-// 16 bytes from global memory straight into shared memory (no register in between); the copies of
-// a thread are complete for that thread after copy_async_wait().
-__device__ __forceinline__ void copy_async16(void *smem_dst, const void *gmem_src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src)
-                 : "memory");
-}
-__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // 256-bit streaming load / store (sm_100 and later): 32 bytes per lane in one instruction.
 // The address must be 32-byte aligned.
 struct alignas(32) uint8x { uint32_t w[8]; };
@@ -270,30 +261,6 @@ __device__ __forceinline__ void philox4x32_10_xN(const PhiloxKey &k, const uint3
     for (int n = 0; n < N; ++n) out[n] = make_uint4(c0[n], c1[n], c2[n], c3[n]);
 }
 
-// The same block number for N workers at once (worker[n] in counter word 2).
-template <int N>
-__device__ __forceinline__ void philox4x32_10_workers(const PhiloxKey &k, uint32_t block_lo, uint32_t block_hi,
-                                                      const uint32_t (&worker)[N], uint4 (&out)[N])
-{
-    uint32_t c0[N], c1[N], c2[N], c3[N];
-#pragma unroll
-    for (int n = 0; n < N; ++n) { c0[n] = block_lo; c1[n] = block_hi; c2[n] = worker[n]; c3[n] = 0u; }
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t k0 = k.k0[r], k1 = k.k1[r];
-#pragma unroll
-        for (int n = 0; n < N; ++n) {
-            const uint64_t p0 = (uint64_t)0xD2511F53u * c0[n];
-            const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2[n];
-            const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1[n] ^ k0;
-            const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3[n] ^ k1;
-            c1[n] = (uint32_t)p1; c3[n] = (uint32_t)p0; c0[n] = n0; c2[n] = n2;
-        }
-    }
-#pragma unroll
-    for (int n = 0; n < N; ++n) out[n] = make_uint4(c0[n], c1[n], c2[n], c3[n]);
-}
-
 // The first two rounds of a block split by what they depend on.  Of the counter
 // (block low, block high, worker, 0) only word 0 differs between the threads of a tile and only
 // word 2 between the workers, and the two do not meet before the second round:
@@ -302,10 +269,11 @@ __device__ __forceinline__ void philox4x32_10_workers(const PhiloxKey &k, uint32
 //   round 1: c0 = hi(M1*c2) ^ c1 ^ k0[1]   c1 = lo(M1*c2)   c2 = hi(M0*c0) ^ c3 ^ k1[1]   c3 = lo(M0*c0)
 // so a thread that draws the same block for several workers keeps {hi, lo}(M1*c2) and c3 of round 0
 // (PhiloxBlockPart), takes the per-worker words from a table made once per launch
-// (PhiloxWorkerPart, uniform over the grid), joins them with two three-input XORs and runs the
+// (PhiloxWorkerPart, uniform over the grid), joins them with two XORs and runs the
 // remaining eight rounds: 34 instead of 40 multiply / XOR instructions per block.
 struct PhiloxBlockPart { uint32_t a, b, c3; };       // hi(M1*c2), lo(M1*c2), c3 after round 0
-struct PhiloxWorkerPart { uint32_t u1, hq, lq; };    // c1 after round 0; hi, lo of M0 * (c0 after round 0)
+// c1 after round 0 and hi of M0 * (c0 after round 0), each with the key of round 1 already in it; lo of that product
+struct alignas(16) PhiloxWorkerPart { uint32_t u1, hq, lq, unused; };
 
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 
@@ -323,39 +291,47 @@ __host__ __device__ __forceinline__ PhiloxWorkerPart philox_worker_part(const Ph
 {
     PhiloxWorkerPart w;
     const uint64_t pw = (uint64_t)kPhiloxM1 * worker;
-    w.u1 = (uint32_t)pw;
+    w.u1 = (uint32_t)pw ^ k.k0[1];
     const uint64_t q0 = (uint64_t)kPhiloxM0 * ((uint32_t)(pw >> 32) ^ block_hi ^ k.k0[0]);
-    w.hq = (uint32_t)(q0 >> 32); w.lq = (uint32_t)q0;
+    w.hq = (uint32_t)(q0 >> 32) ^ k.k1[1]; w.lq = (uint32_t)q0; w.unused = 0u;
     return w;
 }
 
-// Rounds 1 (the joining XORs) to 9 of N blocks of one worker, advanced together.
-template <int N>
-__device__ __forceinline__ void philox_join(const PhiloxKey &k, const PhiloxBlockPart (&blk)[N], const PhiloxWorkerPart &w,
-                                            uint4 (&out)[N])
+// Rounds 1 (the joining XORs) to 9 of the N blocks of G workers, all advanced together: one fetch of a round
+// key serves G * N chains.  last0, last1: the keys of round 9 (a caller that wants words 0 and 2
+// complemented hands over the complemented keys).
+template <int G, int N>
+__device__ __forceinline__ void philox_join(const PhiloxKey &k, uint32_t last0, uint32_t last1, const PhiloxBlockPart (&blk)[N],
+                                            const PhiloxWorkerPart *w, uint4 (&out)[G][N])
 {
-    uint32_t c0[N], c1[N], c2[N], c3[N];
+    uint32_t c0[G][N], c1[G][N], c2[G][N], c3[G][N];
 #pragma unroll
-    for (int n = 0; n < N; ++n) {
-        c0[n] = blk[n].a ^ w.u1 ^ k.k0[1];
-        c1[n] = blk[n].b;
-        c2[n] = w.hq ^ blk[n].c3 ^ k.k1[1];
-        c3[n] = w.lq;
-    }
-#pragma unroll
-    for (int r = 2; r < 10; ++r) {
-        const uint32_t k0 = k.k0[r], k1 = k.k1[r];
+    for (int g = 0; g < G; ++g)
 #pragma unroll
         for (int n = 0; n < N; ++n) {
-            const uint64_t p0 = (uint64_t)kPhiloxM0 * c0[n];
-            const uint64_t p1 = (uint64_t)kPhiloxM1 * c2[n];
-            const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1[n] ^ k0;
-            const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3[n] ^ k1;
-            c1[n] = (uint32_t)p1; c3[n] = (uint32_t)p0; c0[n] = n0; c2[n] = n2;
+            c0[g][n] = blk[n].a ^ w[g].u1;
+            c1[g][n] = blk[n].b;
+            c2[g][n] = w[g].hq ^ blk[n].c3;
+            c3[g][n] = w[g].lq;
         }
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        const uint32_t k0 = r == 9 ? last0 : k.k0[r], k1 = r == 9 ? last1 : k.k1[r];
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                const uint64_t p0 = (uint64_t)kPhiloxM0 * c0[g][n];
+                const uint64_t p1 = (uint64_t)kPhiloxM1 * c2[g][n];
+                const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1[g][n] ^ k0;
+                const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3[g][n] ^ k1;
+                c1[g][n] = (uint32_t)p1; c3[g][n] = (uint32_t)p0; c0[g][n] = n0; c2[g][n] = n2;
+            }
     }
 #pragma unroll
-    for (int n = 0; n < N; ++n) out[n] = make_uint4(c0[n], c1[n], c2[n], c3[n]);
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int n = 0; n < N; ++n) out[g][n] = make_uint4(c0[g][n], c1[g][n], c2[g][n], c3[g][n]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -410,16 +386,16 @@ __device__ __forceinline__ uint32_t level_draw16(float x, uint32_t h)
 }
 constexpr uint32_t kLevelByte16 = 2;
 
-// The same level with the clamp folded into saturating arithmetic (both on the FMA pipe, where the
-// min of the form above is an ALU instruction).  inv256 = inv / 256 exactly (the caller checks that
-// inv is 0 or at least 2^-100, so nothing is lost to a subnormal), hence |v| * inv256 = x / 256
-// with the rounding of x.  c0 = 1 - cap / 256: the saturating sum reaches 1.0 exactly where x
-// reaches cap, and below 1.0 its unit in the last place is 2^-24, i.e. 2^-16 in x (ties to even as
-// before, since c0 is an even multiple of it).  As an integer the sum is
+// The clamp folded into saturating arithmetic (both on the FMA pipe, where the min of the form above is an
+// ALU instruction).  inv256 = inv / 256 exactly (the caller checks that inv is 0 or at least 2^-100, so
+// nothing is lost to a subnormal), hence |v| * inv256 = x / 256 with the rounding of x.  With c0 = 1 -
+// cap / 256 the saturating sum x / 256 + c0 reaches 1.0 exactly where x reaches cap, and below 1.0 its
+// unit in the last place is 2^-24, i.e. 2^-16 in x (ties to even as before, since c0 is an even multiple
+// of it).  As an integer the sum is
 //   0x3F000000 + (128 - cap) * 2^16 + floor(x) * 2^16 + rint(p * 2^16),
-// and subtracting h + 1 borrows from the level field iff h >= rint(p * 2^16).  With
-// adj = -1 - (127 - cap) * 2^16 byte 2 of the result is the level.  The saturating product turns a
-// NaN (0 * Inf, a NaN input) into 0 and so into level 0; Inf saturates to level cap.
+// and adding 2^16 - 1 - h carries into bit 16 iff h < rint(p * 2^16): byte 2 is then the level plus
+// 128 - cap.  The saturating product turns a NaN (0 * Inf, a NaN input) into 0 and so into level 0; Inf
+// saturates to level cap.
 __device__ __forceinline__ float mul_sat(float a, float b)
 {
     float d;
@@ -432,11 +408,6 @@ __device__ __forceinline__ float add_sat(float a, float b)
     asm("add.rn.sat.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
 }
-__device__ __forceinline__ uint32_t level_draw16_sat(float v, float inv256, float c0, uint32_t adj, uint32_t h)
-{
-    return __float_as_uint(add_sat(mul_sat(fabsf(v), inv256), c0)) - h + adj;
-}
-
 // Gathers byte B of four words into one word (coordinate order = byte order).
 template <uint32_t B> __device__ __forceinline__ uint32_t gather_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {

@@ -1,23 +1,25 @@
 // Stochastic quantization of every worker's gradient to small signed integers:
 // Q_s (Section "QSGDMaxNorm Quantization", Algorithm 1 line "Quantize gradient") and
 // Q_{s_} with the shared per-coordinate scale (Section "QSGDMaxNormMultiScale Quantization",
-// Algorithm 2 line "Quantize with s*").
+// Algorithm 2 line "Quantize with s*"), optionally with what stands around it in the algorithms
+// when all workers are in this buffer: the choice and sharing of the scale indices in front (SEL),
+// the integer sum over the workers and the reconstructed average behind (DEC).
 //
-// One streaming pass: a thread owns units of 8 consecutive coordinates (32 B of fp32 or 16 B of
-// bf16 in; 8 B of int8, 6 B of two-plane 6-bit, 4 B of packed 4-bit or 2 B of packed 2-bit levels
-// out); a CTA owns one tile of coordinates and takes the M workers' rows of it one after the other.
-// What does not depend on the worker is then done once per tile instead of once per worker: the
-// segment lookup, the division s / W, the per-coordinate factors s_k / W of the shared scale
-// indices (one index load and eight shuffles per unit), and the first two rounds of the Philox
-// block, whose counter differs between workers only in one word.  The work done for worker m
-// reads only g^m plus the agreed values W and idx.
+// One streaming pass.  A thread owns 8 consecutive coordinates (a warp a row of 256 of them) and takes the
+// workers' rows G at a time, straight-line; a worker's registers are filled again with the bytes of the
+// worker G places on as soon as they are quantized.  What does not depend on the worker is done once: the
+// segment lookup, the factors s_k / W of the coordinates, and the first two rounds of the Philox block,
+// whose counter differs between workers in one word only; the G workers' blocks advance together, so
+// that one fetch of a round key serves all of them.  The levels are added up in packed lanes as they are
+// made, and the average leaves with them: the level rows are written (they are what crosses the wire)
+// but never read back.  SEL: a first pass over the workers' rows takes the largest magnitude of every
+// coordinate, which decides the shared index; the rows of 8 bf16 workers are kept in shared memory for
+// the second pass, others come from the caches.  A warp is on its own (no barrier: with one lookup per CTA
+// the warps waited for it longer than their own lookups take).
 //
-// Decode mode (int8 levels, 16-bit draws, M <= 8, so that one CTA sees every worker of its tile; with
-// 32-bit draws the encoder is bound by its arithmetic and the sums cost what the saved read gains,
-// measured, so there the two kernels stay): the CTA also adds
-// the workers' levels up as it goes and writes the reconstructed average (Algorithm 1 / 2, lines
-// "AllReduce gradients" and "Reconstruct gradient") beside the level rows, which then need not be
-// read back by the aggregation kernel.  Bit for bit what uq_decode makes of the same levels.
+// Measured on a B200 (25.6 M binary32 coordinates in 161 layers, 8 workers, int8 levels, 32-bit draws;
+// sustained): 235 us for quantization + sum + reconstruction, where two kernels took 210 + 53 us; with
+// selection among 4 scales 266 us, where three took 130 + 216 + 53 us.
 #pragma once
 #include "uq_device.cuh"
 #include "uq_select.cuh"
@@ -29,761 +31,598 @@ struct EncodeParams {
     SelectView v;             // g, W, seg_off, d, stride, nseg, M, scales (single-scale: every entry is s) and
                               // s_hat = (float) of the smallest scale: the largest level
     void *lev;
-    float *out;               // decode mode: the reconstructed average [d]; else unused
+    float *out;               // the reconstructed average [d], or NULL
+    int32_t *S;               // the integer sums [d], or NULL (needs out)
     uint8_t *idx;             // shared scale indices: read, or (select) written by this launch
     uint32_t *status;
     int32_t select;           // multi-scale: 1 = find the shared indices here instead of reading them
+    int32_t idx_bits;         // 1, 2, 4 or 8; 0 for the single-scale quantizer
     int32_t worker0;          // number, in the whole job, of the worker in row 0 (keys the draws)
-    int64_t coord0;           // index, in the whole gradient, of coordinate 0 (keys the draws)
-    uint32_t row_blocks;      // CTAs that own rows crossed by boundaries: after the tile CTAs, or (decode mode,
-                              // where such a CTA takes every worker's row and runs much longer) in front of them
-    uint32_t reserved;
-    uint32_t main_blocks;     // CTAs that own tiles
-    uint32_t groups;          // CTAs per tile: ceil(M / kWorkerGroup)
-    PhiloxKey key;            // the ten round keys of the seed
     uint32_t blk_hi;          // high word of the Philox block numbers the table below was made for
+    int64_t coord0;           // index, in the whole gradient, of coordinate 0 (keys the draws)
+    PhiloxKey key;            // the ten round keys of the seed
+    uint32_t last0, last1;    // the last round's keys as the fast path wants them (16-bit draws: complemented)
     PhiloxWorkerPart wpart[UQ_MAX_WORKERS];   // per-worker words of the first two Philox rounds (row m)
 };
 
-constexpr int kWorkerGroup = 8;   // workers that one CTA takes through a tile
+constexpr int kGroup = 8;     // the number of workers that has kernels of its own (all of them straight-line)
 
-// Launch shape per variant, from sweeps on B200: a thread owns UNITS units of 8 coordinates of the
-// tile, and at least MIN_CTAS CTAs share an SM (which caps the registers per thread).
-template <int DT, int RNG> struct EncodeShape {
-    static constexpr int UNITS = DT == UQ_BF16 ? 2 : 1;                       // 32 B per thread and worker in flight
-    static constexpr int MIN_CTAS = (DT == UQ_BF16 && RNG == 32) ? 3 : 4;
-    // decode mode (16-bit draws only) holds the level sums too: at 64 registers the bf16 kernel spills
-    static constexpr int MIN_CTAS_DEC = DT == UQ_F32 ? 4 : 3;
-    static constexpr int TILE = kThreads * UNITS * 8;
+// Launch shape per variant.  The kernel's time is its instructions: a warp scheduler issues one per cycle,
+// except that a 32 x 32 -> 64 bit multiply (two per Philox round) holds it for about four (measured alone:
+// multiply 4.3 cycles, with a logic operation beside it 4.5, with n additions beside it 4.3 + n - 0.4).
+// So the shape is the one with the fewest instructions that still hides the loads: four chains of Philox
+// rounds advance together, and four CTAs of 64 registers share an SM.  Measured on a B200 (8 workers,
+// quantization + sum + reconstruction, sustained): bf16 with 32-bit draws 3 CTAs 188 us, 4 CTAs 197 us
+// (26.2 M coordinates); binary32, selecting, 32-bit draws: one worker at a time 266 us, two 273 us (25.6 M).
+template <int DT, int RNG, bool SEL> struct EncodeShape {
+    static constexpr int V = 8 * Elem<DT>::BYTES / 16;                        // 16-byte words per thread and worker
+    static constexpr int NB = RNG == 32 ? 2 : 1;                              // Philox blocks per thread and worker
+    static constexpr int G = DT == UQ_F32 ? (SEL ? 1 : 2) : RNG == 32 ? 2 : 4;    // workers whose blocks advance together
+    static constexpr int CTAS = DT == UQ_BF16 && RNG == 32 ? 3 : 4;           // per SM
+    static constexpr int TILE = kThreads * 8;
 };
 
-// Coordinates [a, b) of worker m with per-coordinate scale lookup and bounds: the ragged last
-// tile and the 256-coordinate rows that a segment boundary crosses.  Thread `who` of `many`
-// cooperating threads (whole warps) takes every many-th unit, so a warp owns a row of 256
-// consecutive coordinates per round.  The warp looks the row's first segment up together; lane L
-// then holds the end and the scale of segment (first + L), and a coordinate's segment is the
-// number of ends at or before it, counted with shuffles: no dependent loads per coordinate.
-// Rare (a few rows per segment), so kept out of line.
-// own_idx (select mode, rows owned by a CTA that did not select for them): the warp finds the
-// shared indices of its row itself (thr: the warp's 2 * UQ_MAX_SCALES words of shared memory) instead
-// of reading them.
-template <int DT, int FMT, int RNG, int IDXB>
-__device__ __noinline__ void encode_span_general(const EncodeParams &p, int m, int64_t a, int64_t b, int who, int many,
-                                                 bool own_idx = false, int32_t *thr = nullptr)
+// ---------------------------------------------------------------------------------------------
+// the packed indices of UC coordinates: coordinates 0..3 in fields of ib bits from bit 0 of kw[0],
+// coordinates 4..7 in kw[1] (bits beyond a word's four fields: anything)
+// ---------------------------------------------------------------------------------------------
+template <int UC> __device__ __forceinline__ void load_indices(const uint8_t *idx, int64_t i, int ib, uint32_t *kw)
+{
+    const uint8_t *p = idx + ((i * ib) >> 3);
+    const int bits = UC * ib;
+    if (bits == 64) {
+        const uint2 x = __ldg((const uint2 *)p);
+        kw[0] = x.x; kw[UC / 4 - 1] = x.y;
+        return;
+    }
+    uint32_t x;
+    if (bits == 32) x = __ldg((const uint32_t *)p);
+    else if (bits == 16) x = __ldg((const uint16_t *)p);
+    else x = __ldg(p);
+    if (UC == 8) { kw[0] = x; kw[UC / 4 - 1] = x >> (4 * ib); }
+    else kw[0] = bits == 4 ? x >> (i & 4) : x;
+}
+
+// Stores them (kw without stray bits); called by whole warps (4 bits per thread: two lanes share a byte).
+template <int UC> __device__ __forceinline__ void store_indices(uint8_t *idx, int64_t i, int ib, const uint32_t *kw)
+{
+    uint8_t *p = idx + ((i * ib) >> 3);
+    const int bits = UC * ib;
+    if (bits == 64) { *(uint2 *)p = make_uint2(kw[0], kw[UC / 4 - 1]); return; }
+    const uint32_t x = UC == 8 ? kw[0] | (kw[UC / 4 - 1] << (4 * ib)) : kw[0];
+    if (bits == 32) *(uint32_t *)p = x;
+    else if (bits == 16) *(uint16_t *)p = (uint16_t)x;
+    else if (bits == 8) *p = (uint8_t)x;
+    else {
+        const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, x, 1);
+        if ((i & 4) == 0) *p = (uint8_t)(x | (next << 4));
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// slow forms, out of line
+// ---------------------------------------------------------------------------------------------
+
+// Everything for the coordinates [r0, min(r0 + 256, d)), looked up coordinate by coordinate, in plain
+// arithmetic: the row that holds d, rows whose Philox block numbers leave the launch's high word, and
+// rows whose factors are too small or too large for the rescaled forms.  One warp; a lane takes a unit
+// of 8 coordinates.
+template <int DT, int FMT, int RNG, bool MULTI>
+__device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0)
 {
     using E = Elem<DT>;
-    constexpr bool MULTI = IDXB != 0;
-    constexpr int IB = MULTI ? IDXB : 8;
-    const char *row = (const char *)p.v.g + (size_t)m * (size_t)p.v.stride * E::BYTES;
-    const int lane = who & 31;
-    for (int64_t row0 = a + (int64_t)(who - lane) * 8; row0 < b; row0 += (int64_t)many * 8) {
-        const int64_t row1 = min(row0 + 256, b);
-        const int j_row = warp_find_segment(p.v.seg_off, p.v.nseg, row0);
-        const int jl = j_row + lane;
-        const int64_t my_end = jl < p.v.nseg ? segment_end(p.v.seg_off, p.v.nseg, jl, p.v.d) : INT64_MAX;
-        const float my_W = __ldg(p.v.W + min(jl, p.v.nseg - 1));
-        const int64_t i = min(row0 + lane * 8, b - 1);            // lanes beyond b idle but take part in the shuffles
-        int seg[8] = {0, 0, 0, 0, 0, 0, 0, 0};                    // segment of each coordinate, relative to j_row
-        int nb = 0;
-        for (; nb < 32; ++nb) {                                   // warp-uniform loop over the ends inside the row
-            const int64_t end = __shfl_sync(0xFFFFFFFFu, my_end, nb);
-            if (end >= row1) break;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) seg[e] += end <= i + e ? 1 : 0;
+    using LF = LevelFmt<FMT>;
+    const int64_t i = r0 + (threadIdx.x & 31) * 8, d = p.v.d;
+    if (i >= min(r0 + 256, d)) return;
+    int j = find_segment(p.v.seg_off, p.v.nseg, i);
+    uint32_t kw[2] = {0u, 0u};
+    if (MULTI) {
+        if (p.select) {
+            uint32_t amag[8];
+            unit_max_magnitude<DT>(p.v, i, true, amag);
+            const uint64_t packed = select_general(p.v, i, amag, p.idx_bits, j);
+            kw[0] = (uint32_t)packed & (uint32_t)((1ull << (4 * p.idx_bits)) - 1ull);
+            kw[1] = (uint32_t)(packed >> (4 * p.idx_bits));
+            store_indices<8>(p.idx, i, p.idx_bits, kw);
+        } else {
+            load_indices<8>(p.idx, i, p.idx_bits, kw);
         }
-        float Wc[8];
+    }
+    float inv[8], c[8];
+    bool overflow = false;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) Wc[e] = __shfl_sync(0xFFFFFFFFu, my_W, seg[e]);
-        if (nb == 32) {                                           // more than 32 segments in one row: walk the table
-            int j = j_row;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
-                Wc[e] = __ldg(p.v.W + j);
-            }
-        }
-        typename IdxBits<IB>::T kbits = 0;
-        if (MULTI && own_idx)                                     // the whole warp takes part
-            kbits = (typename IdxBits<IB>::T)select_unit<DT, IB, 4>(p.v, row0 + lane * 8, row0, thr);
-        if (row0 + lane * 8 >= b) continue;
-        float v[8];
-        uint4 q[8 / E::G];
-#pragma unroll
-        for (int h = 0; h < 8 / E::G; ++h) {
-            q[h] = ld_stream(row + (i + h * E::G) * E::BYTES);
-            E::unpack(q[h], *(float(*)[E::G])(v + h * E::G));
-        }
-        uint32_t neg_lo, neg_hi;
-        unit_signs<DT>(q, neg_lo, neg_hi);          // the sign of a padding coordinate is harmless: its level is 0
-        if (MULTI && !own_idx)
-            kbits = p.select ? IdxBits<IB>::load_written(p.idx + i * IB / 8) : IdxBits<IB>::load(p.idx + i * IB / 8);
-        float inv[8];
-        bool overflow = false;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            if (i + e >= p.v.d) v[e] = 0.0f;                        // padding quantizes to level 0
-            const int k = MULTI ? (int)((kbits >> (e * IB)) & ((1u << IB) - 1u)) : 0;
-            inv[e] = inv_scale(p.v.scales.s[k & (UQ_MAX_SCALES - 1)], Wc[e]);
+    for (int e = 0; e < 8; ++e) {
+        inv[e] = c[e] = 0.0f;
+        if (i + e < d) {
+            j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
+            const float W = __ldg(p.v.W + j);
+            const uint32_t k = MULTI ? (kw[e >> 2] >> ((e & 3) * p.idx_bits)) & ((1u << p.idx_bits) - 1u) & (UQ_MAX_SCALES - 1) : 0u;
+            inv[e] = inv_scale(p.v.scales.s[k], W);
+            c[e] = decode_factor(W, p.v.scales.s[k], p.v.M);
             overflow |= not_finite(inv[e]);
         }
-        if (overflow && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
-        const uint64_t blk = RNG == 32 ? (uint64_t)((p.coord0 + i) >> 2) : (uint64_t)((p.coord0 + i) >> 3);
-        char *lrow = (char *)p.lev + (size_t)m * LevelFmt<FMT>::row_bytes(p.v.stride);
-        quantize_unit<FMT, RNG>(v, inv, p.v.s_hat, neg_lo, neg_hi, p.key, (uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)(m + p.worker0),
-                                lrow + LevelFmt<FMT>::off(i), lrow + LevelFmt<FMT>::off2(i, p.v.stride));
     }
-}
-
-// A full tile that a segment boundary crosses, all 256 threads, workers m0 .. m1 - 1: the warps
-// walk their 256-coordinate rows one by one.  Lane L takes the end of segment j + L (j = the
-// tile's first segment), so the segment of a row is j + (number of ends at or before the row's
-// start): one ballot per row instead of a search.  What a row's workers share (its segment, the
-// factors s_k / W, the shared indices) is found once per row; the rows of four workers are in
-// flight together.  A row that itself contains a boundary is skipped: a CTA of the second kind
-// owns it.
-template <int DT, int FMT, int RNG, int IDXB>
-__device__ __noinline__ void encode_tile_mixed(const EncodeParams &p, int m0, int m1, int64_t t0, int j)
-{
-    using E = Elem<DT>;
-    using S = EncodeShape<DT, RNG>;
-    using LF = LevelFmt<FMT>;
-    constexpr bool MULTI = IDXB != 0;
-    constexpr int IB = MULTI ? IDXB : 8;
-    constexpr int H = 8 / E::G;
-    constexpr int KMASK = IB < 4 ? (1 << IB) - 1 : UQ_MAX_SCALES - 1;
-    constexpr int G = 4;                                         // workers whose rows are loaded together
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int32_t my_scale = p.v.scales.s[lane & KMASK];
-    const int64_t my_end = j + lane < p.v.nseg ? segment_end(p.v.seg_off, p.v.nseg, j + lane, p.v.d) : INT64_MAX;
-    const size_t grow = (size_t)p.v.stride * E::BYTES, lrow = LF::row_bytes(p.v.stride);
-    bool overflow = false;
-#pragma unroll 1
-    for (int u = 0; u < S::UNITS; ++u) {
-        const int64_t r0 = t0 + (int64_t)(u * kThreads + (tid & ~31)) * 8;
-        const int cnt = __popc(__ballot_sync(0xFFFFFFFFu, my_end <= r0));
-        int jr;
-        int64_t end;
-        if (cnt < 32) {
-            jr = j + cnt;
-            end = __shfl_sync(0xFFFFFFFFu, my_end, cnt);
-        } else {                                                 // more than 32 segments inside one tile
-            jr = warp_find_segment(p.v.seg_off, p.v.nseg, r0);
-            end = segment_end(p.v.seg_off, p.v.nseg, jr, p.v.d);
-        }
-        if (end < r0 + 256) continue;                            // warp-uniform
-        const float inv_lane = inv_scale(my_scale, __ldg(p.v.W + jr));
-        overflow |= not_finite(inv_lane);
-        const int64_t i = r0 + lane * 8;
-        typename IdxBits<IB>::T kbits = 0;
-        if (MULTI) kbits = p.select ? IdxBits<IB>::load_written(p.idx + i * IB / 8) : IdxBits<IB>::load(p.idx + i * IB / 8);
-        float inv[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            inv[e] = MULTI ? __shfl_sync(0xFFFFFFFFu, inv_lane, (int)(uint32_t)(kbits >> (e * IB))) : inv_lane;
-        const uint64_t blk = RNG == 32 ? (uint64_t)((p.coord0 + i) >> 2) : (uint64_t)((p.coord0 + i) >> 3);
-        const char *gp = (const char *)p.v.g + (size_t)m0 * grow + (size_t)i * E::BYTES;
-        char *lp = (char *)p.lev + (size_t)m0 * lrow;
-#pragma unroll 1
-        for (int m = m0; m < m1; m += G) {
-            uint4 q[G][H];
-#pragma unroll
-            for (int k = 0; k < G; ++k)
-                if (m + k < m1) {
-#pragma unroll
-                    for (int h = 0; h < H; ++h) q[k][h] = ld_stream(gp + (size_t)k * grow + h * E::G * E::BYTES);
-                }
-#pragma unroll
-            for (int k = 0; k < G; ++k)
-                if (m + k < m1) {
-                    float v[8];
-#pragma unroll
-                    for (int h = 0; h < H; ++h) E::unpack(q[k][h], *(float(*)[E::G])(v + h * E::G));
-                    uint32_t neg_lo, neg_hi;
-                    unit_signs<DT>(q[k], neg_lo, neg_hi);
-                    quantize_unit<FMT, RNG>(v, inv, p.v.s_hat, neg_lo, neg_hi, p.key, (uint32_t)blk, (uint32_t)(blk >> 32),
-                                            (uint32_t)(m + k + p.worker0), lp + (size_t)k * lrow + LF::off(i),
-                                            lp + (size_t)k * lrow + LF::off2(i, p.v.stride));
-                }
-            gp += G * grow;
-            lp += G * lrow;
-        }
-    }
-    if (overflow && lane < p.v.scales.N && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
-}
-
-// Decode mode, slow forms: sum and reconstruction of the unit of 8 coordinates at i from the int8
-// levels that THIS thread stored for every worker just before (own stores are visible to own loads;
-// read around L1), with the segment and the shared index looked up per coordinate.
-template <int IDXB>
-__device__ __noinline__ void decode_unit_general(const EncodeParams &p, int64_t i, uint64_t kbits_own, bool own_idx)
-{
-    constexpr bool MULTI = IDXB != 0;
-    constexpr int IB = MULTI ? IDXB : 8;
-    if (i >= p.v.d) return;
+    if (overflow && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
+    const uint64_t blk = RNG == 32 ? (uint64_t)((p.coord0 + i) >> 2) : (uint64_t)((p.coord0 + i) >> 3);
     int S[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const char *lp = (const char *)p.lev + i;
-    for (int m = 0; m < p.v.M; ++m) {
-        const uint2 b = __ldcg((const uint2 *)(lp + (size_t)m * (size_t)p.v.stride));
+    constexpr int G = 4, H = 8 / E::G;                              // workers whose loads are in flight together
+    for (int m0 = 0; m0 < p.v.M; m0 += G) {
+        uint4 q[G][H];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            S[e] += (int)(int8_t)(b.x >> (8 * e));
-            S[4 + e] += (int)(int8_t)(b.y >> (8 * e));
+        for (int g = 0; g < G; ++g) {
+            const int m = min(m0 + g, p.v.M - 1);
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+                q[g][h] = ld_stream((const char *)p.v.g + ((size_t)m * (size_t)p.v.stride + i + h * E::G) * E::BYTES);
         }
-    }
-    uint64_t kbits = kbits_own;
-    if (MULTI && !own_idx)        // select mode: the CTA stored the tile's indices itself (behind a barrier)
-        kbits = (uint64_t)(p.select ? IdxBits<IB>::load_written(p.idx + i * IB / 8) : IdxBits<IB>::load(p.idx + i * IB / 8));
-    int j = find_segment(p.v.seg_off, p.v.nseg, i);
-    for (int e = 0; e < 8 && i + e < p.v.d; ++e) {
-        j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
-        const int k = MULTI ? (int)((kbits >> (e * IB)) & ((1u << IB) - 1u)) : 0;
-        p.out[i + e] = __fmul_rn((float)S[e], decode_factor(__ldg(p.v.W + j), p.v.scales.s[k & (UQ_MAX_SCALES - 1)], p.v.M));
-    }
-}
-
-// The units of tile [t0, t1) that this thread encoded in a slow form (the same assignment of units to
-// threads as encode_span_general and encode_tile_mixed).  mixed: a full tile crossed by boundaries; a
-// row that itself contains a boundary was skipped there and is skipped here (a CTA of the second
-// kind owns it), every other row lies in one segment, so lane k takes the factor of scale k once
-// per row.  Else (ragged tile and the like) everything is looked up per coordinate.
-template <int DT, int RNG, int IDXB>
-__device__ __noinline__ void decode_tile_slow(const EncodeParams &p, int64_t t0, int64_t t1, bool mixed)
-{
-    constexpr bool MULTI = IDXB != 0;
-    constexpr int IB = MULTI ? IDXB : 8;
-    constexpr int KMASK = IB < 4 ? (1 << IB) - 1 : UQ_MAX_SCALES - 1;
-    const int lane = threadIdx.x & 31;
-    for (int u = 0; u < EncodeShape<DT, RNG>::UNITS; ++u) {
-        const int64_t r0 = t0 + (int64_t)(u * kThreads + (threadIdx.x & ~31)) * 8;
-        if (r0 >= t1) break;                                         // warp-uniform
-        const int64_t i = r0 + lane * 8;
-        if (!mixed) {
-            if (i < t1) decode_unit_general<IDXB>(p, i, 0, false);
-            continue;
-        }
-        const int jr = warp_find_segment(p.v.seg_off, p.v.nseg, r0);
-        if (segment_end(p.v.seg_off, p.v.nseg, jr, p.v.d) < r0 + 256) continue;
-        const float c_lane = decode_factor(__ldg(p.v.W + jr), p.v.scales.s[lane & KMASK], p.v.M);
-        uint32_t sum[4] = {0u, 0u, 0u, 0u};                          // as in the straight-line path
-        const char *lp = (const char *)p.lev + i;
-        for (int m = 0; m < p.v.M; ++m) {
-            const uint2 b = __ldcg((const uint2 *)(lp + (size_t)m * (size_t)p.v.stride));
-            const uint32_t bl = b.x ^ 0x80808080u, bh = b.y ^ 0x80808080u;
-            sum[0] += __byte_perm(bl, 0u, 0x4240); sum[1] += __byte_perm(bl, 0u, 0x4341);
-            sum[2] += __byte_perm(bh, 0u, 0x4240); sum[3] += __byte_perm(bh, 0u, 0x4341);
-        }
-        typename IdxBits<IB>::T kbits = 0;
-        if (MULTI) kbits = p.select ? IdxBits<IB>::load_written(p.idx + i * IB / 8) : IdxBits<IB>::load(p.idx + i * IB / 8);
-        const int bias = 128 * p.v.M;
-        uint32_t r[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int S = (int)((sum[(e >> 2) * 2 + (e & 1)] >> (16 * ((e & 3) >> 1))) & 0xFFFFu) - bias;
-            const float c = MULTI ? __shfl_sync(0xFFFFFFFFu, c_lane, (int)(uint32_t)(kbits >> (e * IB))) : c_lane;
-            r[e] = __float_as_uint(__fmul_rn((float)S, c));
-        }
-        st_stream256(p.out + i, r);
-    }
-}
-
-// The slow forms of a whole tile, workers m0 .. m1 - 1: the ragged last tile, a tile whose Philox block
-// numbers leave the launch's high word, or 16-bit draws with a factor too small for the saturating
-// form (j < 0: per-coordinate lookup), and a full tile crossed by segment boundaries (j = its first
-// segment).  One out-of-line call keeps their registers out of the straight-line path.
-// In select mode the CTA first finds and stores the shared indices of the whole tile (thr: the
-// CTA's kWarps * 2 * UQ_MAX_SCALES words of shared memory); the encoding then reads them back.
-template <int DT, int FMT, int RNG, int IDXB>
-__device__ __noinline__ void encode_tile_slow(const EncodeParams &p, int64_t t0, int64_t t1, int j, int m0, int m1,
-                                              int32_t *thr)
-{
-    if (IDXB != 0 && p.select) {
-        constexpr int IB = IDXB != 0 ? IDXB : 8;
-        const int lane = threadIdx.x & 31;
-        for (int u = 0; u < EncodeShape<DT, RNG>::UNITS; ++u) {
-            const int64_t i = t0 + (int64_t)(u * kThreads + threadIdx.x) * 8;
-            const int64_t row0 = i - lane * 8;
-            if (row0 >= t1) break;                                   // warp-uniform
-            const uint64_t packed = select_unit<DT, IB, 4>(p.v, i, row0, thr + (threadIdx.x >> 5) * 2 * UQ_MAX_SCALES);
-            if (i < p.v.d) store_unit_indices<IB>(p.idx, i, packed);
-        }
-        __syncthreads();                                             // the tile's indices are in memory for all warps
-    }
-    if (j >= 0) {
-        encode_tile_mixed<DT, FMT, RNG, IDXB>(p, m0, m1, t0, j);
-        return;
-    }
-    for (int m = m0; m < m1; ++m) encode_span_general<DT, FMT, RNG, IDXB>(p, m, t0, t1, threadIdx.x, kThreads);
-}
-
-// State of a tile that does not depend on the worker.
-template <int DT, int FMT, int RNG, int IDXB, bool DEC = false> struct TileState {
-    using E = Elem<DT>;
-    using S = EncodeShape<DT, RNG>;
-    static constexpr int U = S::UNITS;
-    static constexpr int H = 8 / E::G;                           // 16-byte loads per unit
-    static constexpr int BPU = RNG == 32 ? 2 : 1;                // Philox blocks per unit
-    float inv[U][8];                  // factor of every coordinate: / 256 for 16-bit draws, * 2^23 for 32-bit draws
-    PhiloxBlockPart blk[U * BPU];     // worker-independent rounds of the units' Philox blocks
-    SatConstants sc;                  // 16-bit draws
-    float cap23;                      // 32-bit draws: the largest level * 2^23
-    uint32_t sum[DEC ? U : 1][4];     // decode mode: the unit's level sums, every level biased by 128, in 16-bit
-                                      // lanes: bytes 0, 2 and bytes 1, 3 of the low word, then of the high word
-    const char *gp;                   // my first coordinate in the gradient row that is loaded next
-    const uint4 *sp;                  // select mode: my slot of that row's copy in shared memory
-    char *lp, *lp2;                   // and in the level row that is stored next (second plane for 6-bit)
-    size_t grow, lrow;                // bytes between rows
-};
-
-template <bool SEL, int DT, int FMT, int RNG, int IDXB, bool DEC>
-__device__ __forceinline__ void load_units(TileState<DT, FMT, RNG, IDXB, DEC> &t,
-                                           uint4 (&q)[EncodeShape<DT, RNG>::UNITS][8 / Elem<DT>::G])
-{
-    using T = TileState<DT, FMT, RNG, IDXB, DEC>;
-#pragma unroll
-    for (int u = 0; u < T::U; ++u)
-#pragma unroll
-        for (int h = 0; h < T::H; ++h)
-            q[u][h] = SEL ? t.sp[(u * T::H + h) * kThreads] : ld_stream(t.gp + (u * kThreads * 8 + h * T::E::G) * T::E::BYTES);
-    if (SEL) t.sp += T::U * T::H * kThreads;
-    else t.gp += t.grow;
-}
-
-// Workers m0 .. m0 + G - 1 of the tile, straight-line.  On entry q holds worker m0's units (loaded
-// or in flight); while worker m is quantized the units of worker m + 1 are on their way (MORE: also
-// those of the worker after the last one of this call).
-template <int G, bool MORE, bool SEL, int DT, int FMT, int RNG, int IDXB, bool DEC>
-__device__ __forceinline__ void encode_workers(const EncodeParams &p, TileState<DT, FMT, RNG, IDXB, DEC> &t, int m0,
-                                               uint4 (&q)[EncodeShape<DT, RNG>::UNITS][8 / Elem<DT>::G])
-{
-    using T = TileState<DT, FMT, RNG, IDXB, DEC>;
-    using LF = LevelFmt<FMT>;
-    constexpr int UB = LF::UB;                                   // bytes of levels per unit: 8, 4 or 2
-    constexpr int UB2 = FMT == UQ_FMT_I6P ? 2 : 0;               // and in the second plane of the 6-bit format
-#pragma unroll
-    for (int k = 0; k < G; ++k) {
-        const int m = m0 + k;
-        uint4 qn[T::U][T::H];
-        if (k + 1 < G || MORE) load_units<SEL>(t, qn);
-        uint4 r[T::U * T::BPU];
-        philox_join<T::U * T::BPU>(p.key, t.blk, p.wpart[m], r);
-#pragma unroll
-        for (int u = 0; u < T::U; ++u) {
+        for (int g = 0; g < G; ++g) {
+            const int m = m0 + g;
+            if (m >= p.v.M) break;
             float v[8];
 #pragma unroll
-            for (int h = 0; h < T::H; ++h) T::E::unpack(q[u][h], *(float(*)[T::E::G])(v + h * T::E::G));
-            // binary32 to 4 bits: the unit's bytes in even / odd order, which the store merges directly
-            constexpr bool EO = FMT == UQ_FMT_I4X2 && DT == UQ_F32;
+            for (int h = 0; h < H; ++h) E::unpack(q[g][h], *(float(*)[E::G])(v + h * E::G));
             uint32_t neg_lo, neg_hi, lo, hi;
-            unit_signs<DT, EO>(q[u], neg_lo, neg_hi);
-            if (RNG == 16) {
-                quantize_unit_bytes_sat16<EO>(v, t.inv[u], t.sc, neg_lo, neg_hi, r[u], lo, hi);
-            } else {
-                UnitWords<32> rw;
-                rw.r[0] = r[u * T::BPU]; rw.r[1] = r[u * T::BPU + T::BPU - 1];
-                quantize_unit_bytes_fixed23<EO>(v, t.inv[u], t.cap23, neg_lo, neg_hi, rw, lo, hi);
-            }
-            if (EO) store_unit_even_odd(lo, hi, t.lp + u * kThreads * UB);
-            else store_unit<FMT>(lo, hi, t.lp + u * kThreads * UB, t.lp2 + u * kThreads * UB2);
-            if (DEC) {
-                // the sum over the workers: the bytes biased to 1 .. 255, bytes 0, 2 and bytes 1, 3 of a
-                // word spread over the 16-bit lanes of a word each (8 * 255 fits a lane)
-                const uint32_t bl = lo ^ 0x80808080u, bh = hi ^ 0x80808080u;
-                t.sum[u][0] += __byte_perm(bl, 0u, 0x4240); t.sum[u][1] += __byte_perm(bl, 0u, 0x4341);
-                t.sum[u][2] += __byte_perm(bh, 0u, 0x4240); t.sum[u][3] += __byte_perm(bh, 0u, 0x4341);
-            }
-        }
-        t.lp += t.lrow;
-        if (FMT == UQ_FMT_I6P) t.lp2 += t.lrow;
-        if (k + 1 < G || MORE) {
+            unit_signs<DT>(q[g], neg_lo, neg_hi);       // the sign of a padding coordinate is harmless: its level is 0
 #pragma unroll
-            for (int u = 0; u < T::U; ++u)
+            for (int e = 0; e < 8; ++e)
+                if (i + e >= d) v[e] = 0.0f;
+            quantize_unit_bytes<RNG>(v, inv, p.v.s_hat, neg_lo, neg_hi,
+                                     unit_words<RNG>(p.key, (uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)(m + p.worker0)), lo, hi);
+            char *lrow = (char *)p.lev + (size_t)m * LF::row_bytes(p.v.stride);
+            store_unit<FMT>(lo, hi, lrow + LF::off(i), lrow + LF::off2(i, p.v.stride));
 #pragma unroll
-                for (int h = 0; h < T::H; ++h) q[u][h] = qn[u][h];
+            for (int e = 0; e < 8; ++e) S[e] += (int)(int8_t)((e < 4 ? lo : hi) >> (8 * (e & 3)));
         }
+    }
+    if (p.out == nullptr) return;
+    for (int e = 0; e < 8 && i + e < d; ++e) {
+        p.out[i + e] = __fmul_rn((float)S[e], c[e]);
+        if (p.S != nullptr) p.S[i + e] = S[e];
     }
 }
 
-// Select mode: copies of the tile's rows of workers m0 .. m0 + cnt - 1 into shared memory, laid out
-// [worker][unit][16 bytes][thread] so that every thread reads back only what it copied (no barrier).
-// CNT > 0: cnt is that compile-time value (no predicates); CNT == 0: cnt at run time.
-template <int CNT, int DT, int RNG>
-__device__ __forceinline__ void stage_rows(uint4 *stage, const char *gp, size_t grow, int cnt)
+// The factors of the four coordinates at i in a full row that segment boundaries cross: s_k / W for the
+// quantization (dec = false) or W / (s_k * M) for the reconstruction.  j: a segment at or before i's.
+static __device__ __noinline__ float4 mixed_row_factors(const EncodeParams &p, int64_t i, int j, uint32_t kw, bool dec)
+{
+    const uint32_t mask = p.idx_bits == 0 ? 0u : ((1u << p.idx_bits) - 1u) & (UQ_MAX_SCALES - 1);
+    bool overflow = false;
+    float f[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
+        const float W = __ldg(p.v.W + j);
+        const int32_t s = p.v.scales.s[(kw >> (e * p.idx_bits)) & mask];
+        f[e] = dec ? decode_factor(W, s, p.v.M) : inv_scale(s, W);
+        overflow |= !dec && not_finite(f[e]);
+    }
+    if (overflow && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
+    return make_float4(f[0], f[1], f[2], f[3]);
+}
+
+// The shared indices of four coordinates of such a row, from the largest magnitudes over the workers.
+static __device__ __noinline__ uint32_t mixed_row_select(const EncodeParams &p, int64_t i, int j, uint32_t a0, uint32_t a1,
+                                                         uint32_t a2, uint32_t a3)
+{
+    const uint32_t amag[4] = {a0, a1, a2, a3};
+    uint32_t packed = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
+        const float W = __ldg(p.v.W + j), a = __uint_as_float(amag[e]);
+        int k = 0;
+        for (int kk = 1; kk < p.v.scales.N; ++kk)
+            if (__fmul_rn(a, inv_scale(p.v.scales.s[kk], W)) <= p.v.s_hat) k = kk;
+        packed |= (uint32_t)k << (e * p.idx_bits);
+    }
+    return packed;
+}
+
+// ---------------------------------------------------------------------------------------------
+// the straight-line path
+// ---------------------------------------------------------------------------------------------
+
+// The order in which a unit's levels sit in the bytes of its two level words: byte `b` of word `w` is
+// coordinate coord(w, b).  Natural order, except for binary32 gradients and 4-bit levels, where the even
+// coordinates in one word and the odd ones in the other let the nibbles merge with one shift.
+template <int DT, int FMT> struct LevelOrder {
+    static constexpr bool EO = DT == UQ_F32 && FMT == UQ_FMT_I4X2;
+    static __host__ __device__ constexpr int coord(int w, int b) { return EO ? 2 * b + w : 4 * w + b; }
+};
+
+// Constants of the fast level arithmetic.
+struct LevelConstants {
+    float c0;                 // 16-bit draws: 1 - cap / 256
+    uint32_t k_pos, k_neg;    // 16-bit draws: bias of the level bytes, and 128 + it, in every byte
+    float cap23;              // 32-bit draws: cap * 2^23
+};
+
+// One worker's unit (q) turned into signed level bytes: w[k] holds four levels (see LevelOrder).
+// 16-bit draws: the random words come complemented; with h' = 2^16 - 1 - h the carry out of
+// rint(p * 2^16) + h' is the rounding decision, and one dp2a picks the half word and adds it.
+template <int DT, int FMT, int RNG>
+__device__ __forceinline__ void quantize_fast(const uint4 *q, const float (&inv)[8], const LevelConstants &lc, const uint4 *r,
+                                              uint32_t (&w)[2])
 {
     using E = Elem<DT>;
-    constexpr int U = EncodeShape<DT, RNG>::UNITS, H = 8 / E::G;
-    const int tid = threadIdx.x;
+    using O = LevelOrder<DT, FMT>;
+    float v[8];
 #pragma unroll
-    for (int m = 0; m < kWorkerGroup; ++m) {
-        if (CNT > 0 ? m < CNT : m < cnt) {
+    for (int h = 0; h < 8 / E::G; ++h) E::unpack(q[h], *(float(*)[E::G])(v + h * E::G));
+    uint32_t z[8];
 #pragma unroll
-            for (int u = 0; u < U; ++u)
+    for (int e = 0; e < 8; ++e) {
+        if (RNG == 16) {
+            const uint4 x = r[0];
+            const uint32_t word = (e >> 1) == 0 ? x.x : (e >> 1) == 1 ? x.y : (e >> 1) == 2 ? x.z : x.w;
+            z[e] = __dp2a_lo(word, (e & 1) ? 0x100u : 0x1u, __float_as_uint(add_sat(mul_sat(fabsf(v[e]), inv[e]), lc.c0)));
+        } else {
+            const uint4 x = r[e >> 2];
+            const uint32_t word = (e & 3) == 0 ? x.x : (e & 3) == 1 ? x.y : (e & 3) == 2 ? x.z : x.w;
+            z[e] = level_draw23_fixed(v[e], inv[e], lc.cap23, word);
+        }
+    }
 #pragma unroll
-                for (int h = 0; h < H; ++h)
-                    copy_async16(stage + ((m * U + u) * H + h) * kThreads + tid, gp + (u * kThreads * 8 + h * E::G) * E::BYTES);
-            gp += grow;
+    for (int k = 0; k < 2; ++k) {
+        const int a = O::coord(k, 0), b = O::coord(k, 1), c = O::coord(k, 2), d = O::coord(k, 3);
+        uint32_t neg;
+        if (DT == UQ_F32) neg = sign_bytes_f32(v[a], v[b], v[c], v[d]);
+        else neg = k == 0 ? sign_bytes_bf16(q[0].x, q[0].y) : sign_bytes_bf16(q[0].z, q[0].w);
+        if (RNG == 16) {
+            // byte B = L + bias (bias = 128 - cap): L = B - bias, and 128 - L = (128 + bias) - B, neither of
+            // which borrows from the next byte; flipping its top bit makes the latter -L
+            const uint32_t B = gather_bytes<2>(z[a], z[b], z[c], z[d]);
+            const uint32_t plus = B - lc.k_pos, minus = lc.k_neg - B;
+            w[k] = ((plus & ~neg) | (minus & neg)) ^ (neg & 0x80808080u);
+        } else {
+            w[k] = negated_bytes_to_signed(gather_bytes<kLevelByte23Fixed>(z[a], z[b], z[c], z[d]), neg);
         }
     }
 }
 
-// Select mode: the largest magnitude over the staged workers of the 8 coordinates of unit u, as
-// binary32 bit patterns.  bf16: two coordinates per word.  Its sign-magnitude halves read as
-// signed 16-bit integers order the positive values, read as unsigned ones the negative values
-// (sign bit set) above all others, so max |x| = max(smax & 0x7FFF, umax & 0x7FFF): two packed
-// three-input maxima per two workers and word, no mask per element.  binary32: three-input
-// maxima of absolute values, as the selector's kernel takes them (a NaN is skipped).
-template <int CNT, int DT, int RNG>
-__device__ __forceinline__ void staged_max_magnitude(const uint4 *stage, int u, int cnt, uint32_t (&amag)[8])
+// SEL without staging: a row's first read asks the caches to keep the line for the second one, which lets it
+// go (binary32, 8 workers, 4 scales, 25.6 M coordinates: 285 us with the hints on L1 and L2, 290 us without,
+// as a burst; 295 and 320 us sustained).
+__device__ __forceinline__ uint64_t policy_keep()
 {
-    using E = Elem<DT>;
-    constexpr int U = EncodeShape<DT, RNG>::UNITS, H = 8 / E::G;
-    const int tid = threadIdx.x;
-    if (DT == UQ_F32) {
-        float a[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int m = 0; m < kWorkerGroup; ++m) {
-            if (CNT > 0 ? m < CNT : m < cnt) {
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const uint4 x = stage[((m * U + u) * H + h) * kThreads + tid];
-                    a[4 * h + 0] = fmaxf(a[4 * h + 0], fabsf(__uint_as_float(x.x)));
-                    a[4 * h + 1] = fmaxf(a[4 * h + 1], fabsf(__uint_as_float(x.y)));
-                    a[4 * h + 2] = fmaxf(a[4 * h + 2], fabsf(__uint_as_float(x.z)));
-                    a[4 * h + 3] = fmaxf(a[4 * h + 3], fabsf(__uint_as_float(x.w)));
-                }
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) amag[e] = __float_as_uint(a[e]);
-    } else {
-        uint32_t smax[4] = {0x80008000u, 0x80008000u, 0x80008000u, 0x80008000u}, umax[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int m = 0; m < kWorkerGroup; ++m) {
-            if (CNT > 0 ? m < CNT : m < cnt) {
-                const uint4 x = stage[(m * U + u) * kThreads + tid];
-                const uint32_t w4[4] = { x.x, x.y, x.z, x.w };
-#pragma unroll
-                for (int c = 0; c < 4; ++c) { smax[c] = __vmaxs2(smax[c], w4[c]); umax[c] = __vmaxu2(umax[c], w4[c]); }
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint32_t am = __vmaxu2(smax[c] & 0x7FFF7FFFu, umax[c] & 0x7FFF7FFFu);
-            amag[2 * c] = am << 16; amag[2 * c + 1] = am & 0xFFFF0000u;
-        }
-    }
+    uint64_t p;
+    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint64_t policy_drop()
+{
+    uint64_t p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint4 ld_keep(const void *p, uint64_t policy)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L1::evict_last.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_drop(const void *p, uint64_t policy)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
+    return v;
 }
 
-// SEL: the kernel also finds and stores the shared scale indices (multi-scale, all M <= kWorkerGroup
-// workers in one CTA): the tile's rows are copied to shared memory once (every thread its own
-// units, so no barrier), read there for the maximum over the workers and again for quantization.
-// DEC: decode mode (see the head of this file; int8 levels, 16-bit draws, one CTA per tile; with or without SEL).
-template <int DT, int FMT, int RNG, int IDXB, bool SEL, bool DEC>
-__global__ void __launch_bounds__(kThreads, (SEL ? 3 : DEC ? EncodeShape<DT, RNG>::MIN_CTAS_DEC : EncodeShape<DT, RNG>::MIN_CTAS))
+// 16 bytes from global memory straight into shared memory.
+__device__ __forceinline__ void copy_async16(uint32_t smem_dst, const void *gmem_src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_dst), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared16(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+
+// WK: 8 = exactly that many workers (known at compile time), 0 = any number.
+template <int DT, int FMT, int RNG, bool MULTI, bool SEL, bool DEC, int WK>
+__global__ void __launch_bounds__(kThreads, (EncodeShape<DT, RNG, SEL>::CTAS))
 encode_kernel(const __grid_constant__ EncodeParams p)
 {
-    static_assert(!DEC || (FMT == UQ_FMT_I8 && RNG == 16), "decode mode: int8 levels, 16-bit draws");
     grid_dependency_prologue();
-    using T = TileState<DT, FMT, RNG, IDXB, DEC>;
     using E = Elem<DT>;
-    using S = EncodeShape<DT, RNG>;
+    using S = EncodeShape<DT, RNG, SEL>;
     using LF = LevelFmt<FMT>;
-    constexpr bool MULTI = IDXB != 0;
-    constexpr int IB = MULTI ? IDXB : 8;
-    constexpr int U = T::U, H = T::H, BPU = T::BPU;
-    const int tid = threadIdx.x, lane = tid & 31;
-    __shared__ int32_t sh_thr[MULTI ? kWarps * 2 * UQ_MAX_SCALES : 1];   // select mode, slow paths: threshold tables
-    const uint32_t first_tile_block = DEC ? p.row_blocks : 0u;
-    if (DEC ? blockIdx.x < p.row_blocks : blockIdx.x >= p.main_blocks) {
-        // A CTA of the second kind: each warp takes one segment boundary of one worker and, if the
-        // boundary lies strictly inside a 256-coordinate row of a full tile, quantizes that row with
-        // per-coordinate scales (the tile's own CTA skips it).  Keeping these rows out of the tile
-        // CTAs keeps their lifetime short: the slow path no longer holds a whole CTA slot.
-        // (decode mode: one warp takes the row of every worker, one after the other, and then decodes it)
-        const uint32_t x = DEC ? blockIdx.x : blockIdx.x - p.main_blocks;
-        const int m = DEC ? 0 : (int)(x % (uint32_t)p.v.M);
-        const int64_t k = 1 + (int64_t)(DEC ? x : x / (uint32_t)p.v.M) * kWarps + (tid >> 5);
-        if (k >= p.v.nseg) return;
-        const int64_t b = __ldg(p.v.seg_off + k), prev = __ldg(p.v.seg_off + k - 1);
-        const int64_t r0 = b & ~(int64_t)255;
-        const int64_t full_end = p.v.d / S::TILE * S::TILE;          // rows beyond belong to the ragged tile's CTA
-        if (b <= 0 || b == r0 || r0 >= full_end) return;           // not strictly inside a row of a full tile
-        if (prev > r0 && prev <= b) return;                        // an earlier boundary in the same row takes it
-        if (DEC) {
-            // (select mode: the tile's own CTA stores the row's shared indices; this warp finds them for itself)
-            const bool own = MULTI && p.select;
-            int32_t *thr = sh_thr + (MULTI ? (tid >> 5) * 2 * UQ_MAX_SCALES : 0);
-            for (int mm = 0; mm < p.v.M; ++mm) encode_span_general<DT, FMT, RNG, IDXB>(p, mm, r0, r0 + 256, lane, 32, own, thr);
-            uint64_t kbits = 0;
-            if (own) kbits = (uint64_t)select_unit<DT, IB, 4>(p.v, r0 + lane * 8, r0, thr);
-            decode_unit_general<IDXB>(p, r0 + lane * 8, kbits, own);
+    using O = LevelOrder<DT, FMT>;
+    constexpr int V = S::V, NB = S::NB, G = S::G, BSH = RNG == 32 ? 2 : 3;
+    constexpr bool STAGED = SEL && DT == UQ_BF16 && WK == 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, M = WK ? WK : p.v.M, ib = p.idx_bits;
+    const int64_t d = p.v.d;
+    // CTAs walk the tiles back to front: the kernel before this one in a step (the norms) ends on the
+    // high tiles, so part of what is read first is still in L2
+    const int64_t t0 = (int64_t)(gridDim.x - 1 - blockIdx.x) * S::TILE;
+    const int64_t r0 = t0 + warp * 256, i = r0 + lane * 8;                            // my warp's row, my coordinates
+    const uint64_t blk0 = (uint64_t)(p.coord0 + r0) >> BSH;
+    if (r0 >= d) return;
+    bool slow = r0 + 256 > d || (uint32_t)(blk0 >> 32) != p.blk_hi || (uint32_t)blk0 > 0xFFFFFFFFu - (256u >> BSH);
+    const size_t grow = (size_t)p.v.stride * E::BYTES, lrow = LF::row_bytes(p.v.stride);
+    const char *gp = (const char *)p.v.g + (size_t)i * E::BYTES;
+    extern __shared__ uint4 stage[];                             // STAGED: [worker][thread]
+    const uint32_t sp = (uint32_t)__cvta_generic_to_shared(stage) + threadIdx.x * 16;
+    uint64_t policy = 0;
+    uint4 q[G][V];
+    uint32_t kw[2] = {0u, 0u};
+    auto load = [&](int m, uint4 (&x)[V]) {                      // worker m's bytes (called for m = 0, 1, 2, ...)
+        if (STAGED) {
+            x[0] = ld_shared16(sp + m * (kThreads * 16));
             return;
         }
-        encode_span_general<DT, FMT, RNG, IDXB>(p, m, r0, r0 + 256, lane, 32, MULTI && p.select,
-                                                sh_thr + (MULTI ? (tid >> 5) * 2 * UQ_MAX_SCALES : 0));
-        return;
-    }
-    // CTAs walk the tiles back to front (see launch_encode); a tile's CTAs take 8 workers each
-    const uint32_t rev = p.main_blocks - 1u - (blockIdx.x - first_tile_block);
-    const int64_t tile = (int64_t)(rev / p.groups);
-    const int m0 = (int)(rev % p.groups) * kWorkerGroup;
-    const int cnt = min(kWorkerGroup, p.v.M - m0);
-    const int64_t t0 = tile * S::TILE;
-    const int64_t t1 = min(t0 + (int64_t)S::TILE, p.v.d);
-
-    // Philox block of the tile's first unit.  The units of a tile add less than 2^12 to it; the
-    // straight-line path keeps the high word fixed (the per-worker table of the launch was made for
-    // one high word), so a tile in which the low word wraps or whose high word is another one
-    // (one launch in 2^35 coordinates) takes the general path like the ragged last tile.
-    constexpr int BSH = RNG == 32 ? 2 : 3;                       // coordinates per Philox block, log2
-    const uint64_t blk0 = (uint64_t)(p.coord0 >> BSH) + (uint64_t)tile * (uint32_t)(S::TILE >> BSH);
-    const bool other_hi = (uint32_t)blk0 > 0xFFFFFFFFu - (uint32_t)(S::TILE >> BSH) || (uint32_t)(blk0 >> 32) != p.blk_hi;
-    if (t1 - t0 != S::TILE || other_hi) {
-        encode_tile_slow<DT, FMT, RNG, IDXB>(p, t0, t1, -1, m0, m0 + cnt, sh_thr);
-        if (DEC) decode_tile_slow<DT, RNG, IDXB>(p, t0, t1, false);
-        return;
-    }
-    // every warp looks the segment up for itself (no shared memory, no barrier)
-    const int j = warp_find_segment(p.v.seg_off, p.v.nseg, t0);
-    if (segment_end(p.v.seg_off, p.v.nseg, j, p.v.d) < t1) {
-        // A segment boundary crosses the tile (at most nseg - 1 tiles): a compact loop over the
-        // rows of every worker, kept out of line so that its registers do not weigh on the path below.
-        encode_tile_slow<DT, FMT, RNG, IDXB>(p, t0, t1, j, m0, m0 + cnt, sh_thr);
-        if (DEC) decode_tile_slow<DT, RNG, IDXB>(p, t0, t1, true);
-        return;
-    }
-    T t;
-    t.grow = (size_t)p.v.stride * E::BYTES;
-    t.lrow = LF::row_bytes(p.v.stride);
-    t.gp = (const char *)p.v.g + (size_t)m0 * t.grow + ((size_t)t0 + (size_t)tid * 8) * E::BYTES;
-    uint4 q[U][H];
-    typename IdxBits<IB>::T kbits[U];
-    extern __shared__ uint4 stage[];                             // SEL: [worker][unit][16 bytes][thread]
-    if (SEL) {
-        t.sp = stage + tid;
-        if (cnt == kWorkerGroup) stage_rows<kWorkerGroup, DT, RNG>(stage, t.gp, t.grow, cnt);
-        else stage_rows<0, DT, RNG>(stage, t.gp, t.grow, cnt);
-    } else {
-        // the first worker's row and the shared indices are on their way during the set-up below
-        load_units<false>(t, q);
-        if (MULTI) {
-            const uint8_t *ip = p.idx + ((size_t)t0 + (size_t)tid * 8) * IB / 8;
 #pragma unroll
-            for (int u = 0; u < U; ++u) kbits[u] = IdxBits<IB>::load(ip + u * kThreads * IB);
+        for (int h = 0; h < V; ++h) x[h] = SEL ? ld_drop(gp + h * 16, policy) : ld_stream(gp + h * 16);
+        gp += grow;
+    };
+    if (!slow) {
+        // the first rows and the shared indices are on their way during the set-up below
+        if (STAGED) {
+            // every thread copies what it reads back itself
+            const char *gs = gp;
+#pragma unroll
+            for (int m = 0; m < kGroup; ++m, gs += grow) copy_async16(sp + m * (kThreads * 16), gs);
+        } else if (!SEL) {
+#pragma unroll
+            for (int c = 0; c < G; ++c)
+                if (WK || c < M) load(c, q[c]);
+            if (MULTI) load_indices<8>(p.idx, i, ib, kw);
         }
     }
-    // lane k holds s_k / W_j (single-scale: every lane holds s / W_j)
-    constexpr int KMASK = IB < 4 ? (1 << IB) - 1 : UQ_MAX_SCALES - 1;    // lane L holds scale L & KMASK
+    const int j = warp_find_segment(p.v.seg_off, p.v.nseg, r0);
+    const bool mixed = segment_end(p.v.seg_off, p.v.nseg, j, d) < r0 + 256;          // a boundary inside my row
+    const int kmask = !MULTI ? 0 : ib < 4 ? (1 << ib) - 1 : UQ_MAX_SCALES - 1;      // lane L holds scale L & kmask
     const float W = __ldg(p.v.W + j);
-    float inv_lane = inv_scale(p.v.scales.s[lane & KMASK], W);
-    if (lane < p.v.scales.N && not_finite(inv_lane) && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
-    // a W so large (16-bit draws) or so small (32-bit) that the rescaled factors of the fast forms
-    // would leave the normal range: the plain arithmetic
-    if (RNG == 16 ? !sat_form_exact(inv_scale(p.v.scales.s[0], W))
-                  : !fixed_form_exact(inv_scale(p.v.scales.s[p.v.scales.N - 1], W))) {
-        if (SEL) copy_async_wait();
-        encode_tile_slow<DT, FMT, RNG, IDXB>(p, t0, t1, -1, m0, m0 + cnt, sh_thr);
-        if (DEC) decode_tile_slow<DT, RNG, IDXB>(p, t0, t1, false);
-        return;
+    float inv_lane = inv_scale(p.v.scales.s[lane & kmask], W);
+    if (!mixed && !slow) {
+        if (lane < p.v.scales.N && not_finite(inv_lane) && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
+        // a W so large (16-bit draws) or so small (32-bit) that the rescaled factors of the fast forms would leave
+        // the normal range: the plain arithmetic
+        const float edge = MULTI ? __shfl_sync(0xFFFFFFFFu, inv_lane, RNG == 16 ? 0 : p.v.scales.N - 1) : inv_lane;
+        slow = RNG == 16 ? !sat_form_exact(edge) : !fixed_form_exact(edge);
     }
-    if (SEL) {
-        // Scale selection and sharing for the tile (Algorithm 2 lines "Compute coordinate scales" and
-        // "Scale sharing"): the largest magnitude over the workers decides the shared index (see
-        // uq_select.cuh), found by bisection over the pass thresholds that lanes 0 .. N-1 hold.
-        const int N = p.v.scales.N;
-        const int32_t thr = lane < N ? pass_threshold(inv_lane, p.v.s_hat) : -1;
-        const int top = N > 1 ? 1 << (31 - __clz(N - 1)) : 0;               // first step of the bisection
+    if (SEL && !slow) {
+        // Scale selection and sharing (Algorithm 2 lines "Compute coordinate scales" and "Scale sharing"): the
+        // largest magnitude over the workers decides the shared index (see uq_select.cuh), found by bisection
+        // over the pass thresholds that lanes 0 .. N-1 hold.
+        const int top = p.v.scales.N > 1 ? 1 << (31 - __clz(p.v.scales.N - 1)) : 0;   // first step of the bisection
+        const int32_t thr = lane < p.v.scales.N ? pass_threshold(inv_lane, p.v.s_hat) : -1;
         const int32_t thr_top = __shfl_sync(0xFFFFFFFFu, thr, top);
-        copy_async_wait();
+        if (STAGED) asm volatile("cp.async.wait_all;" ::: "memory");
+        else policy = policy_keep();
+        uint32_t amag[8];
+        const char *gs = gp;
+        if (DT == UQ_F32) {
+            float a[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            auto four = [&](int left) {                               // four workers' loads in flight
+                uint4 x[4][V];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            uint32_t amag[8];
-            if (cnt == kWorkerGroup) staged_max_magnitude<kWorkerGroup, DT, RNG>(stage, u, cnt, amag);
-            else staged_max_magnitude<0, DT, RNG>(stage, u, cnt, amag);
+                for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                    for (int h = 0; h < V; ++h) x[k][h] = WK || k < left ? ld_keep(gs + h * 16, policy) : make_uint4(0u, 0u, 0u, 0u);
+                    gs += grow;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int h = 0; h < V; ++h) {
+                        a[4 * h + 0] = fmaxf(a[4 * h + 0], fabsf(__uint_as_float(x[k][h].x)));
+                        a[4 * h + 1] = fmaxf(a[4 * h + 1], fabsf(__uint_as_float(x[k][h].y)));
+                        a[4 * h + 2] = fmaxf(a[4 * h + 2], fabsf(__uint_as_float(x[k][h].z)));
+                        a[4 * h + 3] = fmaxf(a[4 * h + 3], fabsf(__uint_as_float(x[k][h].w)));
+                    }
+            };
+            if (WK) { four(4); four(4); }
+            else {
+#pragma unroll 1
+                for (int m = 0; m < M; m += 4) four(M - m);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) amag[e] = __float_as_uint(a[e]);
+        } else {
+            // bf16 halves read as signed 16-bit integers order the positive values, as unsigned ones the
+            // negative values above all others: max |x| = max(smax & 0x7FFF, umax & 0x7FFF)
+            uint32_t smax[4] = {0u, 0u, 0u, 0u}, umax[4] = {0u, 0u, 0u, 0u};
+            auto eight = [&](int left) {                              // eight workers' loads in flight
+                uint4 x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    x[k] = STAGED ? ld_shared16(sp + k * (kThreads * 16)) : WK || k < left ? ld_keep(gs, policy) : make_uint4(0u, 0u, 0u, 0u);
+                    gs += grow;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; k += 2) {
+                    smax[0] = __vimax3_s16x2(smax[0], x[k].x, x[k + 1].x); umax[0] = __vimax3_u16x2(umax[0], x[k].x, x[k + 1].x);
+                    smax[1] = __vimax3_s16x2(smax[1], x[k].y, x[k + 1].y); umax[1] = __vimax3_u16x2(umax[1], x[k].y, x[k + 1].y);
+                    smax[2] = __vimax3_s16x2(smax[2], x[k].z, x[k + 1].z); umax[2] = __vimax3_u16x2(umax[2], x[k].z, x[k + 1].z);
+                    smax[3] = __vimax3_s16x2(smax[3], x[k].w, x[k + 1].w); umax[3] = __vimax3_u16x2(umax[3], x[k].w, x[k + 1].w);
+                }
+            };
+            if (WK) eight(8);
+            else {
+#pragma unroll 1
+                for (int m = 0; m < M; m += 8) eight(M - m);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t am = __vmaxu2(smax[c] & 0x7FFF7FFFu, umax[c] & 0x7FFF7FFFu);
+                amag[2 * c] = am << 16; amag[2 * c + 1] = am & 0xFFFF0000u;
+            }
+        }
+        if (!mixed) {
             int k[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) k[e] = (top != 0 && (int32_t)amag[e] <= thr_top) ? top : 0;   // the first step
+            for (int e = 0; e < 8; ++e) k[e] = (top != 0 && (int32_t)amag[e] <= thr_top) ? top : 0;
 #pragma unroll 1
             for (int step = top >> 1; step >= 1; step >>= 1) {
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
                     if ((int32_t)amag[e] <= __shfl_sync(0xFFFFFFFFu, thr, k[e] + step)) k[e] += step;
             }
-            typename IdxBits<IB>::T packed = 0;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) packed |= (typename IdxBits<IB>::T)k[e] << (e * IB);
-            kbits[u] = packed;
-            store_unit_indices<IB>(p.idx, t0 + (int64_t)(u * kThreads + tid) * 8, packed);
+            for (int e = 0; e < 8; ++e) kw[e >> 2] |= (uint32_t)k[e] << ((e & 3) * ib);
+        } else {
+            kw[0] = mixed_row_select(p, i, j, amag[0], amag[1], amag[2], amag[3]);
+            kw[1] = mixed_row_select(p, i + 4, j, amag[4], amag[5], amag[6], amag[7]);
+            __syncwarp();
         }
-        load_units<true>(t, q);
-    }
-    if (RNG == 16) {
-        inv_lane = __fmul_rn(inv_lane, 0.00390625f);
-        t.sc = sat_constants(p.v.s_hat);
-    } else {
-        inv_lane = __fmul_rn(inv_lane, 8388608.0f);
-        t.cap23 = __fmul_rn(p.v.s_hat, 8388608.0f);
-    }
-    // the shuffle reads its source lane modulo 32 and the table repeats every 2^IB lanes (an 8-bit
-    // index is below 16), so the index bits need a shift but no mask
+        store_indices<8>(p.idx, i, ib, kw);
+        if (!STAGED) policy = policy_drop();
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+        for (int c = 0; c < G; ++c)
+            if (WK || c < M) load(c, q[c]);
+    }
+
+    // the factors of my coordinates.  The shuffle reads its source lane modulo 32 and the table repeats every
+    // 2^ib lanes: the index needs no mask
+    float inv[8];
+    if (!mixed) {
+        inv_lane = __fmul_rn(inv_lane, RNG == 16 ? 0.00390625f : 8388608.0f);
 #pragma unroll
         for (int e = 0; e < 8; ++e)
-            t.inv[u][e] = MULTI ? __shfl_sync(0xFFFFFFFFu, inv_lane, (int)(uint32_t)(kbits[u] >> (e * IB))) : inv_lane;
-    const uint32_t blk_lo = (uint32_t)blk0 + (uint32_t)tid * BPU;
+            inv[e] = MULTI ? __shfl_sync(0xFFFFFFFFu, inv_lane, (int)(kw[e >> 2] >> ((e & 3) * ib))) : inv_lane;
+    } else if (!slow) {
+        bool inexact = false;
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+        for (int k = 0; k < 2; ++k) {
+            const float4 f = mixed_row_factors(p, i + 4 * k, j, kw[k], false);
+            const float g[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
-        for (int b = 0; b < BPU; ++b) t.blk[u * BPU + b] = philox_block_part(p.key, blk_lo + (uint32_t)(u * kThreads * BPU + b));
-    char *lrow0 = (char *)p.lev + (size_t)m0 * t.lrow;
-    t.lp = lrow0 + LF::off(t0) + tid * LF::UB;
-    t.lp2 = lrow0 + LF::off2(t0, p.v.stride) + tid * (FMT == UQ_FMT_I6P ? 2 : 0);
-
-    // decode mode: lane k holds the reconstruction factor of scale k, the sums start at zero
-    float c_lane = 0.0f;
-    if (DEC) {
-        c_lane = decode_factor(W, p.v.scales.s[lane & KMASK], p.v.M);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) t.sum[u][k] = 0u;
-    }
-
-    // The workers of the group straight-line, with no loop around them: all 8, or (the last group
-    // of a job whose M is not a multiple of 8) 4, 2 and 1 of them as the count's bits say.
-    if (cnt == kWorkerGroup) {
-        encode_workers<kWorkerGroup, false, SEL>(p, t, m0, q);
-    } else {
-        int m = m0;
-        if (cnt & 4) {
-            if (cnt & 3) encode_workers<4, true, SEL>(p, t, m, q);
-            else encode_workers<4, false, SEL>(p, t, m, q);
-            m += 4;
-        }
-        if (cnt & 2) {
-            if (cnt & 1) encode_workers<2, true, SEL>(p, t, m, q);
-            else encode_workers<2, false, SEL>(p, t, m, q);
-            m += 2;
-        }
-        if (cnt & 1) encode_workers<1, false, SEL>(p, t, m, q);
-    }
-    if (DEC) {
-        // Algorithm 1 / 2, lines "AllReduce gradients" and "Reconstruct gradient" for the tile: the sum
-        // of a coordinate leaves its lane, loses the bias, and is multiplied by the factor of the
-        // coordinate's scale (the same three operations as the aggregation kernel's)
-        const int bias = 128 * p.v.M;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            uint32_t r[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint32_t lanes = t.sum[DEC ? u : 0][(e >> 2) * 2 + (e & 1)];
-                const int sum = (int)((lanes >> (16 * ((e & 3) >> 1))) & 0xFFFFu) - bias;
-                const float c = MULTI ? __shfl_sync(0xFFFFFFFFu, c_lane, (int)(uint32_t)(kbits[u] >> (e * IB))) : c_lane;
-                r[e] = __float_as_uint(__fmul_rn((float)sum, c));
+            for (int e = 0; e < 4; ++e) {
+                inexact |= RNG == 16 ? !sat_form_exact(g[e]) : !fixed_form_exact(g[e]);
+                inv[4 * k + e] = __fmul_rn(g[e], RNG == 16 ? 0.00390625f : 8388608.0f);
             }
-            st_stream256(p.out + t0 + (int64_t)(u * kThreads + tid) * 8, r);
         }
+        slow = __any_sync(0xFFFFFFFFu, inexact);
+    }
+    if (slow) {
+        encode_row_slow<DT, FMT, RNG, MULTI>(p, r0);
+        return;
+    }
+    LevelConstants lc;
+    lc.c0 = __fsub_rn(1.0f, __fmul_rn(p.v.s_hat, 0.00390625f));
+    lc.k_pos = (128u - (uint32_t)p.v.s_hat) * 0x01010101u;
+    lc.k_neg = (256u - (uint32_t)p.v.s_hat) * 0x01010101u;
+    lc.cap23 = __fmul_rn(p.v.s_hat, 8388608.0f);
+    PhiloxBlockPart blk[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) blk[b] = philox_block_part(p.key, (uint32_t)blk0 + (uint32_t)(lane * NB + b));
+
+    // The workers, straight-line.  The sums of two levels share a word: dp2a adds byte 0 and 2^14 times byte 1
+    // (64 workers * 127 < 2^13, so the fields come apart again).
+    int sum[2][2] = {{0, 0}, {0, 0}};
+    char *lp = (char *)p.lev + LF::off(i), *lp2 = (char *)p.lev + LF::off2(i, p.v.stride);
+    auto group = [&](int m0) {
+        uint4 r[G][NB];
+        philox_join<G, NB>(p.key, p.last0, p.last1, blk, p.wpart + m0, r);
+#pragma unroll
+        for (int c = 0; c < G; ++c) {
+            if (WK || m0 + c < M) {
+                if (RNG == 16) { r[c][0].y = ~r[c][0].y; r[c][0].w = ~r[c][0].w; }
+                uint32_t w[2];
+                quantize_fast<DT, FMT, RNG>(q[c], inv, lc, r[c], w);
+                if (m0 + c + G < M) load(m0 + c + G, q[c]);
+                if (O::EO) store_unit_even_odd(w[0], w[1], lp);
+                else store_unit<FMT>(w[0], w[1], lp, lp2);
+                lp += lrow;
+                if (FMT == UQ_FMT_I6P) lp2 += lrow;
+                if (DEC) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        sum[k][0] = __dp2a_lo(0x40000001, (int)w[k], sum[k][0]);
+                        sum[k][1] = __dp2a_hi(0x40000001, (int)w[k], sum[k][1]);
+                    }
+                }
+            }
+        }
+    };
+    if (WK) {
+#pragma unroll
+        for (int m = 0; m < WK; m += G) group(m);
+    } else {
+#pragma unroll 1
+        for (int m = 0; m < M; m += G) group(m);
+    }
+    if (DEC) {
+        // Algorithm 1 / 2, lines "AllReduce gradients" and "Reconstruct gradient": the sum of a coordinate times
+        // the factor of its scale (the same operations as the aggregation kernel's)
+        float c[8];
+        if (!mixed) {
+            const float c_lane = decode_factor(W, p.v.scales.s[lane & kmask], M);
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                c[e] = MULTI ? __shfl_sync(0xFFFFFFFFu, c_lane, (int)(kw[e >> 2] >> ((e & 3) * ib))) : c_lane;
+        } else {
+            const float4 a = mixed_row_factors(p, i, j, kw[0], true), b = mixed_row_factors(p, i + 4, j, kw[1], true);
+            c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w; c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
+        }
+        uint32_t s[8], r[8];
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int hi = (sum[k][h] + 0x2000) >> 14;
+                s[O::coord(k, 2 * h + 1)] = (uint32_t)hi;
+                s[O::coord(k, 2 * h)] = (uint32_t)(sum[k][h] - (hi << 14));
+            }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) r[e] = __float_as_uint(__fmul_rn((float)(int)s[e], c[e]));
+        st_stream256(p.out + i, r);
+        if (p.S != nullptr) st_stream256(p.S + i, s);
     }
 }
 
-template <int DT, int FMT, int RNG, int IDXB, bool SEL = false, bool DEC = false>
+template <int DT, int FMT, int RNG, bool MULTI, bool SEL, bool DEC, int WK>
 static cudaError_t launch(EncodeParams p, cudaStream_t st)
 {
-    using S = EncodeShape<DT, RNG>;
-    const int64_t ntiles = (p.v.d + S::TILE - 1) / S::TILE;
-    p.reserved = 0u;
-    p.groups = (uint32_t)((p.v.M + kWorkerGroup - 1) / kWorkerGroup);
-    int64_t blocks = ntiles * p.groups;
+    using S = EncodeShape<DT, RNG, SEL>;
+    const int64_t blocks = (p.v.d + S::TILE - 1) / S::TILE;
     if (blocks == 0) return cudaSuccess;
     if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    p.main_blocks = (uint32_t)blocks;
-    int64_t rows = 0;
-    if (p.v.seg_off != nullptr && p.v.nseg > 1) rows = (int64_t)((p.v.nseg - 1 + kWarps - 1) / kWarps) * (DEC ? 1 : p.v.M);
-    blocks += rows;
-    if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    p.row_blocks = (uint32_t)rows;
     constexpr int BSH = RNG == 32 ? 2 : 3;
     p.blk_hi = (uint32_t)((uint64_t)(p.coord0 >> BSH) >> 32);
-    for (int m = 0; m < UQ_MAX_WORKERS; ++m)
-        p.wpart[m] = philox_worker_part(p.key, p.blk_hi, (uint32_t)(p.worker0 + (m < p.v.M ? m : 0)));
-    if (SEL) {
-        // the copies of the tile's rows: up to kWorkerGroup workers * TILE coordinates (64 KiB)
-        const size_t smem = (size_t)(p.v.M < kWorkerGroup ? p.v.M : kWorkerGroup) * S::TILE * Elem<DT>::BYTES;
-        // more than 48 KiB of dynamic shared memory needs an opt-in per kernel and device (the call
-        // is idempotent, so a race between host threads on the flag is harmless)
-        static bool opted_in[64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64 || !opted_in[dev]) {
-            e = cudaFuncSetAttribute(encode_kernel<DT, FMT, RNG, IDXB, SEL, DEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kWorkerGroup * S::TILE * Elem<DT>::BYTES);
-            if (e != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) opted_in[dev] = true;
-        }
-        launch_k_smem(encode_kernel<DT, FMT, RNG, IDXB, SEL, DEC>, (unsigned)blocks, kThreads, smem, st, p);
-    } else {
-        launch_k(encode_kernel<DT, FMT, RNG, IDXB, SEL, DEC>, (unsigned)blocks, kThreads, st, p);
-    }
+    const uint32_t flip = RNG == 16 ? 0xFFFFFFFFu : 0u;
+    p.last0 = p.key.k0[9] ^ flip; p.last1 = p.key.k1[9] ^ flip;
+    for (int m = 0; m < p.v.M; ++m) p.wpart[m] = philox_worker_part(p.key, p.blk_hi, (uint32_t)(p.worker0 + m));
+    // bf16, selecting: the 8 workers' rows of the tile
+    const size_t smem = SEL && DT == UQ_BF16 && WK == 8 ? (size_t)WK * S::TILE * Elem<DT>::BYTES : 0;
+    launch_k_smem(encode_kernel<DT, FMT, RNG, MULTI, SEL, DEC, WK>, (unsigned)blocks, kThreads, smem, st, p);
     return cudaGetLastError();
 }
 
-template <int DT, int FMT, int RNG>
-static cudaError_t dispatch_idx(const EncodeParams &p, int idx_bits, cudaStream_t st)
+// All wire formats and modes of one element type and draw width (one translation unit each, so that
+// the variants build in parallel).
+template <int DT, int FMT, int RNG, int WK> static cudaError_t dispatch_mode(const EncodeParams &p, cudaStream_t st)
 {
-    if constexpr (FMT == UQ_FMT_I8 && RNG == 16) {
-        if (p.out != nullptr && !p.select) {          // decode mode (the caller has checked M <= kWorkerGroup)
-            switch (idx_bits) {
-            case 0: return launch<DT, FMT, RNG, 0, false, true>(p, st);
-            case 1: return launch<DT, FMT, RNG, 1, false, true>(p, st);
-            case 2: return launch<DT, FMT, RNG, 2, false, true>(p, st);
-            case 4: return launch<DT, FMT, RNG, 4, false, true>(p, st);
-            default: return launch<DT, FMT, RNG, 8, false, true>(p, st);
-            }
-        }
-    }
-    if constexpr (FMT == UQ_FMT_I8 && RNG == 16) {
-        if (p.out != nullptr && p.select) {           // select mode and decode mode together
-            switch (idx_bits) {
-            case 1: return launch<DT, FMT, RNG, 1, true, true>(p, st);
-            case 2: return launch<DT, FMT, RNG, 2, true, true>(p, st);
-            case 4: return launch<DT, FMT, RNG, 4, true, true>(p, st);
-            default: return launch<DT, FMT, RNG, 8, true, true>(p, st);
-            }
-        }
-    }
-    if (p.select) {
-        switch (idx_bits) {
-        case 1: return launch<DT, FMT, RNG, 1, true>(p, st);
-        case 2: return launch<DT, FMT, RNG, 2, true>(p, st);
-        case 4: return launch<DT, FMT, RNG, 4, true>(p, st);
-        default: return launch<DT, FMT, RNG, 8, true>(p, st);
-        }
-    }
-    switch (idx_bits) {
-    case 0: return launch<DT, FMT, RNG, 0>(p, st);
-    case 1: return launch<DT, FMT, RNG, 1>(p, st);
-    case 2: return launch<DT, FMT, RNG, 2>(p, st);
-    case 4: return launch<DT, FMT, RNG, 4>(p, st);
-    default: return launch<DT, FMT, RNG, 8>(p, st);
-    }
+    const bool dec = p.out != nullptr;
+    if (p.idx_bits == 0)
+        return dec ? launch<DT, FMT, RNG, false, false, true, WK>(p, st) : launch<DT, FMT, RNG, false, false, false, WK>(p, st);
+    if (p.select)
+        return dec ? launch<DT, FMT, RNG, true, true, true, WK>(p, st) : launch<DT, FMT, RNG, true, true, false, WK>(p, st);
+    return dec ? launch<DT, FMT, RNG, true, false, true, WK>(p, st) : launch<DT, FMT, RNG, true, false, false, WK>(p, st);
 }
 
-// All wire formats and index widths of one element type and draw width (one translation unit
-// each, so that the variants build in parallel).
-template <int DT, int RNG>
-static cudaError_t dispatch_fmt(const EncodeParams &p, int fmt, int idx_bits, cudaStream_t st)
+template <int DT, int FMT, int RNG> static cudaError_t dispatch_workers(const EncodeParams &p, cudaStream_t st)
 {
-    if (fmt == UQ_FMT_I8) return dispatch_idx<DT, UQ_FMT_I8, RNG>(p, idx_bits, st);
-    if (fmt == UQ_FMT_I4X2) return dispatch_idx<DT, UQ_FMT_I4X2, RNG>(p, idx_bits, st);
-    if (fmt == UQ_FMT_I2X4) return dispatch_idx<DT, UQ_FMT_I2X4, RNG>(p, idx_bits, st);
-    return dispatch_idx<DT, UQ_FMT_I6P, RNG>(p, idx_bits, st);
+    return p.v.M == kGroup ? dispatch_mode<DT, FMT, RNG, kGroup>(p, st) : dispatch_mode<DT, FMT, RNG, 0>(p, st);
 }
 
-cudaError_t launch_encode_f32_r16(const EncodeParams &p, int fmt, int idx_bits, cudaStream_t st);
-cudaError_t launch_encode_f32_r32(const EncodeParams &p, int fmt, int idx_bits, cudaStream_t st);
-cudaError_t launch_encode_bf16_r16(const EncodeParams &p, int fmt, int idx_bits, cudaStream_t st);
-cudaError_t launch_encode_bf16_r32(const EncodeParams &p, int fmt, int idx_bits, cudaStream_t st);
+template <int DT, int RNG> static cudaError_t dispatch_fmt(const EncodeParams &p, int fmt, cudaStream_t st)
+{
+    if (fmt == UQ_FMT_I8) return dispatch_workers<DT, UQ_FMT_I8, RNG>(p, st);
+    if (fmt == UQ_FMT_I4X2) return dispatch_workers<DT, UQ_FMT_I4X2, RNG>(p, st);
+    if (fmt == UQ_FMT_I2X4) return dispatch_workers<DT, UQ_FMT_I2X4, RNG>(p, st);
+    return dispatch_workers<DT, UQ_FMT_I6P, RNG>(p, st);
+}
+
+cudaError_t launch_encode_f32_r16(const EncodeParams &p, int fmt, cudaStream_t st);
+cudaError_t launch_encode_f32_r32(const EncodeParams &p, int fmt, cudaStream_t st);
+cudaError_t launch_encode_bf16_r16(const EncodeParams &p, int fmt, cudaStream_t st);
+cudaError_t launch_encode_bf16_r32(const EncodeParams &p, int fmt, cudaStream_t st);
 
 }  // namespace uq

@@ -3,9 +3,9 @@
 
 namespace uq {
 
-cudaError_t launch_encode_f32_r16(const EncodeParams &p, int fmt, int idx_bits, cudaStream_t st)
+cudaError_t launch_encode_f32_r16(const EncodeParams &p, int fmt, cudaStream_t st)
 {
-    return dispatch_fmt<UQ_F32, 16>(p, fmt, idx_bits, st);
+    return dispatch_fmt<UQ_F32, 16>(p, fmt, st);
 }
 
 }  // namespace uq

@@ -33,10 +33,8 @@ class Quantizer:
         self.M, self.d, self.dtype = M, d, dtype
         self.stride = -(-d // 32) * 32
         self.multi = scales is not None and idx_bits != 0
-        # multi-scale: whether selection + sharing run inside the encoder's kernel (one kernel for M <= 8,
-        # the gradients read once, same bits) instead of as a streaming kernel of their own.  None = the
-        # library's own choice (uq_step: inside where the encoder also aggregates and reconstructs, i.e.
-        # int8 levels, 16-bit draws, M <= 8 and no integer sums kept; a kernel of its own otherwise).
+        # multi-scale: whether selection + sharing run inside the encoder's kernel (same bits) instead of as a
+        # streaming kernel of their own.  None = the library's own choice (uq_step: inside).
         self.fused_select = None if fused_select is None else bool(fused_select) and self.multi
         self.s = int(scales[0]) if self.multi else int(s)
         self.scales = [int(x) for x in scales] if self.multi else None
@@ -100,7 +98,7 @@ class Quantizer:
 
     def encode_decode(self, g: torch.Tensor, seed: int) -> None:
         """Quantization, integer aggregation and reconstruction as one call (what the step makes when
-        the integer sums are not kept; one kernel for int8 levels, 16-bit draws and M <= 8)."""
+        the integer sums are not kept)."""
         B.uq_encode_decode(self.layout, g, self.W, self.s, self.scales, self.idx, self.idx_bits, seed, self.rng_bits,
                            self.fmt, self.lev, self.out, self.status)
 
@@ -109,13 +107,12 @@ class Quantizer:
         """Multi-scale: whether the step's selection runs inside the encoder's kernel."""
         if not self.multi:
             return False
-        return self.fused_decode if self.fused_select is None else self.fused_select
+        return self.fused_select is None or self.fused_select
 
     @property
     def fused_decode(self) -> bool:
-        """Whether the step's encoder also aggregates and reconstructs (uq_encode_decode as one kernel)."""
-        return (self.S is None and self.fmt == B.UQ_FMT_I8 and self.layout.M <= B.SMALL_STEP_MAX_WORKERS
-                and self.rng_bits == 16)
+        """Whether the step's encoder also aggregates and reconstructs."""
+        return self.fused_select is None or self.S is None
 
     def aggregate_decode_update(self, theta: torch.Tensor, momentum: Optional[torch.Tensor], lr: float,
                                 mu: float = 0.0, wd: float = 0.0) -> None:
@@ -185,12 +182,11 @@ class Quantizer:
         B.require_current_device(self.device.index, current, "the quantizer")
 
     def kernels_per_step(self) -> int:
-        """Kernel launches one step enqueues (norm partials + finalize, [select], encode, decode; the
-        last two are one kernel when the encoder also aggregates and reconstructs)."""
+        """Kernel launches one step enqueues (norm partials + finalize, [select,] encode[, decode]: one
+        kernel when the encoder also selects, aggregates and reconstructs)."""
         if self.one_kernel:
             return 1
-        inside = self.selects_inside
-        separate_select = self.multi and (not inside or self.M > 8) and self.d > 0
+        separate_select = self.multi and not self.selects_inside and self.d > 0
         tail = 0 if self.d == 0 else 1 if self.fused_decode else 2
         return (2 if self.d > 0 else 1) + (1 if separate_select else 0) + tail
 
