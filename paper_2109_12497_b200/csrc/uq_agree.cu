@@ -103,48 +103,69 @@ norm_partials_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int 
     }
 }
 
+// One CTA per segment: every worker's slots are added up by `nwarps / M` warps (at least one), eight loads in
+// flight per lane, in an order that depends on the launch's size only.  (With one warp per worker and the
+// loads one after the other a segment of 1600 tiles took 9.8 us, all of it load latency.)
 template <int NORM>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(1024)
 norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg,
                      const int64_t *__restrict__ seg_off, int64_t ntiles, float *__restrict__ W,
                      uint32_t *__restrict__ status, int tile_coords)       // tile_coords: coordinates per partial
 {
     grid_dependency_prologue();
     const int j = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     int64_t a = seg_off ? __ldg(seg_off + j) : 0;
     int64_t b = seg_off ? __ldg(seg_off + j + 1) : d;
     const bool bad = a < 0 || b > d || a > b || (j == 0 && a != 0) || (j == nseg - 1 && b != d);
     a = min(max(a, (int64_t)0), d);
     b = min(max(b, a), d);
 
-    double best = 0.0;
+    __shared__ double sh[UQ_MAX_WORKERS + 32];                             // [worker][warp of the worker]
+    const int share = max(nwarps / M, 1);                                   // warps per worker
+    const int sub = warp % share;
     if (a < b) {
-        const int64_t first = a / tile_coords, last = (b - 1) / tile_coords;
-        for (int m = warp; m < M; m += kWarps) {
+        const int first = (int)(a / tile_coords), last = (int)((b - 1) / tile_coords), step = 32 * share;
+        for (int m = warp / share; m < M; m += max(nwarps / share, 1)) {
             const double *prow = part + (size_t)m * (size_t)(ntiles + nseg) + j;
             double acc = 0.0;
-            for (int64_t t = first + lane; t <= last; t += 32) acc = combine<NORM>(acc, prow[t]);
+            for (int t = first + sub * 32 + lane; t <= last; t += 8 * step) {
+                double v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = t + k * step <= last ? __ldcg(prow + t + k * step) : 0.0;    // 0 is neutral for both norms
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc = combine<NORM>(acc, v[k]);
+            }
             const double r = warp_reduce<NORM>(acc);
-            best = (r != r || best != best) ? r + best : fmax(best, r);   // keep a NaN alive
+            if (lane == 0) sh[m * share + sub] = r;
         }
+    } else {
+        for (int k = tid; k < M * share; k += blockDim.x) sh[k] = 0.0;
     }
-    __shared__ double sh[kWarps];
-    if (lane == 0) sh[warp] = best;
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0) {
         // fmax drops NaN, so look for it explicitly
         bool nan = false;
         double top = 0.0;
-        for (int k = 0; k < kWarps; ++k) { nan |= sh[k] != sh[k]; top = fmax(top, sh[k]); }
-        float w;
-        if (NORM == UQ_NORM_L2) w = nan ? __uint_as_float(0x7FC00000u) : __double2float_rn(sqrt(top));
-        else w = __uint_as_float((uint32_t)top);
-        W[j] = w;
-        uint32_t flags = 0;
-        if ((__float_as_uint(w) & 0x7F800000u) == 0x7F800000u) flags |= UQ_STATUS_NONFINITE;
-        if (bad) flags |= UQ_STATUS_BAD_SEGMENTS;
-        if (flags && status) atomicOr(status, flags);
+        for (int m = lane; m < M; m += 32) {
+            double tot = sh[m * share];
+            for (int k = 1; k < share; ++k) tot = combine<NORM>(tot, sh[m * share + k]);
+            nan |= tot != tot;
+            top = fmax(top, tot);
+        }
+        nan = __any_sync(0xFFFFFFFFu, nan);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+        if (lane == 0) {
+            float w;
+            if (NORM == UQ_NORM_L2) w = nan ? __uint_as_float(0x7FC00000u) : __double2float_rn(sqrt(top));
+            else w = __uint_as_float((uint32_t)top);
+            W[j] = w;
+            uint32_t flags = 0;
+            if ((__float_as_uint(w) & 0x7F800000u) == 0x7F800000u) flags |= UQ_STATUS_NONFINITE;
+            if (bad) flags |= UQ_STATUS_BAD_SEGMENTS;
+            if (flags && status) atomicOr(status, flags);
+        }
     }
 }
 
@@ -159,10 +180,11 @@ static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t 
         dim3 grid((unsigned)ntiles, (unsigned)L.M);
         if (DT == UQ_F32)
             grid = dim3((unsigned)L.M * (unsigned)min(ntiles, (int64_t)kSlab), (unsigned)((ntiles + kSlab - 1) / kSlab));
-        launch_k(norm_partials_kernel<DT, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg,
-                                                                 L.seg_off, ntiles, part);
+        launch_k(norm_partials_kernel<DT, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
     }
-    launch_k(norm_finalize_kernel<NORM>, L.nseg, kThreads, st, part, L.M, L.d, L.nseg, L.seg_off, ntiles, W,
+    // few long segments: more warps per worker
+    const int threads = ntiles / L.nseg * L.M >= 2048 ? 1024 : kThreads;
+    launch_k(norm_finalize_kernel<NORM>, L.nseg, threads, st, part, L.M, L.d, L.nseg, L.seg_off, ntiles, W,
                                                           status, kNormTile);
     return cudaGetLastError();
 }
