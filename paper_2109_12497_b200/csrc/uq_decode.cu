@@ -274,6 +274,20 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
     const size_t row_bytes = LevelFmt<FMT>::row_bytes(p.stride);
 
     const bool want_values = p.out != nullptr || UPDATE;           // else: the integer sums only
+    const bool full = i + C <= p.d;
+    const bool has_mom = UPDATE && p.mom != nullptr;
+    // UPDATE with 32 coordinates per thread: there are few threads, so all parameters (and momenta) are on
+    // their way while the levels are summed (23.5 M coordinates, 8 workers: 2-bit levels 96 -> 84 us, 4-bit 99 -> 87;
+    // not 6-bit ones, whose two planes leave no registers for it: 108 -> 123)
+    constexpr bool AHEAD = UPDATE && C > 16 && FMT != UQ_FMT_I6P;
+    float th[AHEAD ? C / 8 : 1][8], bf[AHEAD ? C / 8 : 1][8];
+    if (AHEAD && full) {
+#pragma unroll
+        for (int e = 0; e < C / 8; ++e) {
+            ld256(p.theta + i + 8 * e, th[AHEAD ? e : 0]);
+            if (has_mom) ld256(p.mom + i + 8 * e, bf[AHEAD ? e : 0]);
+        }
+    }
     U unit;
     uint32_t kw[WORDS];
     if (active) {
@@ -305,7 +319,6 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
     // stored (256 bits per array) and forgotten, which keeps the registers of a thread low enough for
     // more CTAs per SM than 32 sums and 32 values held at once would allow.
     unit.prepare();
-    const bool full = i + C <= p.d;
     // every warp looks up the segment of its own row of 32*C coordinates; lane k holds the
     // reconstruction factor of scale k (single-scale: every lane holds the same factor)
     const int64_t row1 = min(row0 + 32 * C, p.d);
@@ -317,7 +330,6 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
         uniform = segment_end(p.seg_off, p.nseg, j, p.d) >= row1;
         if (uniform) c_lane = decode_factor(__ldg(p.W + j), p.scales.s[lane & (UQ_MAX_SCALES - 1)], p.M);
     }
-    const bool has_mom = UPDATE && p.mom != nullptr;
     auto group = [&](auto e0_tag) {
         constexpr int E0 = decltype(e0_tag)::value;
         int s[8];
@@ -354,20 +366,22 @@ __global__ void __launch_bounds__(kThreads) aggregate_decode_kernel(const __grid
             // from registers into the parameters (and the momentum buffer), 8 coordinates as one
             // 256-bit access per array: a lane's 32 bytes are one whole sector
             if (full) {
-                float th[8], bf[8] = {};
-                ld256(p.theta + i + E0, th);
-                if (has_mom) ld256(p.mom + i + E0, bf);
+                constexpr int S = AHEAD ? E0 / 8 : 0;
+                if (!AHEAD) {
+                    ld256(p.theta + i + E0, th[0]);
+                    if (has_mom) ld256(p.mom + i + E0, bf[0]);
+                }
 #pragma unroll
-                for (int t = 0; t < 8; ++t) sgd_coordinate(r[t], th[t], bf[t], has_mom, p.lr, p.mu, p.wd);
-                st256(p.theta + i + E0, th);
-                if (has_mom) st256(p.mom + i + E0, bf);
+                for (int t = 0; t < 8; ++t) sgd_coordinate(r[t], th[S][t], bf[S][t], has_mom, p.lr, p.mu, p.wd);
+                st256(p.theta + i + E0, th[S]);
+                if (has_mom) st256(p.mom + i + E0, bf[S]);
             } else {
                 for (int e = 0; e < 8; ++e) {
                     if (i + E0 + e >= p.d) break;
-                    float th = p.theta[i + E0 + e], bf = has_mom ? p.mom[i + E0 + e] : 0.0f;
-                    sgd_coordinate(r[e], th, bf, has_mom, p.lr, p.mu, p.wd);
-                    p.theta[i + E0 + e] = th;
-                    if (has_mom) p.mom[i + E0 + e] = bf;
+                    float x = p.theta[i + E0 + e], y = has_mom ? p.mom[i + E0 + e] : 0.0f;
+                    sgd_coordinate(r[e], x, y, has_mom, p.lr, p.mu, p.wd);
+                    p.theta[i + E0 + e] = x;
+                    if (has_mom) p.mom[i + E0 + e] = y;
                 }
             }
         }
