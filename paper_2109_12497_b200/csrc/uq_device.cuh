@@ -204,9 +204,10 @@ __device__ __forceinline__ int64_t segment_end(const int64_t *__restrict__ seg_o
 // Philox4x32-10, counter = (block low, block high, worker, tag), key = seed; the rounding draws use tag 0
 // ---------------------------------------------------------------------------------------------
 
-// The ten round keys (uniform over the grid).  8-byte aligned: inside kernel parameters the keys are
-// fetched two at a time, and a table that starts on an odd word costs the encoders 6-9 % (measured).
-struct alignas(8) PhiloxKey { uint32_t k0[10], k1[10]; };
+// The ten round keys (uniform over the grid), a round's two words side by side.  16-byte aligned: inside
+// kernel parameters they are fetched four at a time (two rounds); a table that starts 8 bytes off costs
+// the encoders 7 % (measured), one on an odd word 6-9 %.
+struct alignas(16) PhiloxKey { uint32_t k[20]; };      // k[2 r], k[2 r + 1]: words 0 and 1 of round r
 
 __host__ __device__ __forceinline__ PhiloxKey philox_key(uint64_t seed)
 {
@@ -214,7 +215,7 @@ __host__ __device__ __forceinline__ PhiloxKey philox_key(uint64_t seed)
     uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        k.k0[r] = a; k.k1[r] = b;
+        k.k[2 * r] = a; k.k[2 * r + 1] = b;
         a += 0x9E3779B9u; b += 0xBB67AE85u;
     }
     return k;
@@ -228,8 +229,8 @@ __device__ __forceinline__ uint4 philox4x32_10(const PhiloxKey &k, uint32_t bloc
     for (int r = 0; r < 10; ++r) {
         uint64_t p0 = (uint64_t)0xD2511F53u * c0;
         uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
-        uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.k0[r];
-        uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.k1[r];
+        uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.k[2 * r];
+        uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.k[2 * r + 1];
         c1 = (uint32_t)p1; c3 = (uint32_t)p0; c0 = n0; c2 = n2;
     }
     return make_uint4(c0, c1, c2, c3);
@@ -247,7 +248,7 @@ __device__ __forceinline__ void philox4x32_10_xN(const PhiloxKey &k, const uint3
     for (int n = 0; n < N; ++n) { c0[n] = block_lo[n]; c1[n] = block_hi; c2[n] = worker; c3[n] = 0u; }
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t k0 = k.k0[r], k1 = k.k1[r];
+        const uint32_t k0 = k.k[2 * r], k1 = k.k[2 * r + 1];
 #pragma unroll
         for (int n = 0; n < N; ++n) {
             const uint64_t p0 = (uint64_t)0xD2511F53u * c0[n];
@@ -282,7 +283,7 @@ __device__ __forceinline__ PhiloxBlockPart philox_block_part(const PhiloxKey &k,
     PhiloxBlockPart r;
     const uint64_t p0 = (uint64_t)kPhiloxM0 * block_lo;
     r.c3 = (uint32_t)p0;
-    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ k.k1[0]);
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ k.k[1]);
     r.a = (uint32_t)(p1 >> 32); r.b = (uint32_t)p1;
     return r;
 }
@@ -291,17 +292,16 @@ __host__ __device__ __forceinline__ PhiloxWorkerPart philox_worker_part(const Ph
 {
     PhiloxWorkerPart w;
     const uint64_t pw = (uint64_t)kPhiloxM1 * worker;
-    w.u1 = (uint32_t)pw ^ k.k0[1];
-    const uint64_t q0 = (uint64_t)kPhiloxM0 * ((uint32_t)(pw >> 32) ^ block_hi ^ k.k0[0]);
-    w.hq = (uint32_t)(q0 >> 32) ^ k.k1[1]; w.lq = (uint32_t)q0; w.unused = 0u;
+    w.u1 = (uint32_t)pw ^ k.k[2];
+    const uint64_t q0 = (uint64_t)kPhiloxM0 * ((uint32_t)(pw >> 32) ^ block_hi ^ k.k[0]);
+    w.hq = (uint32_t)(q0 >> 32) ^ k.k[3]; w.lq = (uint32_t)q0; w.unused = 0u;
     return w;
 }
 
 // Rounds 1 (the joining XORs) to 9 of the N blocks of G workers, all advanced together: one fetch of a round
-// key serves G * N chains.  last0, last1: the keys of round 9 (a caller that wants words 0 and 2
-// complemented hands over the complemented keys).
+// key serves G * N chains.
 template <int G, int N>
-__device__ __forceinline__ void philox_join(const PhiloxKey &k, uint32_t last0, uint32_t last1, const PhiloxBlockPart (&blk)[N],
+__device__ __forceinline__ void philox_join(const PhiloxKey &k, const PhiloxBlockPart (&blk)[N],
                                             const PhiloxWorkerPart *w, uint4 (&out)[G][N])
 {
     uint32_t c0[G][N], c1[G][N], c2[G][N], c3[G][N];
@@ -316,7 +316,7 @@ __device__ __forceinline__ void philox_join(const PhiloxKey &k, uint32_t last0, 
         }
 #pragma unroll
     for (int r = 2; r < 10; ++r) {
-        const uint32_t k0 = r == 9 ? last0 : k.k0[r], k1 = r == 9 ? last1 : k.k1[r];
+        const uint32_t k0 = k.k[2 * r], k1 = k.k[2 * r + 1];
 #pragma unroll
         for (int g = 0; g < G; ++g)
 #pragma unroll

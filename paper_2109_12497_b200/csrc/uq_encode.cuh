@@ -39,10 +39,11 @@ struct EncodeParams {
     int32_t idx_bits;         // 1, 2, 4 or 8; 0 for the single-scale quantizer
     int32_t worker0;          // number, in the whole job, of the worker in row 0 (keys the draws)
     uint32_t blk_hi;          // high word of the Philox block numbers the table below was made for
+    int32_t split;            // workers per CTA (grid.y = ceil(M / split)); M unless only the levels are wanted
     int64_t coord0;           // index, in the whole gradient, of coordinate 0 (keys the draws)
-    PhiloxKey key;            // the ten round keys of the seed
-    uint32_t last0, last1;    // the last round's keys as the fast path wants them (16-bit draws: complemented)
-    PhiloxWorkerPart wpart[UQ_MAX_WORKERS];   // per-worker words of the first two Philox rounds (row m)
+    PhiloxKey key;            // the ten round keys of the seed; 16-bit draws: the last round's complemented, so that
+                              // words 0 and 2 of a block come out complemented
+    alignas(16) PhiloxWorkerPart wpart[UQ_MAX_WORKERS];   // per-worker words of the first two Philox rounds (row m)
 };
 
 constexpr int kGroup = 8;     // the number of workers that has kernels of its own (all of them straight-line)
@@ -105,10 +106,10 @@ template <int UC> __device__ __forceinline__ void store_indices(uint8_t *idx, in
 
 // Everything for the coordinates [r0, min(r0 + 256, d)), looked up coordinate by coordinate, in plain
 // arithmetic: the row that holds d, rows whose Philox block numbers leave the launch's high word, and
-// rows whose factors are too small or too large for the rescaled forms.  One warp; a lane takes a unit
-// of 8 coordinates.
+// rows whose factors are too small or too large for the rescaled forms.  Workers m_first .. m_last - 1 (all of
+// them if the sums are wanted).  One warp; a lane takes a unit of 8 coordinates.
 template <int DT, int FMT, int RNG, bool MULTI>
-__device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0)
+__device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0, int m_first, int m_last)
 {
     using E = Elem<DT>;
     using LF = LevelFmt<FMT>;
@@ -146,11 +147,11 @@ __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0)
     const uint64_t blk = RNG == 32 ? (uint64_t)((p.coord0 + i) >> 2) : (uint64_t)((p.coord0 + i) >> 3);
     int S[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     constexpr int G = 4, H = 8 / E::G;                              // workers whose loads are in flight together
-    for (int m0 = 0; m0 < p.v.M; m0 += G) {
+    for (int m0 = m_first; m0 < m_last; m0 += G) {
         uint4 q[G][H];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const int m = min(m0 + g, p.v.M - 1);
+            const int m = min(m0 + g, m_last - 1);
 #pragma unroll
             for (int h = 0; h < H; ++h)
                 q[g][h] = ld_stream((const char *)p.v.g + ((size_t)m * (size_t)p.v.stride + i + h * E::G) * E::BYTES);
@@ -158,7 +159,7 @@ __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0)
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const int m = m0 + g;
-            if (m >= p.v.M) break;
+            if (m >= m_last) break;
             float v[8];
 #pragma unroll
             for (int h = 0; h < H; ++h) E::unpack(q[g][h], *(float(*)[E::G])(v + h * E::G));
@@ -167,8 +168,9 @@ __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0)
 #pragma unroll
             for (int e = 0; e < 8; ++e)
                 if (i + e >= d) v[e] = 0.0f;
-            quantize_unit_bytes<RNG>(v, inv, p.v.s_hat, neg_lo, neg_hi,
-                                     unit_words<RNG>(p.key, (uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)(m + p.worker0)), lo, hi);
+            UnitWords<RNG> words = unit_words<RNG>(p.key, (uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)(m + p.worker0));
+            if (RNG == 16) { words.r[0].x = ~words.r[0].x; words.r[0].z = ~words.r[0].z; }
+            quantize_unit_bytes<RNG>(v, inv, p.v.s_hat, neg_lo, neg_hi, words, lo, hi);
             char *lrow = (char *)p.lev + (size_t)m * LF::row_bytes(p.v.stride);
             store_unit<FMT>(lo, hi, lrow + LF::off(i), lrow + LF::off2(i, p.v.stride));
 #pragma unroll
@@ -345,7 +347,10 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     if (r0 >= d) return;
     bool slow = r0 + 256 > d || (uint32_t)(blk0 >> 32) != p.blk_hi || (uint32_t)blk0 > 0xFFFFFFFFu - (256u >> BSH);
     const size_t grow = (size_t)p.v.stride * E::BYTES, lrow = LF::row_bytes(p.v.stride);
-    const char *gp = (const char *)p.v.g + (size_t)i * E::BYTES;
+    // my workers: all of them, or (only the levels wanted) one of grid.y groups
+    constexpr bool SPLIT = !WK && !SEL && !DEC;
+    const int m_first = SPLIT ? blockIdx.y * p.split : 0, m_last = SPLIT ? min(m_first + p.split, M) : M;
+    const char *gp = (const char *)p.v.g + (size_t)i * E::BYTES + (SPLIT ? m_first * grow : 0);
     extern __shared__ uint4 stage[];                             // STAGED: [worker][thread]
     const uint32_t sp = (uint32_t)__cvta_generic_to_shared(stage) + threadIdx.x * 16;
     uint64_t policy = 0;
@@ -370,7 +375,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         } else if (!SEL) {
 #pragma unroll
             for (int c = 0; c < G; ++c)
-                if (WK || c < M) load(c, q[c]);
+                if (WK || m_first + c < m_last) load(c, q[c]);
             if (MULTI) load_indices<8>(p.idx, i, ib, kw);
         }
     }
@@ -501,7 +506,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         slow = __any_sync(0xFFFFFFFFu, inexact);
     }
     if (slow) {
-        encode_row_slow<DT, FMT, RNG, MULTI>(p, r0);
+        encode_row_slow<DT, FMT, RNG, MULTI>(p, r0, m_first, m_last);
         return;
     }
     LevelConstants lc;
@@ -516,17 +521,17 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     // The workers, straight-line.  The sums of two levels share a word: dp2a adds byte 0 and 2^14 times byte 1
     // (64 workers * 127 < 2^13, so the fields come apart again).
     int sum[2][2] = {{0, 0}, {0, 0}};
-    char *lp = (char *)p.lev + LF::off(i), *lp2 = (char *)p.lev + LF::off2(i, p.v.stride);
+    char *lp = (char *)p.lev + LF::off(i) + (SPLIT ? m_first * lrow : 0), *lp2 = lp + (LF::off2(i, p.v.stride) - LF::off(i));
     auto group = [&](int m0) {
         uint4 r[G][NB];
-        philox_join<G, NB>(p.key, p.last0, p.last1, blk, p.wpart + m0, r);
+        philox_join<G, NB>(p.key, blk, p.wpart + m0, r);
 #pragma unroll
         for (int c = 0; c < G; ++c) {
-            if (WK || m0 + c < M) {
+            if (WK || m0 + c < m_last) {
                 if (RNG == 16) { r[c][0].y = ~r[c][0].y; r[c][0].w = ~r[c][0].w; }
                 uint32_t w[2];
                 quantize_fast<DT, FMT, RNG>(q[c], inv, lc, r[c], w);
-                if (m0 + c + G < M) load(m0 + c + G, q[c]);
+                if (m0 + c + G < m_last) load(m0 + c + G, q[c]);
                 if (O::EO) store_unit_even_odd(w[0], w[1], lp);
                 else store_unit<FMT>(w[0], w[1], lp, lp2);
                 lp += lrow;
@@ -546,7 +551,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         for (int m = 0; m < WK; m += G) group(m);
     } else {
 #pragma unroll 1
-        for (int m = 0; m < M; m += G) group(m);
+        for (int m = m_first; m < m_last; m += G) group(m);
     }
     if (DEC) {
         // Algorithm 1 / 2, lines "AllReduce gradients" and "Reconstruct gradient": the sum of a coordinate times
@@ -586,12 +591,15 @@ static cudaError_t launch(EncodeParams p, cudaStream_t st)
     if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
     constexpr int BSH = RNG == 32 ? 2 : 3;
     p.blk_hi = (uint32_t)((uint64_t)(p.coord0 >> BSH) >> 32);
-    const uint32_t flip = RNG == 16 ? 0xFFFFFFFFu : 0u;
-    p.last0 = p.key.k0[9] ^ flip; p.last1 = p.key.k1[9] ^ flip;
+    if (RNG == 16) { p.key.k[18] = ~p.key.k[18]; p.key.k[19] = ~p.key.k[19]; }
     for (int m = 0; m < p.v.M; ++m) p.wpart[m] = philox_worker_part(p.key, p.blk_hi, (uint32_t)(p.worker0 + m));
     // bf16, selecting: the 8 workers' rows of the tile
     const size_t smem = SEL && DT == UQ_BF16 && WK == 8 ? (size_t)WK * S::TILE * Elem<DT>::BYTES : 0;
-    launch_k_smem(encode_kernel<DT, FMT, RNG, MULTI, SEL, DEC, WK>, (unsigned)blocks, kThreads, smem, st, p);
+    // only the levels wanted: groups of 8 workers are independent, which gives small gradients of many workers
+    // as many warps as they have groups
+    p.split = !WK && !SEL && !DEC ? kGroup : p.v.M;
+    const dim3 grid((unsigned)blocks, (unsigned)((p.v.M + p.split - 1) / p.split));
+    launch_k_smem(encode_kernel<DT, FMT, RNG, MULTI, SEL, DEC, WK>, grid, kThreads, smem, st, p);
     return cudaGetLastError();
 }
 
