@@ -12,17 +12,27 @@ namespace uq {
 // Programmatic dependent launch: every kernel of the library is launched with the attribute that
 // lets the GPU schedule its CTAs while the kernel before it in the stream is still draining, and
 // starts with grid_dependency_prologue(): it first lets the kernel AFTER it be scheduled the same
-// way, then waits until the kernel before it has completed and its writes are visible.  No read of
-// global memory may come before the prologue.  What overlaps is launch latency and the ramp of the
+// way, then waits until the kernel before it has completed and its writes are visible.  No access to
+// global memory may come before the wait.  What overlaps is launch latency and the ramp of the
 // CTAs, not the work; a predecessor that knows nothing of this (a framework kernel, a copy) simply
 // counts as complete when it ends.  -DUQ_NO_PDL launches the plain way.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void grid_dependency_prologue()
+__device__ __forceinline__ void grid_dependency_trigger()
 {
 #ifndef UQ_NO_PDL
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void grid_dependency_wait()
+{
+#ifndef UQ_NO_PDL
     asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
+}
+__device__ __forceinline__ void grid_dependency_prologue()
+{
+    grid_dependency_trigger();
+    grid_dependency_wait();
 }
 
 template <typename... P, typename... A>

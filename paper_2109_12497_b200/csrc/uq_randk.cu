@@ -41,25 +41,32 @@ struct RandkParams {
     PhiloxKey key;
 };
 
+// The choice reads nothing but the kernel's parameters, so it is made before the wait for the kernel in front:
+// its chain (8 rounds of a 10-round Philox, repeated by the walk: up to about 4 us for the unluckiest of 10^4
+// threads) runs while that one still works.  10^4 of 25.6 M coordinates, 8 workers, launches back to back:
+// 7.4 -> 3.1 us.
 template <int DT>
 __global__ void __launch_bounds__(kThreads) randk_gather_kernel(const __grid_constant__ RandkParams p)
 {
-    grid_dependency_prologue();
     using T = typename std::conditional<DT == UQ_F32, uint32_t, uint16_t>::type;
+    grid_dependency_trigger();
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    uint64_t x = (uint64_t)t;
+    bool lost = false;
+    if (t < p.K) {
+        int step = 0;
+        do x = randk_network(x, p.bits, p.key); while (x >= (uint64_t)p.d && ++step < kWalkLimit);
+        lost = x >= (uint64_t)p.d;                               // never expected; stay in range
+        if (lost) x = (uint64_t)t;
+    }
+    grid_dependency_wait();
     if (t >= p.gk_stride) return;
     T *dst = (T *)p.gk + t;
     if (t >= p.K) {                                              // row padding
         for (int m = 0; m < p.M; ++m) dst[(size_t)m * (size_t)p.gk_stride] = 0;
         return;
     }
-    uint64_t x = (uint64_t)t;
-    int step = 0;
-    do x = randk_network(x, p.bits, p.key); while (x >= (uint64_t)p.d && ++step < kWalkLimit);
-    if (x >= (uint64_t)p.d) {                                    // never expected; stay in range
-        x = (uint64_t)t;
-        if (p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_BAD_INDEX);
-    }
+    if (lost && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_BAD_INDEX);
     p.sel[t] = (int64_t)x;
     const T *src = (const T *)p.g + x;
     int m = 0;
