@@ -28,12 +28,9 @@ cudaError_t launch_randk_scatter(int64_t d, int64_t K, const int64_t *sel, const
                                  float lr, uint32_t *status, cudaStream_t st);
 bool small_step_supported(const uq_layout &L, int fmt);
 size_t small_workspace_bytes();
-cudaError_t launch_small_step(const uq_layout &L, const void *g, int norm, int s, uint64_t seed, int rng_bits, int fmt,
-                              float *W, void *lev, float *out, int32_t *S, uint32_t *status, void *workspace,
-                              cudaStream_t st);
-cudaError_t launch_small_step_multi(const uq_layout &L, const void *g, int norm, const ScaleSet &scales, int idx_bits,
-                                    uint64_t seed, int rng_bits, int fmt, float *W, uint8_t *idx, void *lev, float *out,
-                                    int32_t *S, uint32_t *status, void *workspace, cudaStream_t st);
+cudaError_t launch_small_step(const uq_layout &L, const void *g, int norm, const ScaleSet &scales, int idx_bits,
+                              uint64_t seed, int rng_bits, int fmt, float *W, uint8_t *idx, void *lev, float *out,
+                              int32_t *S, uint32_t *status, void *workspace, cudaStream_t st);
 }  // namespace uq
 
 namespace {
@@ -355,11 +352,13 @@ int uq_step_small(const uq_layout *L, const void *g, int norm, int s, const int3
     if (!uq::small_step_supported(*L, fmt)) return UQ_ERR_UNSUPPORTED;
     if (workspace == nullptr || !aligned(workspace, 8) || workspace_bytes < uq_workspace_bytes_small())
         return UQ_ERR_WORKSPACE;
-    const cudaError_t e = scales != nullptr
-        ? uq::launch_small_step_multi(*L, g, norm, set, idx_bits, seed, rng_bits, fmt, W, idx, lev, out, S_opt, status,
-                                      workspace, (cudaStream_t)stream)
-        : uq::launch_small_step(*L, g, norm, s, seed, rng_bits, fmt, W, lev, out, S_opt, status, workspace,
-                                (cudaStream_t)stream);
+    if (scales == nullptr) {
+        set = single_scale(s);
+        idx_bits = 0;
+        idx = nullptr;
+    }
+    const cudaError_t e = uq::launch_small_step(*L, g, norm, set, idx_bits, seed, rng_bits, fmt, W, idx, lev, out, S_opt, status,
+                                                workspace, (cudaStream_t)stream);
     if (e == cudaErrorNotSupported) return UQ_ERR_UNSUPPORTED;
     return finish(e);
 }

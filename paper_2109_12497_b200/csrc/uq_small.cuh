@@ -1,15 +1,37 @@
-// Shared by the one-kernel steps of the two quantizers (uq_small.cu, uq_small_multi.cu): the kernel
-// parameters, the bounded grid-wide barrier and the scale agreement in front of it.
+// One whole step of either quantizer in ONE kernel, for gradients so small that the launches of the regular
+// step cost more than its arithmetic (Algorithm 1 / 2, lines "MaxAllReduce Norm" to "Reconstruct gradient";
+// one segment, at most 8 workers).
+//
+// A thread owns units of 8 coordinates of all workers, loads them once and keeps them in registers (8
+// unit-rows: UPT units of MW workers) across the scale agreement:
+//   phase 1  the norm accumulators of the workers, reduced over the CTA
+//   exchange the CTAs' partials: CLUSTER (8 or 16 CTAs): through distributed shared memory, behind the
+//            cluster barrier; otherwise a cooperative grid through the scratch, behind an arrival counter
+//            (zero when the kernel starts: the caller zeroes the scratch once, the last CTA through the
+//            barrier zeroes the counters again); that wait is bounded: a CTA that gives up sets
+//            UQ_STATUS_TIMEOUT and returns.  All warps add up the partials in the same fixed order, so all of
+//            them hold the same bits of W
+//   phase 2  [the shared indices from the maxima over the workers,] quantization of the workers' units, level
+//            rows, sums in packed lanes, average
+// Only a gradient with more units than the grid holds is read again in phase 2.  Levels, indices, sums and the
+// reconstruction are bit for bit those of the separate calls given the same W; W itself is summed in another
+// fixed order (L2: within one unit in the last place of the regular kernel's).
+//
+// What bounds it is latency: one trip to memory, the barrier, the chains of the Philox rounds.  Measured on a
+// B200, launches back to back (a grid with a counter in memory, every value loaded twice -> this form):
+// 4 x 4099 bf16, 8 scales 8.8 -> 5.2 us, 8 x 10^4 fp32 10.1 -> 6.8 us (one cluster); 2 x 2^20 fp32 10.9 -> 10.5 us.
 #pragma once
 #include "uq_device.cuh"
-#include "uq_unit.cuh"
 #include "uq_norm.cuh"
+#include "uq_select.cuh"
+#include "uq_unit.cuh"
 
 namespace uq {
 
 constexpr int kSmallMaxWorkers = 8;
 constexpr int kSmallHeader = 64;                  // bytes in front of the partials: arrival and departure counters
 constexpr uint32_t kSmallSpinLimit = 1u << 20;    // polls of the counter before a CTA gives up (about a second)
+constexpr int kSmallThreads = 512;                // most threads per CTA
 
 struct SmallParams {
     const void *g;
@@ -21,8 +43,9 @@ struct SmallParams {
     uint32_t *counter;        // scratch: [0] arrivals, [1] departures
     double *part;             // scratch: [gridDim.x][kSmallMaxWorkers]
     int64_t d, stride, coord0;
-    int32_t M, worker0, s, fmt;
-    ScaleSet scales;          // multi-scale only; s = scales.s[0] there
+    int32_t M, worker0, fmt, idx_bits;
+    int32_t rounds;           // units per thread / UPT, rounded up; 1: everything stays in registers
+    ScaleSet scales;          // single-scale: every entry is s
     PhiloxKey key;
 };
 
@@ -33,128 +56,402 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
     return v;
 }
 
-// Phase 1, the barrier and phase 2a of a one-kernel step: every thread adds its units into one norm
-// accumulator per worker, the CTAs exchange their partials through the scratch and every CTA adds
-// them up in the same order.  Returns false if the wait at the barrier ran out (the CTA must
-// return); otherwise W is the agreed scale, the same bits in every thread of the grid.
-// Must be called by all threads of every CTA of a cooperative grid.
-template <int DT, int NORM>
-__device__ __forceinline__ bool small_agree(const SmallParams &p, float &W_out)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// A double of CTA `rank`'s shared memory, at the place of `p` in mine.
+__device__ __forceinline__ double ld_cluster(const double *p, uint32_t rank)
 {
+    uint32_t a;
+    double v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void store_unit_any(int fmt, uint32_t lo, uint32_t hi, char *row, int64_t i)
+{
+    if (fmt == UQ_FMT_I8) store_unit<UQ_FMT_I8>(lo, hi, row + i, nullptr);
+    else if (fmt == UQ_FMT_I4X2) store_unit<UQ_FMT_I4X2>(lo, hi, row + (i >> 1), nullptr);
+    else store_unit<UQ_FMT_I2X4>(lo, hi, row + (i >> 2), nullptr);
+}
+
+// One warp: the sums of partials k = first, first + step, .. < n of each of MW workers (value(k, m)); lane L
+// ends with that of worker L % MW.  The order depends on the arguments only.
+template <int NORM, int MW, typename F> __device__ __forceinline__ double sum_partials(int first, int step, int n, F value)
+{
+    const int lane = threadIdx.x & 31, m = lane & (MW - 1);
+    constexpr int PARTS = 32 / MW;
+    double a = 0.0;
+    for (int k0 = first + step * (lane / MW); k0 < n; k0 += 4 * step * PARTS) {      // four loads in flight, added in order
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = k0 + k * step * PARTS < n ? value(k0 + k * step * PARTS, m) : 0.0;   // 0 is neutral for both norms
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a = combine<NORM>(a, v[k]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o >= MW; o >>= 1) a = combine<NORM>(a, __shfl_xor_sync(0xFFFFFFFFu, a, o));
+    return a;
+}
+
+// W from the workers' sums (lane L: worker L % MW).
+template <int NORM, int MW> __device__ __forceinline__ float scale_from_sums(double a, int M)
+{
+    const int m = threadIdx.x & (MW - 1);
+    const bool nan = __any_sync(0xFFFFFFFFu, m < M && a != a);            // (fmax drops a NaN)
+    double top = m < M ? a : 0.0;
+#pragma unroll
+    for (int o = MW / 2; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+    if (NORM == UQ_NORM_L2) return nan ? __uint_as_float(0x7FC00000u) : __double2float_rn(sqrt(top));
+    return __uint_as_float((uint32_t)top);
+}
+
+template <int DT, int NORM, int RNG, bool MULTI, bool CLUSTER, int MW>
+__global__ void __launch_bounds__(kSmallThreads, 1)
+small_step_kernel(const __grid_constant__ SmallParams p)
+{
+    if (CLUSTER) grid_dependency_prologue();
     using E = Elem<DT>;
-    constexpr int H = 8 / E::G;
-    constexpr int MW = kSmallMaxWorkers;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t nunits = (p.d + 7) >> 3;
-    const int64_t u0 = (int64_t)blockIdx.x * kThreads + tid, ustep = (int64_t)gridDim.x * kThreads;
-    __shared__ double sh[32][MW];
-    __shared__ float sh_w;
+    constexpr int H = 8 / E::G, UPT = kSmallMaxWorkers / MW;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int M = p.M, ib = p.idx_bits;
+    const int64_t d = p.d, nunits = (d + 7) >> 3;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + tid, T = (int64_t)gridDim.x * blockDim.x;
+    __shared__ double sh[kSmallThreads / 32][MW], sh2[kSmallThreads / 32][MW];
+    __shared__ double sh_part[MW];
     __shared__ int sh_fail;
 
-    // ---- phase 1: per-worker norm partials of my units
-    Acc<NORM> acc[MW];
-    for (int64_t u = u0; u < nunits; u += ustep) {
-        const int64_t i = u << 3;
-        const char *col = (const char *)p.g + (size_t)i * E::BYTES;
-        const int valid = (int)min((int64_t)8, p.d - i);
+    uint4 q[UPT][MW][H];
+    auto load = [&](int round) {
 #pragma unroll
-        for (int m = 0; m < MW; ++m) {
-            if (m < p.M) {
-                float v[8];
+        for (int k = 0; k < UPT; ++k) {
+            const int64_t u = (int64_t)(round * UPT + k) * T + t, i = u << 3;
+#pragma unroll
+            for (int m = 0; m < MW; ++m)
 #pragma unroll
                 for (int h = 0; h < H; ++h)
-                    E::unpack(ld_stream(col + ((size_t)m * (size_t)p.stride + h * E::G) * E::BYTES),
-                              *(float(*)[E::G])(v + h * E::G));
+                    q[k][m][h] = u < nunits && m < M
+                        ? ld_stream((const char *)p.g + ((size_t)m * (size_t)p.stride + (size_t)i + h * E::G) * E::BYTES) : make_uint4(0u, 0u, 0u, 0u);
+            if (u < nunits && i + 8 > d) {                             // the row's padding counts as zeros
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (e < valid) acc[m].add(v[e]);
+                for (int m = 0; m < MW; ++m)
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        uint32_t w[4] = {q[k][m][h].x, q[k][m][h].y, q[k][m][h].z, q[k][m][h].w};
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const int64_t e = i + h * E::G + c * (4 / E::BYTES);      // first coordinate of the word
+                            if (e >= d) w[c] = 0u;
+                            else if (DT == UQ_BF16 && e + 1 >= d) w[c] &= 0xFFFFu;
+                        }
+                        q[k][m][h] = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
             }
         }
-    }
+    };
+
+    // ---- phase 1: per-worker norm partials of my units
+    {
+        Acc<NORM> acc[MW];
+        for (int round = 0; round < p.rounds; ++round) {
+            load(round);
 #pragma unroll
-    for (int m = 0; m < MW; ++m) {
-        const double w = m < p.M ? warp_reduce<NORM>(acc[m].value()) : 0.0;     // uniform: idle workers cost nothing
-        if (lane == 0) sh[warp][m] = w;
+            for (int m = 0; m < MW; ++m)
+#pragma unroll
+                for (int k = 0; k < UPT; ++k)
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        float v[E::G];
+                        E::unpack(q[k][m][h], v);
+#pragma unroll
+                        for (int e = 0; e < E::G; ++e) acc[m].add(v[e]);
+                    }
+        }
+#pragma unroll
+        for (int m = 0; m < MW; ++m) {
+            const double w = m < M ? warp_reduce<NORM>(acc[m].value()) : 0.0;
+            if (lane == 0) sh[warp][m] = w;
+        }
     }
     __syncthreads();
     if (tid < MW) {
         double tot = sh[0][tid];
-        for (int k = 1; k < kWarps; ++k) tot = combine<NORM>(tot, sh[k][tid]);
-        p.part[(size_t)blockIdx.x * MW + tid] = tot;
+        for (int k = 1; k < nwarps; ++k) tot = combine<NORM>(tot, sh[k][tid]);
+        if (CLUSTER) sh_part[tid] = tot;
+        else p.part[(size_t)blockIdx.x * kSmallMaxWorkers + tid] = tot;
     }
 
-    // ---- the grid-wide barrier (bounded)
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();                  // release: this CTA's partials (ordered before the barrier above) before its arrival
-        atomicAdd(p.counter, 1u);
-        uint32_t polls = 0;
-        int fail = 0;
-        while (ld_acquire(p.counter) < gridDim.x) {
-            if (++polls > kSmallSpinLimit) { fail = 1; break; }
-            __nanosleep(32);
-        }
-        __threadfence();                  // acquire: the other CTAs' partials after their arrivals
-        if (fail) atomicOr(p.status, (uint32_t)UQ_STATUS_TIMEOUT);
-        sh_fail = fail;
-        // the last CTA to leave the barrier puts both counters back to zero for the next call
-        // (every CTA has read its last value of the arrival counter by then)
-        if (!fail && atomicAdd(p.counter + 1, 1u) == gridDim.x - 1) {
-            p.counter[1] = 0u;
-            __threadfence();
-            p.counter[0] = 0u;
-        }
-    }
-    __syncthreads();
-    if (sh_fail) return false;
-
-    // ---- phase 2a: W from all partials, in an order that depends on the grid size only
-    {
-        const int m = tid & (MW - 1), part = tid >> 3;             // 32 strided partial sums per worker
-        double a = 0.0;
-        for (unsigned c0 = part; c0 < gridDim.x; c0 += 32 * 10) {    // ten loads in flight, added in index order
-            double v[10];
-#pragma unroll
-            for (int k = 0; k < 10; ++k) {
-                const unsigned c = c0 + 32u * k;
-                v[k] = c < gridDim.x ? __ldcg(p.part + (size_t)c * MW + m) : 0.0;     // 0 is neutral for both norms
+    // ---- the exchange, and W
+    float W;
+    if (CLUSTER) {
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+        W = scale_from_sums<NORM, MW>(sum_partials<NORM, MW>(0, 1, (int)gridDim.x, [&](int c, int m) { return ld_cluster(sh_part + m, c); }), M);
+        cluster_arrive();                          // waited for at the end: my shared memory may be read until then
+    } else {
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();                  // release: this CTA's partials (ordered before the barrier above) before its arrival
+            atomicAdd(p.counter, 1u);
+            uint32_t polls = 0;
+            int fail = 0;
+            while (ld_acquire(p.counter) < gridDim.x) {
+                if (++polls > kSmallSpinLimit) { fail = 1; break; }
+                __nanosleep(32);
             }
-#pragma unroll
-            for (int k = 0; k < 10; ++k) a = combine<NORM>(a, v[k]);
+            __threadfence();                  // acquire: the other CTAs' partials after their arrivals
+            if (fail) atomicOr(p.status, (uint32_t)UQ_STATUS_TIMEOUT);
+            sh_fail = fail;
+            // the last CTA to leave the barrier puts both counters back to zero for the next call
+            // (every CTA has read its last value of the arrival counter by then)
+            if (!fail && atomicAdd(p.counter + 1, 1u) == gridDim.x - 1) {
+                p.counter[1] = 0u;
+                __threadfence();
+                p.counter[0] = 0u;
+            }
         }
-        sh[part][m] = a;
+        __syncthreads();
+        if (sh_fail) return;
+        // each warp every nwarps-th CTA's partials, then every warp all warps' sums
+        const double a = sum_partials<NORM, MW>(warp, nwarps, (int)gridDim.x,
+                                                [&](int c, int m) { return __ldcg(p.part + (size_t)c * kSmallMaxWorkers + m); });
+        if (lane < MW) sh2[warp][lane] = a;
+        __syncthreads();
+        W = scale_from_sums<NORM, MW>(sum_partials<NORM, MW>(0, 1, nwarps, [&](int w, int m) { return sh2[w][m]; }), M);
     }
-    __syncthreads();
-    if (tid < MW) {                                  // thread m: worker m's 32 sums in index order
-        double tot = sh[0][tid];
-        for (int k = 1; k < 32; ++k) tot = combine<NORM>(tot, sh[k][tid]);
-        sh[0][tid] = tot;                            // only thread m touches column m
-    }
-    __syncthreads();
-    if (tid == 0) {
-        bool nan = false;
-        double top = 0.0;
-        for (int m = 0; m < p.M; ++m) {
-            const double tot = sh[0][m];
-            nan |= tot != tot;
-            top = fmax(top, tot);
-        }
-        float w;
-        if (NORM == UQ_NORM_L2) w = nan ? __uint_as_float(0x7FC00000u) : __double2float_rn(sqrt(top));
-        else w = __uint_as_float((uint32_t)top);
-        sh_w = w;
-        if (blockIdx.x == 0) {
-            p.W[0] = w;
-            uint32_t flags = 0;
-            if (not_finite(w)) flags |= UQ_STATUS_NONFINITE;
-            if (not_finite(inv_scale(p.s, w))) flags |= UQ_STATUS_SCALE_OVERFLOW;
+
+    // ---- phase 2.  Lane k holds the factor s_k / W, the reconstruction factor W / (s_k * M) and the pass
+    // threshold of scale k (single-scale: every lane the same factors)
+    const float cap = (float)p.scales.s[0];
+    const int32_t s_lane = p.scales.s[lane & (UQ_MAX_SCALES - 1)];
+    const float inv_lane = inv_scale(s_lane, W), c_lane = decode_factor(W, s_lane, M);
+    if (blockIdx.x == 0 && warp == 0) {
+        const bool overflow = __any_sync(0xFFFFFFFFu, lane < p.scales.N && not_finite(inv_lane));
+        if (lane == 0) {
+            p.W[0] = W;
+            const uint32_t flags = (not_finite(W) ? UQ_STATUS_NONFINITE : 0u) | (overflow ? UQ_STATUS_SCALE_OVERFLOW : 0u);
             if (flags && p.status) atomicOr(p.status, flags);
         }
+        __syncwarp();
     }
-    __syncthreads();
-    W_out = sh_w;
-    return true;
+    int32_t thr = -1;
+    int top = 0;                                                        // the bisection's first step
+    if (MULTI) {
+        if (lane < p.scales.N) thr = pass_threshold(inv_lane, cap);
+        top = p.scales.N > 1 ? 1 << (31 - __clz(p.scales.N - 1)) : 0;
+        __syncwarp();
+    }
+    const size_t row_bytes = (size_t)(p.stride >> p.fmt);
+    for (int round = 0; round < p.rounds; ++round) {
+        if (p.rounds > 1) load(round);
+#pragma unroll
+        for (int k = 0; k < UPT; ++k) {
+            const int64_t u = (int64_t)(round * UPT + k) * T + t, i = u << 3;
+            const bool active = u < nunits;
+            if (!__any_sync(0xFFFFFFFFu, active)) break;                // the same for all lanes
+            float inv[8], c[8];
+            if (MULTI) {
+                // the shared indices from the maxima over the workers (see uq_select.cuh)
+                uint32_t amag[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) amag[e] = 0u;
+#pragma unroll
+                for (int m = 0; m < MW; ++m)
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        const uint32_t w[4] = {q[k][m][h].x, q[k][m][h].y, q[k][m][h].z, q[k][m][h].w};
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            if (DT == UQ_F32) amag[(4 * h + x) & 7] = max(amag[(4 * h + x) & 7], w[x] & 0x7FFFFFFFu);
+                            else {
+                                amag[(2 * x) & 7] = max(amag[(2 * x) & 7], (w[x] << 16) & 0x7FFFFFFFu);
+                                amag[(2 * x + 1) & 7] = max(amag[(2 * x + 1) & 7], w[x] & 0x7FFF0000u);
+                            }
+                        }
+                    }
+                uint64_t packed = 0;
+                int ks[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) ks[e] = 0;
+                for (int step = top; step >= 1; step >>= 1)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if ((int32_t)amag[e] <= __shfl_sync(0xFFFFFFFFu, thr, ks[e] + step)) ks[e] += step;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if (!active || i + e >= d) ks[e] = 0;                // padding keeps index 0
+                    packed |= (uint64_t)ks[e] << (e * ib);
+                    inv[e] = __shfl_sync(0xFFFFFFFFu, inv_lane, ks[e]);
+                    c[e] = __shfl_sync(0xFFFFFFFFu, c_lane, ks[e]);
+                }
+                if (active) {
+                    if (ib == 1) p.idx[i >> 3] = (uint8_t)packed;
+                    else if (ib == 2) *(uint16_t *)(p.idx + (i >> 2)) = (uint16_t)packed;
+                    else if (ib == 4) *(uint32_t *)(p.idx + (i >> 1)) = (uint32_t)packed;
+                    else *(uint64_t *)(p.idx + i) = packed;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) { inv[e] = inv_lane; c[e] = c_lane; }
+            }
+            if (active) {                                               // no warp-wide operation in here
+                const uint64_t blk = RNG == 32 ? (uint64_t)((p.coord0 + i) >> 2) : (uint64_t)((p.coord0 + i) >> 3);
+                int sum[2][2] = {{0, 0}, {0, 0}};                       // two levels share a word (see the encoder)
+#pragma unroll
+                for (int m = 0; m < MW; ++m) {
+                    if (m < M) {
+                        float v[8];
+#pragma unroll
+                        for (int h = 0; h < H; ++h) E::unpack(q[k][m][h], *(float(*)[E::G])(v + h * E::G));
+                        uint32_t neg_lo, neg_hi, w[2];
+                        unit_signs<DT>(q[k][m], neg_lo, neg_hi);
+                        quantize_unit_bytes<RNG>(v, inv, cap, neg_lo, neg_hi,
+                                                 unit_words<RNG>(p.key, (uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)(m + p.worker0)), w[0], w[1]);
+                        store_unit_any(p.fmt, w[0], w[1], (char *)p.lev + (size_t)m * row_bytes, i);
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) {
+                            sum[x][0] = __dp2a_lo(0x40000001, (int)w[x], sum[x][0]);
+                            sum[x][1] = __dp2a_hi(0x40000001, (int)w[x], sum[x][1]);
+                        }
+                    }
+                }
+                uint32_t s[8], r[8];
+#pragma unroll
+                for (int x = 0; x < 2; ++x)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int hi = (sum[x][h] + 0x2000) >> 14;
+                        s[4 * x + 2 * h + 1] = (uint32_t)hi;
+                        s[4 * x + 2 * h] = (uint32_t)(sum[x][h] - (hi << 14));
+                    }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) r[e] = __float_as_uint(__fmul_rn((float)(int)s[e], c[e]));
+                if (i + 8 <= d) {
+                    st_stream256(p.out + i, r);
+                    if (p.S != nullptr) st_stream256(p.S + i, s);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (i + e < d) {
+                            p.out[i + e] = __uint_as_float(r[e]);
+                            if (p.S != nullptr) p.S[i + e] = (int32_t)s[e];
+                        }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    if (CLUSTER) {
+        __syncwarp();
+        cluster_wait();
+    }
 }
+
+// ---------------------------------------------------------------------------------------------
+// launch
+// ---------------------------------------------------------------------------------------------
+constexpr int kSmallMaxCtas = 148 * 8 * 2;            // bound used to size the scratch (far above today's largest part)
+
+// CTAs of one instantiation that fit the device at once (cooperative launches need the whole grid resident);
+// looked up once per device and instantiation.
+template <typename K> static int resident_ctas(K kernel, int *cache)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (cache[dev] == 0) {
+        int sms = 0, per_sm = 0, coop = 0;
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kSmallThreads, 0);
+        cache[dev] = coop && sms > 0 && per_sm > 0 ? sms * per_sm : -1;
+    }
+    return cache[dev] > 0 ? cache[dev] : 0;
+}
+
+// The largest cluster that the device schedules: 16 CTAs (an opt-in) or the portable 8; once per device and
+// instantiation.
+template <typename K> static int cluster_ctas(K kernel, int *cache)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+    if (cache[dev] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(16);
+        cfg.blockDim = dim3(kSmallThreads);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0;
+        if (!ok) cudaGetLastError();
+        cache[dev] = ok ? 16 : 8;
+    }
+    return cache[dev];
+}
+
+template <int DT, int NORM, int RNG, bool MULTI, int MW>
+static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
+{
+    constexpr int UPT = kSmallMaxWorkers / MW;
+    const int64_t nunits = (p.d + 7) / 8;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    // One cluster, a unit per thread, while its few SMs take no longer than a grid over all of them loses in its
+    // barrier and its cooperative launch (about 3 us): a unit-row is 8 coordinates at about 35 cycles per warp
+    // and scheduler, so 40 k of them are 5.5 k cycles on 16 SMs.
+    if (nunits * p.M <= 40000 && nunits <= 8 * kSmallThreads) {
+        static int ccache[64] = {};
+        // one warp per scheduler of 8 SMs is not worth spreading further
+        const int ctas = nunits <= 8 * 128 ? 8 : cluster_ctas(small_step_kernel<DT, NORM, RNG, MULTI, true, MW>, ccache);
+        const int64_t want = (nunits + ctas - 1) / ctas;
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3((unsigned)max((want + 31) / 32 * 32, (int64_t)32));
+        p.rounds = 1;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)ctas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 2;
+        return cudaLaunchKernelEx(&cfg, small_step_kernel<DT, NORM, RNG, MULTI, true, MW>, p);
+    }
+    static int cache[64] = {};
+    const int resident = min(resident_ctas(small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, cache), kSmallMaxCtas);
+    if (resident <= 0) return cudaErrorNotSupported;
+    const int64_t per = (nunits + kSmallThreads - 1) / kSmallThreads;     // CTAs at one unit per thread
+    p.rounds = (int)((per + (int64_t)resident * UPT - 1) / ((int64_t)resident * UPT));
+    const int64_t units = (per + resident - 1) / resident;                // units per thread that the grid needs
+    cfg.gridDim = dim3((unsigned)min((int64_t)resident, (per + units - 1) / units));
+    cfg.blockDim = dim3(kSmallThreads);
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, p);
+}
+
+template <int DT, int NORM, int RNG, bool MULTI> static cudaError_t launch_small_workers(const SmallParams &p, cudaStream_t st)
+{
+    if (p.M <= 2) return launch_small_one<DT, NORM, RNG, MULTI, 2>(p, st);
+    if (p.M <= 4) return launch_small_one<DT, NORM, RNG, MULTI, 4>(p, st);
+    return launch_small_one<DT, NORM, RNG, MULTI, 8>(p, st);
+}
+
+template <int DT, int NORM> static cudaError_t launch_small_mode(const SmallParams &p, int rng_bits, cudaStream_t st)
+{
+    if (p.idx_bits != 0)
+        return rng_bits == 32 ? launch_small_workers<DT, NORM, 32, true>(p, st) : launch_small_workers<DT, NORM, 16, true>(p, st);
+    return rng_bits == 32 ? launch_small_workers<DT, NORM, 32, false>(p, st) : launch_small_workers<DT, NORM, 16, false>(p, st);
+}
+
+cudaError_t launch_small_f32(const SmallParams &p, int norm, int rng_bits, cudaStream_t st);
+cudaError_t launch_small_bf16(const SmallParams &p, int norm, int rng_bits, cudaStream_t st);
 
 }  // namespace uq
