@@ -375,6 +375,30 @@ int uq_step_small(const uq_layout *layout, const void *g, int norm, int s, const
                   void *stream);
 
 /*
+ * uq_step / uq_step_small for callers that make the same step over and over and to whom passing some twenty
+ * arguments every time is a cost (a scripting language's foreign-function interface): what stays the
+ * same between steps is gathered in a struct, and a step passes the gradients, the seed and the stream.
+ *   N           0: single-scale (Algorithm 1, s); else the number of entries of scales (Algorithm 2)
+ *   one_kernel  0: uq_step with workspace of uq_workspace_bytes(); 1: uq_step_small with its own kind
+ * The other fields are the arguments of those calls of the same names; the plan is only read.
+ * Errors: those of the call made; UQ_ERR_BAD_ARG also for a null plan or N outside 0..UQ_MAX_SCALES.
+ */
+typedef struct uq_step_plan {
+    uq_layout layout;
+    int32_t norm, s, N, idx_bits, rng_bits, fmt, one_kernel, reserved;
+    int32_t scales[UQ_MAX_SCALES];
+    float *W;
+    uint8_t *idx;
+    void *lev;
+    float *out;
+    int32_t *S_opt;
+    uint32_t *status;
+    void *workspace;
+    size_t workspace_bytes;
+} uq_step_plan;
+int uq_step_run(const uq_step_plan *plan, const void *g, uint64_t seed, void *stream);
+
+/*
  * GlobalRandKMaxNorm / GlobalRandKMaxNormMultiScale — Sections "GlobalRandKMaxNorm Compression"
  * and "GlobalRandKMaxNormMultiScale Compression": every worker keeps the same K coordinates,
  * chosen uniformly at every iteration, and the quantizer of Algorithm 1 / 2 runs on them.

@@ -29,7 +29,7 @@ EXPORTS = (
     "uq_workspace_bytes_small",
     "uq_agree_scale", "uq_agree_scale_static", "uq_encode_single", "uq_select_scale_multi", "uq_encode_multi",
     "uq_aggregate", "uq_decode", "uq_decode_update", "uq_randk_gather", "uq_randk_scatter", "uq_randk_update", "uq_index_min", "uq_decode_rows", "uq_select_encode_multi", "uq_encode_decode", "uq_select_encode_decode_multi", "uq_step",
-    "uq_step_small",
+    "uq_step_small", "uq_step_run",
 )
 
 
@@ -44,6 +44,15 @@ class uq_layout(C.Structure):
         ("worker0", C.c_int32),
         ("coord0", C.c_int64),
     ]
+
+
+class uq_step_plan(C.Structure):
+    """What stays the same between the steps of one configuration (uq_step_run)."""
+    _fields_ = ([("layout", uq_layout)]
+                + [(n, C.c_int32) for n in ("norm", "s", "N", "idx_bits", "rng_bits", "fmt", "one_kernel", "reserved")]
+                + [("scales", C.c_int32 * 16)]
+                + [(n, C.c_void_p) for n in ("W", "idx", "lev", "out", "S_opt", "status", "workspace")]
+                + [("workspace_bytes", C.c_size_t)])
 
 
 class UqError(RuntimeError):
@@ -80,6 +89,7 @@ def lib() -> C.CDLL:
         L.uq_agree_scale.argtypes = [LP, P, I, P, P, P, SZ, P]
         L.uq_step.argtypes = [LP, P, I, I, P, I, I, U64, I, I, P, P, P, P, P, P, P, SZ, P]
         L.uq_step_small.argtypes = [LP, P, I, I, P, I, I, U64, I, I, P, P, P, P, P, P, P, SZ, P]
+        L.uq_step_run.argtypes = [P, P, U64, P]
         L.uq_workspace_bytes_small.restype = SZ
         L.uq_workspace_bytes_small.argtypes = []
         L.uq_agree_scale_static.argtypes = [LP, P, I, P, P, P]

@@ -363,6 +363,15 @@ int uq_step_small(const uq_layout *L, const void *g, int norm, int s, const int3
     return finish(e);
 }
 
+int uq_step_run(const uq_step_plan *p, const void *g, uint64_t seed, void *stream)
+{
+    if (p == nullptr || p->N < 0 || p->N > UQ_MAX_SCALES) return UQ_ERR_BAD_ARG;
+    const int32_t *scales = p->N > 0 ? p->scales : nullptr;
+    return (p->one_kernel ? uq_step_small : uq_step)(&p->layout, g, p->norm, p->s, scales, p->N, p->idx_bits, seed, p->rng_bits,
+                                                     p->fmt, p->W, p->idx, p->lev, p->out, p->S_opt, p->status, p->workspace,
+                                                     p->workspace_bytes, stream);
+}
+
 int uq_index_min(const uint8_t *rows, int R, int64_t row_bytes, int64_t nbytes, int idx_bits, uint8_t *idx, void *stream)
 {
     if (R < 1 || R > UQ_MAX_WORKERS || nbytes < 0 || (nbytes & 3) != 0 || row_bytes < nbytes || (row_bytes & 3) != 0)

@@ -7,6 +7,7 @@ into the CUDA library.
 """
 from __future__ import annotations
 
+import ctypes as C
 from typing import Optional, Sequence
 
 import numpy as np
@@ -14,6 +15,9 @@ import torch
 
 from . import binding as B
 
+
+_current_device = torch._C._cuda_getDevice
+_raw_stream = torch._C._cuda_getCurrentRawStream
 
 ONE_KERNEL_MAX_BYTES = 8 << 20      # gradients of all workers up to this size take the one-kernel step
 
@@ -63,8 +67,8 @@ class Quantizer:
                     if self.multi else None)
         self.out = torch.empty(max(d, 1), dtype=torch.float32, device=dev)
         self.S = torch.empty(max(d, 1), dtype=torch.int32, device=dev) if keep_sums else None
-        self._small_call = None
-        self._step_call = None
+        self._plan = None                               # the step's arguments, gathered at the first step
+        self._g_shape = torch.Size((M, self.stride))
         self._out_view = self.out[: self.d]
 
     # the four stages, each one C-ABI call -------------------------------------------------------
@@ -122,35 +126,17 @@ class Quantizer:
 
     def step(self, g: torch.Tensor, seed: int = 0) -> torch.Tensor:
         """g: [M, stride] gradients of all workers -> the reconstructed average gradient [d]."""
-        if self.one_kernel:
-            # every buffer but g is this object's own: their addresses are marshalled once, not per
-            # step (the checked wrapper B.uq_step_small costs about as much host time as the kernel runs)
-            self._check_devices(g)
-            if self._small_call is None:
-                ptr = lambda t: None if t is None else t.data_ptr()
-                arr, N = B._scales(self.scales) if self.multi else (None, 0)
-                self._small_call = (B.lib().uq_step_small, self.layout.ref(), arr, N,
-                                    (ptr(self.W), ptr(self.idx), ptr(self.lev), ptr(self.out), ptr(self.S),
-                                     ptr(self.status), ptr(self.small_workspace), self.small_workspace.numel()))
-            fn, ref, arr, N, tail = self._small_call
-            rc = fn(ref, g.data_ptr(), self.norm, self.s, arr, N, self.idx_bits, seed, self.rng_bits, self.fmt, *tail,
-                    B._stream())
+        if self.one_kernel or self.fused_select is None:      # the library's sequence: one trip through the binding
+            # every buffer but g is this object's own: their addresses are gathered in a plan once, not marshalled
+            # per step (for small gradients the host's share of a step is as long as the GPU's)
+            plan = self._plan or self._make_plan()
+            index = g.get_device()
+            if not (g.shape == self._g_shape and g.dtype is self.dtype and g.is_contiguous() and index == self.device.index
+                    and index == _current_device()):
+                self._check_devices(g)
+            rc = plan[0](plan[1], g.data_ptr(), seed, _raw_stream(index))
             if rc != B.UQ_OK:
-                raise B.UqError("uq_step_small", rc)
-            return self._out_view
-        if self.fused_select is None:                         # the library's sequence: one trip through the binding (uq_step)
-            self._check_devices(g)
-            if self._step_call is None:                      # addresses of my own buffers, marshalled once
-                ptr = lambda t: None if t is None else t.data_ptr()
-                arr, N = B._scales(self.scales) if self.multi else (None, 0)
-                self._step_call = (B.lib().uq_step, self.layout.ref(), arr, N,
-                                   (ptr(self.W), ptr(self.idx), ptr(self.lev), ptr(self.out), ptr(self.S),
-                                    ptr(self.status), ptr(self.workspace), self.workspace.numel()))
-            fn, ref, arr, N, tail = self._step_call
-            rc = fn(ref, g.data_ptr(), self.norm, self.s, arr, N, self.idx_bits, seed, self.rng_bits, self.fmt, *tail,
-                    B._stream())
-            if rc != B.UQ_OK:
-                raise B.UqError("uq_step", rc)
+                raise B.UqError("uq_step_small" if self.one_kernel else "uq_step", rc)
             return self._out_view
         # the caller's choice of where selection runs, call by call
         self.agree_scale(g)
@@ -169,6 +155,18 @@ class Quantizer:
             self.encode(g, seed)
             self.aggregate_decode()
         return self.out[: self.d]
+
+    def _make_plan(self):
+        ptr = lambda t: None if t is None else t.data_ptr()
+        ws = self.small_workspace if self.one_kernel else self.workspace
+        p = B.uq_step_plan(layout=self.layout.c, norm=self.norm, s=self.s, N=len(self.scales) if self.multi else 0,
+                           idx_bits=self.idx_bits, rng_bits=self.rng_bits, fmt=self.fmt, one_kernel=int(self.one_kernel),
+                           W=ptr(self.W), idx=ptr(self.idx), lev=ptr(self.lev), out=ptr(self.out), S_opt=ptr(self.S),
+                           status=ptr(self.status), workspace=ptr(ws), workspace_bytes=ws.numel())
+        if self.multi:
+            p.scales[: p.N] = self.scales
+        self._plan = (B.lib().uq_step_run, C.addressof(p), p)
+        return self._plan
 
     def _check_devices(self, g: torch.Tensor) -> None:
         """The checks of the marshalling wrappers for the paths that call the library directly: the
@@ -214,9 +212,22 @@ class RandKQuantizer:
         self.sel = torch.empty(max(K, 1), dtype=torch.int64, device=dev)
         self.gk = torch.empty((M, self.inner.stride), dtype=dtype, device=dev)
         self.status = self.inner.status
+        self._g_shape = torch.Size((M, self.dense_layout.worker_stride))
+        self._tail = (self.sel.data_ptr(), self.gk.data_ptr(), self.gk.shape[1], self.status.data_ptr())
+
+    def _mine(self, t: torch.Tensor, dtype: torch.dtype) -> bool:
+        """Whether t is contiguous, of that type, and on this object's device, which is the current one (else
+        the marshalling wrappers are called, whose checks say what is wrong)."""
+        index = t.get_device()
+        return t.dtype is dtype and t.is_contiguous() and index == self.inner.device.index and index == _current_device()
 
     def gather(self, g: torch.Tensor, seed: int) -> None:
-        B.uq_randk_gather(self.dense_layout, g, self.K, seed, self.sel, self.gk, self.status)
+        if not (g.shape == self._g_shape and self._mine(g, self.dense_layout.dtype)):
+            B.uq_randk_gather(self.dense_layout, g, self.K, seed, self.sel, self.gk, self.status)
+            return
+        rc = B.lib().uq_randk_gather(self.dense_layout.ref(), g.data_ptr(), self.K, seed, *self._tail, _raw_stream(g.get_device()))
+        if rc != B.UQ_OK:
+            raise B.UqError("uq_randk_gather", rc)
 
     def quantize(self, seed: int) -> torch.Tensor:
         """Agree-scale, [select], encode, aggregate + reconstruct on the compact buffer -> [K] values."""
@@ -230,7 +241,13 @@ class RandKQuantizer:
         B.uq_randk_scatter(self.d, self.K, self.sel, None, out, self.status)
 
     def update(self, theta: torch.Tensor, lr: float) -> None:
-        B.uq_randk_update(self.d, self.K, self.sel, self.inner.out, theta, lr, self.status)
+        if not (theta.dim() == 1 and theta.shape[0] >= self.d and self._mine(theta, torch.float32)):
+            B.uq_randk_update(self.d, self.K, self.sel, self.inner.out, theta, lr, self.status)
+            return
+        rc = B.lib().uq_randk_update(self.d, self.K, self._tail[0], self.inner.out.data_ptr(), theta.data_ptr(), lr, self._tail[3],
+                                     _raw_stream(theta.get_device()))
+        if rc != B.UQ_OK:
+            raise B.UqError("uq_randk_update", rc)
 
     def step(self, g: torch.Tensor, out: torch.Tensor, seed: int = 0) -> torch.Tensor:
         """g: [M, stride] gradients -> out (dense [d], zero off the chosen set if it was zero before)."""

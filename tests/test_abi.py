@@ -149,6 +149,27 @@ def test_later_entry_points_reject_bad_arguments_on_the_host(lib):
     assert lib.uq_randk_update(100, 10, p, p, p, F(float("nan")), None, None) == B.UQ_ERR_BAD_ARG
 
 
+def test_step_plan_is_checked_on_the_host(lib):
+    """uq_step_run makes the call that its plan describes: the same argument checks, nothing launched."""
+    p = 0x10000
+    def plan(**kw):
+        f = dict(layout=_layout(), norm=B.UQ_NORM_L2, s=127, rng_bits=16, fmt=B.UQ_FMT_I8, W=p, lev=p, out=p, status=p, workspace=p,
+                 workspace_bytes=1 << 20)
+        f.update(kw)
+        return B.uq_step_plan(**f)
+    run = lambda q: lib.uq_step_run(C.addressof(q), p, 0, None)
+    assert lib.uq_step_run(None, p, 0, None) == B.UQ_ERR_BAD_ARG
+    assert run(plan(N=17)) == B.UQ_ERR_BAD_ARG and run(plan(N=-1)) == B.UQ_ERR_BAD_ARG
+    assert run(plan(layout=_layout(M=0))) == B.UQ_ERR_BAD_ARG
+    assert run(plan(workspace_bytes=8)) == B.UQ_ERR_WORKSPACE
+    assert run(plan(one_kernel=1, s=128)) == B.UQ_ERR_BAD_ARG
+    assert run(plan(one_kernel=1, workspace_bytes=64)) == B.UQ_ERR_WORKSPACE
+    assert run(plan(one_kernel=1, layout=_layout(M=9))) == B.UQ_ERR_UNSUPPORTED
+    multi = plan(one_kernel=1, N=2, idx_bits=3, idx=p)                                       # idx_bits
+    multi.scales[:2] = [127, 1016]
+    assert run(multi) == B.UQ_ERR_BAD_ARG
+
+
 def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", tmp_path / "missing.so")
