@@ -1,7 +1,7 @@
 // Shared scale W[j] = max_m || g^m on segment j ||   (Algorithm 1, line "MaxAllReduce Norm").
 //
-// Two launches.  (1) norm_partials: the coordinate axis is cut into fixed tiles of kNormTile
-// coordinates; the CTA of (tile t, worker m) reduces every segment that crosses its tile and
+// Two launches.  (1) norm_partials (a CTA per tile and worker) or norm_rows (a CTA per tile and four workers):
+// the coordinate axis is cut into fixed tiles of kNormTile coordinates; the CTA of (tile t, worker m) reduces every segment that crosses its tile and
 // stores one partial per (tile, segment) pair in slot t + j of worker m's scratch row.  Tiles and
 // segments are both ordered, so t + j is unique for every pair and the row needs
 // ntiles + nseg slots.  (2) norm_finalize: one CTA per segment adds that segment's slots in a
@@ -12,7 +12,8 @@
 
 namespace uq {
 
-constexpr int kSlab = 32768;       // tiles per grid.y step of the tile-major order (keeps grid.x below 2^31)
+constexpr int kNormItems = 4;      // rows of a tile that a CTA takes
+constexpr int kSlab = 32768;       // tiles per grid.y step (keeps grid.x below 2^31)
 
 template <int DT, int NORM>
 __global__ void __launch_bounds__(kThreads, 8)     // 32 registers: eight CTAs per SM keep HBM busy
@@ -103,6 +104,105 @@ norm_partials_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int 
     }
 }
 
+// The ragged last tile of a CTA's workers, inside one segment (out of line: one tile of the grid).
+template <int DT, int NORM>
+__device__ __noinline__ void norm_ragged_tile(const char *__restrict__ row, int64_t row_bytes, double *__restrict__ slot, int64_t slots,
+                                              int n, int64_t t0, int64_t t1)
+{
+    using E = Elem<DT>;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ double sh[kNormItems][kWarps];
+    for (int k = 0; k < n; ++k) {
+        Acc<NORM> acc;
+#pragma unroll 4
+        for (int64_t i = t0 + (int64_t)tid * E::G; i < t1; i += kThreads * E::G) {
+            float v[E::G];
+            E::unpack(ld_stream(row + k * row_bytes + i * E::BYTES), v);      // (rows are padded to whole vectors)
+#pragma unroll
+            for (int e = 0; e < E::G; ++e)
+                if (i + e < t1) acc.add(v[e]);
+        }
+        __syncwarp();
+        const double w = warp_reduce<NORM>(acc.value());
+        if (lane == 0) sh[k][warp] = w;
+    }
+    __syncthreads();
+    if (tid < n) {
+        double tot = sh[tid][0];
+        for (int x = 1; x < kWarps; ++x) tot = combine<NORM>(tot, sh[tid][x]);
+        slot[tid * slots] = tot;
+    }
+}
+
+// A CTA takes up to kNormItems workers' rows of one tile.  A full tile inside one segment (the common case) has no
+// bounds checks, one segment lookup and one barrier for all rows, and a vector's registers are filled again
+// with the next row's as soon as it is added.  (With a CTA per row and checked elements a binary32 element
+// cost 18 instructions, of which it needs 2.3: the kernel reached 0.95 of the copy peak in a burst and lost
+// a tenth of it at the board's power cap.)
+template <int DT, int NORM>
+__global__ void __launch_bounds__(kThreads, 4)
+norm_rows_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int M, int nseg,
+                 const int64_t *__restrict__ seg_off, int64_t ntiles, double *__restrict__ part)
+{
+    grid_dependency_prologue();
+    using E = Elem<DT>;
+    constexpr int UNITS = kNormTile / (kThreads * E::G);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // tiles front to back, a tile's groups of workers side by side (grid.x = groups * tiles of one slab of kSlab
+    // tiles, grid.y = slab): the kernel ends on the high coordinates of all workers, which the encoder reads first
+    const uint32_t groups = (uint32_t)(M + kNormItems - 1) / kNormItems;
+    const int m = (int)(blockIdx.x % groups) * kNormItems;
+    const int64_t tile = (int64_t)blockIdx.y * kSlab + blockIdx.x / groups;
+    if (tile >= ntiles) return;                                       // the last slab may be ragged
+    const int n = min(kNormItems, M - m);
+    const int64_t t0 = tile * kNormTile, t1 = min(t0 + (int64_t)kNormTile, d);
+    const int64_t row_bytes = stride * E::BYTES, slots = ntiles + nseg;
+    const char *row = (const char *)g + m * row_bytes;
+    double *prow = part + m * slots;
+    uint4 q[UNITS];
+    const char *p = row + (t0 + tid * E::G) * E::BYTES;
+    if (t1 - t0 == kNormTile) {
+#pragma unroll
+        for (int u = 0; u < UNITS; ++u) q[u] = ld_stream(p + u * (kThreads * 16));
+    }
+    const int j = warp_find_segment(seg_off, nseg, t0);
+    if (segment_end(seg_off, nseg, j, d) < t1) {
+        for (int k = 0; k < n; ++k) {
+            norm_mixed_tile<DT, NORM>(row + k * row_bytes, prow + k * slots, tile, t0, t1, d, nseg, seg_off);
+            __syncthreads();                                            // its shared memory is free again
+        }
+        return;
+    }
+    if (t1 - t0 != kNormTile) {
+        norm_ragged_tile<DT, NORM>(row, row_bytes, prow + tile + j, slots, n, t0, t1);
+        return;
+    }
+    __shared__ double sh[kNormItems][kWarps];
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+        p += row_bytes;
+        const bool more = k + 1 < n;
+        Acc<NORM> acc;
+#pragma unroll
+        for (int u = 0; u < UNITS; ++u) {
+            float v[E::G];
+            E::unpack(q[u], v);
+#pragma unroll
+            for (int e = 0; e < E::G; ++e) acc.add(v[e]);
+            if (more) q[u] = ld_stream(p + u * (kThreads * 16));
+        }
+        const double w = warp_reduce<NORM>(acc.value());
+        if (lane == 0) sh[k][warp] = w;
+    }
+    __syncthreads();
+    if (tid < n) {
+        double tot = sh[tid][0];
+#pragma unroll
+        for (int x = 1; x < kWarps; ++x) tot = combine<NORM>(tot, sh[tid][x]);
+        prow[tile + j + tid * slots] = tot;
+    }
+}
+
 // One CTA per segment: every worker's slots are added up by `nwarps / M` warps (at least one), eight loads in
 // flight per lane, in an order that depends on the launch's size only.  (With one warp per worker and the
 // loads one after the other a segment of 1600 tiles took 9.8 us, all of it load latency.)
@@ -175,12 +275,24 @@ static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t 
 {
     if (L.d > 0) {
         if (ntiles > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-        // fp32: tile-major order is 5 % faster on the layer-segmented workloads and neutral on the
-        // one-segment ones; bf16: it is 20 % slower than worker-major order
-        dim3 grid((unsigned)ntiles, (unsigned)L.M);
-        if (DT == UQ_F32)
-            grid = dim3((unsigned)L.M * (unsigned)min(ntiles, (int64_t)kSlab), (unsigned)((ntiles + kSlab - 1) / kSlab));
-        launch_k(norm_partials_kernel<DT, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
+        // binary32 takes several rows per CTA where that leaves eight waves and boundaries are rare (the rows of a
+        // tile that one crosses are worked through one after the other): 16 rows of 33.6 M coordinates 342 ->
+        // 300 us, 2 of 60 M 86 -> 71 us, sustained; with 161 segments in 25.6 M the slow tiles cost what the
+        // others gain.  bf16 does not: its conversions to binary64 (8 cycles each per warp and scheduler) bound
+        // it either way, and it wants a worker's row streamed front to back (13 M coordinates, 8 workers: 34 us
+        // against 42)
+        const int groups = (L.M + kNormItems - 1) / kNormItems;
+        if (DT == UQ_F32 && L.M > 1 && ntiles * groups >= 148 * 4 * 8 && (int64_t)L.nseg * 64 <= ntiles) {
+            const dim3 grid((unsigned)groups * (unsigned)min(ntiles, (int64_t)kSlab), (unsigned)((ntiles + kSlab - 1) / kSlab));
+            launch_k(norm_rows_kernel<UQ_F32, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.M, L.nseg, L.seg_off, ntiles, part);
+        } else {
+            // fp32: tile-major order is 5 % faster on the layer-segmented workloads and neutral on the
+            // one-segment ones; bf16: it is 20 % slower than worker-major order
+            dim3 grid((unsigned)ntiles, (unsigned)L.M);
+            if (DT == UQ_F32)
+                grid = dim3((unsigned)L.M * (unsigned)min(ntiles, (int64_t)kSlab), (unsigned)((ntiles + kSlab - 1) / kSlab));
+            launch_k(norm_partials_kernel<DT, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
+        }
     }
     // few long segments: more warps per worker
     const int threads = ntiles / L.nseg * L.M >= 2048 ? 1024 : kThreads;

@@ -1,0 +1,96 @@
+"""The sizes at which the library changes from one kernel, grid or access width to another, each side of the
+line against the CPU oracle (parity.py: integers and scale bits equal, values within its derived bound)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import uq_oracle as o
+from paper_2109_12497_b200 import binding as B
+from paper_2109_12497_b200 import workloads as wl
+from parity import _check_parity, check_parity, ulp_distance
+
+pytestmark = pytest.mark.gpu
+
+
+# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 40 000 unit-rows and 4096 units,
+# a cooperative grid above, and more than one pass per thread (values read again) beyond one unit per register set
+@pytest.mark.parametrize("M,d", [(2, 8 * 1024), (2, 8 * 1024 + 1), (2, 8 * 4096), (2, 8 * 4096 + 1), (8, 8 * 4096 - 7),
+                                 (3, 8 * 4097), (1, 8 * 4096), (8, 8 * 148 * 512 + 1), (8, 2 * 8 * 148 * 512 + 9)])
+@pytest.mark.parametrize("dtype,scales,rng_bits", [(wl.F32, (127,), 16), (wl.BF16, (7, 56), 32), (wl.F32, (7, 56, 448), 32),
+                                                   (wl.BF16, (127,), 16)])
+def test_one_kernel_step_at_the_edges_of_its_grids(M, d, dtype, scales, rng_bits):
+    w = wl.scaled("c3" if len(scales) > 1 else "c1", d, M=M, dtype=dtype, norm=wl.NORM_L2, fmt="i8", s=scales[0],
+                  scales=scales, idx_bits=2, rng_bits=rng_bits, segments="one", seed=d)
+    assert _check_parity(w, wl.generate(w), None, "one")["q"].one_kernel
+
+
+# many workers of a small gradient: separate kernels up to 148 * 4 * 256 coordinates and above 24 workers
+@pytest.mark.parametrize("M", [24, 25, 64])
+@pytest.mark.parametrize("d", [148 * 4 * 256, 148 * 4 * 256 + 1])
+@pytest.mark.parametrize("name", ["c2", "c3"])
+def test_many_workers_of_a_small_gradient(name, d, M):
+    w = wl.scaled(name, d, M=M)
+    check_parity(w, wl.generate(w))
+
+
+# norms of large binary32 gradients: four workers' rows per CTA from 148 * 4 * 8 groups of a tile of 8192
+# coordinates, with few segments; one row per CTA below.  Maximum exact, Euclidean within one unit in the last place
+@pytest.mark.parametrize("M", [2, 5, 8])
+@pytest.mark.parametrize("extra", [-8192, 0, 8192 + 1])
+@pytest.mark.parametrize("nseg", [1, 7])
+def test_norms_of_large_gradients(M, extra, nseg):
+    groups = (M + 3) // 4
+    d = (148 * 4 * 8 // groups) * 8192 + extra
+    stride = (d + 31) // 32 * 32
+    g = torch.randn(M, stride, device="cuda", generator=torch.Generator("cuda").manual_seed(d + M))
+    seg = None if nseg == 1 else np.array([0, 5, 8192, 8192, 16384 * 3 + 1, d // 2, d - 3, d], dtype=np.int64)
+    lay = B.Layout(M, d, stride, torch.float32, None if seg is None else torch.from_numpy(seg).cuda())
+    W, status = torch.empty(nseg, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(lay.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    g_np = g.cpu().numpy()[:, :d]
+    for norm, onorm, ulps in ((B.UQ_NORM_LINF, o.NORM_LINF, 0), (B.UQ_NORM_L2, o.NORM_L2, 1)):
+        B.uq_agree_scale(lay, g, norm, W, status, ws)
+        assert ulp_distance(W.cpu().numpy(), o.agree_scale(g_np, seg, onorm)).max() <= ulps
+    assert int(status.item()) == 0
+
+
+# shared index: 16-, 8- and 4-byte accesses by alignment and length, each number of rows that is unrolled, and more
+@pytest.mark.parametrize("offset", [0, 4, 8])
+@pytest.mark.parametrize("nbytes", [4, 8, 12, 16, 4096 + 4, 65536 + 16])
+@pytest.mark.parametrize("R", [1, 2, 3, 4, 5, 9])
+def test_index_min_access_widths(offset, nbytes, R):
+    rng = np.random.default_rng(nbytes + R)
+    raw = rng.integers(0, 4, size=(R, nbytes * 4), dtype=np.uint8)
+    flat = torch.zeros(offset + R * (nbytes + 2 * offset), dtype=torch.uint8, device="cuda")     # row pitch as aligned as the base
+    rows = flat[offset:].view(R, nbytes + 2 * offset)
+    rows[:, :nbytes] = torch.from_numpy(np.stack([o.pack_index(r, 2) for r in raw])).cuda()
+    idx = torch.full((nbytes + 32,), 0xEE, dtype=torch.uint8, device="cuda")
+    B.uq_index_min(rows, 2, idx[offset: offset + nbytes], nbytes=nbytes)
+    got = idx.cpu().numpy()
+    assert np.array_equal(got[offset: offset + nbytes], o.pack_index(o.index_min(raw), 2))
+    assert (got[:offset] == 0xEE).all() and (got[offset + nbytes:] == 0xEE).all()
+
+
+# the levels alone: the workers are dealt out in groups of eight over the grid
+@pytest.mark.parametrize("M", [7, 8, 9, 17])
+@pytest.mark.parametrize("fmt,s", [("i8", 127), ("i6p", 31), ("i4x2", 7), ("i2x4", 1)])
+def test_levels_alone_of_many_workers(M, fmt, s):
+    w = wl.scaled("c2", 70_001, M=M, fmt=fmt, s=s, scales=(s,))
+    check_parity(w, wl.generate(w))
+
+
+# update of parameters: with 2- and 4-bit levels a thread requests its parameters before the sums; coordinates
+# around one thread's 32 and one CTA's share, and none at all in the last vector
+@pytest.mark.parametrize("d", [1, 31, 32, 33, 8191, 8193])
+@pytest.mark.parametrize("fmt,s", [("i2x4", 1), ("i4x2", 7), ("i6p", 31), ("i8", 127)])
+def test_update_at_the_edges_of_its_vectors(d, fmt, s):
+    w = wl.scaled("c1", d, M=8, fmt=fmt, s=s, scales=(s,))
+    g_np = wl.generate(w)
+    r = _check_parity(w, g_np, None, "separate")
+    q = r["q"]
+    theta = torch.ones(d + 16, device="cuda")
+    mom = torch.full((d + 16,), 0.5, device="cuda")
+    B.uq_decode_update(q.layout, q.lev, q.fmt, q.W, q.s, q.scales, None, 0, theta[8: 8 + d], mom[8: 8 + d], 0.1, 0.9, 5e-4, None)
+    want, want_m = o.sgd_update(r["ref"]["out"], np.ones(d, np.float32), np.full(d, 0.5, np.float32), lr=0.1, mu=0.9, wd=5e-4)
+    assert np.array_equal(theta.cpu().numpy()[8: 8 + d], want) and np.array_equal(mom.cpu().numpy()[8: 8 + d], want_m)
+    assert (theta[:8] == 1).all() and (theta[8 + d:] == 1).all() and (mom[8 + d:] == 0.5).all()
