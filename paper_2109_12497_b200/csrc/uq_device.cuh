@@ -370,18 +370,18 @@ __device__ __forceinline__ uint32_t level_draw23(float x, uint32_t word)
 constexpr uint32_t kLevelByte23 = 0;      // which byte of the returned word holds the level
 
 // The same level from the fixed-point form of x (the fast path of the encoder).  inv23 = inv * 2^23
-// and cap23 = cap * 2^23, both exact, so |v| * inv23 = x * 2^23 with the rounding of x (the caller
+// and cap23 = cap * 2^23, both exact, so xs = v * inv23 = +- x * 2^23 with the rounding of x (the caller
 // checks that inv23 is finite; a product below the normal range gives threshold 0 either way), and
 //   T = rint(min(x, cap) * 2^23) = floor(x) * 2^23 + rint(p * 2^23)
 // by one conversion (ties to even; x >= 1 is a multiple of 2^-23, so only p < 1 is rounded, and a
 // p that rounds up to 1 carries into the level, as it must: then every draw rounds up).  With
 // r = word >> 9 the level is L = (T + 2^23 - 1 - r) >> 23 = ceil((T - r) / 2^23), so
-// -L = floor((r - T) / 2^23).  The function converts the negated product (-T, exactly) and returns
+// -L = floor((r - T) / 2^23).  The function converts the negated magnitude (-T, exactly) and returns
 // y = 2 (-T) + (word >> 8) = 2 (r - T) + (0 or 1): byte 3 of y is -L as a two's-complement byte
 // (-127 .. 0), the stray low bit changes no floor.  negated_bytes_to_signed puts the signs on.
-__device__ __forceinline__ uint32_t level_draw23_fixed(float v, float inv23, float cap23, uint32_t word)
+__device__ __forceinline__ uint32_t level_draw23_fixed(float xs, float cap23, uint32_t word)
 {
-    const uint32_t Tn = (uint32_t)__float2int_rn(fmaxf(__fmul_rn(-fabsf(v), inv23), -cap23));
+    const uint32_t Tn = (uint32_t)__float2int_rn(fmaxf(-fabsf(xs), -cap23));
     return Tn + Tn + (word >> 8);
 }
 constexpr uint32_t kLevelByte23Fixed = 3;
@@ -411,6 +411,15 @@ __device__ __forceinline__ float mul_sat(float a, float b)
     float d;
     asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
     return d;
+}
+// Two products by one instruction.  (It has no absolute values: the sign comes off in the clamp, which does.)
+__device__ __forceinline__ void mul_pair(float a0, float a1, float b0, float b1, float &r0, float &r1)
+{
+    uint64_t a, b, r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "f"(a0), "f"(a1));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(b0), "f"(b1));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r0), "=f"(r1) : "l"(r));
 }
 __device__ __forceinline__ float add_sat(float a, float b)
 {

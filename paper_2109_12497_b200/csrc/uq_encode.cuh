@@ -243,26 +243,32 @@ struct LevelConstants {
 // One worker's unit (q) turned into signed level bytes: w[k] holds four levels (see LevelOrder).
 // 16-bit draws: the random words come complemented; with h' = 2^16 - 1 - h the carry out of
 // rint(p * 2^16) + h' is the rounding decision, and one dp2a picks the half word and adds it.
+// 32-bit draws: half an instruction per coordinate less with the products taken in pairs (8 workers, 25.6 M
+// coordinates, binary32: 238 -> 230.6 us; 13.1 M bf16: 97.2 -> 95.1 us).
 template <int DT, int FMT, int RNG>
 __device__ __forceinline__ void quantize_fast(const uint4 *q, const float (&inv)[8], const LevelConstants &lc, const uint4 *r,
                                               uint32_t (&w)[2])
 {
     using E = Elem<DT>;
     using O = LevelOrder<DT, FMT>;
-    float v[8];
+    float v[8], x[8];
 #pragma unroll
     for (int h = 0; h < 8 / E::G; ++h) E::unpack(q[h], *(float(*)[E::G])(v + h * E::G));
+    if (RNG == 32) {
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) mul_pair(v[e], v[e + 1], inv[e], inv[e + 1], x[e], x[e + 1]);
+    }
     uint32_t z[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         if (RNG == 16) {
-            const uint4 x = r[0];
-            const uint32_t word = (e >> 1) == 0 ? x.x : (e >> 1) == 1 ? x.y : (e >> 1) == 2 ? x.z : x.w;
+            const uint4 b = r[0];
+            const uint32_t word = (e >> 1) == 0 ? b.x : (e >> 1) == 1 ? b.y : (e >> 1) == 2 ? b.z : b.w;
             z[e] = __dp2a_lo(word, (e & 1) ? 0x100u : 0x1u, __float_as_uint(add_sat(mul_sat(fabsf(v[e]), inv[e]), lc.c0)));
         } else {
-            const uint4 x = r[e >> 2];
-            const uint32_t word = (e & 3) == 0 ? x.x : (e & 3) == 1 ? x.y : (e & 3) == 2 ? x.z : x.w;
-            z[e] = level_draw23_fixed(v[e], inv[e], lc.cap23, word);
+            const uint4 b = r[e >> 2];
+            const uint32_t word = (e & 3) == 0 ? b.x : (e & 3) == 1 ? b.y : (e & 3) == 2 ? b.z : b.w;
+            z[e] = level_draw23_fixed(x[e], lc.cap23, word);
         }
     }
 #pragma unroll
