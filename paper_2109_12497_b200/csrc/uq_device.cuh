@@ -539,16 +539,18 @@ __device__ __forceinline__ float decode_factor(float W, int32_t s, int M)
 
 // Largest non-negative binary32 bit pattern t with fl(t * inv) <= s_hat, or -1 if not even 0
 // passes.  fl(t * inv) is non-decreasing in t, so "passes" is a prefix of the magnitudes and the
-// test |v| * inv <= s_hat is the integer compare bits(|v|) <= t.  The quotient s_hat / inv lands
-// within a few units of the answer; the two bounded loops settle it exactly.
+// test |v| * inv <= s_hat is the integer compare bits(|v|) <= t.  A product passes up to s_hat plus half a unit in
+// the last place (s_hat, a level count, is even there), which moves the bound by at most one unit of t, and the
+// quotient s_hat / inv is within half a unit: the answer is b - 1, b or b + 1.  (With two loops that walked to it and the
+// factors shuffled by the packed index the selecting encoders were 1 to 2 % slower.)
 __device__ __forceinline__ int32_t pass_threshold(float inv, float s_hat)
 {
     if (!(inv > 0.0f)) return inv == 0.0f ? 0x7F7FFFFF : -1;       // W = 0: every finite value passes
     if (!(__fmul_rn(0.0f, inv) <= s_hat)) return -1;                // inv = Inf: 0 * Inf is NaN
-    int32_t b = __float_as_int(fminf(__fdiv_rn(s_hat, inv), 3.402823466e38f));
-    for (int it = 0; it < 64 && b < 0x7F7FFFFF && __fmul_rn(__int_as_float(b + 1), inv) <= s_hat; ++it) ++b;
-    for (int it = 0; it < 64 && b >= 0 && !(__fmul_rn(__int_as_float(b), inv) <= s_hat); ++it) --b;
-    return b;
+    const int32_t b = __float_as_int(fminf(__fdiv_rn(s_hat, inv), 3.402823466e38f));
+    const bool up = b < 0x7F7FFFFF && __fmul_rn(__int_as_float(b + 1), inv) <= s_hat;
+    const bool ok = __fmul_rn(__int_as_float(b), inv) <= s_hat;
+    return up ? b + 1 : ok ? b : b - 1;
 }
 
 }  // namespace uq

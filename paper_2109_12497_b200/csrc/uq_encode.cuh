@@ -397,6 +397,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         const float edge = MULTI ? __shfl_sync(0xFFFFFFFFu, inv_lane, RNG == 16 ? 0 : p.v.scales.N - 1) : inv_lane;
         slow = RNG == 16 ? !sat_form_exact(edge) : !fixed_form_exact(edge);
     }
+    float inv[8];
     if (SEL && !slow) {
         // Scale selection and sharing (Algorithm 2 lines "Compute coordinate scales" and "Scale sharing"): the
         // largest magnitude over the workers decides the shared index (see uq_select.cuh), found by bisection
@@ -475,8 +476,12 @@ encode_kernel(const __grid_constant__ EncodeParams p)
                 for (int e = 0; e < 8; ++e)
                     if ((int32_t)amag[e] <= __shfl_sync(0xFFFFFFFFu, thr, k[e] + step)) k[e] += step;
             }
+            const float f = __fmul_rn(inv_lane, RNG == 16 ? 0.00390625f : 8388608.0f);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) kw[e >> 2] |= (uint32_t)k[e] << ((e & 3) * ib);
+            for (int e = 0; e < 8; ++e) {
+                kw[e >> 2] |= (uint32_t)k[e] << ((e & 3) * ib);
+                inv[e] = __shfl_sync(0xFFFFFFFFu, f, k[e]);
+            }
         } else {
             kw[0] = mixed_row_select(p, i, j, amag[0], amag[1], amag[2], amag[3]);
             kw[1] = mixed_row_select(p, i + 4, j, amag[4], amag[5], amag[6], amag[7]);
@@ -491,8 +496,9 @@ encode_kernel(const __grid_constant__ EncodeParams p)
 
     // the factors of my coordinates.  The shuffle reads its source lane modulo 32 and the table repeats every
     // 2^ib lanes: the index needs no mask
-    float inv[8];
-    if (!mixed) {
+    if (!mixed && SEL && !slow) {
+        // known from the selection
+    } else if (!mixed) {
         inv_lane = __fmul_rn(inv_lane, RNG == 16 ? 0.00390625f : 8388608.0f);
 #pragma unroll
         for (int e = 0; e < 8; ++e)
