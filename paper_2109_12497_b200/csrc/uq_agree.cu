@@ -1,7 +1,7 @@
 // Shared scale W[j] = max_m || g^m on segment j ||   (Algorithm 1, line "MaxAllReduce Norm").
 //
-// Two launches.  (1) norm_partials (a CTA per tile and worker) or norm_rows (a CTA per tile and four workers):
-// the coordinate axis is cut into fixed tiles of kNormTile coordinates; the CTA of (tile t, worker m) reduces every segment that crosses its tile and
+// Two launches.  (1) norm_partials (a CTA per tile and worker), norm_rows (a CTA per tile and four workers) or
+// norm_row_warps (a warp per row, which is then the tile): the coordinate axis is cut into fixed tiles of kNormTile coordinates; the CTA of (tile t, worker m) reduces every segment that crosses its tile and
 // stores one partial per (tile, segment) pair in slot t + j of worker m's scratch row.  Tiles and
 // segments are both ordered, so t + j is unique for every pair and the row needs
 // ntiles + nseg slots.  (2) norm_finalize: one CTA per segment adds that segment's slots in a
@@ -13,6 +13,7 @@
 namespace uq {
 
 constexpr int kNormItems = 4;      // rows of a tile that a CTA takes
+constexpr int kNormRow = 256;      // coordinates per partial where a warp takes a row
 constexpr int kSlab = 32768;       // tiles per grid.y step (keeps grid.x below 2^31)
 
 template <int DT, int NORM>
@@ -203,6 +204,54 @@ norm_rows_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int M, i
     }
 }
 
+// Small gradients in several segments: a warp per row of kNormRow coordinates and worker, 8 coordinates per lane.
+// What bounds them is latency: with tiles of 8192 coordinates a layer table crosses nearly every tile, and a
+// warp then walks its pieces one after the other, each with a trip to memory.  Here a row's values and its first
+// 32 boundaries arrive together and the pieces of a row cost one warp reduction each.  Norms of 8 workers in 161
+// layers: 12 778 coordinates 27.5 -> 9.8 us, 100 003 14.6 -> 9.7 us, 255 570 11.9 -> 9.7 us.
+template <int DT, int NORM>
+__global__ void __launch_bounds__(kThreads)
+norm_row_warps_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int nseg, const int64_t *__restrict__ seg_off,
+                      int64_t nrows, double *__restrict__ part)
+{
+    grid_dependency_prologue();
+    using E = Elem<DT>;
+    constexpr int V = 8 / E::G;
+    const int lane = threadIdx.x & 31, m = blockIdx.y;
+    const int64_t row = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    if (row >= nrows) return;
+    const int64_t r0 = row * kNormRow, r1 = min(r0 + (int64_t)kNormRow, d), i = r0 + lane * 8;
+    const char *p = (const char *)g + ((size_t)m * (size_t)stride + (size_t)i) * E::BYTES;
+    uint4 q[V];
+#pragma unroll
+    for (int h = 0; h < V; ++h) q[h] = i < d ? ld_stream(p + h * 16) : make_uint4(0, 0, 0, 0);    // (rows are padded)
+    double *slot = part + (size_t)m * (size_t)(nrows + nseg) + row;
+    int j = warp_find_segment(seg_off, nseg, r0);
+    int64_t ends = segment_end(seg_off, nseg, min(j + lane, nseg - 1), d);      // lane l: where segment j0 + l ends
+    float v[8];
+#pragma unroll
+    for (int h = 0; h < V; ++h) E::unpack(q[h], *(float(*)[E::G])(v + h * E::G));
+    int64_t a = r0;
+    for (int k = 0; a < r1; ++j, ++k) {                            // the pieces of my row; j stays below nseg:
+        if (k == 32) {
+            ends = segment_end(seg_off, nseg, min(j + lane, nseg - 1), d);
+            k = 0;
+        }
+        const int64_t end = __shfl_sync(0xFFFFFFFFu, ends, k);
+        const int64_t b = j >= nseg - 1 ? r1 : min(max(end, a), r1);             // the last one takes the rest
+        if (b > a) {
+            const int lo = (int)max((int64_t)0, min((int64_t)8, a - i)), hi = (int)max((int64_t)0, min((int64_t)8, b - i));
+            Acc<NORM> acc;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (e >= lo && e < hi) acc.add(v[e]);
+            const double w = warp_reduce<NORM>(acc.value());
+            if (lane == 0) slot[j] = w;
+        }
+        a = b;
+    }
+}
+
 // One CTA per segment: every worker's slots are added up by `nwarps / M` warps (at least one), eight loads in
 // flight per lane, in an order that depends on the launch's size only.  (With one warp per worker and the
 // loads one after the other a segment of 1600 tiles took 9.8 us, all of it load latency.)
@@ -269,11 +318,22 @@ norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg
     }
 }
 
+// A warp per row: up to 16384 rows of all workers (24 000 of them 14.2 us by tiles and 14.4 by rows, 62 000 18.2 and
+// 29.3), in segments of 64 coordinates or more on average (a row has one slot, and a segment one, in the scratch:
+// M * (16384 / M + d / 64) of them stay below what the tiles of larger gradients take).
+static bool by_rows(const uq_layout &L)
+{
+    return L.nseg > 1 && (int64_t)L.nseg * 64 <= L.d && (L.d + kNormRow - 1) / kNormRow * L.M <= 16384;
+}
+
 template <int DT, int NORM>
 static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t *status, double *part,
                           int64_t ntiles, cudaStream_t st)
 {
-    if (L.d > 0) {
+    if (L.d > 0 && by_rows(L)) {
+        launch_k(norm_row_warps_kernel<DT, NORM>, dim3((unsigned)((ntiles + kWarps - 1) / kWarps), (unsigned)L.M), kThreads, st,
+                 g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
+    } else if (L.d > 0) {
         if (ntiles > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
         // binary32 takes several rows per CTA where that leaves eight waves and boundaries are rare (the rows of a
         // tile that one crosses are worked through one after the other): 16 rows of 33.6 M coordinates 342 ->
@@ -297,16 +357,20 @@ static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t 
     // few long segments: more warps per worker
     const int threads = ntiles / L.nseg * L.M >= 2048 ? 1024 : kThreads;
     launch_k(norm_finalize_kernel<NORM>, L.nseg, threads, st, part, L.M, L.d, L.nseg, L.seg_off, ntiles, W,
-                                                          status, kNormTile);
+             status, by_rows(L) ? kNormRow : kNormTile);
     return cudaGetLastError();
 }
 
-int64_t norm_tiles(int64_t d) { return (d + kNormTile - 1) / kNormTile; }
+int64_t norm_tiles(const uq_layout &L)
+{
+    const int64_t tile = by_rows(L) ? kNormRow : kNormTile;
+    return (L.d + tile - 1) / tile;
+}
 
 cudaError_t launch_agree_scale(const uq_layout &L, const void *g, int norm, float *W, uint32_t *status,
                                void *workspace, cudaStream_t st)
 {
-    const int64_t ntiles = norm_tiles(L.d);
+    const int64_t ntiles = norm_tiles(L);
     double *part = (double *)workspace;
     if (L.dtype == UQ_F32)
         return norm == UQ_NORM_L2 ? launch<UQ_F32, UQ_NORM_L2>(L, g, W, status, part, ntiles, st)

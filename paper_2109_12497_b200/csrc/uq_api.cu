@@ -3,7 +3,7 @@
 #include "uq_device.cuh"
 
 namespace uq {
-int64_t norm_tiles(int64_t d);
+int64_t norm_tiles(const uq_layout &L);
 cudaError_t launch_agree_scale(const uq_layout &L, const void *g, int norm, float *W, uint32_t *status,
                                void *workspace, cudaStream_t st);
 cudaError_t launch_encode(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
@@ -127,7 +127,7 @@ const char *uq_error_string(int code)
 size_t uq_workspace_bytes(const uq_layout *L)
 {
     if (!layout_ok(L)) return 0;
-    return (size_t)L->M * (size_t)(uq::norm_tiles(L->d) + L->nseg) * sizeof(double);
+    return (size_t)L->M * (size_t)(uq::norm_tiles(*L) + L->nseg) * sizeof(double);
 }
 
 size_t uq_index_bytes(const uq_layout *L, int idx_bits)

@@ -54,6 +54,29 @@ def test_norms_of_large_gradients(M, extra, nseg):
     assert int(status.item()) == 0
 
 
+# norms of small gradients in segments: a warp per row of 256 coordinates; empty segments, segments of one
+# coordinate, more than 32 pieces in a row, boundaries around a row's end, a ragged last row; and both sides of the
+# line at 16384 rows
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("M,d,cuts", [
+    (3, 20_003, [*range(1, 81), 255, 256, 256, 256, 257, 511, 513, 1024, 5000, 5003, 20_000, 20_002]),
+    (1, 128, [128]), (2, 257, [256]), (7, 4_096, [8, 8, 4_095]),
+    (4, 256 * 4096, [3, 700_001]), (4, 256 * 4096 + 1, [3, 700_001]),
+])
+def test_norms_of_small_gradients_in_segments(dtype, M, d, cuts):
+    seg = np.array([0, *cuts, d], dtype=np.int64)
+    stride = (d + 31) // 32 * 32
+    g = torch.randn(M, stride, device="cuda", generator=torch.Generator("cuda").manual_seed(d)).to(dtype)
+    lay = B.Layout(M, d, stride, dtype, torch.from_numpy(seg).cuda())
+    W, status = torch.empty(len(seg) - 1, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.full((lay.workspace_bytes(),), 0xFF, dtype=torch.uint8, device="cuda")
+    g_np = (g if dtype == torch.float32 else g.view(torch.uint16)).cpu().numpy()[:, :d]
+    for norm, onorm, ulps in ((B.UQ_NORM_LINF, o.NORM_LINF, 0), (B.UQ_NORM_L2, o.NORM_L2, 1)):
+        B.uq_agree_scale(lay, g, norm, W, status, ws)
+        assert ulp_distance(W.cpu().numpy(), o.agree_scale(g_np, seg, onorm)).max() <= ulps
+    assert int(status.item()) == 0
+
+
 # shared index: 16-, 8- and 4-byte accesses by alignment and length, each number of rows that is unrolled, and more
 @pytest.mark.parametrize("offset", [0, 4, 8])
 @pytest.mark.parametrize("nbytes", [4, 8, 12, 16, 4096 + 4, 65536 + 16])
