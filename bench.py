@@ -42,7 +42,7 @@ FALLBACK_HBM_GBS = 6650.0          # earlier measurement on this machine, used only
 # bytes per coordinate * d, since every byte of these kernels belongs to a coordinate.
 # Keyed by (workload, kernel); absent = not captured.
 NCU_TRAFFIC_BYTES_PER_COORD = {
-    ("c5", "select_encode_decode"): 27.64,   # profiles/kernel_select_encode_decode_c5_small_ncu.md: 1381.8 MB for d = 50,000,000
+    ("c5", "select_encode_decode"): 27.68,   # profiles/kernel_select_encode_decode_c5_small_ncu.md: 1384.0 MB for d = 50,000,000
     ("c5", "encode_decode"): 27.39,   # profiles/kernel_encode_decode_c5_small_ncu.md: 1369.4 MB for d = 50,000,000
     ("c5", "encode"): 23.39,      # profiles/kernel_encode_c5_small_ncu.md: 1169.7 MB for d = 50,000,000
     ("c2", "encode"): 38.15,      # profiles/kernel_encode_c2_rng32_ncu.md: 975.7 MB at full size (d = 25,557,032)
@@ -54,7 +54,7 @@ NCU_TRAFFIC_BYTES_PER_COORD = {
 # pipe's peak: 16 lanes per scheduler (measured: such an instruction occupies its scheduler's pipe for
 # 2 cycles), 4 schedulers per SM, 148 SMs, at the SM clock sampled during the run.
 NCU_ALU_OPS_PER_COORD_WORKER = {
-    ("c5", "select_encode_decode"): 9.99,    # profiles/kernel_select_encode_decode_c5_small_ncu.md
+    ("c5", "select_encode_decode"): 8.37,    # profiles/kernel_select_encode_decode_c5_small_ncu.md
 }
 ALU_LANES_PER_SM = 64
 SM_COUNT = 148
@@ -159,18 +159,10 @@ class ClockSampler:
 # GPU arm
 # ---------------------------------------------------------------------------------------------
 
-def encoder_decodes(w) -> bool:
-    """Whether the step's encoder also aggregates and reconstructs (uq_encode_decode as one kernel:
-    int8 levels, 16-bit draws, at most 8 workers; pipeline.Quantizer.fused_decode says the same of its object)."""
-    return w.fmt == "i8" and w.M <= 8 and w.rng_bits == 16
-
-
 def stages_of(w):
-    """The calls uq_step makes for this workload (without the integer sums among its outputs)."""
-    if w.quantizer == "multi" and encoder_decodes(w):
-        return ["agree_scale", "select_encode_decode"]      # the encoder also selects: two calls do the step
-    head = ["agree_scale", "select_scale"] if w.quantizer == "multi" else ["agree_scale"]
-    return head + (["encode_decode"] if encoder_decodes(w) else ["encode", "aggregate_decode"])
+    """The calls uq_step makes for this workload (without the integer sums among its outputs): the encoder also
+    selects, aggregates and reconstructs, whatever the wire format."""
+    return ["agree_scale", "select_encode_decode" if w.quantizer == "multi" else "encode_decode"]
 
 
 def stage_calls(q, g):
@@ -373,15 +365,9 @@ def time_two_kernel_tail(q, g, w, reps):
 
 
 def time_fused_select_encode(q, g, w, reps):
-    """Multi-scale: mean ms of selection + encoding as one call (uq_select_encode_multi: one kernel
-    for M <= 8; the step runs the two streaming kernels), timed alone."""
+    """Multi-scale: mean ms of selection + encoding as one call (uq_select_encode_multi: one kernel),
+    timed alone."""
     return time_alone(lambda k: q.select_encode(g, w.seed + k), reps)
-
-
-def time_fused_select_encode_decode(q, g, w, reps):
-    """Multi-scale: mean ms of everything behind the scale agreement as one call
-    (uq_select_encode_decode_multi), timed alone."""
-    return time_alone(lambda k: q.select_encode_decode(g, w.seed + k), reps)
 
 
 def time_graph_replay(q, g, w, reps, stats=False):
@@ -584,9 +570,6 @@ def bench_workload(w, steps, warmup, barrier, threads, want_e2e, flush_between=F
     res["update_ms"] = time_fused_update(q, w, min(steps, 10))
     if q.multi:
         res["fused_select_ms"] = time_fused_select_encode(q, g_dev, w, min(steps, 10))
-        if q.fused_decode and not q.one_kernel and "select_encode_decode" not in res["stages_ms"]:
-            time.sleep(BURST_IDLE_S)
-            res["fused_all_ms"] = time_fused_select_encode_decode(q, g_dev, w, min(steps, 10))
     if randk_K:
         res["randk"] = time_randk(w, g_dev, min(randk_K, w.d), 50)
         if w.quantizer == "single":               # the same choice quantized with a two-scale set (GlobalRandK-MN-TS)
@@ -629,7 +612,7 @@ def summarize(res, peak_gbs):
     out = {"gradient_GBps": w.in_bytes / res["ms"] / 1e6, "ms_per_step": res["ms"],
            "step_roofline": step_roofline(w, res["ms"], peak_gbs), "kernels": {}}
     if res["q"].one_kernel:
-        out["step_form"] = ("one cooperative kernel (uq_step_small): ms_per_step is that kernel; the entries under "
+        out["step_form"] = ("one kernel (uq_step_small): ms_per_step is that kernel; the entries under "
                             "kernels are the separate calls, timed one by one for comparison")
     for s, ms in res["stages_ms"].items():
         gbs = ab[s] / ms / 1e6
@@ -675,40 +658,20 @@ def summarize(res, peak_gbs):
                 "selection + encoding + aggregation + reconstruction as one kernel: the gradients are read once and "
                 "nothing is read back; bound by instruction issue (ALU pipe), not by memory, so its fraction of the HBM "
                 "peak is lower than that of the streaming kernels it replaces (timed alone beside it), and its time shorter")
-    if "fused_select_ms" in res:
+    if "fused_select_ms" in res and "two_kernel_tail_ms" in res:
         ms = res["fused_select_ms"]
         sel = res["stages_ms"].get("select_scale", res.get("alone_ms", {}).get("select_scale", 0.0))
-        if "select_encode_decode" in res["stages_ms"]:      # the step already selects inside its second call
-            enc_alone, dec_alone = res["two_kernel_tail_ms"]
-            two = sel + enc_alone
-            step_with = res["ms"] - res["stages_ms"]["select_encode_decode"] + ms + dec_alone
-        elif "two_kernel_tail_ms" in res:       # the step's tail is one kernel: compare with selector + encoder alone
-            enc_alone, dec_alone = res["two_kernel_tail_ms"]
-            two = sel + enc_alone
-            step_with = res["ms"] - sel - res["stages_ms"]["encode_decode"] + ms + dec_alone
-        else:
-            two = sel + res["stages_ms"].get("encode", 0.0)
-            step_with = res["ms"] - two + ms
+        enc_alone, dec_alone = res["two_kernel_tail_ms"]    # the step already selects inside its second call
+        two = sel + enc_alone
+        step_with = res["ms"] - res["stages_ms"]["select_encode_decode"] + ms + dec_alone
         out["kernels"]["select_encode"] = {
             "ms": round(ms, 5), "algorithmic_MB": round(ab["select_encode"] / 1e6, 2),
             "GBps": round(ab["select_encode"] / ms / 1e6, 1),
             "frac_of_hbm_peak": round(ab["select_encode"] / ms / 1e6 / peak_gbs, 4),
             "ms_of_the_two_kernels_it_replaces": round(two, 5),
             "gradient_GBps_of_a_step_with_it": round(w.in_bytes / step_with / 1e6, 1),
-            "note": "selection + encoding as one call (one kernel for M <= 8: the gradients are read once; bound by "
+            "note": "selection + encoding as one call (one kernel: the gradients are read once; bound by "
                     "instruction issue, not by memory), timed alone, not part of the step"}
-    if "fused_all_ms" in res:
-        ms = res["fused_all_ms"]
-        nbytes = ab["select_encode"] + 4 * w.d
-        two = res["stages_ms"]["select_scale"] + res["stages_ms"]["encode_decode"]
-        out["kernels"]["select_encode_decode"] = {
-            "ms": round(ms, 5), "algorithmic_MB": round(nbytes / 1e6, 2), "GBps": round(nbytes / ms / 1e6, 1),
-            "frac_of_hbm_peak": round(nbytes / ms / 1e6 / peak_gbs, 4),
-            "ms_of_the_two_kernels_it_replaces": round(two, 5),
-            "gradient_GBps_of_a_step_with_it": round(w.in_bytes / (res["ms"] - two + ms) / 1e6, 1),
-            "note": "selection + encoding + aggregation + reconstruction as one call (uq_select_encode_decode_multi: one "
-                    "kernel, the gradients are read once and nothing is read back; bound by instruction issue, not by "
-                    "memory), timed alone, not part of the step"}
     lev = {"i8": 1.0, "i4x2": 0.5, "i2x4": 0.25, "i6p": 0.75}[w.fmt]
     upd_bytes = lev * w.M * w.d + w.idx_bits / 8.0 * w.d + 16 * w.d      # levels, index, theta and momentum r/w
     ms = res["update_ms"]
@@ -957,8 +920,8 @@ def gpu_main(args):
         mhz = (clocks or {}).get("sm_mhz") or 1965.0
         alu_peak = SM_COUNT * ALU_LANES_PER_SM * mhz * 1e6
         alu_rate = alu_ops * w.M * w.d / (res["stages_ms"][dom] * 1e-3)
-        line["roofline"]["limiter"] = ("ALU pipe and instruction issue, not memory (ncu on a smaller case: ALU pipe 70 %, "
-                                       "DRAM 49 % busy); the streaming kernels whose work it does are timed alone under "
+        line["roofline"]["limiter"] = ("ALU pipe and instruction issue, not memory (ncu on a smaller case: ALU pipe 64 %, "
+                                       "integer-multiply pipe 57 %, 0.75 instructions issued per cycle); the streaming kernels whose work it does are timed alone under "
                                        "kernels: select_scale, encode, aggregate_decode")
         line["roofline"]["alu"] = {"achieved": round(alu_rate / 1e12, 2), "peak": round(alu_peak / 1e12, 2),
                                    "unit": "T ALU-pipe thread instructions/s", "frac": round(alu_rate / alu_peak, 4),
