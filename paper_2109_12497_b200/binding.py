@@ -123,18 +123,24 @@ def require_current_device(index: Optional[int], current: int, what: str = "tens
                          f"make its device current first (torch.cuda.device / set_device)")
 
 
+_current_device = torch._C._cuda_getDevice
+
+
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
-    if not t.is_cuda:
+    index = t.get_device()
+    if index < 0:
         raise ValueError("uq: tensors must live on a CUDA device")
-    require_current_device(t.device.index, torch.cuda.current_device())
+    if index != _current_device():                # asked directly: the public wrappers around it and around the
+                                                  # tensor's device made a call of eight tensors 1.3 us slower
+        require_current_device(index, torch.cuda.current_device())
     return t.data_ptr()
 
 
 def _stream() -> int:
     """The raw handle of the current stream of the current CUDA device."""
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return torch._C._cuda_getCurrentRawStream(_current_device())
 
 
 def _check(fn: str, code: int) -> None:
