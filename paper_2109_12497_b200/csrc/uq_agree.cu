@@ -252,11 +252,14 @@ norm_row_warps_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int
     }
 }
 
-// One CTA per segment: every worker's slots are added up by `nwarps / M` warps (at least one), eight loads in
-// flight per lane, in an order that depends on the launch's size only.  (With one warp per worker and the
-// loads one after the other a segment of 1600 tiles took 9.8 us, all of it load latency.)
+// One CTA per segment, one warp per worker: lane l adds up the slots of the segment's tiles l, l + 32, .. one after
+// the other, and then the lanes' sums are added.  That order depends on the segment's tiles alone: a worker's sum has
+// the same bits whatever else is in the buffer.  What bounds it is the latency of the loads, of which a lane has eight
+// in flight.  (Several warps fetching a worker's slots into shared memory for the one that adds: 1 worker 14.9 -> 13.4
+// us, 2 to 4 workers no faster, and with 40 KB of it the kernel in front, beside whose CTAs these start, took 4 %
+// longer; norms of 25.6 M bf16 coordinates in one segment.)
 template <int NORM>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(512)
 norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg,
                      const int64_t *__restrict__ seg_off, int64_t ntiles, float *__restrict__ W,
                      uint32_t *__restrict__ status, int tile_coords)       // tile_coords: coordinates per partial
@@ -270,26 +273,21 @@ norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg
     a = min(max(a, (int64_t)0), d);
     b = min(max(b, a), d);
 
-    __shared__ double sh[UQ_MAX_WORKERS + 32];                             // [worker][warp of the worker]
-    const int share = max(nwarps / M, 1);                                   // warps per worker
-    const int sub = warp % share;
-    if (a < b) {
-        const int first = (int)(a / tile_coords), last = (int)((b - 1) / tile_coords), step = 32 * share;
-        for (int m = warp / share; m < M; m += max(nwarps / share, 1)) {
-            const double *prow = part + (size_t)m * (size_t)(ntiles + nseg) + j;
-            double acc = 0.0;
-            for (int t = first + sub * 32 + lane; t <= last; t += 8 * step) {
-                double v[8];
+    __shared__ double sh[UQ_MAX_WORKERS];
+    const int first = (int)(a / tile_coords), last = a < b ? (int)((b - 1) / tile_coords) : first - 1;
+    for (int m = warp; m < M; m += nwarps) {
+        const double *prow = part + (size_t)m * (size_t)(ntiles + nseg) + j;
+        double acc = 0.0;
+        for (int t = first + lane; t <= last; t += 32 * 8) {
+            double v[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = t + k * step <= last ? __ldcg(prow + t + k * step) : 0.0;    // 0 is neutral for both norms
+            for (int k = 0; k < 8; ++k) v[k] = t + k * 32 <= last ? __ldcg(prow + t + k * 32) : 0.0;      // 0 is neutral for both norms
 #pragma unroll
-                for (int k = 0; k < 8; ++k) acc = combine<NORM>(acc, v[k]);
-            }
-            const double r = warp_reduce<NORM>(acc);
-            if (lane == 0) sh[m * share + sub] = r;
+            for (int k = 0; k < 8; ++k) acc = combine<NORM>(acc, v[k]);
         }
-    } else {
-        for (int k = tid; k < M * share; k += blockDim.x) sh[k] = 0.0;
+        __syncwarp();
+        const double r = warp_reduce<NORM>(acc);
+        if (lane == 0) sh[m] = r;
     }
     __syncthreads();
     if (warp == 0) {
@@ -297,10 +295,8 @@ norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg
         bool nan = false;
         double top = 0.0;
         for (int m = lane; m < M; m += 32) {
-            double tot = sh[m * share];
-            for (int k = 1; k < share; ++k) tot = combine<NORM>(tot, sh[m * share + k]);
-            nan |= tot != tot;
-            top = fmax(top, tot);
+            nan |= sh[m] != sh[m];
+            top = fmax(top, sh[m]);
         }
         nan = __any_sync(0xFFFFFFFFu, nan);
 #pragma unroll
@@ -354,10 +350,9 @@ static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t 
             launch_k(norm_partials_kernel<DT, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
         }
     }
-    // few long segments: more warps per worker
-    const int threads = ntiles / L.nseg * L.M >= 2048 ? 1024 : kThreads;
-    launch_k(norm_finalize_kernel<NORM>, L.nseg, threads, st, part, L.M, L.d, L.nseg, L.seg_off, ntiles, W,
-             status, by_rows(L) ? kNormRow : kNormTile);
+    // segments of more than eight loads per lane: 16 workers side by side
+    launch_k(norm_finalize_kernel<NORM>, L.nseg, ntiles / L.nseg >= 256 ? 32 * min(L.M, 16) : kThreads, st, part, L.M, L.d, L.nseg,
+             L.seg_off, ntiles, W, status, by_rows(L) ? kNormRow : kNormTile);
     return cudaGetLastError();
 }
 

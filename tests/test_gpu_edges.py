@@ -77,6 +77,25 @@ def test_norms_of_small_gradients_in_segments(dtype, M, d, cuts):
     assert int(status.item()) == 0
 
 
+# a worker's squares are added in an order that does not depend on how many other workers the buffer holds.  One tile's
+# squares sum to (2^24 + 1)^2, whose root lies half way between two binary32 values (the even one is 2^24); the
+# other squares are 2^-6, a quarter of the last place of that sum: added to it one by one, as lane 0 of the tiles 0, 32,
+# 64, .. does, they vanish, and added among themselves first they would tip the root to 2^24 + 2
+@pytest.mark.parametrize("M", [1, 2, 3, 8, 16, 17])
+def test_order_of_a_sum_does_not_depend_on_the_number_of_workers(M):
+    d = 32 * 32 * 8192 + 7
+    stride = (d + 31) // 32 * 32
+    g = torch.zeros(M, stride, dtype=torch.bfloat16, device="cuda")
+    g[:-1] = 0.5
+    g[-1, :4] = torch.tensor([2.0 ** 24, 2.0 ** 12, 2.0 ** 12, 1.0])
+    g[-1, 32 * 8192:: 32 * 8192] = 0.125
+    W, status = torch.empty(1, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    lay = B.Layout(M, d, stride, torch.bfloat16)
+    ws = torch.empty(lay.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    B.uq_agree_scale(lay, g, B.UQ_NORM_L2, W, status, ws)
+    assert float(W.item()) == 2.0 ** 24 and int(status.item()) == 0
+
+
 # shared index: 16-, 8- and 4-byte accesses by alignment and length, each number of rows that is unrolled, and more
 @pytest.mark.parametrize("offset", [0, 4, 8])
 @pytest.mark.parametrize("nbytes", [4, 8, 12, 16, 4096 + 4, 65536 + 16])
