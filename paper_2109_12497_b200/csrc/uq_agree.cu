@@ -1,19 +1,24 @@
 // Shared scale W[j] = max_m || g^m on segment j ||   (Algorithm 1, line "MaxAllReduce Norm").
 //
-// Two launches.  (1) norm_partials (a CTA per tile and worker), norm_rows (a CTA per tile and four workers) or
-// norm_row_warps (a warp per row, which is then the tile): the coordinate axis is cut into fixed tiles of kNormTile coordinates; the CTA of (tile t, worker m) reduces every segment that crosses its tile and
+// Two launches.  (1) norm_partials, norm_rows (large binary32 gradients: a CTA takes a tile of four workers) or
+// norm_staged (small gradients in segments): the coordinate axis is cut into fixed tiles of kNormTile coordinates; the
+// CTA of (tile t, worker m) reduces every segment that crosses its tile and
 // stores one partial per (tile, segment) pair in slot t + j of worker m's scratch row.  Tiles and
 // segments are both ordered, so t + j is unique for every pair and the row needs
 // ntiles + nseg slots.  (2) norm_finalize: one CTA per segment adds that segment's slots in a
 // fixed order, takes the max over workers, and writes W[j].  The summation tree depends only on
 // (d, seg_off), never on the grid or on timing, so W is reproducible bit for bit.
+#include <type_traits>
+
 #include "uq_device.cuh"
 #include "uq_norm.cuh"
 
 namespace uq {
 
 constexpr int kNormItems = 4;      // rows of a tile that a CTA takes
-constexpr int kNormRow = 256;      // coordinates per partial where a warp takes a row
+constexpr int kStagedTiles = 512;  // most tiles of all workers that norm_staged_kernel takes (where few boundaries cross many tiles it
+                                   // loses: 1.5 M coordinates in 3 segments, 8 workers 10.9 -> 11.6 us)
+constexpr int kDealtTiles = 256;   // and that it gives two warps per chunk: more CTAs than that fill the GPU (100 003 coordinates, 16 workers: 9.1 us with two, 9.0 with one)
 constexpr int kSlab = 32768;       // tiles per grid.y step (keeps grid.x below 2^31)
 
 template <int DT, int NORM>
@@ -204,51 +209,124 @@ norm_rows_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int M, i
     }
 }
 
-// Small gradients in several segments: a warp per row of kNormRow coordinates and worker, 8 coordinates per lane.
-// What bounds them is latency: with tiles of 8192 coordinates a layer table crosses nearly every tile, and a
-// warp then walks its pieces one after the other, each with a trip to memory.  Here a row's values and its first
-// 32 boundaries arrive together and the pieces of a row cost one warp reduction each.  Norms of 8 workers in 161
-// layers: 12 778 coordinates 27.5 -> 9.8 us, 100 003 14.6 -> 9.7 us, 255 570 11.9 -> 9.7 us.
-template <int DT, int NORM>
-__global__ void __launch_bounds__(kThreads)
-norm_row_warps_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int nseg, const int64_t *__restrict__ seg_off,
-                      int64_t nrows, double *__restrict__ part)
+// Small gradients in several segments.  What bounds them is latency: a layer table crosses nearly every tile, and a
+// warp that walks the pieces of its chunk in memory makes a trip there for every few of them.  Here the whole tile
+// is on its way to shared memory while the segment is looked up, the pieces are walked there, and the pieces of a
+// chunk are dealt out to WPC warps.  The additions are those of norm_partials_kernel in the same order, so which of the
+// two runs is a matter of speed alone.  Norms of 8 binary32 workers in 161 layers, both kernels, launches without gaps,
+// by norm_partials_kernel / here with one / with two warps per chunk: 20 011 coordinates 15.0 / 11.1 / 9.2 us, 100 003
+// 10.8 / 7.6 / 7.0 us, 400 003 14.8 / 8.9 / 8.9 us.
+template <int DT, int NORM, int WPC>
+__global__ void __launch_bounds__(kThreads * WPC)
+norm_staged_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int nseg, const int64_t *__restrict__ seg_off,
+                   int64_t ntiles, double *__restrict__ part)
 {
     grid_dependency_prologue();
     using E = Elem<DT>;
-    constexpr int V = 8 / E::G;
-    const int lane = threadIdx.x & 31, m = blockIdx.y;
-    const int64_t row = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
-    if (row >= nrows) return;
-    const int64_t r0 = row * kNormRow, r1 = min(r0 + (int64_t)kNormRow, d), i = r0 + lane * 8;
-    const char *p = (const char *)g + ((size_t)m * (size_t)stride + (size_t)i) * E::BYTES;
-    uint4 q[V];
+    using T = typename std::conditional<DT == UQ_F32, float, uint16_t>::type;
+    constexpr int VECS = kNormTile / E::G, UNITS = VECS / kThreads, CHUNK = kNormTile / kWarps;
+    __shared__ uint4 stage[VECS];
+    __shared__ double sh_head[kWarps], sh_tail[kWarps];                  // as in norm_mixed_tile
+    __shared__ int sh_head_seg[kWarps], sh_tail_seg[kWarps], sh_head_open[kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t tile = blockIdx.x, t0 = tile * kNormTile, t1 = min(t0 + (int64_t)kNormTile, d);
+    const char *row = (const char *)g + (size_t)blockIdx.y * (size_t)stride * E::BYTES;
+    double *prow = part + (size_t)blockIdx.y * (size_t)(ntiles + nseg);
+    const uint32_t sp = (uint32_t)__cvta_generic_to_shared(stage);
 #pragma unroll
-    for (int h = 0; h < V; ++h) q[h] = i < d ? ld_stream(p + h * 16) : make_uint4(0, 0, 0, 0);    // (rows are padded)
-    double *slot = part + (size_t)m * (size_t)(nrows + nseg) + row;
-    int j = warp_find_segment(seg_off, nseg, r0);
-    int64_t ends = segment_end(seg_off, nseg, min(j + lane, nseg - 1), d);      // lane l: where segment j0 + l ends
-    float v[8];
-#pragma unroll
-    for (int h = 0; h < V; ++h) E::unpack(q[h], *(float(*)[E::G])(v + h * E::G));
-    int64_t a = r0;
-    for (int k = 0; a < r1; ++j, ++k) {                            // the pieces of my row; j stays below nseg:
-        if (k == 32) {
-            ends = segment_end(seg_off, nseg, min(j + lane, nseg - 1), d);
-            k = 0;
+    for (int v = tid; v < VECS; v += kThreads * WPC)                             // (rows are padded to whole vectors)
+        if (t0 + v * E::G < t1) copy_async16(sp + v * 16, row + (t0 + v * E::G) * E::BYTES);
+    if (tid < kWarps) sh_head_seg[tid] = sh_tail_seg[tid] = -1;
+    const int chunk = warp / WPC, sub = warp % WPC;
+    const int64_t c0 = t0 + (int64_t)chunk * CHUNK, c1 = min(c0 + CHUNK, t1);
+    const int jt = warp_find_segment(seg_off, nseg, t0);
+    int64_t ends = segment_end(seg_off, nseg, min(jt + lane, nseg - 1), d);                     // lane l: where segment jt + l ends
+    const int64_t start = __ldg(seg_off + jt);
+    const bool uniform = __shfl_sync(0xFFFFFFFFu, ends, 0) >= t1;
+    int j0 = jt, base = jt;                                         // my chunk's first segment, and lane 0's
+    int64_t seg_b = start;                                                                      // and where the one before it ends
+    if (!uniform && c0 < c1) {
+        const int before = __popc(__ballot_sync(0xFFFFFFFFu, ends <= c0 && jt + lane < nseg - 1));
+        if (before == 32) {
+            j0 = warp_find_segment(seg_off, nseg, c0);
+            seg_b = __ldg(seg_off + j0);
+        } else {
+            j0 = jt + before;
+            if (before > 0) seg_b = __shfl_sync(0xFFFFFFFFu, ends, before - 1);
         }
-        const int64_t end = __shfl_sync(0xFFFFFFFFu, ends, k);
-        const int64_t b = j >= nseg - 1 ? r1 : min(max(end, a), r1);             // the last one takes the rest
-        if (b > a) {
-            const int lo = (int)max((int64_t)0, min((int64_t)8, a - i)), hi = (int)max((int64_t)0, min((int64_t)8, b - i));
-            Acc<NORM> acc;
+        if (j0 - jt >= 16) {
+            ends = segment_end(seg_off, nseg, min(j0 + lane, nseg - 1), d);
+            base = j0;
+        }
+    }
+    copy_async_wait();
+    __syncthreads();
+    if (uniform) {
+        Acc<NORM> acc;
+        if (warp < kWarps) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (e >= lo && e < hi) acc.add(v[e]);
+            for (int u = 0; u < UNITS; ++u) {
+                const int64_t i = t0 + (int64_t)(u * kThreads + tid) * E::G;
+                if (i >= t1) break;
+                float v[E::G];
+                E::unpack(stage[u * kThreads + tid], v);
+#pragma unroll
+                for (int e = 0; e < E::G; ++e)
+                    if (i + e < t1) acc.add(v[e]);
+            }
+            __syncwarp();
             const double w = warp_reduce<NORM>(acc.value());
-            if (lane == 0) slot[j] = w;
+            if (lane == 0) sh_head[warp] = w;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            double tot = sh_head[0];
+#pragma unroll
+            for (int k = 1; k < kWarps; ++k) tot = combine<NORM>(tot, sh_head[k]);
+            prow[tile + jt] = tot;
+        }
+        return;
+    }
+    int64_t a = c0;
+    for (int j = j0, k = 0; a < c1; ++j) {                                       // the pieces of my chunk
+        const int64_t seg_a = seg_b;
+        seg_b = j - base < 32 ? __shfl_sync(0xFFFFFFFFu, ends, (j - base) & 31) : segment_end(seg_off, nseg, j, d);
+        const int64_t b = min(max(seg_b, a), c1);
+        if (b > a && k++ % WPC == sub) {
+            Acc<NORM> acc;
+#pragma unroll 8
+            for (int i = (int)(a - t0) + lane; i < (int)(b - t0); i += 32) {
+                const T x = *((const T *)stage + i);
+                acc.add(DT == UQ_F32 ? (float)x : __uint_as_float((uint32_t)x << 16));
+            }
+            __syncwarp();
+            const double w = warp_reduce<NORM>(acc.value());
+            const bool goes_on = b == c1 && seg_b > c1;                            // may continue in the right chunk
+            if (lane == 0) {
+                if (a == c0 && seg_a < c0) { sh_head[chunk] = w; sh_head_seg[chunk] = j; sh_head_open[chunk] = goes_on; }   // may continue one from the left
+                else if (goes_on) { sh_tail[chunk] = w; sh_tail_seg[chunk] = j; }
+                else prow[tile + j] = w;
+            }
         }
         a = b;
+        if (j + 1 >= nseg) break;
+    }
+    __syncthreads();
+    // What goes on to the right is added up in chunk order, a thread per piece that starts one: the tail of a chunk, or
+    // the head of the tile's first.
+    if (tid < 2 * kWarps) {
+        int w = tid >> 1;
+        const bool from_head = (tid & 1) != 0;
+        const int j = from_head ? (w == 0 ? sh_head_seg[0] : -1) : sh_tail_seg[w];
+        if (j >= 0) {
+            double sum = from_head ? sh_head[0] : sh_tail[w];
+            bool open = !from_head || sh_head_open[0];
+            for (++w; open && w < kWarps && sh_head_seg[w] == j; ++w) {
+                sum = combine<NORM>(sum, sh_head[w]);
+                open = sh_head_open[w];
+            }
+            prow[tile + j] = sum;
+        }
     }
 }
 
@@ -261,8 +339,7 @@ norm_row_warps_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int
 template <int NORM>
 __global__ void __launch_bounds__(512)
 norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg,
-                     const int64_t *__restrict__ seg_off, int64_t ntiles, float *__restrict__ W,
-                     uint32_t *__restrict__ status, int tile_coords)       // tile_coords: coordinates per partial
+                     const int64_t *__restrict__ seg_off, int64_t ntiles, float *__restrict__ W, uint32_t *__restrict__ status)
 {
     grid_dependency_prologue();
     const int j = blockIdx.x;
@@ -274,7 +351,7 @@ norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg
     b = min(max(b, a), d);
 
     __shared__ double sh[UQ_MAX_WORKERS];
-    const int first = (int)(a / tile_coords), last = a < b ? (int)((b - 1) / tile_coords) : first - 1;
+    const int first = (int)(a / kNormTile), last = a < b ? (int)((b - 1) / kNormTile) : first - 1;
     for (int m = warp; m < M; m += nwarps) {
         const double *prow = part + (size_t)m * (size_t)(ntiles + nseg) + j;
         double acc = 0.0;
@@ -314,21 +391,16 @@ norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg
     }
 }
 
-// A warp per row: up to 16384 rows of all workers (24 000 of them 14.2 us by tiles and 14.4 by rows, 62 000 18.2 and
-// 29.3), in segments of 64 coordinates or more on average (a row has one slot, and a segment one, in the scratch:
-// M * (16384 / M + d / 64) of them stay below what the tiles of larger gradients take).
-static bool by_rows(const uq_layout &L)
-{
-    return L.nseg > 1 && (int64_t)L.nseg * 64 <= L.d && (L.d + kNormRow - 1) / kNormRow * L.M <= 16384;
-}
-
 template <int DT, int NORM>
 static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t *status, double *part,
                           int64_t ntiles, cudaStream_t st)
 {
-    if (L.d > 0 && by_rows(L)) {
-        launch_k(norm_row_warps_kernel<DT, NORM>, dim3((unsigned)((ntiles + kWarps - 1) / kWarps), (unsigned)L.M), kThreads, st,
-                 g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
+    if (L.d > 0 && L.nseg > 1 && ntiles * L.M <= kStagedTiles) {
+        const dim3 grid((unsigned)ntiles, (unsigned)L.M);
+        if (ntiles * L.M <= kDealtTiles)
+            launch_k(norm_staged_kernel<DT, NORM, 2>, grid, kThreads * 2, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
+        else
+            launch_k(norm_staged_kernel<DT, NORM, 1>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
     } else if (L.d > 0) {
         if (ntiles > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
         // binary32 takes several rows per CTA where that leaves eight waves and boundaries are rare (the rows of a
@@ -352,15 +424,11 @@ static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t 
     }
     // segments of more than eight loads per lane: 16 workers side by side
     launch_k(norm_finalize_kernel<NORM>, L.nseg, ntiles / L.nseg >= 256 ? 32 * min(L.M, 16) : kThreads, st, part, L.M, L.d, L.nseg,
-             L.seg_off, ntiles, W, status, by_rows(L) ? kNormRow : kNormTile);
+             L.seg_off, ntiles, W, status);
     return cudaGetLastError();
 }
 
-int64_t norm_tiles(const uq_layout &L)
-{
-    const int64_t tile = by_rows(L) ? kNormRow : kNormTile;
-    return (L.d + tile - 1) / tile;
-}
+int64_t norm_tiles(const uq_layout &L) { return (L.d + kNormTile - 1) / kNormTile; }
 
 cudaError_t launch_agree_scale(const uq_layout &L, const void *g, int norm, float *W, uint32_t *status,
                                void *workspace, cudaStream_t st)

@@ -121,6 +121,14 @@ __device__ __forceinline__ uint2 ld_coherent64(const void *p)
 
 template <typename T> __device__ __forceinline__ void st_stream(T *p, T v) { __stcs(p, v); }
 
+// 16 bytes from global memory straight into shared memory; a thread's copies are complete for that thread after
+// copy_async_wait().
+__device__ __forceinline__ void copy_async16(uint32_t smem_dst, const void *gmem_src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_dst), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // 256-bit streaming load / store (sm_100 and later): 32 bytes per lane in one instruction.
 // The address must be 32-byte aligned.
 struct alignas(32) uint8x { uint32_t w[8]; };

@@ -319,11 +319,6 @@ __device__ __forceinline__ uint4 ld_drop(const void *p, uint64_t policy)
     return v;
 }
 
-// 16 bytes from global memory straight into shared memory.
-__device__ __forceinline__ void copy_async16(uint32_t smem_dst, const void *gmem_src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_dst), "l"(gmem_src) : "memory");
-}
 __device__ __forceinline__ uint4 ld_shared16(uint32_t a)
 {
     uint4 v;
@@ -405,7 +400,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         const int top = p.v.scales.N > 1 ? 1 << (31 - __clz(p.v.scales.N - 1)) : 0;   // first step of the bisection
         const int32_t thr = lane < p.v.scales.N ? pass_threshold(inv_lane, p.v.s_hat) : -1;
         const int32_t thr_top = __shfl_sync(0xFFFFFFFFu, thr, top);
-        if (STAGED) asm volatile("cp.async.wait_all;" ::: "memory");
+        if (STAGED) copy_async_wait();
         else policy = policy_keep();
         uint32_t amag[8];
         const char *gs = gp;

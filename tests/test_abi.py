@@ -57,6 +57,14 @@ def test_sizes(lib):
     assert lib.uq_error_string(B.UQ_ERR_BAD_ARG) == b"bad argument"
 
 
+def test_scratch_of_the_norms_grows_with_the_layout(lib):
+    """M * (ceil(d / 8192) + nseg) doubles for every layout: scratch sized for the largest gradient does for all."""
+    for M, nseg in ((1, 1), (8, 1), (8, 161), (64, 161), (3, 5000)):
+        for d in (1, 8191, 8193, 10304, 100_003, 262_145, 524_288, 524_289, 600_000, 2_000_000, 25_557_032):
+            L = _layout(d=d, worker_stride=-(-d // 32) * 32, M=M, nseg=nseg, seg_off=0x10000 if nseg > 1 else None)
+            assert lib.uq_workspace_bytes(C.byref(L)) == M * (-(-d // 8192) + nseg) * 8
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     """None of these reaches a launch, so they run without a GPU (pointers are fake but aligned)."""
     p = 0x10000

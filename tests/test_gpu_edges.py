@@ -54,9 +54,9 @@ def test_norms_of_large_gradients(M, extra, nseg):
     assert int(status.item()) == 0
 
 
-# norms of small gradients in segments: a warp per row of 256 coordinates; empty segments, segments of one
-# coordinate, more than 32 pieces in a row, boundaries around a row's end, a ragged last row; and both sides of the
-# line at 16384 rows
+# norms of small gradients in segments: tiles of 8192 coordinates through shared memory; empty segments, segments of
+# one coordinate, more than 32 pieces in a warp's chunk, boundaries around a chunk's end, a ragged last tile, tiles
+# without a boundary; and both sides of the line at 512 tiles
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("M,d,cuts", [
     (3, 20_003, [*range(1, 81), 255, 256, 256, 256, 257, 511, 513, 1024, 5000, 5003, 20_000, 20_002]),
@@ -94,6 +94,24 @@ def test_order_of_a_sum_does_not_depend_on_the_number_of_workers(M):
     ws = torch.empty(lay.workspace_bytes(), dtype=torch.uint8, device="cuda")
     B.uq_agree_scale(lay, g, B.UQ_NORM_L2, W, status, ws)
     assert float(W.item()) == 2.0 ** 24 and int(status.item()) == 0
+
+
+# the same in segments, where the kernel that takes the tiles depends on how many of them there are.  Here every fourth
+# tile holds one of the small squares and each lane of the second kernel adds up two tiles, so the lanes' sums
+# tip the root: by three units of the last place of the sum, to 2^24 + 2
+@pytest.mark.parametrize("M", [1, 8, 9, 64])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_order_of_a_sum_in_segments_does_not_depend_on_the_number_of_workers(M, dtype):
+    d = 64 * 8192
+    g = torch.zeros(M, d, dtype=dtype, device="cuda")
+    g[:-1] = 0.5
+    g[-1, :4] = torch.tensor([2.0 ** 24, 2.0 ** 12, 2.0 ** 12, 1.0])
+    g[-1, 4 * 8192:: 4 * 8192] = 0.125
+    W, status = torch.empty(2, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    lay = B.Layout(M, d, d, dtype, torch.tensor([0, d - 1, d], device="cuda"))
+    ws = torch.empty(lay.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    B.uq_agree_scale(lay, g, B.UQ_NORM_L2, W, status, ws)
+    assert float(W[0].item()) == 2.0 ** 24 + 2 and int(status.item()) == 0
 
 
 # shared index: 16-, 8- and 4-byte accesses by alignment and length, each number of rows that is unrolled, and more
