@@ -35,24 +35,32 @@ __device__ __forceinline__ void grid_dependency_prologue()
     grid_dependency_wait();
 }
 
+// The launch attribute that goes with the wait inside the kernels; returns how many attributes it filled in (-DUQ_NO_PDL:
+// neither the attribute nor the wait).
+inline unsigned grid_dependency_attribute(cudaLaunchAttribute *attr)
+{
+#ifdef UQ_NO_PDL
+    (void)attr;
+    return 0;
+#else
+    attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr->val.programmaticStreamSerializationAllowed = 1;
+    return 1;
+#endif
+}
+
 template <typename... P, typename... A>
 inline void launch_k_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem_bytes, cudaStream_t st, A &&...args)
 {
-#ifdef UQ_NO_PDL
-    kernel<<<grid, block, smem_bytes, st>>>(static_cast<A &&>(args)...);
-#else
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = grid_dependency_attribute(attr);
     cudaLaunchKernelEx(&cfg, kernel, static_cast<A &&>(args)...);    // an error stays for cudaGetLastError()
-#endif
 }
 
 template <typename... P, typename... A>

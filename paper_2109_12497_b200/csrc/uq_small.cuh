@@ -418,9 +418,7 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
         p.rounds = 1;
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)ctas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.numAttrs = 2;
+        cfg.numAttrs = 1 + grid_dependency_attribute(attr + 1);
         return cudaLaunchKernelEx(&cfg, small_step_kernel<DT, NORM, RNG, MULTI, true, MW>, p);
     }
     static int cache[64] = {};

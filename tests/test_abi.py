@@ -2,6 +2,8 @@
 host-side argument validation rejects bad calls before any launch."""
 import ctypes as C
 import re
+import subprocess
+from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
 import pytest
@@ -176,6 +178,20 @@ def test_step_plan_is_checked_on_the_host(lib):
     multi = plan(one_kernel=1, N=2, idx_bits=3, idx=p)                                       # idx_bits
     multi.scales[:2] = [127, 1016]
     assert run(multi) == B.UQ_ERR_BAD_ARG
+
+
+def test_launches_overlap_only_where_the_kernels_wait():
+    """-DUQ_NO_PDL: no launch asks for the overlap with the kernel in front, since no kernel waits for it then."""
+    def preprocessed(src, *flags):
+        cmd = [uq_build._nvcc(), "-E", "-std=c++17", *flags, "-I", str(uq_build.INCLUDE), "-I", str(uq_build.CSRC),
+               str(uq_build.CSRC / src)]
+        text = subprocess.run(cmd, capture_output=True, text=True, check=True).stdout
+        return re.search(r"programmaticStreamSerializationAllowed\s*=", text), re.search(r'griddepcontrol\.wait;" :::', text)   # (CUDA's own headers spell it without blanks)
+    with ThreadPoolExecutor() as pool:
+        for asks, waits in pool.map(lambda s: preprocessed(s, "-DUQ_NO_PDL"), uq_build.SOURCES):
+            assert not asks and not waits
+    asks, waits = preprocessed("uq_small_f32.cu")
+    assert asks and waits
 
 
 def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
