@@ -67,9 +67,13 @@ class Quantizer:
                     if self.multi else None)
         self.out = torch.empty(max(d, 1), dtype=torch.float32, device=dev)
         self.S = torch.empty(max(d, 1), dtype=torch.int32, device=dev) if keep_sums else None
-        self._plan = None                               # the step's arguments, gathered at the first step
-        self._g_shape = torch.Size((M, self.stride))
-        self._out_view = self.out[: self.d]
+        self._plan = None                               # the step's arguments, gathered at the next step
+
+    def __setattr__(self, name, value):
+        # whatever is assigned, the next step gathers its arguments anew
+        object.__setattr__(self, name, value)
+        if name != "_plan":
+            object.__setattr__(self, "_plan", None)
 
     # the four stages, each one C-ABI call -------------------------------------------------------
     def agree_scale(self, g: torch.Tensor) -> None:
@@ -127,17 +131,19 @@ class Quantizer:
     def step(self, g: torch.Tensor, seed: int = 0) -> torch.Tensor:
         """g: [M, stride] gradients of all workers -> the reconstructed average gradient [d]."""
         if self.one_kernel or self.fused_select is None:      # the library's sequence: one trip through the binding
-            # every buffer but g is this object's own: their addresses are gathered in a plan once, not marshalled
-            # per step (for small gradients the host's share of a step is as long as the GPU's)
-            plan = self._plan or self._make_plan()
+            # every buffer but g is this object's own: their addresses and the settings are gathered in a plan when
+            # one of them has been assigned, not marshalled per step (for small gradients the host's share of a step
+            # is as long as the GPU's).  The layout is copied each time: its worker0 and coord0 may be set in place.
+            call, address, plan, shape, dtype, out = self._plan or self._make_plan()
+            plan.layout = self.layout.c
             index = g.get_device()
-            if not (g.shape == self._g_shape and g.dtype is self.dtype and g.is_contiguous() and index == self.device.index
+            if not (g.shape == shape and g.dtype is dtype and g.is_contiguous() and index == self.device.index
                     and index == _current_device()):
                 self._check_devices(g)
-            rc = plan[0](plan[1], g.data_ptr(), seed, _raw_stream(index))
+            rc = call(address, g.data_ptr(), seed, _raw_stream(index))
             if rc != B.UQ_OK:
                 raise B.UqError("uq_step_small" if self.one_kernel else "uq_step", rc)
-            return self._out_view
+            return out
         # the caller's choice of where selection runs, call by call
         self.agree_scale(g)
         if self.fused_select:                                 # inside the encoder's kernel
@@ -165,7 +171,8 @@ class Quantizer:
                            status=ptr(self.status), workspace=ptr(ws), workspace_bytes=ws.numel())
         if self.multi:
             p.scales[: p.N] = self.scales
-        self._plan = (B.lib().uq_step_run, C.addressof(p), p)
+        self._plan = (B.lib().uq_step_run, C.addressof(p), p, torch.Size((self.layout.M, self.layout.worker_stride)),
+                      self.layout.dtype, self.out[: self.d])
         return self._plan
 
     def _check_devices(self, g: torch.Tensor) -> None:
