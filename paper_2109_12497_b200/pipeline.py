@@ -170,7 +170,8 @@ class Quantizer:
                            W=ptr(self.W), idx=ptr(self.idx), lev=ptr(self.lev), out=ptr(self.out), S_opt=ptr(self.S),
                            status=ptr(self.status), workspace=ptr(ws), workspace_bytes=ws.numel())
         if self.multi:
-            p.scales[: p.N] = self.scales
+            kept = self.scales[: len(p.scales)]         # (the library refuses an N beyond them)
+            p.scales[: len(kept)] = kept
         self._plan = (B.lib().uq_step_run, C.addressof(p), p, torch.Size((self.layout.M, self.layout.worker_stride)),
                       self.layout.dtype, self.out[: self.d])
         return self._plan

@@ -91,3 +91,13 @@ def test_a_step_uses_the_buffers_as_they_are(calls):
     assert (p.W, p.idx, p.lev, p.status, p.S_opt, p.out, p.workspace) == tuple(
         getattr(q, n).data_ptr() for n in ("W", "idx", "lev", "status", "S", "out", "small_workspace"))
     assert out.data_ptr() == q.out.data_ptr()
+
+
+def test_too_many_scales_are_refused_by_the_library(monkeypatch):
+    """N > 16 is the library's argument error, found on the host before anything is launched."""
+    monkeypatch.setattr(pipeline, "_current_device", lambda: 0)
+    monkeypatch.setattr(pipeline, "_raw_stream", lambda index: 0)
+    q = quantizer(scales=[7 * 2 ** k for k in range(17)], idx_bits=8)
+    with pytest.raises(B.UqError) as e:
+        q.step(FakeGradients(q), 0)
+    assert e.value.code == B.UQ_ERR_BAD_ARG
