@@ -220,8 +220,13 @@ class RandKQuantizer:
         self.sel = torch.empty(max(K, 1), dtype=torch.int64, device=dev)
         self.gk = torch.empty((M, self.inner.stride), dtype=dtype, device=dev)
         self.status = self.inner.status
-        self._g_shape = torch.Size((M, self.dense_layout.worker_stride))
-        self._tail = (self.sel.data_ptr(), self.gk.data_ptr(), self.gk.shape[1], self.status.data_ptr())
+        self._own = None                                     # my buffers' addresses, once a call has checked them
+
+    def __setattr__(self, name, value):
+        # whatever is assigned, the next call checks my buffers anew
+        object.__setattr__(self, name, value)
+        if name != "_own":
+            object.__setattr__(self, "_own", None)
 
     def _mine(self, t: torch.Tensor, dtype: torch.dtype) -> bool:
         """Whether t is contiguous, of that type, and on this object's device, which is the current one (else
@@ -230,10 +235,14 @@ class RandKQuantizer:
         return t.dtype is dtype and t.is_contiguous() and index == self.inner.device.index and index == _current_device()
 
     def gather(self, g: torch.Tensor, seed: int) -> None:
-        if not (g.shape == self._g_shape and self._mine(g, self.dense_layout.dtype)):
-            B.uq_randk_gather(self.dense_layout, g, self.K, seed, self.sel, self.gk, self.status)
+        lay, own = self.dense_layout, self._own
+        fits = g.shape == (lay.M, lay.worker_stride) and self._mine(g, lay.dtype)
+        if own is None or not fits:
+            B.uq_randk_gather(lay, g, self.K, seed, self.sel, self.gk, self.status)
+            if fits:
+                self._own = (self.sel.data_ptr(), self.gk.data_ptr(), self.gk.shape[1], B._ptr(self.status))
             return
-        rc = B.lib().uq_randk_gather(self.dense_layout.ref(), g.data_ptr(), self.K, seed, *self._tail, _raw_stream(g.get_device()))
+        rc = B.lib().uq_randk_gather(lay.ref(), g.data_ptr(), self.K, seed, *own, _raw_stream(g.get_device()))
         if rc != B.UQ_OK:
             raise B.UqError("uq_randk_gather", rc)
 
@@ -249,10 +258,12 @@ class RandKQuantizer:
         B.uq_randk_scatter(self.d, self.K, self.sel, None, out, self.status)
 
     def update(self, theta: torch.Tensor, lr: float) -> None:
-        if not (theta.dim() == 1 and theta.shape[0] >= self.d and self._mine(theta, torch.float32)):
-            B.uq_randk_update(self.d, self.K, self.sel, self.inner.out, theta, lr, self.status)
+        own, vals = self._own, self.inner.out
+        if own is None or not (theta.dim() == 1 and theta.shape[0] >= self.d and self._mine(theta, torch.float32)
+                               and vals.dim() == 1 and vals.shape[0] >= self.K and self._mine(vals, torch.float32)):
+            B.uq_randk_update(self.d, self.K, self.sel, vals, theta, lr, self.status)
             return
-        rc = B.lib().uq_randk_update(self.d, self.K, self._tail[0], self.inner.out.data_ptr(), theta.data_ptr(), lr, self._tail[3],
+        rc = B.lib().uq_randk_update(self.d, self.K, own[0], vals.data_ptr(), theta.data_ptr(), lr, own[3],
                                      _raw_stream(theta.get_device()))
         if rc != B.UQ_OK:
             raise B.UqError("uq_randk_update", rc)

@@ -1,5 +1,5 @@
-"""What Quantizer.step hands to the library, on the host (the call itself is replaced by a recorder): the object's
-settings, buffers and layout as they are at that step, whatever was assigned or set in place since the last one."""
+"""What the objects of pipeline.py hand to the library, on the host (the calls themselves are replaced by recorders): their
+settings, buffers and layout as they are at that call, whatever was assigned or set in place since the last one."""
 import ctypes as C
 from types import SimpleNamespace
 
@@ -29,9 +29,9 @@ def calls(monkeypatch):
         made.append(B.uq_step_plan.from_buffer_copy(C.cast(address, C.POINTER(B.uq_step_plan)).contents))
         return B.UQ_OK
     real = B.lib()
-    monkeypatch.setattr(B, "lib", lambda: SimpleNamespace(uq_step_run=uq_step_run, uq_workspace_bytes=real.uq_workspace_bytes,
-                                                          uq_index_bytes=real.uq_index_bytes, uq_error_string=real.uq_error_string,
-                                                          uq_workspace_bytes_small=real.uq_workspace_bytes_small))
+    fake = SimpleNamespace(uq_step_run=uq_step_run, **{n: getattr(real, n) for n in (
+        "uq_workspace_bytes", "uq_workspace_bytes_small", "uq_index_bytes", "uq_error_string")})
+    monkeypatch.setattr(B, "lib", lambda: fake)
     monkeypatch.setattr(pipeline, "_current_device", lambda: 0)
     monkeypatch.setattr(pipeline, "_raw_stream", lambda index: 0)
     return made
@@ -101,3 +101,33 @@ def test_too_many_scales_are_refused_by_the_library(monkeypatch):
     with pytest.raises(B.UqError) as e:
         q.step(FakeGradients(q), 0)
     assert e.value.code == B.UQ_ERR_BAD_ARG
+
+
+def test_sparse_calls_use_the_buffers_as_they_are(monkeypatch, calls):
+    made = {}
+    lib = B.lib()
+    lib.uq_randk_gather = lambda lay, g, K, seed, sel, gk, gk_stride, status, stream: made.update(
+        sel=sel, gk=gk, gk_stride=gk_stride, status=status) or B.UQ_OK
+    lib.uq_randk_update = lambda d, K, sel, vals, theta, lr, status, stream: made.update(sel=sel, vals=vals, status=status) or B.UQ_OK
+    monkeypatch.setattr(B, "_ptr", lambda t: None if t is None else t.data_ptr())
+    monkeypatch.setattr(B, "_stream", lambda: 0)
+    monkeypatch.setattr(pipeline.RandKQuantizer, "_mine", lambda self, t, dtype: t.dtype is dtype and t.is_contiguous())
+    rq = pipeline.RandKQuantizer(2, 1000, 100, device="cpu")
+    g = FakeGradients(SimpleNamespace(layout=rq.dense_layout))
+    theta = torch.zeros(1000)
+    theta.get_device = lambda: 0
+    for _ in range(2):
+        for _ in range(2):
+            rq.gather(g, 0)
+            assert (made["sel"], made["gk"], made["gk_stride"], made["status"]) == (rq.sel.data_ptr(), rq.gk.data_ptr(), 128,
+                                                                                      rq.status.data_ptr())
+            rq.update(theta, 0.1)
+            assert (made["sel"], made["vals"], made["status"]) == (rq.sel.data_ptr(), rq.inner.out.data_ptr(), rq.status.data_ptr())
+        rq.sel, rq.gk, rq.status, rq.inner.out = rq.sel.clone(), rq.gk.clone(), rq.status.clone(), rq.inner.out.clone()
+    rq.gather(g, 0)
+    rq.inner.out = torch.zeros(99)
+    with pytest.raises(ValueError, match="vals"):
+        rq.update(theta, 0.1)
+    rq.sel = torch.zeros(99, dtype=torch.int64)
+    with pytest.raises(ValueError, match="sel"):
+        rq.gather(g, 0)
