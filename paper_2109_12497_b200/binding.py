@@ -123,7 +123,8 @@ def require_current_device(index: Optional[int], current: int, what: str = "tens
                          f"make its device current first (torch.cuda.device / set_device)")
 
 
-_current_device = torch._C._cuda_getDevice
+# (a torch built without CUDA has only the public wrapper)
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

@@ -16,8 +16,8 @@ import torch
 from . import binding as B
 
 
-_current_device = torch._C._cuda_getDevice
-_raw_stream = torch._C._cuda_getCurrentRawStream
+_current_device = B._current_device
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # (a torch built without CUDA has none)
 
 ONE_KERNEL_MAX_BYTES = 8 << 20      # gradients of all workers up to this size take the one-kernel step
 

@@ -3,6 +3,7 @@ host-side argument validation rejects bad calls before any launch."""
 import ctypes as C
 import re
 import subprocess
+import sys
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
@@ -199,6 +200,16 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "LIB_PATH", tmp_path / "missing.so")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         B.lib()
+
+
+def test_the_package_imports_with_a_torch_built_without_cuda():
+    """The layouts, the workloads and the exchange logic are of use without a GPU."""
+    code = ("import torch\n"
+            "for name in ('_cuda_getDevice', '_cuda_getCurrentRawStream'):\n"
+            "    delattr(torch._C, name)\n"
+            "from paper_2109_12497_b200 import binding, distributed, pipeline, workloads\n"
+            "assert binding.Layout(2, 100, 128, torch.float32).nseg == 1\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
 
 
 def test_a_tensor_on_another_device_is_refused_before_any_launch():
