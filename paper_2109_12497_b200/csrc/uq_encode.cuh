@@ -513,6 +513,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         slow = __any_sync(0xFFFFFFFFu, inexact);
     }
     if (slow) {
+        if (STAGED) copy_async_wait();                           // copies may be on their way: W came after them
         encode_row_slow<DT, FMT, RNG, MULTI>(p, r0, m_first, m_last);
         return;
     }

@@ -131,6 +131,17 @@ def test_index_min_access_widths(offset, nbytes, R):
     assert (got[:offset] == 0xEE).all() and (got[offset + nbytes:] == 0xEE).all()
 
 
+# 8 bf16 workers, selecting: a row's bytes are on their way to shared memory before its scale is known; scales that the
+# fast arithmetic cannot take, in the first half of the layers, over more CTAs than the GPU holds at a time
+@pytest.mark.parametrize("rng_bits,power", [(16, 110), (32, -98)])
+def test_staged_rows_whose_scales_the_fast_forms_cannot_take(rng_bits, power):
+    w = wl.scaled("c3", 2_600_003, M=8, dtype=wl.BF16, rng_bits=rng_bits)
+    g = wl.generate(w)
+    half = wl.segment_offsets(w)[len(wl.segment_offsets(w)) // 2]
+    g[:, :half] = wl.f32_to_bf16_bits(wl.bf16_bits_to_f32(g[:, :half]) * np.float32(2.0 ** power))
+    check_parity(w, g)
+
+
 # the levels alone: the workers are dealt out in groups of eight over the grid
 @pytest.mark.parametrize("M", [7, 8, 9, 17])
 @pytest.mark.parametrize("fmt,s", [("i8", 127), ("i6p", 31), ("i4x2", 7), ("i2x4", 1)])
