@@ -21,6 +21,8 @@
 // sustained): 235 us for quantization + sum + reconstruction, where two kernels took 210 + 53 us; with
 // selection among 4 scales 266 us, where three took 130 + 216 + 53 us.
 #pragma once
+#include <type_traits>
+
 #include "uq_device.cuh"
 #include "uq_select.cuh"
 #include "uq_unit.cuh"
@@ -530,36 +532,54 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     // (64 workers * 127 < 2^13, so the fields come apart again).
     int sum[2][2] = {{0, 0}, {0, 0}};
     char *lp = (char *)p.lev + LF::off(i) + (SPLIT ? m_first * lrow : 0), *lp2 = lp + (LF::off2(i, p.v.stride) - LF::off(i));
-    auto group = [&](int m0) {
-        uint4 r[G][NB];
-        philox_join<G, NB>(p.key, blk, p.wpart + m0, r);
+    // workers m0 .. m0 + GG - 1; ahead: the worker GG places on, if there is one, is fetched into the registers that become free
+    auto group = [&](auto gg_tag, int m0, auto ahead) {
+        constexpr int GG = decltype(gg_tag)::value;
+        uint4 r[GG][NB];
+        philox_join<GG, NB>(p.key, blk, p.wpart + m0, r);
 #pragma unroll
-        for (int c = 0; c < G; ++c) {
-            if (WK || m0 + c < m_last) {
-                if (RNG == 16) { r[c][0].y = ~r[c][0].y; r[c][0].w = ~r[c][0].w; }
-                uint32_t w[2];
-                quantize_fast<DT, FMT, RNG>(q[c], inv, lc, r[c], w);
-                if (m0 + c + G < m_last) load(m0 + c + G, q[c]);
-                if (O::EO) store_unit_even_odd(w[0], w[1], lp);
-                else store_unit<FMT>(w[0], w[1], lp, lp2);
-                lp += lrow;
-                if (FMT == UQ_FMT_I6P) lp2 += lrow;
-                if (DEC) {
+        for (int c = 0; c < GG; ++c) {
+            if (RNG == 16) { r[c][0].y = ~r[c][0].y; r[c][0].w = ~r[c][0].w; }
+            uint32_t w[2];
+            quantize_fast<DT, FMT, RNG>(q[c], inv, lc, r[c], w);
+            if (ahead(m0 + c + GG)) load(m0 + c + GG, q[c]);
+            if (O::EO) store_unit_even_odd(w[0], w[1], lp);
+            else store_unit<FMT>(w[0], w[1], lp, lp2);
+            lp += lrow;
+            if (FMT == UQ_FMT_I6P) lp2 += lrow;
+            if (DEC) {
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        sum[k][0] = __dp2a_lo(0x40000001, (int)w[k], sum[k][0]);
-                        sum[k][1] = __dp2a_hi(0x40000001, (int)w[k], sum[k][1]);
-                    }
+                for (int k = 0; k < 2; ++k) {
+                    sum[k][0] = __dp2a_lo(0x40000001, (int)w[k], sum[k][0]);
+                    sum[k][1] = __dp2a_hi(0x40000001, (int)w[k], sum[k][1]);
                 }
             }
         }
     };
     if (WK) {
 #pragma unroll
-        for (int m = 0; m < WK; m += G) group(m);
+        for (int m = 0; m < WK; m += G) group(std::integral_constant<int, G>(), m, [](int m) { return m < WK; });
     } else {
+        // Eight workers whose levels alone are wanted go straight-line; else whole groups, and the rest by twos and
+        // one, so that a worker that is not there costs no draws.  (With groups of four chains for whoever is there: one
+        // bf16 worker of 25.6 M coordinates, levels alone, 16-bit draws 53 us, 34 like this; five of them 1.2 times as long.
+        // With a loop around the eight: 16 binary32 workers 3 % longer.)
+        int m = m_first;
+        if (SPLIT && m_last - m_first == kGroup) {
+#pragma unroll
+            for (int k = 0; k < kGroup; k += G) group(std::integral_constant<int, G>(), m_first + k, [&](int x) { return x < m_first + kGroup; });
+            return;
+        }
 #pragma unroll 1
-        for (int m = m_first; m < m_last; m += G) group(m);
+        for (; m + G <= m_last; m += G) group(std::integral_constant<int, G>(), m, [&](int m) { return m < m_last; });
+        const auto never = [](int) { return false; };
+        if (G > 2 && ((m_last - m) & 2)) {
+            group(std::integral_constant<int, (G > 2 ? 2 : 1)>(), m, never);
+            m += 2;
+#pragma unroll
+            for (int h = 0; h < V; ++h) q[0][h] = q[G > 2 ? 2 : 0][h];
+        }
+        if (G > 1 && m < m_last) group(std::integral_constant<int, 1>(), m, never);
     }
     if (DEC) {
         // Algorithm 1 / 2, lines "AllReduce gradients" and "Reconstruct gradient": the sum of a coordinate times

@@ -150,6 +150,17 @@ def test_levels_alone_of_many_workers(M, fmt, s):
     check_parity(w, wl.generate(w))
 
 
+# the encoder's ways through the workers: straight-line ones by number and element type, and groups of four, two and one
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 6, 7, 9, 15, 16])
+@pytest.mark.parametrize("dtype", [wl.F32, wl.BF16])
+@pytest.mark.parametrize("rng_bits", [16, 32])
+@pytest.mark.parametrize("name,fmt,s", [("c2", "i8", 127), ("c3", "i8", 127), ("c3", "i4x2", 7), ("c3", "i6p", 31)])
+def test_encoder_at_every_number_of_workers(name, fmt, s, rng_bits, dtype, M):
+    scales = (s, 8 * s, 64 * s) if name == "c3" else (s,)
+    w = wl.scaled(name, 9_001, M=M, dtype=dtype, fmt=fmt, s=s, scales=scales, rng_bits=rng_bits)
+    check_parity(w, wl.generate(w))
+
+
 # update of parameters: with 2- and 4-bit levels a thread requests its parameters before the sums; coordinates
 # around one thread's 32 and one CTA's share, and none at all in the last vector
 @pytest.mark.parametrize("d", [1, 31, 32, 33, 8191, 8193])
