@@ -57,11 +57,19 @@ constexpr int kGroup = 8;     // the number of workers that has kernels of its o
 // rounds advance together, and four CTAs of 64 registers share an SM.  Measured on a B200 (8 workers,
 // quantization + sum + reconstruction, sustained): bf16 with 32-bit draws 3 CTAs 188 us, 4 CTAs 197 us
 // (26.2 M coordinates); binary32, selecting, 32-bit draws: one worker at a time 266 us, two 273 us (25.6 M).
-template <int DT, int RNG, bool SEL> struct EncodeShape {
+//
+// Few workers (1 to 4 of bf16): what does not depend on the worker is then most of a lane's work, so all workers' blocks
+// go together straight-line, their rows are staged as the eight's are, and fewer registers let more warps hide the way
+// to memory.  25.6 M coordinates, 16-bit draws, general kernel / this / an encoder of two units per lane: levels alone,
+// one worker in 161 layers 40.9 / 33.2 / 32.9 us, two workers in one segment 47.9 / 41.5 / 38.2; with selection, two
+// workers 88.6 / 66.4 / 67.4.
+template <int DT, int RNG, bool SEL, int WK> struct EncodeShape {
+    static constexpr bool FEW = WK > 0 && WK < kGroup;
     static constexpr int V = 8 * Elem<DT>::BYTES / 16;                        // 16-byte words per thread and worker
     static constexpr int NB = RNG == 32 ? 2 : 1;                              // Philox blocks per thread and worker
-    static constexpr int G = DT == UQ_F32 ? (SEL ? 1 : 2) : RNG == 32 ? 2 : 4;    // workers whose blocks advance together
-    static constexpr int CTAS = DT == UQ_BF16 && RNG == 32 ? 3 : 4;           // per SM
+    static constexpr int G = FEW ? (RNG == 16 ? WK : WK % 2 == 0 ? 2 : 1)      // workers whose blocks advance together
+                                 : DT == UQ_F32 ? (SEL ? 1 : 2) : RNG == 32 ? 2 : 4;
+    static constexpr int CTAS = FEW ? (WK <= 2 ? 5 : 4) : DT == UQ_BF16 && RNG == 32 ? 3 : 4;           // per SM
     static constexpr int TILE = kThreads * 8;
 };
 
@@ -328,18 +336,18 @@ __device__ __forceinline__ uint4 ld_shared16(uint32_t a)
     return v;
 }
 
-// WK: 8 = exactly that many workers (known at compile time), 0 = any number.
+// WK: 8, or with bf16 1 to 4 = exactly that many workers (known at compile time), 0 = any number.
 template <int DT, int FMT, int RNG, bool MULTI, bool SEL, bool DEC, int WK>
-__global__ void __launch_bounds__(kThreads, (EncodeShape<DT, RNG, SEL>::CTAS))
+__global__ void __launch_bounds__(kThreads, (EncodeShape<DT, RNG, SEL, WK>::CTAS))
 encode_kernel(const __grid_constant__ EncodeParams p)
 {
     grid_dependency_prologue();
     using E = Elem<DT>;
-    using S = EncodeShape<DT, RNG, SEL>;
+    using S = EncodeShape<DT, RNG, SEL, WK>;
     using LF = LevelFmt<FMT>;
     using O = LevelOrder<DT, FMT>;
     constexpr int V = S::V, NB = S::NB, G = S::G, BSH = RNG == 32 ? 2 : 3;
-    constexpr bool STAGED = SEL && DT == UQ_BF16 && WK == 8;
+    constexpr bool STAGED = SEL && DT == UQ_BF16 && WK > 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, M = WK ? WK : p.v.M, ib = p.idx_bits;
     const int64_t d = p.v.d;
     // CTAs walk the tiles back to front: the kernel before this one in a step (the norms) ends on the
@@ -374,7 +382,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
             // every thread copies what it reads back itself
             const char *gs = gp;
 #pragma unroll
-            for (int m = 0; m < kGroup; ++m, gs += grow) copy_async16(sp + m * (kThreads * 16), gs);
+            for (int m = 0; m < WK; ++m, gs += grow) copy_async16(sp + m * (kThreads * 16), gs);
         } else if (!SEL) {
 #pragma unroll
             for (int c = 0; c < G; ++c)
@@ -441,7 +449,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
                 uint4 x[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    x[k] = STAGED ? ld_shared16(sp + k * (kThreads * 16)) : WK || k < left ? ld_keep(gs, policy) : make_uint4(0u, 0u, 0u, 0u);
+                    x[k] = STAGED && k < WK ? ld_shared16(sp + k * (kThreads * 16)) : !STAGED && k < left ? ld_keep(gs, policy) : make_uint4(0u, 0u, 0u, 0u);
                     gs += grow;
                 }
 #pragma unroll
@@ -613,7 +621,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
 template <int DT, int FMT, int RNG, bool MULTI, bool SEL, bool DEC, int WK>
 static cudaError_t launch(EncodeParams p, cudaStream_t st)
 {
-    using S = EncodeShape<DT, RNG, SEL>;
+    using S = EncodeShape<DT, RNG, SEL, WK>;
     const int64_t blocks = (p.v.d + S::TILE - 1) / S::TILE;
     if (blocks == 0) return cudaSuccess;
     if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
@@ -621,8 +629,8 @@ static cudaError_t launch(EncodeParams p, cudaStream_t st)
     p.blk_hi = (uint32_t)((uint64_t)(p.coord0 >> BSH) >> 32);
     if (RNG == 16) { p.key.k[18] = ~p.key.k[18]; p.key.k[19] = ~p.key.k[19]; }
     for (int m = 0; m < p.v.M; ++m) p.wpart[m] = philox_worker_part(p.key, p.blk_hi, (uint32_t)(p.worker0 + m));
-    // bf16, selecting: the 8 workers' rows of the tile
-    const size_t smem = SEL && DT == UQ_BF16 && WK == 8 ? (size_t)WK * S::TILE * Elem<DT>::BYTES : 0;
+    // bf16, selecting: the workers' rows of the tile, where their number is known
+    const size_t smem = SEL && DT == UQ_BF16 && WK > 0 ? (size_t)WK * S::TILE * Elem<DT>::BYTES : 0;
     // only the levels wanted: groups of 8 workers are independent, which gives small gradients of many workers
     // as many warps as they have groups
     p.split = !WK && !SEL && !DEC ? kGroup : p.v.M;
@@ -645,6 +653,12 @@ template <int DT, int FMT, int RNG, int WK> static cudaError_t dispatch_mode(con
 
 template <int DT, int FMT, int RNG> static cudaError_t dispatch_workers(const EncodeParams &p, cudaStream_t st)
 {
+    if constexpr (DT == UQ_BF16) {
+        if (p.v.M == 1) return dispatch_mode<DT, FMT, RNG, 1>(p, st);
+        if (p.v.M == 2) return dispatch_mode<DT, FMT, RNG, 2>(p, st);
+        if (p.v.M == 3) return dispatch_mode<DT, FMT, RNG, 3>(p, st);
+        if (p.v.M == 4) return dispatch_mode<DT, FMT, RNG, 4>(p, st);
+    }
     return p.v.M == kGroup ? dispatch_mode<DT, FMT, RNG, kGroup>(p, st) : dispatch_mode<DT, FMT, RNG, 0>(p, st);
 }
 
