@@ -42,7 +42,8 @@
  *   - Stream order.  The kernels are launched so that the GPU may schedule the blocks of one while
  *     the kernel before it in the stream is still draining (programmatic dependent launch); each
  *     kernel waits for that predecessor to complete before it reads or writes anything, so the
- *     results are those of plain stream order.
+ *     results are those of plain stream order.  (uq_randk_gather computes which coordinates it takes, from
+ *     its arguments alone, before that wait.)
  */
 #ifndef UQ_H
 #define UQ_H
@@ -113,6 +114,11 @@ size_t uq_workspace_bytes(const uq_layout *layout);
 
 /* Bytes of a packed scale-index stream for this layout: worker_stride * idx_bits / 8. */
 size_t uq_index_bytes(const uq_layout *layout, int idx_bits);
+
+/* Kernels that the encoding calls launch for this layout (0 on a bad layout or d = 0): uq_select_encode_multi (select = 1,
+ * reconstruct = 0), uq_encode_decode (0, 1), uq_select_encode_decode_multi and the part of uq_step behind the norms (1 with
+ * several scales, 1).  One, or one per stage: many workers of a small gradient. */
+int uq_encode_launches(const uq_layout *layout, int select, int reconstruct);
 
 /*
  * Shared scale — Algorithm 1 / Algorithm 2, line "MaxAllReduce Norm":
@@ -219,12 +225,13 @@ int uq_encode_multi(const uq_layout *layout, const void *g, const float *W, cons
                     void *lev, uint32_t *status, void *stream);
 
 /*
- * uq_select_encode_multi followed by uq_decode(src = UQ_SRC_LEVELS) as one kernel — Algorithm 2 from
+ * uq_select_encode_multi followed by uq_decode(src = UQ_SRC_LEVELS) as one call — Algorithm 2 from
  * "Compute coordinate scales" to "Reconstruct gradient", everything of a multi-scale step behind
- * the scale agreement.  The gradients are read once (with 8 bf16 workers; otherwise twice, the
- * second time from the caches as far as they hold them), the indices, the level rows and the
- * average are written, nothing is read back.  idx, lev and out receive, bit for bit, what the
- * separate calls write; arguments and errors are theirs.  uq_step makes this call.
+ * the scale agreement.  As one kernel (unless uq_encode_launches says otherwise) it reads the
+ * gradients once (with 8 bf16 workers, or 1 to 4; otherwise twice, the second time from the caches
+ * as far as they hold them), writes the indices, the level rows and the average, and reads nothing
+ * back.  idx, lev and out receive, bit for bit, what the separate calls write; arguments and errors
+ * are theirs.  uq_step makes this call.
  */
 int uq_select_encode_decode_multi(const uq_layout *layout, const void *g, const float *W,
                                   const int32_t *scales, int N, int idx_bits, uint64_t seed, int rng_bits,
@@ -233,11 +240,12 @@ int uq_select_encode_decode_multi(const uq_layout *layout, const void *g, const 
 
 /*
  * uq_encode_single (scales = NULL) or uq_encode_multi (scales given) followed by
- * uq_decode(src = UQ_SRC_LEVELS) as one kernel — Algorithm 1 lines "Quantize gradient", "AllReduce
+ * uq_decode(src = UQ_SRC_LEVELS) as one call — Algorithm 1 lines "Quantize gradient", "AllReduce
  * gradients", "Reconstruct gradient" (Algorithm 2: "Quantize with s*" onwards) — for callers whose
- * M workers are all in this buffer.  The warp that takes a row of coordinates through the workers
- * adds their levels up in registers and writes the reconstructed average beside the level rows, so
- * the levels are written (they are what would cross the wire) but never read back.  lev and out
+ * M workers are all in this buffer.  One kernel (unless uq_encode_launches says otherwise): the warp
+ * that takes a row of coordinates through the workers adds their levels up in registers and writes
+ * the reconstructed average beside the level rows, so the levels are written (they are what would
+ * cross the wire) but never read back.  lev and out
  * receive, bit for bit, what the two separate calls write; arguments and errors are theirs (the
  * integer sums are not available here: use uq_step, uq_decode or uq_aggregate).
  */
@@ -246,11 +254,11 @@ int uq_encode_decode(const uq_layout *layout, const void *g, const float *W, int
                      void *lev, float *out, uint32_t *status, void *stream);
 
 /*
- * uq_select_scale_multi followed by uq_encode_multi as one kernel — Algorithm 2 lines "Compute
+ * uq_select_scale_multi followed by uq_encode_multi as one call — Algorithm 2 lines "Compute
  * coordinate scales", "Scale sharing" and "Quantize with s*" — for callers whose M workers are all
- * in this buffer: a first pass over the workers' rows takes the maximum over the workers of every
- * magnitude, which decides the shared index, and the second pass quantizes.  idx and lev receive,
- * bit for bit, what the two separate calls write; arguments and errors are theirs.
+ * in this buffer.  As one kernel (unless uq_encode_launches says otherwise): a first pass over the
+ * workers' rows takes the maximum over the workers of every magnitude, which decides the shared
+ * index, and the second pass quantizes.  idx and lev receive, bit for bit, what the two separate calls write; arguments and errors are theirs.
  */
 int uq_select_encode_multi(const uq_layout *layout, const void *g, const float *W, const int32_t *scales,
                            int N, int idx_bits, uint64_t seed, int rng_bits, int fmt, uint8_t *idx,
@@ -337,7 +345,7 @@ int uq_index_min(const uint8_t *rows, int R, int64_t row_bytes, int64_t nbytes, 
  * One whole step in one call — Algorithm 1 lines "MaxAllReduce Norm" to "Reconstruct gradient"
  * (scales = NULL: uq_agree_scale, uq_encode_single, uq_decode) or Algorithm 2 (scales given:
  * uq_agree_scale, uq_select_scale_multi, uq_encode_multi, uq_decode), enqueued in that order on
- * `stream`, as three kernels: two for the norms, and one for everything else.  Nothing is computed
+ * `stream`: two kernels for the norms and uq_encode_launches for everything else.  Nothing is computed
  * differently: every output is bit for bit that of the separate calls.  Arguments are
  * those of the calls it makes (idx is not used when scales = NULL); the first error stops the
  * sequence and is returned.
@@ -350,9 +358,13 @@ int uq_step(const uq_layout *layout, const void *g, int norm, int s, const int32
 /*
  * One whole step as ONE kernel — Algorithm 1 (scales = NULL) or Algorithm 2 (scales given), lines
  * "MaxAllReduce Norm" to "Reconstruct gradient" — for gradients so small that the launches of
- * uq_step cost more than its arithmetic.  A cooperative grid reads the gradients for the norms,
- * meets at one grid-wide barrier, and reads them again (from L2) to [select and share the scale
- * indices,] quantize, store the level rows, add the levels and write the reconstructed average.
+ * uq_step cost more than its arithmetic.  Every thread reads its coordinates of all workers, and
+ * keeps them in registers while the norms are agreed on, across one thread-block cluster (up to
+ * 32768 coordinates) or a cooperative grid with one grid-wide barrier; then it [selects and shares the
+ * scale indices,] quantizes, stores the level rows, adds the levels and writes the reconstructed average.
+ * A gradient beyond the grid's registers is read again.  The first call of a configuration on a
+ * device asks for its occupancy and may set a kernel attribute: make it during set-up, before any
+ * stream capture.
  * Arguments as in uq_step.  Supported: one segment (layout->nseg = 1), M <= 8, formats
  * UQ_FMT_I8 / I4X2 / I2X4, both dtypes, norms, draw widths, every index width; worker0 and coord0
  * key the draws as in the encoders.  Anything else returns UQ_ERR_UNSUPPORTED, as does a device
@@ -364,7 +376,7 @@ int uq_step(const uq_layout *layout, const void *g, int norm, int s, const int32
  *                 one that reports UQ_STATUS_TIMEOUT: zero them again after that.
  * Results: idx, lev, S_opt and out are bit for bit those of uq_step given the same W; W is added
  * up in another fixed order (L-inf: identical; L2: within one unit in the last place).
- * The wait at the barrier is bounded: a CTA that gives up sets UQ_STATUS_TIMEOUT and returns
+ * The wait at the grid's barrier is bounded: a CTA that gives up sets UQ_STATUS_TIMEOUT and returns
  * (outputs then incomplete).  For that reason status must not be NULL here (UQ_ERR_BAD_ARG).
  * Errors: UQ_ERR_BAD_ARG, UQ_ERR_UNSUPPORTED, UQ_ERR_WORKSPACE, UQ_ERR_CUDA.
  */

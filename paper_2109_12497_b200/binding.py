@@ -26,7 +26,7 @@ UQ_STATUS_TIMEOUT = 16
 
 EXPORTS = (
     "uq_version", "uq_last_cuda_error", "uq_error_string", "uq_workspace_bytes", "uq_index_bytes",
-    "uq_workspace_bytes_small",
+    "uq_workspace_bytes_small", "uq_encode_launches",
     "uq_agree_scale", "uq_agree_scale_static", "uq_encode_single", "uq_select_scale_multi", "uq_encode_multi",
     "uq_aggregate", "uq_decode", "uq_decode_update", "uq_randk_gather", "uq_randk_scatter", "uq_randk_update", "uq_index_min", "uq_decode_rows", "uq_select_encode_multi", "uq_encode_decode", "uq_select_encode_decode_multi", "uq_step",
     "uq_step_small", "uq_step_run",
@@ -86,6 +86,7 @@ def lib() -> C.CDLL:
         L.uq_workspace_bytes.argtypes = [LP]
         L.uq_index_bytes.restype = SZ
         L.uq_index_bytes.argtypes = [LP, I]
+        L.uq_encode_launches.argtypes = [LP, I, I]
         L.uq_agree_scale.argtypes = [LP, P, I, P, P, P, SZ, P]
         L.uq_step.argtypes = [LP, P, I, I, P, I, I, U64, I, I, P, P, P, P, P, P, P, SZ, P]
         L.uq_step_small.argtypes = [LP, P, I, I, P, I, I, U64, I, I, P, P, P, P, P, P, P, SZ, P]

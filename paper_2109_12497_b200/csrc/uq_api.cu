@@ -9,6 +9,7 @@ cudaError_t launch_agree_scale(const uq_layout &L, const void *g, int norm, floa
 cudaError_t launch_encode(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
                           uint8_t *idx, int idx_bits, bool select, uint64_t seed, int rng_bits, int fmt,
                           void *lev, float *out, int32_t *S, uint32_t *status, cudaStream_t st);
+int encode_launches(const uq_layout &L, bool select, bool reconstruct);
 cudaError_t launch_select(const uq_layout &L, const void *g, const float *W, const ScaleSet &scales,
                           int idx_bits, uint8_t *idx, uint32_t *status, cudaStream_t st);
 cudaError_t launch_aggregate_decode(const uq_layout &L, const void *lev, int fmt, const float *W,
@@ -136,6 +137,11 @@ size_t uq_index_bytes(const uq_layout *L, int idx_bits)
     return (size_t)L->worker_stride * (size_t)idx_bits / 8;
 }
 
+int uq_encode_launches(const uq_layout *L, int select, int reconstruct)
+{
+    return layout_ok(L) ? uq::encode_launches(*L, select != 0, reconstruct != 0) : 0;
+}
+
 int uq_agree_scale(const uq_layout *L, const void *g, int norm, float *W, uint32_t *status, void *workspace,
                    size_t workspace_bytes, void *stream)
 {
@@ -235,8 +241,8 @@ int uq_decode(const uq_layout *L, const void *src, int src_kind, int fmt, const 
                                               (cudaStream_t)stream));
 }
 
-// Quantization, sum over the workers and reconstruction as one kernel; select: the shared indices are
-// found by that kernel too (by a kernel of their own in front with more than 8 workers).
+// Quantization, sum over the workers and reconstruction; select: the shared indices are found too.  One kernel, or one
+// per stage (uq_encode_launches).
 static int encode_decode(const uq_layout *L, const void *g, const float *W, int s, const int32_t *scales, int N,
                          uint8_t *idx, int idx_bits, bool select, uint64_t seed, int rng_bits, int fmt, void *lev,
                          float *out, int32_t *S_opt, uint32_t *status, void *stream)

@@ -188,13 +188,14 @@ class Quantizer:
         B.require_current_device(self.device.index, current, "the quantizer")
 
     def kernels_per_step(self) -> int:
-        """Kernel launches one step enqueues (norm partials + finalize, [select,] encode[, decode]: one
-        kernel when the encoder also selects, aggregates and reconstructs)."""
+        """Kernel launches one step enqueues: norm partials + their sum, and what follows as one kernel or as one per
+        stage (the library's choice by size, or the caller's)."""
         if self.one_kernel:
             return 1
-        separate_select = self.multi and not self.selects_inside and self.d > 0
-        tail = 0 if self.d == 0 else 1 if self.fused_decode else 2
-        return (2 if self.d > 0 else 1) + (1 if separate_select else 0) + tail
+        if self.d == 0:
+            return 1
+        n = 2 + B.lib().uq_encode_launches(self.layout.ref(), self.selects_inside, self.fused_decode)
+        return n + (self.multi and not self.selects_inside) + (not self.fused_decode)
 
     def status_bits(self) -> int:
         """Synchronizes and returns the device status word (0 = clean)."""

@@ -11,6 +11,7 @@ import pytest
 
 from paper_2109_12497_b200 import binding as B
 from paper_2109_12497_b200 import build as uq_build
+from paper_2109_12497_b200 import pipeline
 
 ROOT = Path(__file__).resolve().parent.parent
 
@@ -66,6 +67,24 @@ def test_scratch_of_the_norms_grows_with_the_layout(lib):
         for d in (1, 8191, 8193, 10304, 100_003, 262_145, 524_288, 524_289, 600_000, 2_000_000, 25_557_032):
             L = _layout(d=d, worker_stride=-(-d // 32) * 32, M=M, nseg=nseg, seg_off=0x10000 if nseg > 1 else None)
             assert lib.uq_workspace_bytes(C.byref(L)) == M * (-(-d // 8192) + nseg) * 8
+
+
+def test_kernels_behind_the_norms(lib):
+    """One kernel, or one per stage for many workers of a small gradient (the count that Quantizer.kernels_per_step reports)."""
+    def n(M, d, select, reconstruct, nseg=1):
+        return lib.uq_encode_launches(C.byref(_layout(M=M, d=d, worker_stride=-(-d // 32) * 32, nseg=nseg, seg_off=0x10000)), select,
+                                      reconstruct)
+    assert [n(8, 25_557_032, s, r) for s in (0, 1) for r in (0, 1)] == [1, 1, 1, 1]
+    assert [n(64, 50_001, s, r) for s in (0, 1) for r in (0, 1)] == [1, 2, 2, 3]
+    assert [n(20, d, 1, 1) for d in (50_001, 239_999, 240_001)] == [3, 3, 1] and n(19, 50_001, 1, 1) == 1
+    assert [n(25, d, 1, 1, 7) for d in (50_001, 124_999, 125_001)] == [3, 3, 1] and n(24, 50_001, 1, 1, 7) == 1
+    assert [n(32, 256 * k, 1, 1) for k in (93, 94)] == [3, 1] and n(28, 256, 1, 1) == 1
+    assert [n(8, d, 1, 0) for d in (239_999, 240_001)] == [2, 1] and n(7, 9_001, 1, 0) == 1
+    assert [n(M, 9_001, 1, 0, 7) for M in (15, 16)] == [1, 2]
+    assert [n(25, 256 * k, 1, 0) for k in (351, 352)] == [2, 1] and n(8, 0, 1, 1) == 0 and n(65, 100, 0, 1) == 0
+    q = pipeline.Quantizer(25, 1000, device="cpu", scales=[127, 1016], idx_bits=2)
+    assert [q.kernels_per_step(), pipeline.Quantizer(64, 1001, device="cpu").kernels_per_step(),
+            pipeline.Quantizer(8, 1001, device="cpu", one_kernel=False).kernels_per_step()] == [5, 4, 3]
 
 
 def test_bad_arguments_are_rejected_on_the_host(lib):

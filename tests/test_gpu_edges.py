@@ -12,8 +12,7 @@ from parity import _check_parity, check_parity, ulp_distance
 pytestmark = pytest.mark.gpu
 
 
-# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 40 000 unit-rows and 4096 units,
-# a cooperative grid above, and more than one pass per thread (values read again) beyond one unit per register set
+# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 4096 units, a cooperative grid above, and more than one pass per thread (values read again) beyond one unit per register set
 @pytest.mark.parametrize("M,d", [(2, 8 * 1024), (2, 8 * 1024 + 1), (2, 8 * 4096), (2, 8 * 4096 + 1), (8, 8 * 4096 - 7),
                                  (3, 8 * 4097), (1, 8 * 4096), (8, 8 * 148 * 512 + 1), (8, 2 * 8 * 148 * 512 + 9)])
 @pytest.mark.parametrize("dtype,scales,rng_bits", [(wl.F32, (127,), 16), (wl.BF16, (7, 56), 32), (wl.F32, (7, 56, 448), 32),
@@ -24,12 +23,17 @@ def test_one_kernel_step_at_the_edges_of_its_grids(M, d, dtype, scales, rng_bits
     assert _check_parity(w, wl.generate(w), None, "one")["q"].one_kernel
 
 
-# many workers of a small gradient: separate kernels up to 148 * 4 * 256 coordinates and above 24 workers
-@pytest.mark.parametrize("M", [24, 25, 64])
-@pytest.mark.parametrize("d", [148 * 4 * 256, 148 * 4 * 256 + 1])
+# many workers of a small gradient: both sides of the lines between one kernel and one per stage, with the sums (20
+# workers or more) and for selection and levels alone (8 or more), with and without a row that d ends in
+@pytest.mark.parametrize("M,d", [
+    (24, 148 * 4 * 256), (25, 148 * 4 * 256), (64, 148 * 4 * 256), (64, 148 * 4 * 256 + 1), (19, 50_001), (20, 50_001), (20, 239_999),
+    (20, 240_001), (32, 93 * 256), (32, 94 * 256), (7, 9_001), (8, 239_999), (8, 240_001), (25, 351 * 256), (25, 352 * 256), (16, 9_001),
+    (25, 124_999), (25, 125_001),
+])
 @pytest.mark.parametrize("name", ["c2", "c3"])
-def test_many_workers_of_a_small_gradient(name, d, M):
-    w = wl.scaled(name, d, M=M)
+@pytest.mark.parametrize("segments", ["one", "layers161"])
+def test_many_workers_of_a_small_gradient(name, d, M, segments):
+    w = wl.scaled(name, d, M=M, segments=segments)
     check_parity(w, wl.generate(w))
 
 
