@@ -133,3 +133,15 @@ def test_benchmark_times_the_real_exchange_when_there_are_several_processes(name
             expect += 2 * (world - 1) * (P * w.idx_bits // 8)
         assert rec["slices"]["wire_bytes_received_per_process_and_step"] == expect
         assert np.allclose(res[: w.d], want, rtol=1e-6, atol=0)
+
+
+def test_the_line_on_stdout_is_short(capsys):
+    """Details, which are many times as long, go to stderr."""
+    import json
+    import bench
+    line = {"metric": bench.METRIC, "value": 1.0, "kernels": {"k": "x" * 10_000}, "other_workloads": {"c1": "x" * 10_000},
+            "cold_l2": {}, "cuda_graph_warm_l2": {}, "roofline": {"frac": 0.5}}
+    bench.print_line(line)
+    out, err = capsys.readouterr()
+    assert json.loads(out) == {"metric": bench.METRIC, "value": 1.0, "roofline": {"frac": 0.5}}
+    assert set(json.loads(err)["details"]) == {"kernels", "other_workloads", "cold_l2", "cuda_graph_warm_l2"}
