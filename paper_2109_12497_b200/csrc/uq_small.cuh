@@ -32,6 +32,7 @@ constexpr int kSmallMaxWorkers = 8;
 constexpr int kSmallHeader = 64;                  // bytes in front of the partials: arrival and departure counters
 constexpr uint32_t kSmallSpinLimit = 1u << 20;    // polls of the counter before a CTA gives up (about a second)
 constexpr int kSmallThreads = 512;                // most threads per CTA
+constexpr int kSmallMinThreads = 128;             // least threads per CTA of a cooperative grid
 
 struct SmallParams {
     const void *g;
@@ -405,10 +406,10 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    // One cluster, a unit per thread, while its few SMs take no longer than a grid over all of them loses in its
-    // barrier and its cooperative launch (about 3 us): a unit-row is 8 coordinates at about 35 cycles per warp
-    // and scheduler, so 40 k of them are 5.5 k cycles on 16 SMs.
-    if (nunits * p.M <= 40000 && nunits <= 8 * kSmallThreads) {
+    // One cluster, a unit per thread, up to 4096 units: its few SMs then take no longer than a grid over all of them
+    // loses in its barrier and its cooperative launch (about 3 us; a unit-row is 8 coordinates at about 35 cycles per
+    // warp and scheduler, so 8 workers are 4.5 k cycles on 16 SMs).
+    if (nunits <= 8 * kSmallThreads) {
         static int ccache[64] = {};
         // one warp per scheduler of 8 SMs is not worth spreading further
         const int ctas = nunits <= 8 * 128 ? 8 : cluster_ctas(small_step_kernel<DT, NORM, RNG, MULTI, true, MW>, ccache);
@@ -424,11 +425,16 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
     static int cache[64] = {};
     const int resident = min(resident_ctas(small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, cache), kSmallMaxCtas);
     if (resident <= 0) return cudaErrorNotSupported;
-    const int64_t per = (nunits + kSmallThreads - 1) / kSmallThreads;     // CTAs at one unit per thread
+    // As many CTAs as the GPU takes before any has more than kSmallMinThreads threads: with 512 threads in each, a
+    // gradient of 60 000 coordinates was left to a tenth of the SMs.  512 / 256 / 128 / 64 threads, launches without
+    // gaps, against an older kernel of 256: 1 binary32 worker of 60 000 coordinates 1.16 / 0.99 / 0.98 / 0.97, 8 workers
+    // 1.09 / 0.84 / 0.78 / 0.81, 8 bf16 workers of 151 552 1.07 / 0.84 / 0.86 / 0.86.
+    const int64_t threads = max((int64_t)kSmallMinThreads, min((int64_t)kSmallThreads, ((nunits + resident - 1) / resident + 31) / 32 * 32));
+    const int64_t per = (nunits + threads - 1) / threads;                 // CTAs at one unit per thread
     p.rounds = (int)((per + (int64_t)resident * UPT - 1) / ((int64_t)resident * UPT));
     const int64_t units = (per + resident - 1) / resident;                // units per thread that the grid needs
     cfg.gridDim = dim3((unsigned)min((int64_t)resident, (per + units - 1) / units));
-    cfg.blockDim = dim3(kSmallThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.numAttrs = 1;

@@ -12,9 +12,12 @@ from parity import _check_parity, check_parity, ulp_distance
 pytestmark = pytest.mark.gpu
 
 
-# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 4096 units, a cooperative grid above, and more than one pass per thread (values read again) beyond one unit per register set
-@pytest.mark.parametrize("M,d", [(2, 8 * 1024), (2, 8 * 1024 + 1), (2, 8 * 4096), (2, 8 * 4096 + 1), (8, 8 * 4096 - 7),
-                                 (3, 8 * 4097), (1, 8 * 4096), (8, 8 * 148 * 512 + 1), (8, 2 * 8 * 148 * 512 + 9)])
+# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 4096 units, a cooperative grid above: of 128
+# threads per CTA up to 148 * 128 units, then more, and more than one pass per thread (values read again) beyond one unit
+# per register set
+@pytest.mark.parametrize("M,d", [(2, 8 * 1024), (2, 8 * 1024 + 1), (2, 8 * 4096), (2, 8 * 4096 + 1), (8, 8 * 4096 - 7), (3, 8 * 4097),
+                                 (1, 8 * 4096), (2, 8 * 148 * 128), (1, 8 * 148 * 128 + 1), (5, 8 * 148 * 160 + 9), (8, 8 * 148 * 480 + 1),
+                                 (8, 8 * 148 * 512 + 1), (8, 2 * 8 * 148 * 512 + 9)])
 @pytest.mark.parametrize("dtype,scales,rng_bits", [(wl.F32, (127,), 16), (wl.BF16, (7, 56), 32), (wl.F32, (7, 56, 448), 32),
                                                    (wl.BF16, (127,), 16)])
 def test_one_kernel_step_at_the_edges_of_its_grids(M, d, dtype, scales, rng_bits):
