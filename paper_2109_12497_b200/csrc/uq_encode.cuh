@@ -74,40 +74,29 @@ template <int DT, int RNG, bool SEL, int WK> struct EncodeShape {
 };
 
 // ---------------------------------------------------------------------------------------------
-// the packed indices of UC coordinates: coordinates 0..3 in fields of ib bits from bit 0 of kw[0],
-// coordinates 4..7 in kw[1] (bits beyond a word's four fields: anything)
+// the packed indices of a unit: coordinates 0..3 in fields of ib bits from bit 0 of kw[0],
+// coordinates 4..7 in kw[1] (loaded: bits beyond a word's four fields are anything; stored: they must be 0)
 // ---------------------------------------------------------------------------------------------
-template <int UC> __device__ __forceinline__ void load_indices(const uint8_t *idx, int64_t i, int ib, uint32_t *kw)
+__device__ __forceinline__ void load_indices(const uint8_t *idx, int64_t i, int ib, uint32_t (&kw)[2])
 {
     const uint8_t *p = idx + ((i * ib) >> 3);
-    const int bits = UC * ib;
-    if (bits == 64) {
+    if (ib == 8) {
         const uint2 x = __ldg((const uint2 *)p);
-        kw[0] = x.x; kw[UC / 4 - 1] = x.y;
+        kw[0] = x.x; kw[1] = x.y;
         return;
     }
-    uint32_t x;
-    if (bits == 32) x = __ldg((const uint32_t *)p);
-    else if (bits == 16) x = __ldg((const uint16_t *)p);
-    else x = __ldg(p);
-    if (UC == 8) { kw[0] = x; kw[UC / 4 - 1] = x >> (4 * ib); }
-    else kw[0] = bits == 4 ? x >> (i & 4) : x;
+    kw[0] = ib == 4 ? __ldg((const uint32_t *)p) : ib == 2 ? __ldg((const uint16_t *)p) : __ldg(p);
+    kw[1] = kw[0] >> (4 * ib);
 }
 
-// Stores them (kw without stray bits); called by whole warps (4 bits per thread: two lanes share a byte).
-template <int UC> __device__ __forceinline__ void store_indices(uint8_t *idx, int64_t i, int ib, const uint32_t *kw)
+__device__ __forceinline__ void store_indices(uint8_t *idx, int64_t i, int ib, const uint32_t (&kw)[2])
 {
     uint8_t *p = idx + ((i * ib) >> 3);
-    const int bits = UC * ib;
-    if (bits == 64) { *(uint2 *)p = make_uint2(kw[0], kw[UC / 4 - 1]); return; }
-    const uint32_t x = UC == 8 ? kw[0] | (kw[UC / 4 - 1] << (4 * ib)) : kw[0];
-    if (bits == 32) *(uint32_t *)p = x;
-    else if (bits == 16) *(uint16_t *)p = (uint16_t)x;
-    else if (bits == 8) *p = (uint8_t)x;
-    else {
-        const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, x, 1);
-        if ((i & 4) == 0) *p = (uint8_t)(x | (next << 4));
-    }
+    if (ib == 8) { *(uint2 *)p = make_uint2(kw[0], kw[1]); return; }
+    const uint32_t x = kw[0] | (kw[1] << (4 * ib));
+    if (ib == 4) *(uint32_t *)p = x;
+    else if (ib == 2) *(uint16_t *)p = (uint16_t)x;
+    else *p = (uint8_t)x;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -134,9 +123,9 @@ __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0, 
             const uint64_t packed = select_general(p.v, i, amag, p.idx_bits, j);
             kw[0] = (uint32_t)packed & (uint32_t)((1ull << (4 * p.idx_bits)) - 1ull);
             kw[1] = (uint32_t)(packed >> (4 * p.idx_bits));
-            store_indices<8>(p.idx, i, p.idx_bits, kw);
+            store_indices(p.idx, i, p.idx_bits, kw);
         } else {
-            load_indices<8>(p.idx, i, p.idx_bits, kw);
+            load_indices(p.idx, i, p.idx_bits, kw);
         }
     }
     float inv[8], c[8];
@@ -387,7 +376,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
 #pragma unroll
             for (int c = 0; c < G; ++c)
                 if (WK || m_first + c < m_last) load(c, q[c]);
-            if (MULTI) load_indices<8>(p.idx, i, ib, kw);
+            if (MULTI) load_indices(p.idx, i, ib, kw);
         }
     }
     const int j = warp_find_segment(p.v.seg_off, p.v.nseg, r0);
@@ -492,7 +481,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
             kw[1] = mixed_row_select(p, i + 4, j, amag[4], amag[5], amag[6], amag[7]);
             __syncwarp();
         }
-        store_indices<8>(p.idx, i, ib, kw);
+        store_indices(p.idx, i, ib, kw);
         if (!STAGED) policy = policy_drop();
 #pragma unroll
         for (int c = 0; c < G; ++c)

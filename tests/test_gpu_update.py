@@ -56,15 +56,14 @@ def _fused_update_case(w, lr, mu, wd, use_mom):
 @pytest.mark.parametrize("fmt,s", [("i8", 127), ("i4x2", 7), ("i2x4", 1), ("i6p", 31)])
 @pytest.mark.parametrize("N,idx_bits", [(2, 1), (4, 2), (8, 4), (3, 8)])
 def test_update_without_the_gradient_output(fmt, s, N, idx_bits):
-    """out = NULL (the update a training loop makes): the same parameters and momentum as with it."""
+    """out = NULL (the update a training loop makes): the oracle's parameters and momentum."""
     w = wl.scaled("c3", 33_001, M=8, fmt=fmt, s=s, scales=tuple(s * 8 ** k for k in range(N)), idx_bits=idx_bits)
-    q = run_gpu(w, wl.generate(w))["q"]
-    got = []
-    for out in (torch.empty(w.d, device="cuda"), None):
-        theta, mom = torch.ones(w.d, device="cuda"), torch.zeros(w.d, device="cuda")
-        B.uq_decode_update(q.layout, q.lev, q.fmt, q.W, q.s, q.scales, q.idx, q.idx_bits, theta, mom, 0.1, 0.9, 5e-4, out)
-        got.append((theta, mom))
-    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    r = check_parity(w, wl.generate(w))
+    q = r["q"]
+    theta, mom = torch.ones(w.d, device="cuda"), torch.zeros(w.d, device="cuda")
+    B.uq_decode_update(q.layout, q.lev, q.fmt, q.W, q.s, q.scales, q.idx, q.idx_bits, theta, mom, 0.1, 0.9, 5e-4, None)
+    want, want_m = o.sgd_update(r["ref"]["out"], np.ones(w.d, np.float32), np.zeros(w.d, np.float32), lr=0.1, mu=0.9, wd=5e-4)
+    assert np.array_equal(theta.cpu().numpy(), want) and np.array_equal(mom.cpu().numpy(), want_m)
 
 
 def test_update_rejects_bad_arguments():
