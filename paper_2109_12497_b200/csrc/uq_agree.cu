@@ -287,29 +287,55 @@ norm_staged_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int ns
         }
         return;
     }
+    // The pieces of my chunk that are mine, four at a time: their reductions over the lanes overlap.
     int64_t a = c0;
-    for (int j = j0, k = 0; a < c1; ++j) {                                       // the pieces of my chunk
-        const int64_t seg_a = seg_b;
-        seg_b = j - base < 32 ? __shfl_sync(0xFFFFFFFFu, ends, (j - base) & 31) : segment_end(seg_off, nseg, j, d);
-        const int64_t b = min(max(seg_b, a), c1);
-        if (b > a && k++ % WPC == sub) {
+    int j = j0, k = 0;
+    bool more = a < c1;
+    while (more) {
+        double w[4];
+        int seg[4];                                                              // -1: no piece
+        bool first[4], goes_on[4];                                               // may continue one from the left; may continue to the right
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
             Acc<NORM> acc;
+            seg[n] = -1;
+            while (more && seg[n] < 0) {
+                const int64_t seg_a = seg_b;
+                if (j - base == 32) {
+                    ends = segment_end(seg_off, nseg, min(j + lane, nseg - 1), d);
+                    base = j;
+                }
+                seg_b = __shfl_sync(0xFFFFFFFFu, ends, j - base);
+                const int64_t b = min(max(seg_b, a), c1);
+                if (b > a && k++ % WPC == sub) {
+                    seg[n] = j;
+                    first[n] = a == c0 && seg_a < c0;
+                    goes_on[n] = b == c1 && seg_b > c1;
 #pragma unroll 8
-            for (int i = (int)(a - t0) + lane; i < (int)(b - t0); i += 32) {
-                const T x = *((const T *)stage + i);
-                acc.add(DT == UQ_F32 ? (float)x : __uint_as_float((uint32_t)x << 16));
+                    for (int i = (int)(a - t0) + lane; i < (int)(b - t0); i += 32) {
+                        const T x = *((const T *)stage + i);
+                        acc.add(DT == UQ_F32 ? (float)x : __uint_as_float((uint32_t)x << 16));
+                    }
+                    __syncwarp();
+                }
+                a = b;
+                more = a < c1 && j + 1 < nseg;
+                ++j;
             }
-            __syncwarp();
-            const double w = warp_reduce<NORM>(acc.value());
-            const bool goes_on = b == c1 && seg_b > c1;                            // may continue in the right chunk
-            if (lane == 0) {
-                if (a == c0 && seg_a < c0) { sh_head[chunk] = w; sh_head_seg[chunk] = j; sh_head_open[chunk] = goes_on; }   // may continue one from the left
-                else if (goes_on) { sh_tail[chunk] = w; sh_tail_seg[chunk] = j; }
-                else prow[tile + j] = w;
+            w[n] = acc.value();
+        }
+#pragma unroll
+        for (int n = 0; n < 4; ++n) w[n] = warp_reduce<NORM>(w[n]);
+        if (lane == 0) {
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                if (seg[n] < 0) continue;
+                if (first[n]) { sh_head[chunk] = w[n]; sh_head_seg[chunk] = seg[n]; sh_head_open[chunk] = goes_on[n]; }
+                else if (goes_on[n]) { sh_tail[chunk] = w[n]; sh_tail_seg[chunk] = seg[n]; }
+                else prow[tile + seg[n]] = w[n];
             }
         }
-        a = b;
-        if (j + 1 >= nseg) break;
+        __syncwarp();
     }
     __syncthreads();
     // What goes on to the right is added up in chunk order, a thread per piece that starts one: the tail of a chunk, or
