@@ -360,16 +360,15 @@ int uq_step(const uq_layout *layout, const void *g, int norm, int s, const int32
  * "MaxAllReduce Norm" to "Reconstruct gradient" — for gradients so small that the launches of
  * uq_step cost more than its arithmetic.  Every thread reads its coordinates of all workers, and
  * keeps them in registers while the norms are agreed on, across one thread-block cluster (up to
- * 32768 coordinates) or a cooperative grid with one grid-wide barrier; then it [selects and shares the
+ * 32768 coordinates) or a grid with one grid-wide barrier (whose CTAs need not all be resident); then it [selects and shares the
  * scale indices,] quantizes, stores the level rows, adds the levels and writes the reconstructed average.
  * A gradient beyond the grid's registers is read again.  The first call of a configuration on a
  * device asks for its occupancy and may set a kernel attribute: make it during set-up, before any
  * stream capture.
  * Arguments as in uq_step.  Supported: one segment (layout->nseg = 1), M <= 8, formats
  * UQ_FMT_I8 / I4X2 / I2X4, both dtypes, norms, draw widths, every index width; worker0 and coord0
- * key the draws as in the encoders.  Anything else returns UQ_ERR_UNSUPPORTED, as does a device
- * without cooperative launches.  Any size is computed correctly; it pays while M * d elements are
- * a few megabytes.
+ * key the draws as in the encoders.  Anything else returns UQ_ERR_UNSUPPORTED.  Any size is computed
+ * correctly; it pays while M * d elements are a few megabytes.
  *   workspace     scratch, device, 8-byte aligned, >= uq_workspace_bytes_small() bytes, used by one
  *                 call at a time.  Its first 64 bytes must be ZERO before the first call (zero
  *                 the scratch once after allocating it); every call leaves them zero again, except

@@ -462,7 +462,7 @@ def uq_step_small(layout: Layout, g: torch.Tensor, norm: int, s: int, scales: Op
                   seed: int, rng_bits: int, fmt: int, W: torch.Tensor, idx: Optional[torch.Tensor], lev: torch.Tensor,
                   out: torch.Tensor, S_opt: Optional[torch.Tensor], status: Optional[torch.Tensor],
                   workspace: torch.Tensor) -> None:
-    """The whole step of either quantizer as one cooperative kernel (small gradients); arguments as
+    """The whole step of either quantizer as one kernel (small gradients); arguments as
     uq_step.  ``workspace``: zero-filled before its first use (the kernel leaves its counters
     zero), one call at a time."""
     layout.check_g(g)

@@ -6,20 +6,25 @@
 // unit-rows: UPT units of MW workers) across the scale agreement:
 //   phase 1  the norm accumulators of the workers, reduced over the CTA
 //   exchange the CTAs' partials: CLUSTER (8 or 16 CTAs): through distributed shared memory, behind the
-//            cluster barrier; otherwise a cooperative grid through the scratch, behind an arrival counter
-//            (zero when the kernel starts: the caller zeroes the scratch once, the last CTA through the
-//            barrier zeroes the counters again); that wait is bounded: a CTA that gives up sets
+//            cluster barrier; otherwise through the scratch, behind an arrival counter (zero when the kernel
+//            starts: the caller zeroes the scratch once, the last CTA to go zeroes it again).  Nothing is assumed
+//            about which CTAs are resident: a CTA marks its share as taken before it begins, and one that has
+//            waited for long takes a share that nobody has, so the grid gets on with whatever part of it runs (a
+//            CTA whose share was taken returns).  The wait is bounded all the same: a CTA that gives up sets
 //            UQ_STATUS_TIMEOUT and returns.  All warps add up the partials in the same fixed order, so all of
 //            them hold the same bits of W
 //   phase 2  [the shared indices from the maxima over the workers,] quantization of the workers' units, level
 //            rows, sums in packed lanes, average
-// Only a gradient with more units than the grid holds is read again in phase 2.  Levels, indices, sums and the
+// Only a gradient with more units than the grid holds, and shares taken from others, are read again in phase 2.  Levels, indices, sums and the
 // reconstruction are bit for bit those of the separate calls given the same W; W itself is summed in another
 // fixed order (L2: within one unit in the last place of the regular kernel's).
 //
 // What bounds it is latency: one trip to memory, the barrier, the chains of the Philox rounds.  Measured on a
 // B200, launches back to back (a grid with a counter in memory, every value loaded twice -> this form):
-// 4 x 4099 bf16, 8 scales 8.8 -> 5.2 us, 8 x 10^4 fp32 10.1 -> 6.8 us (one cluster); 2 x 2^20 fp32 10.9 -> 10.5 us.
+// 4 x 4099 bf16, 8 scales 8.8 -> 5.2 us, 8 x 10^4 fp32 10.1 -> 6.8 us (one cluster).  A step of 2 x 2^20 binary32 took
+// 12.3 us as a cooperative launch, which is what such launches take one after the other whatever the kernel does; as
+// an ordinary one, whose launch overlaps the kernel in front, 10.1.  (The draws of the first units made while their
+// loads are on their way, kept in shared memory: no gain on the grid, one cluster 5.5 -> 6.0 us.)
 #pragma once
 #include "uq_device.cuh"
 #include "uq_norm.cuh"
@@ -29,10 +34,13 @@
 namespace uq {
 
 constexpr int kSmallMaxWorkers = 8;
-constexpr int kSmallHeader = 64;                  // bytes in front of the partials: arrival and departure counters
+constexpr int kSmallHeader = 64;                  // bytes in front of the partials: arrival and departure counters, shares taken
+constexpr int kSmallTaken = 2;                    // the header's first word of the bits of shares taken
+constexpr int kSmallShares = (kSmallHeader / 4 - kSmallTaken) * 32;
 constexpr uint32_t kSmallSpinLimit = 1u << 20;    // polls of the counter before a CTA gives up (about a second)
+constexpr uint32_t kSmallPatience = 64;           // polls before it looks for a share that nobody has taken (about 50 us)
 constexpr int kSmallThreads = 512;                // most threads per CTA
-constexpr int kSmallMinThreads = 128;             // least threads per CTA of a cooperative grid
+constexpr int kSmallMinThreads = 128;             // least threads per CTA of a grid
 
 struct SmallParams {
     const void *g;
@@ -41,7 +49,7 @@ struct SmallParams {
     float *W, *out;
     int32_t *S;
     uint32_t *status;
-    uint32_t *counter;        // scratch: [0] arrivals, [1] departures
+    uint32_t *counter;        // scratch: [0] arrivals, [1] departures, [kSmallTaken ..] shares taken
     double *part;             // scratch: [gridDim.x][kSmallMaxWorkers]
     int64_t d, stride, coord0;
     int32_t M, worker0, fmt, idx_bits;
@@ -113,16 +121,18 @@ template <int DT, int NORM, int RNG, bool MULTI, bool CLUSTER, int MW>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 small_step_kernel(const __grid_constant__ SmallParams p)
 {
-    if (CLUSTER) grid_dependency_prologue();
+    grid_dependency_prologue();
     using E = Elem<DT>;
     constexpr int H = 8 / E::G, UPT = kSmallMaxWorkers / MW;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int M = p.M, ib = p.idx_bits;
     const int64_t d = p.d, nunits = (d + 7) >> 3;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + tid, T = (int64_t)gridDim.x * blockDim.x;
+    int64_t t = (int64_t)blockIdx.x * blockDim.x + tid;                 // of the share that I am at
+    const int64_t T = (int64_t)gridDim.x * blockDim.x;
     __shared__ double sh[kSmallThreads / 32][MW], sh2[kSmallThreads / 32][MW];
     __shared__ double sh_part[MW];
-    __shared__ int sh_fail;
+    __shared__ int sh_next;                                              // after the wait: -1 go on, below: return, else a share to take
+    __shared__ uint16_t sh_taken[kSmallShares];                        // shares that I took from others
 
     uint4 q[UPT][MW][H];
     auto load = [&](int round) {
@@ -153,8 +163,8 @@ small_step_kernel(const __grid_constant__ SmallParams p)
         }
     };
 
-    // ---- phase 1: per-worker norm partials of my units
-    {
+    // ---- phase 1: per-worker norm partials of a share's units
+    auto norms = [&](int share) {
         Acc<NORM> acc[MW];
         for (int round = 0; round < p.rounds; ++round) {
             load(round);
@@ -175,48 +185,71 @@ small_step_kernel(const __grid_constant__ SmallParams p)
             const double w = m < M ? warp_reduce<NORM>(acc[m].value()) : 0.0;
             if (lane == 0) sh[warp][m] = w;
         }
-    }
-    __syncthreads();
-    if (tid < MW) {
-        double tot = sh[0][tid];
-        for (int k = 1; k < nwarps; ++k) tot = combine<NORM>(tot, sh[k][tid]);
-        if (CLUSTER) sh_part[tid] = tot;
-        else p.part[(size_t)blockIdx.x * kSmallMaxWorkers + tid] = tot;
-    }
+        __syncthreads();
+        if (tid < MW) {
+            double tot = sh[0][tid];
+            for (int k = 1; k < nwarps; ++k) tot = combine<NORM>(tot, sh[k][tid]);
+            if (CLUSTER) sh_part[tid] = tot;
+            else __stcg(p.part + (size_t)share * kSmallMaxWorkers + tid, tot);
+        }
+    };
+    uint32_t mine = 1;                                                  // whether my share is still mine
+    if (!CLUSTER && tid == 0) mine = !(atomicOr(p.counter + kSmallTaken + (blockIdx.x >> 5), 1u << (blockIdx.x & 31)) >> (blockIdx.x & 31) & 1u);
 
     // ---- the exchange, and W
+    int taken = 0;
     float W;
     if (CLUSTER) {
+        norms(0);
         __syncwarp();
         cluster_arrive();
         cluster_wait();
         W = scale_from_sums<NORM, MW>(sum_partials<NORM, MW>(0, 1, (int)gridDim.x, [&](int c, int m) { return ld_cluster(sh_part + m, c); }), M);
         cluster_arrive();                          // waited for at the end: my shared memory may be read until then
     } else {
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) {
-            __threadfence();                  // release: this CTA's partials (ordered before the barrier above) before its arrival
-            atomicAdd(p.counter, 1u);
-            uint32_t polls = 0;
-            int fail = 0;
-            while (ld_acquire(p.counter) < gridDim.x) {
-                if (++polls > kSmallSpinLimit) { fail = 1; break; }
-                __nanosleep(32);
+        int share = blockIdx.x;
+        while (true) {
+            norms(share);
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) {
+                if (mine) {
+                    __threadfence();          // release: this share's partials (ordered before the barrier above) before its arrival
+                    atomicAdd(p.counter, 1u);
+                }
+                int next = mine ? -1 : -3;
+                for (uint32_t polls = 0; mine && ld_acquire(p.counter) < gridDim.x; ++polls) {
+                    if (polls > kSmallSpinLimit) { next = -2; break; }
+                    if (polls % kSmallPatience == kSmallPatience - 1) {
+                        // a share that nobody has: its CTA may be waiting for an SM that I hold
+                        for (int w = 0; w * 32 < (int)gridDim.x && next < 0; ++w) {
+                            const uint32_t all = gridDim.x - w * 32 >= 32 ? 0xFFFFFFFFu : (1u << (gridDim.x - w * 32)) - 1u;
+                            const uint32_t open = all & ~ld_acquire(p.counter + kSmallTaken + w);
+                            if (open == 0u) continue;
+                            const uint32_t bit = open & (0u - open);
+                            if (!(atomicOr(p.counter + kSmallTaken + w, bit) & bit)) next = w * 32 + __ffs((int)bit) - 1;
+                        }
+                        if (next >= 0) break;
+                    }
+                    __nanosleep(32);
+                }
+                __threadfence();              // acquire: the other CTAs' partials after their arrivals
+                if (next == -2) atomicOr(p.status, (uint32_t)UQ_STATUS_TIMEOUT);
+                sh_next = next;
+                // the last CTA to go puts the counters and the marks back to zero for the next call (every CTA has
+                // looked at its mark and read its last value of the arrival counter by then)
+                if ((next == -1 || next == -3) && atomicAdd(p.counter + 1, 1u) == gridDim.x - 1) {
+                    for (int w = kSmallHeader / 4 - 1; w >= 0; --w) p.counter[w] = 0u;
+                }
             }
-            __threadfence();                  // acquire: the other CTAs' partials after their arrivals
-            if (fail) atomicOr(p.status, (uint32_t)UQ_STATUS_TIMEOUT);
-            sh_fail = fail;
-            // the last CTA to leave the barrier puts both counters back to zero for the next call
-            // (every CTA has read its last value of the arrival counter by then)
-            if (!fail && atomicAdd(p.counter + 1, 1u) == gridDim.x - 1) {
-                p.counter[1] = 0u;
-                __threadfence();
-                p.counter[0] = 0u;
-            }
+            __syncthreads();
+            share = sh_next;
+            if (share < -1) return;
+            if (share == -1) break;
+            if (tid == 0) sh_taken[taken] = (uint16_t)share;
+            ++taken;
+            t = (int64_t)share * blockDim.x + tid;
         }
-        __syncthreads();
-        if (sh_fail) return;
         // each warp every nwarps-th CTA's partials, then every warp all warps' sums
         const double a = sum_partials<NORM, MW>(warp, nwarps, (int)gridDim.x,
                                                 [&](int c, int m) { return __ldcg(p.part + (size_t)c * kSmallMaxWorkers + m); });
@@ -247,8 +280,11 @@ small_step_kernel(const __grid_constant__ SmallParams p)
         __syncwarp();
     }
     const size_t row_bytes = (size_t)(p.stride >> p.fmt);
+    const bool again = p.rounds > 1 || taken > 0;                       // the values have left the registers
+    for (int share = 0; share <= taken; ++share) {
+    t = (int64_t)(share == 0 ? blockIdx.x : sh_taken[share - 1]) * blockDim.x + tid;
     for (int round = 0; round < p.rounds; ++round) {
-        if (p.rounds > 1) load(round);
+        if (again) load(round);
 #pragma unroll
         for (int k = 0; k < UPT; ++k) {
             const int64_t u = (int64_t)(round * UPT + k) * T + t, i = u << 3;
@@ -346,6 +382,7 @@ small_step_kernel(const __grid_constant__ SmallParams p)
             __syncwarp();
         }
     }
+    }
     if (CLUSTER) {
         __syncwarp();
         cluster_wait();
@@ -357,18 +394,17 @@ small_step_kernel(const __grid_constant__ SmallParams p)
 // ---------------------------------------------------------------------------------------------
 constexpr int kSmallMaxCtas = 148 * 8 * 2;            // bound used to size the scratch (far above today's largest part)
 
-// CTAs of one instantiation that fit the device at once (cooperative launches need the whole grid resident);
-// looked up once per device and instantiation.
+// CTAs of one instantiation that fit the device at once (with more, shares would wait for one another); looked up once
+// per device and instantiation.
 template <typename K> static int resident_ctas(K kernel, int *cache)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     if (cache[dev] == 0) {
-        int sms = 0, per_sm = 0, coop = 0;
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        int sms = 0, per_sm = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kSmallThreads, 0);
-        cache[dev] = coop && sms > 0 && per_sm > 0 ? sms * per_sm : -1;
+        cache[dev] = sms > 0 && per_sm > 0 ? sms * per_sm : -1;
     }
     return cache[dev] > 0 ? cache[dev] : 0;
 }
@@ -407,7 +443,7 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     // One cluster, a unit per thread, up to 4096 units: its few SMs then take no longer than a grid over all of them
-    // loses in its barrier and its cooperative launch (about 3 us; a unit-row is 8 coordinates at about 35 cycles per
+    // loses in its barrier (about 3 us; a unit-row is 8 coordinates at about 35 cycles per
     // warp and scheduler, so 8 workers are 4.5 k cycles on 16 SMs).
     if (nunits <= 8 * kSmallThreads) {
         static int ccache[64] = {};
@@ -423,7 +459,7 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
         return cudaLaunchKernelEx(&cfg, small_step_kernel<DT, NORM, RNG, MULTI, true, MW>, p);
     }
     static int cache[64] = {};
-    const int resident = min(resident_ctas(small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, cache), kSmallMaxCtas);
+    const int resident = min(resident_ctas(small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, cache), kSmallShares);
     if (resident <= 0) return cudaErrorNotSupported;
     // As many CTAs as the GPU takes before any has more than kSmallMinThreads threads: with 512 threads in each, a
     // gradient of 60 000 coordinates was left to a tenth of the SMs.  512 / 256 / 128 / 64 threads, launches without
@@ -435,9 +471,7 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
     const int64_t units = (per + resident - 1) / resident;                // units per thread that the grid needs
     cfg.gridDim = dim3((unsigned)min((int64_t)resident, (per + units - 1) / units));
     cfg.blockDim = dim3((unsigned)threads);
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = grid_dependency_attribute(attr);
     return cudaLaunchKernelEx(&cfg, small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, p);
 }
 

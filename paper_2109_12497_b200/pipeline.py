@@ -50,7 +50,7 @@ class Quantizer:
         nseg = self.layout.nseg
         self.W = torch.zeros(nseg, dtype=torch.float32, device=dev)
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
-        # one segment, few workers, and so small that the step is bound by its launches: the whole step as one cooperative kernel (uq_step_small).  None = decide by size.
+        # one segment, few workers, and so small that the step is bound by its launches: the whole step as one kernel (uq_step_small).  None = decide by size.
         fits = B.small_step_supported(self.layout, fmt)
         if one_kernel and not fits:
             raise ValueError("uq: the one-kernel step takes one segment, M <= 8 and one-plane level formats")

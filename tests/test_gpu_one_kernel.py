@@ -215,3 +215,27 @@ def test_agree_scale_between_steps_does_not_disturb_the_barrier():
         assert np.array_equal(q.lev.cpu().numpy()[:, : w.d], lev)
         assert np.array_equal(q.S.cpu().numpy()[: w.d], o.aggregate(lev))
         assert int(q.small_workspace[:64].sum().item()) == 0  # the counters are back at zero after every step
+
+
+@pytest.mark.parametrize("d,M,dtype", [(1 << 20, 2, wl.F32), (100_003, 8, wl.F32), (500_009, 4, wl.BF16)])
+def test_steps_on_several_streams_at_once(d, M, dtype):
+    """Grids that compete for the SMs: no CTA of a step needs another one of it to be resident.  Every stream's last step
+    is compared with the oracle."""
+    w = wl.scaled("c1", d, M=M, dtype=dtype)
+    g_np = wl.generate(w)
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    qs = [from_workload(w, keep_sums=True, one_kernel=True) for _ in streams]
+    gs = [to_device(w, g_np) for _ in streams]
+    torch.cuda.synchronize()
+    for step in range(60):
+        for k, (st, q, g) in enumerate(zip(streams, qs, gs)):
+            with torch.cuda.stream(st):
+                q.step(g, 1000 * k + step)
+    torch.cuda.synchronize()
+    W_ref = o.agree_scale(g_np[:, : w.d], None, o.NORM_LINF)
+    for k, q in enumerate(qs):
+        assert q.status_bits() == 0 and int(q.small_workspace[:64].sum().item()) == 0
+        assert np.array_equal(q.W.cpu().numpy(), W_ref)
+        lev = o.encode_single(g_np[:, : w.d], W_ref, w.s, 1000 * k + 59, w.rng_bits)
+        assert np.array_equal(q.lev.cpu().numpy()[:, : w.d], lev)
+        assert np.array_equal(q.S.cpu().numpy()[: w.d], o.aggregate(lev))
