@@ -23,7 +23,7 @@
 // B200, launches back to back (a grid with a counter in memory, every value loaded twice -> this form):
 // 4 x 4099 bf16, 8 scales 8.8 -> 5.2 us, 8 x 10^4 fp32 10.1 -> 6.8 us (one cluster).  A step of 2 x 2^20 binary32 took
 // 12.3 us as a cooperative launch, which is what such launches take one after the other whatever the kernel does; as
-// an ordinary one, whose launch overlaps the kernel in front, 10.1.  (The draws of the first units made while their
+// an ordinary one, whose launch overlaps the kernel in front, 10.1, and with one fence at the barrier instead of three 9.7.  (The draws of the first units made while their
 // loads are on their way, kept in shared memory: no gain on the grid, one cluster 5.5 -> 6.0 us.)
 #pragma once
 #include "uq_device.cuh"
@@ -210,11 +210,10 @@ small_step_kernel(const __grid_constant__ SmallParams p)
         int share = blockIdx.x;
         while (true) {
             norms(share);
-            __threadfence();
-            __syncthreads();
+            __syncwarp();                     // (the partials are this warp's)
             if (tid == 0) {
                 if (mine) {
-                    __threadfence();          // release: this share's partials (ordered before the barrier above) before its arrival
+                    __threadfence();          // release: this share's partials before its arrival
                     atomicAdd(p.counter, 1u);
                 }
                 int next = mine ? -1 : -3;
@@ -233,7 +232,6 @@ small_step_kernel(const __grid_constant__ SmallParams p)
                     }
                     __nanosleep(32);
                 }
-                __threadfence();              // acquire: the other CTAs' partials after their arrivals
                 if (next == -2) atomicOr(p.status, (uint32_t)UQ_STATUS_TIMEOUT);
                 sh_next = next;
                 // the last CTA to go puts the counters and the marks back to zero for the next call (every CTA has
