@@ -358,11 +358,12 @@ norm_staged_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int ns
 
 // One CTA per segment, one warp per worker: lane l adds up the slots of the segment's tiles l, l + 32, .. one after
 // the other, and then the lanes' sums are added.  That order depends on the segment's tiles alone: a worker's sum has
-// the same bits whatever else is in the buffer.  What bounds it is the latency of the loads, of which a lane has up to 32
-// in flight (8 at a time: 8 workers of 13.1 M coordinates in one segment 7.0 us, with up to 32 5.0).  (Several warps fetching a worker's slots into shared memory for the one that adds: 1 worker 14.9 -> 13.4
+// the same bits whatever else is in the buffer.  What bounds it is the latency of the loads, of which a lane has K
+// in flight: 8 workers of 13.1 M coordinates in one segment 7.0 us with 8, 5.0 with 32.  (With 32 throughout, a CTA's
+// registers do not fit beside the kernel in front of it: a step of 64 workers of 114 688 coordinates 46.5 -> 48 us.)  (Several warps fetching a worker's slots into shared memory for the one that adds: 1 worker 14.9 -> 13.4
 // us, 2 to 4 workers no faster, and with 40 KB of it the kernel in front, beside whose CTAs these start, took 4 %
 // longer; norms of 25.6 M bf16 coordinates in one segment.)
-template <int NORM>
+template <int NORM, int K>
 __global__ void __launch_bounds__(512)
 norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg,
                      const int64_t *__restrict__ seg_off, int64_t ntiles, float *__restrict__ W, uint32_t *__restrict__ status)
@@ -381,17 +382,13 @@ norm_finalize_kernel(const double *__restrict__ part, int M, int64_t d, int nseg
     for (int m = warp; m < M; m += nwarps) {
         const double *prow = part + (size_t)m * (size_t)(ntiles + nseg) + j;
         double acc = 0.0;
-        auto add = [&](auto n, int t) {                                // n of the lane's slots
-            constexpr int K = decltype(n)::value;
+        for (int t = first + lane; t <= last; t += 32 * K) {
             double v[K];
 #pragma unroll
             for (int k = 0; k < K; ++k) v[k] = t + k * 32 <= last ? __ldcg(prow + t + k * 32) : 0.0;      // 0 is neutral for both norms
 #pragma unroll
             for (int k = 0; k < K; ++k) acc = combine<NORM>(acc, v[k]);
-        };
-        int t = first + lane;
-        for (; t + 32 * 8 <= last; t += 32 * 32) add(std::integral_constant<int, 32>(), t);
-        if (t <= last) add(std::integral_constant<int, 8>(), t);
+        }
         __syncwarp();
         const double r = warp_reduce<NORM>(acc);
         if (lane == 0) sh[m] = r;
@@ -452,9 +449,11 @@ static cudaError_t launch(const uq_layout &L, const void *g, float *W, uint32_t 
             launch_k(norm_partials_kernel<DT, NORM>, grid, kThreads, st, g, L.d, L.worker_stride, L.nseg, L.seg_off, ntiles, part);
         }
     }
-    // segments of more than eight loads per lane: 16 workers side by side
-    launch_k(norm_finalize_kernel<NORM>, L.nseg, ntiles / L.nseg >= 256 ? 32 * min(L.M, 16) : kThreads, st, part, L.M, L.d, L.nseg,
-             L.seg_off, ntiles, W, status);
+    // segments of more than eight loads per lane: 16 workers side by side, and more loads
+    if (ntiles / L.nseg >= 256)
+        launch_k(norm_finalize_kernel<NORM, 32>, L.nseg, 32 * min(L.M, 16), st, part, L.M, L.d, L.nseg, L.seg_off, ntiles, W, status);
+    else
+        launch_k(norm_finalize_kernel<NORM, 8>, L.nseg, kThreads, st, part, L.M, L.d, L.nseg, L.seg_off, ntiles, W, status);
     return cudaGetLastError();
 }
 
