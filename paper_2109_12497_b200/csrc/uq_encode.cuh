@@ -58,13 +58,17 @@ constexpr int kGroup = 8;     // the number of workers that has kernels of its o
 // quantization + sum + reconstruction, sustained): bf16 with 32-bit draws 3 CTAs 188 us, 4 CTAs 197 us
 // (26.2 M coordinates); binary32, selecting, 32-bit draws: one worker at a time 266 us, two 273 us (25.6 M).
 //
+// binary32, 2 and 4 workers: the kernels of 8 with fewer of them, no loop, nothing spilled.  Steps, general kernel / these:
+// 4 workers of 25 M coordinates 176 / 173 us, of 25 M in 161 layers with 4 scales 247 / 218, 4-bit levels 171 / 165; 14.7 M with
+// two scales and 6-bit levels 156.6 / 141.0; of 40 003, whose last row is no slow one now, 12.5 / 9.6 and with 4 scales 17.6 / 9.8.
+//
 // Few workers (1 to 4 of bf16): what does not depend on the worker is then most of a lane's work, so all workers' blocks
 // go together straight-line, their rows are staged as the eight's are, and fewer registers let more warps hide the way
 // to memory.  25.6 M coordinates, 16-bit draws, general kernel / this / an encoder of two units per lane: levels alone,
 // one worker in 161 layers 40.9 / 33.2 / 32.9 us, two workers in one segment 47.9 / 41.5 / 38.2; with selection, two
 // workers 88.6 / 66.4 / 67.4.
 template <int DT, int RNG, bool SEL, int WK> struct EncodeShape {
-    static constexpr bool FEW = WK > 0 && WK < kGroup;
+    static constexpr bool FEW = DT == UQ_BF16 && WK > 0 && WK < kGroup;
     static constexpr int V = 8 * Elem<DT>::BYTES / 16;                        // 16-byte words per thread and worker
     static constexpr int NB = RNG == 32 ? 2 : 1;                              // Philox blocks per thread and worker
     static constexpr int G = FEW ? (RNG == 16 ? WK : WK % 2 == 0 ? 2 : 1)      // workers whose blocks advance together
@@ -104,8 +108,8 @@ __device__ __forceinline__ void store_indices(uint8_t *idx, int64_t i, int ib, c
 // ---------------------------------------------------------------------------------------------
 
 // Everything for the coordinates [r0, min(r0 + 256, d)), looked up coordinate by coordinate, in plain
-// arithmetic: the row that holds d, rows whose Philox block numbers leave the launch's high word, and
-// rows whose factors are too small or too large for the rescaled forms.  Workers m_first .. m_last - 1 (all of
+// arithmetic: the row that d ends in, in the kernels that do not take it as the others, rows whose Philox
+// block numbers leave the launch's high word, and rows whose factors are too small or too large for the rescaled forms.  Workers m_first .. m_last - 1 (all of
 // them if the sums are wanted).  One warp; a lane takes a unit of 8 coordinates.
 template <int DT, int FMT, int RNG, bool MULTI>
 __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0, int m_first, int m_last)
@@ -183,41 +187,102 @@ __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0, 
     }
 }
 
-// The factors of the four coordinates at i in a full row that segment boundaries cross: s_k / W for the
-// quantization (dec = false) or W / (s_k * M) for the reconstruction.  j: a segment at or before i's.
+// The scales of the four coordinates at i (the first or the second half of a lane's unit) in a row that segment
+// boundaries cross.  j: the segment that the row starts in.  The whole warp: lane l holds where segment j + l ends and its
+// scale, and a coordinate's segment is the number of ends at or before it.  (Before, every lane walked along the table for
+// every coordinate, loads behind each other, and the row that d ends in took the slow form above.  Steps of 8 binary32
+// workers in 161 layers, before / with both changed: 100 003 coordinates 22.9 / 21.2 us, 16 384 coordinates with 6-bit
+// levels 28.2 / 25.4; of 4 workers of 14.7 M with two scales, where it is the boundaries alone, 157.2 / 155.4.)
+__device__ __forceinline__ float4 mixed_row_scales(const SelectView &v, int64_t i, int j)
+{
+    const int lane = threadIdx.x & 31, c = (int)(i & 255), at = min(j + lane, v.nseg - 1);
+    const int64_t r0 = i - c, r1 = min(r0 + 256, v.d), end = segment_end(v.seg_off, v.nseg, at, v.d);
+    const float W = __ldg(v.W + at);
+    const int n = __popc(__ballot_sync(0xFFFFFFFFu, end < r1 && j + lane < v.nseg - 1));     // boundaries (a sorted table's are the first lanes)
+    if (n < 32) {
+        const int rel = (int)(end - r0);
+        int k[4] = {0, 0, 0, 0};
+        for (int b = 0; b < n; ++b) {
+            const int e = __shfl_sync(0xFFFFFFFFu, rel, b);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) k[x] += e <= c + x;
+        }
+        return make_float4(__shfl_sync(0xFFFFFFFFu, W, k[0]), __shfl_sync(0xFFFFFFFFu, W, k[1]), __shfl_sync(0xFFFFFFFFu, W, k[2]),
+                           __shfl_sync(0xFFFFFFFFu, W, k[3]));
+    }
+    float f[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        j = advance_segment(v.seg_off, v.nseg, j, i + x);
+        f[x] = __ldg(v.W + j);
+    }
+    __syncwarp();
+    return make_float4(f[0], f[1], f[2], f[3]);
+}
+
+// The factors of these coordinates: s_k / W for the quantization (dec = false) or W / (s_k * M) for the reconstruction.
 static __device__ __noinline__ float4 mixed_row_factors(const EncodeParams &p, int64_t i, int j, uint32_t kw, bool dec)
 {
     const uint32_t mask = p.idx_bits == 0 ? 0u : ((1u << p.idx_bits) - 1u) & (UQ_MAX_SCALES - 1);
+    const float4 w = mixed_row_scales(p.v, i, j);
+    const float W[4] = {w.x, w.y, w.z, w.w};
     bool overflow = false;
     float f[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
-        const float W = __ldg(p.v.W + j);
         const int32_t s = p.v.scales.s[(kw >> (e * p.idx_bits)) & mask];
-        f[e] = dec ? decode_factor(W, s, p.v.M) : inv_scale(s, W);
-        overflow |= !dec && not_finite(f[e]);
+        f[e] = dec ? decode_factor(W[e], s, p.v.M) : inv_scale(s, W[e]);
+        overflow |= !dec && i + e < p.v.d && not_finite(f[e]);
     }
     if (overflow && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
     return make_float4(f[0], f[1], f[2], f[3]);
 }
 
-// The shared indices of four coordinates of such a row, from the largest magnitudes over the workers.
-static __device__ __noinline__ uint32_t mixed_row_select(const EncodeParams &p, int64_t i, int j, uint32_t a0, uint32_t a1,
-                                                         uint32_t a2, uint32_t a3)
+// The shared indices of these coordinates, from the largest magnitudes over the workers: the largest index that passes,
+// by bisection (see uq_select.cuh: those that pass are the first ones).
+static __device__ __noinline__ uint32_t mixed_row_select(const EncodeParams &p, int64_t i, int j, uint32_t a0, uint32_t a1, uint32_t a2,
+                                                         uint32_t a3)
 {
+    const float4 w = mixed_row_scales(p.v, i, j);
+    const float W[4] = {w.x, w.y, w.z, w.w};
     const uint32_t amag[4] = {a0, a1, a2, a3};
     uint32_t packed = 0;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
-        const float W = __ldg(p.v.W + j), a = __uint_as_float(amag[e]);
+        const float a = __uint_as_float(amag[e]);
         int k = 0;
-        for (int kk = 1; kk < p.v.scales.N; ++kk)
-            if (__fmul_rn(a, inv_scale(p.v.scales.s[kk], W)) <= p.v.s_hat) k = kk;
+        for (int step = UQ_MAX_SCALES / 2; step >= 1; step >>= 1)
+            if (k + step < p.v.scales.N && __fmul_rn(a, inv_scale(p.v.scales.s[k + step], W[e])) <= p.v.s_hat) k += step;
         packed |= (uint32_t)k << (e * p.idx_bits);
     }
     return packed;
+}
+
+// What is left to do in the unit that d ends in, after the straight-line path: level 0 (and index 0, where this launch has
+// found the indices) for the coordinates d and up, whatever the padding held.
+template <int FMT> static __device__ __noinline__ void clear_padding(const EncodeParams &p, int64_t i)
+{
+    using LF = LevelFmt<FMT>;
+    const int live = (int)(p.v.d - i), M = p.v.M;
+    const size_t lrow = LF::row_bytes(p.v.stride);
+    char *row = (char *)p.lev;
+    for (int m = 0; m < M; ++m, row += lrow) {
+        char *a = row + LF::off(i);
+        if (FMT == UQ_FMT_I8) {
+            for (int e = live; e < 8; ++e) a[e] = 0;
+        } else if (FMT == UQ_FMT_I2X4) {
+            *(uint16_t *)a &= (uint16_t)((1u << (2 * live)) - 1u);
+        } else {
+            *(uint32_t *)a &= (1u << (4 * live)) - 1u;
+            if (FMT == UQ_FMT_I6P) *(uint16_t *)(row + LF::off2(i, p.v.stride)) &= (uint16_t)((1u << (2 * live)) - 1u);
+        }
+    }
+    if (p.select) {
+        const int ib = p.idx_bits;
+        uint8_t *k = p.idx + ((i * ib) >> 3);
+        if (ib == 8) for (int e = live; e < 8; ++e) k[e] = 0;
+        else for (int b = 0; b < ib; ++b) k[b] &= (uint8_t)((1u << min(max(live * ib - b * 8, 0), 8)) - 1u);
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -325,7 +390,7 @@ __device__ __forceinline__ uint4 ld_shared16(uint32_t a)
     return v;
 }
 
-// WK: 8, or with bf16 1 to 4 = exactly that many workers (known at compile time), 0 = any number.
+// WK: 8, with bf16 also 1 to 4, with binary32 2 and 4 = exactly that many workers (known at compile time), 0 = any number.
 template <int DT, int FMT, int RNG, bool MULTI, bool SEL, bool DEC, int WK>
 __global__ void __launch_bounds__(kThreads, (EncodeShape<DT, RNG, SEL, WK>::CTAS))
 encode_kernel(const __grid_constant__ EncodeParams p)
@@ -342,10 +407,15 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     // CTAs walk the tiles back to front: the kernel before this one in a step (the norms) ends on the
     // high tiles, so part of what is read first is still in L2
     const int64_t t0 = (int64_t)(gridDim.x - 1 - blockIdx.x) * S::TILE;
-    const int64_t r0 = t0 + warp * 256, i = r0 + lane * 8;                            // my warp's row, my coordinates
+    // my warp's row and my coordinates.  In the row that d ends in, the lanes beyond d do what the last one before it does,
+    // down to the bytes that they store: such a row runs as the others do.  Only in a step of binary32 gradients whose number
+    // of workers is known: with a loop around the workers the kernels have no register left for it (16 workers of 67 M
+    // coordinates 1.2 % slower), and 8 bf16 workers of 335 M coordinates or levels alone lose 0.7 % by it.
+    constexpr bool RAGGED = DT == UQ_F32 && DEC && WK > 0;
+    const int64_t r0 = t0 + warp * 256, i = RAGGED ? min(r0 + lane * 8, (d - 1) & ~(int64_t)7) : r0 + lane * 8;
     const uint64_t blk0 = (uint64_t)(p.coord0 + r0) >> BSH;
     if (r0 >= d) return;
-    bool slow = r0 + 256 > d || (uint32_t)(blk0 >> 32) != p.blk_hi || (uint32_t)blk0 > 0xFFFFFFFFu - (256u >> BSH);
+    bool slow = (!RAGGED && r0 + 256 > d) || (uint32_t)(blk0 >> 32) != p.blk_hi || (uint32_t)blk0 > 0xFFFFFFFFu - (256u >> BSH);
     const size_t grow = (size_t)p.v.stride * E::BYTES, lrow = LF::row_bytes(p.v.stride);
     // my workers: all of them, or (only the levels wanted) one of grid.y groups
     constexpr bool SPLIT = !WK && !SEL && !DEC;
@@ -380,7 +450,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         }
     }
     const int j = warp_find_segment(p.v.seg_off, p.v.nseg, r0);
-    const bool mixed = segment_end(p.v.seg_off, p.v.nseg, j, d) < r0 + 256;          // a boundary inside my row
+    const bool mixed = segment_end(p.v.seg_off, p.v.nseg, j, d) < (RAGGED ? min(r0 + 256, d) : r0 + 256);          // a boundary inside my row
     const int kmask = !MULTI ? 0 : ib < 4 ? (1 << ib) - 1 : UQ_MAX_SCALES - 1;      // lane L holds scale L & kmask
     const float W = __ldg(p.v.W + j);
     float inv_lane = inv_scale(p.v.scales.s[lane & kmask], W);
@@ -410,7 +480,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
 #pragma unroll
-                    for (int h = 0; h < V; ++h) x[k][h] = WK || k < left ? ld_keep(gs + h * 16, policy) : make_uint4(0u, 0u, 0u, 0u);
+                    for (int h = 0; h < V; ++h) x[k][h] = (WK ? k < WK : k < left) ? ld_keep(gs + h * 16, policy) : make_uint4(0u, 0u, 0u, 0u);
                     gs += grow;
                 }
 #pragma unroll
@@ -423,7 +493,8 @@ encode_kernel(const __grid_constant__ EncodeParams p)
                         a[4 * h + 3] = fmaxf(a[4 * h + 3], fabsf(__uint_as_float(x[k][h].w)));
                     }
             };
-            if (WK) { four(4); four(4); }
+            if (WK == kGroup) { four(4); four(4); }
+            else if (WK) four(WK);
             else {
 #pragma unroll 1
                 for (int m = 0; m < M; m += 4) four(M - m);
@@ -523,7 +594,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     lc.cap23 = __fmul_rn(p.v.s_hat, 8388608.0f);
     PhiloxBlockPart blk[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) blk[b] = philox_block_part(p.key, (uint32_t)blk0 + (uint32_t)(lane * NB + b));
+    for (int b = 0; b < NB; ++b) blk[b] = philox_block_part(p.key, RAGGED ? (uint32_t)((uint64_t)(p.coord0 + i) >> BSH) + (uint32_t)b : (uint32_t)blk0 + (uint32_t)(lane * NB + b));
 
     // The workers, straight-line.  The sums of two levels share a word: dp2a adds byte 0 and 2^14 times byte 1
     // (64 workers * 127 < 2^13, so the fields come apart again).
@@ -602,6 +673,17 @@ encode_kernel(const __grid_constant__ EncodeParams p)
             }
 #pragma unroll
         for (int e = 0; e < 8; ++e) r[e] = __float_as_uint(__fmul_rn((float)(int)s[e], c[e]));
+        if (RAGGED && i + 8 > p.v.d) {                           // d ends in my unit
+            __shared__ uint32_t part[16];                         // (lanes of this unit hold the same values)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { part[e] = r[e]; part[8 + e] = s[e]; }
+            for (int e = 0; i + e < p.v.d; ++e) {
+                p.out[i + e] = __uint_as_float(part[e]);
+                if (p.S != nullptr) p.S[i + e] = (int32_t)part[8 + e];
+            }
+            clear_padding<FMT>(p, i);
+            return;
+        }
         st_stream256(p.out + i, r);
         if (p.S != nullptr) st_stream256(p.S + i, s);
     }
@@ -646,6 +728,9 @@ template <int DT, int FMT, int RNG> static cudaError_t dispatch_workers(const En
         if (p.v.M == 1) return dispatch_mode<DT, FMT, RNG, 1>(p, st);
         if (p.v.M == 2) return dispatch_mode<DT, FMT, RNG, 2>(p, st);
         if (p.v.M == 3) return dispatch_mode<DT, FMT, RNG, 3>(p, st);
+        if (p.v.M == 4) return dispatch_mode<DT, FMT, RNG, 4>(p, st);
+    } else {
+        if (p.v.M == 2) return dispatch_mode<DT, FMT, RNG, 2>(p, st);
         if (p.v.M == 4) return dispatch_mode<DT, FMT, RNG, 4>(p, st);
     }
     return p.v.M == kGroup ? dispatch_mode<DT, FMT, RNG, kGroup>(p, st) : dispatch_mode<DT, FMT, RNG, 0>(p, st);

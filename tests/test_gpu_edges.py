@@ -183,3 +183,47 @@ def test_update_at_the_edges_of_its_vectors(d, fmt, s):
     want, want_m = o.sgd_update(r["ref"]["out"], np.ones(d, np.float32), np.full(d, 0.5, np.float32), lr=0.1, mu=0.9, wd=5e-4)
     assert np.array_equal(theta.cpu().numpy()[8: 8 + d], want) and np.array_equal(mom.cpu().numpy()[8: 8 + d], want_m)
     assert (theta[:8] == 1).all() and (theta[8 + d:] == 1).all() and (mom[8 + d:] == 0.5).all()
+
+
+# rows of 256 coordinates: the row that d ends in runs as the others do (binary32 steps of 2, 4 and 8 workers), whatever its
+# padding holds, and a row's boundaries are counted by its lanes (up to 31) or walked along the table (32 and more)
+@pytest.mark.parametrize("d", [1, 7, 255, 257, 2047, 2048, 4001, 4345, 6009])
+@pytest.mark.parametrize("dtype,fmt,s,N,idx_bits,rng_bits", [
+    (torch.float32, "i8", 127, 1, 0, 32), (torch.float32, "i4x2", 7, 1, 0, 16), (torch.bfloat16, "i8", 127, 8, 4, 16),
+    (torch.float32, "i6p", 31, 2, 1, 32), (torch.bfloat16, "i2x4", 1, 4, 2, 32), (torch.float32, "i8", 127, 3, 8, 32),
+])
+@pytest.mark.parametrize("segments", [False, True])
+@pytest.mark.parametrize("M", [2, 4, 8])
+def test_rows_that_end_early_or_hold_boundaries(M, d, dtype, fmt, s, N, idx_bits, rng_bits, segments):
+    from paper_2109_12497_b200.pipeline import Quantizer
+    cuts = [*range(3, 520, 7), 520, 520, 1024, 1500, 2000, 2001, 2009, d - 5, d - 1] if segments else []
+    seg = [0, *sorted(min(max(c, 0), d) for c in cuts), d]
+    scales = [s * 8 ** k for k in range(N)] if N > 1 else None
+    q = Quantizer(M, d, dtype, seg, s=s, scales=scales, idx_bits=idx_bits, rng_bits=rng_bits, keep_sums=True, one_kernel=False,
+                  fmt={"i8": B.UQ_FMT_I8, "i4x2": B.UQ_FMT_I4X2, "i2x4": B.UQ_FMT_I2X4, "i6p": B.UQ_FMT_I6P}[fmt])
+    gen = torch.Generator("cuda").manual_seed(d)
+    g = (torch.randn(M, q.stride, device="cuda", generator=gen) * torch.rand(q.stride, device="cuda", generator=gen) ** 6).to(dtype)
+    g[:, d:] = torch.tensor([np.nan, np.inf, -np.inf, 3e38] * 8, device="cuda")[: q.stride - d].to(dtype)
+    q.lev.fill_(0x55)
+    out = q.step(g, 11).cpu().numpy()
+    W, lev = q.W.cpu().numpy(), q.lev.cpu().numpy().view(np.uint8)
+    assert q.status_bits() == 0
+    g_np = g[:, :d].float().cpu().numpy()
+    table = None if q.layout.nseg == 1 else np.array(seg, dtype=np.int64)
+    assert ulp_distance(W, o.agree_scale(g_np, table, o.NORM_L2)).max() <= 1
+    if N > 1:
+        idx = o.select_scale_multi(g_np, W, scales, seg_off=table)
+        want, packed = o.encode_multi(g_np, W, scales, idx, 11, rng_bits, seg_off=table), o.pack_index(idx, idx_bits)
+        assert np.array_equal(q.idx.cpu().numpy()[: len(packed)], packed)
+        ref = o.decode(o.aggregate(want), M, W, scales=scales, idx=idx, seg_off=table)
+    else:
+        want = o.encode_single(g_np, W, s, 11, rng_bits, seg_off=table)
+        ref = o.decode(o.aggregate(want), M, W, s=s, seg_off=table)
+    unit = np.pad(want, ((0, 0), (0, -d % 8)))                          # the last unit's padding: level 0
+    bits = {"i8": lambda x: np.ascontiguousarray(x).view(np.uint8), "i4x2": o.pack_levels_i4, "i2x4": o.pack_levels_i2,
+            "i6p": lambda x: o.pack_levels_i6p(x, q.stride)}[fmt](unit)
+    n = unit.shape[1]
+    parts = [(0, n // 2), (q.stride // 2, n // 4)] if fmt == "i6p" else [(0, bits.shape[1])]
+    for a, k in parts:
+        assert np.array_equal(lev[:, a: a + k], bits[:, a: a + k])
+    assert np.array_equal(q.S.cpu().numpy()[:d], o.aggregate(want)) and np.array_equal(out, ref)
