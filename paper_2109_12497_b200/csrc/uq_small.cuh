@@ -10,7 +10,7 @@
 //            starts: the caller zeroes the scratch once, the last CTA to go zeroes it again).  Nothing is assumed
 //            about which CTAs are resident: a CTA marks its share as taken before it begins, and one that has
 //            waited for long takes a share that nobody has, so the grid gets on with whatever part of it runs (a
-//            CTA whose share was taken returns).  The wait is bounded all the same: a CTA that gives up sets
+//            CTA whose share was taken returns; W and the status flags are written by whoever holds share 0).  The wait is bounded all the same: a CTA that gives up sets
 //            UQ_STATUS_TIMEOUT and returns.  All warps add up the partials in the same fixed order, so all of
 //            them hold the same bits of W
 //   phase 2  [the shared indices from the maxima over the workers,] quantization of the workers' units, level
@@ -198,6 +198,7 @@ small_step_kernel(const __grid_constant__ SmallParams p)
 
     // ---- the exchange, and W
     int taken = 0;
+    bool holds_first = blockIdx.x == 0;                                 // share 0 is mine, from the start or taken
     float W;
     if (CLUSTER) {
         norms(0);
@@ -246,6 +247,7 @@ small_step_kernel(const __grid_constant__ SmallParams p)
             if (share == -1) break;
             if (tid == 0) sh_taken[taken] = (uint16_t)share;
             ++taken;
+            holds_first |= share == 0;
             t = (int64_t)share * blockDim.x + tid;
         }
         // each warp every nwarps-th CTA's partials, then every warp all warps' sums
@@ -261,7 +263,7 @@ small_step_kernel(const __grid_constant__ SmallParams p)
     const float cap = (float)p.scales.s[0];
     const int32_t s_lane = p.scales.s[lane & (UQ_MAX_SCALES - 1)];
     const float inv_lane = inv_scale(s_lane, W), c_lane = decode_factor(W, s_lane, M);
-    if (blockIdx.x == 0 && warp == 0) {
+    if (holds_first && warp == 0) {
         const bool overflow = __any_sync(0xFFFFFFFFu, lane < p.scales.N && not_finite(inv_lane));
         if (lane == 0) {
             p.W[0] = W;

@@ -2,6 +2,7 @@
 and against the separate calls."""
 import ctypes as C
 import dataclasses
+import time
 
 import numpy as np
 import pytest
@@ -239,3 +240,51 @@ def test_steps_on_several_streams_at_once(d, M, dtype):
         lev = o.encode_single(g_np[:, : w.d], W_ref, w.s, 1000 * k + 59, w.rng_bits)
         assert np.array_equal(q.lev.cpu().numpy()[:, : w.d], lev)
         assert np.array_equal(q.S.cpu().numpy()[: w.d], o.aggregate(lev))
+
+
+@pytest.mark.parametrize("late", [0x1, 0x90000401, 0xFFFFFFFF])
+@pytest.mark.parametrize("name,d,M,dtype,norm", [
+    ("c1", 1_500_003, 2, wl.F32, wl.NORM_LINF), ("c1", 2_000_003, 8, wl.F32, wl.NORM_L2),          # (more than the grid's registers)
+    ("c5", 700_001, 4, wl.BF16, wl.NORM_L2), ("c1", 33_790, 3, wl.F32, wl.NORM_L2), ("c3", 40_009, 8, wl.F32, wl.NORM_LINF),
+])
+def test_shares_that_change_hands(name, d, M, dtype, norm, late):
+    """Blocks that find their shares marked as taken return at once.  The marks are put there before the step and cleared while
+    it waits: the blocks that are left have to take those shares, share 0 among them (of 33 blocks, one has all).  The results
+    are complete and as if every block had kept its own."""
+    w = wl.scaled(name, d, M=M, segments="one", dtype=dtype, norm=norm)
+    g_np = wl.generate(w)
+    q = from_workload(w, keep_sums=True, one_kernel=True)
+    word = lambda x: torch.from_numpy(np.array([x], dtype=np.uint32).view(np.uint8))          # the marks of shares 0 .. 31
+    side, others = torch.cuda.Stream(), word(0xFFFFFFFF ^ late).pin_memory()
+    for step, bad in enumerate((False, True)):
+        if bad:
+            g_np[1, 1234] = np.inf if dtype == wl.F32 else 0x7F80
+        g = to_device(w, g_np)
+        for t in (q.W, q.out, q.S, q.lev):
+            t.fill_(77)
+        q.small_workspace[8:12] = word(late).cuda()
+        torch.cuda.synchronize()
+        q.step(g, 40 + step)
+        time.sleep(0.02)                                      # (the wait lasts up to a second)
+        with torch.cuda.stream(side):
+            q.small_workspace[8:12].copy_(others, non_blocking=True)
+        torch.cuda.synchronize()
+        W = q.W.cpu().numpy()
+        assert int(q.small_workspace[:64].sum().item()) == 0
+        if bad:
+            assert not np.isfinite(W[0]) and q.status_bits() == B.UQ_STATUS_NONFINITE
+            continue
+        assert q.status_bits() == 0
+        W_ref = o.agree_scale(g_np[:, :d], None, o.NORM_L2 if norm == wl.NORM_L2 else o.NORM_LINF)
+        assert abs(int(W.view(np.int32)[0]) - int(W_ref.view(np.int32)[0])) <= (norm == wl.NORM_L2)
+        if q.multi:
+            idx = o.select_scale_multi(g_np[:, :d], W, w.scales)
+            lev = o.encode_multi(g_np[:, :d], W, w.scales, idx, 40 + step, w.rng_bits)
+            packed = o.pack_index(idx, w.idx_bits)
+            assert np.array_equal(q.idx.cpu().numpy()[: len(packed)], packed)
+            out = o.decode(o.aggregate(lev), M, W, scales=w.scales, idx=idx)
+        else:
+            lev = o.encode_single(g_np[:, :d], W, w.s, 40 + step, w.rng_bits)
+            out = o.decode(o.aggregate(lev), M, W, s=w.s)
+        assert np.array_equal(q.lev.cpu().numpy()[:, :d], lev) and np.array_equal(q.S.cpu().numpy()[:d], o.aggregate(lev))
+        assert np.array_equal(q.out.cpu().numpy()[:d], out)
