@@ -163,8 +163,10 @@ small_step_kernel(const __grid_constant__ SmallParams p)
         }
     };
 
-    // ---- phase 1: per-worker norm partials of a share's units
-    auto norms = [&](int share) {
+    // ---- phase 1: per-worker norm partials of a share's units.  mine (thread 0's counts): nobody else has the share.  A CTA
+    // that came late for its own reads it all the same, since the answer takes as long as the loads, but stores nothing:
+    // others may be reading.
+    auto norms = [&](int share, uint32_t mine) {
         Acc<NORM> acc[MW];
         for (int round = 0; round < p.rounds; ++round) {
             load(round);
@@ -186,11 +188,12 @@ small_step_kernel(const __grid_constant__ SmallParams p)
             if (lane == 0) sh[warp][m] = w;
         }
         __syncthreads();
+        if (!CLUSTER && warp == 0) mine = __shfl_sync(0xFFFFFFFFu, mine, 0);
         if (tid < MW) {
             double tot = sh[0][tid];
             for (int k = 1; k < nwarps; ++k) tot = combine<NORM>(tot, sh[k][tid]);
             if (CLUSTER) sh_part[tid] = tot;
-            else __stcg(p.part + (size_t)share * kSmallMaxWorkers + tid, tot);
+            else if (mine) __stcg(p.part + (size_t)share * kSmallMaxWorkers + tid, tot);
         }
     };
     uint32_t mine = 1;                                                  // whether my share is still mine
@@ -201,7 +204,7 @@ small_step_kernel(const __grid_constant__ SmallParams p)
     bool holds_first = blockIdx.x == 0;                                 // share 0 is mine, from the start or taken
     float W;
     if (CLUSTER) {
-        norms(0);
+        norms(0, 1u);
         __syncwarp();
         cluster_arrive();
         cluster_wait();
@@ -210,7 +213,7 @@ small_step_kernel(const __grid_constant__ SmallParams p)
     } else {
         int share = blockIdx.x;
         while (true) {
-            norms(share);
+            norms(share, mine);
             __syncwarp();                     // (the partials are this warp's)
             if (tid == 0) {
                 if (mine) {
