@@ -12,7 +12,8 @@ namespace uq {
 // Programmatic dependent launch: the kernels of the library are launched with the attribute that
 // lets the GPU schedule their CTAs while the kernel before in the stream is still draining, and
 // start with grid_dependency_prologue(): a kernel first lets the one AFTER it be scheduled the same
-// way, then waits until the one before it has completed and its writes are visible.  No access to
+// way, then waits until the one before it has completed and its writes are visible (the grid of the
+// one-kernel step lets the next one be scheduled later).  No access to
 // global memory may come before the wait; what needs none may (randk_gather).  What overlaps is launch latency and the ramp of the
 // CTAs, not the work; a predecessor that knows nothing of this (a framework kernel, a copy) simply
 // counts as complete when it ends.  -DUQ_NO_PDL launches the plain way.

@@ -121,7 +121,8 @@ template <int DT, int NORM, int RNG, bool MULTI, bool CLUSTER, int MW>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 small_step_kernel(const __grid_constant__ SmallParams p)
 {
-    grid_dependency_prologue();
+    if (CLUSTER) grid_dependency_prologue();
+    else grid_dependency_wait();
     using E = Elem<DT>;
     constexpr int H = 8 / E::G, UPT = kSmallMaxWorkers / MW;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -253,6 +254,11 @@ small_step_kernel(const __grid_constant__ SmallParams p)
             holds_first |= share == 0;
             t = (int64_t)share * blockDim.x + tid;
         }
+        // The next kernel's CTAs may come now and no sooner: where two fit an SM (up to 256 threads), those that came while
+        // the grid was starting piled up on the SMs that it left free, and the next step ran at the pace of these.  8
+        // binary32 workers of 122 880 / 262 144 coordinates, steps without gaps: 11.4 / 12.7 us with the kernel's first
+        // instruction, 9.1 / 10.0 from here; 1 worker of 262 144 6.6 / 6.1, of 2^20 (512 threads) 7.8 / 7.9.
+        grid_dependency_trigger();
         // each warp every nwarps-th CTA's partials, then every warp all warps' sums
         const double a = sum_partials<NORM, MW>(warp, nwarps, (int)gridDim.x,
                                                 [&](int c, int m) { return __ldcg(p.part + (size_t)c * kSmallMaxWorkers + m); });
