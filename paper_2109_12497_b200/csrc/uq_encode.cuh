@@ -221,18 +221,24 @@ __device__ __forceinline__ float4 mixed_row_scales(const SelectView &v, int64_t 
 }
 
 // The factors of these coordinates: s_k / W for the quantization (dec = false) or W / (s_k * M) for the reconstruction.
+// LANES: the scales come from the lanes; else every lane walks along the table, which leaves more registers to the caller.
+template <bool LANES>
 static __device__ __noinline__ float4 mixed_row_factors(const EncodeParams &p, int64_t i, int j, uint32_t kw, bool dec)
 {
     const uint32_t mask = p.idx_bits == 0 ? 0u : ((1u << p.idx_bits) - 1u) & (UQ_MAX_SCALES - 1);
-    const float4 w = mixed_row_scales(p.v, i, j);
-    const float W[4] = {w.x, w.y, w.z, w.w};
+    const float4 w = LANES ? mixed_row_scales(p.v, i, j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float W[4] = {w.x, w.y, w.z, w.w};
     bool overflow = false;
     float f[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
+        if (!LANES) {
+            j = advance_segment(p.v.seg_off, p.v.nseg, j, i + e);
+            W[e] = __ldg(p.v.W + j);
+        }
         const int32_t s = p.v.scales.s[(kw >> (e * p.idx_bits)) & mask];
         f[e] = dec ? decode_factor(W[e], s, p.v.M) : inv_scale(s, W[e]);
-        overflow |= !dec && i + e < p.v.d && not_finite(f[e]);
+        overflow |= !dec && (!LANES || i + e < p.v.d) && not_finite(f[e]);     // (a walked row is a whole one)
     }
     if (overflow && p.status) atomicOr(p.status, (uint32_t)UQ_STATUS_SCALE_OVERFLOW);
     return make_float4(f[0], f[1], f[2], f[3]);
@@ -412,6 +418,11 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     // of workers is known: with a loop around the workers the kernels have no register left for it (16 workers of 67 M
     // coordinates 1.2 % slower), and 8 bf16 workers of 335 M coordinates or levels alone lose 0.7 % by it.
     constexpr bool RAGGED = DT == UQ_F32 && DEC && WK > 0;
+    // Where the callee's registers cost the rows without boundaries more than the lanes give the others, rows with
+    // boundaries walk.  From the lanes / walking, us: levels alone, 16 workers of 5 715 coordinates 10.3 / 10.0; a step of 32
+    // workers of 131 355 25.8 / 25.3, of 3 workers of 2 465 in 161 layers 47.3 / 46.3; levels alone inside a training step, 8
+    // workers of 1.1 M 28.5 / 27.8.  With selection the lanes win: 12 workers of 172 032 in 161 layers 28.5 / 29.8.
+    constexpr bool LANES = DT == UQ_BF16 || SEL || RAGGED;
     const int64_t r0 = t0 + warp * 256, i = RAGGED ? min(r0 + lane * 8, (d - 1) & ~(int64_t)7) : r0 + lane * 8;
     const uint64_t blk0 = (uint64_t)(p.coord0 + r0) >> BSH;
     if (r0 >= d) return;
@@ -572,7 +583,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
         bool inexact = false;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const float4 f = mixed_row_factors(p, i + 4 * k, j, kw[k], false);
+            const float4 f = mixed_row_factors<LANES>(p, i + 4 * k, j, kw[k], false);
             const float g[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -659,7 +670,7 @@ encode_kernel(const __grid_constant__ EncodeParams p)
             for (int e = 0; e < 8; ++e)
                 c[e] = MULTI ? __shfl_sync(0xFFFFFFFFu, c_lane, (int)(kw[e >> 2] >> ((e & 3) * ib))) : c_lane;
         } else {
-            const float4 a = mixed_row_factors(p, i, j, kw[0], true), b = mixed_row_factors(p, i + 4, j, kw[1], true);
+            const float4 a = mixed_row_factors<LANES>(p, i, j, kw[0], true), b = mixed_row_factors<LANES>(p, i + 4, j, kw[1], true);
             c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w; c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
         }
         uint32_t s[8], r[8];
