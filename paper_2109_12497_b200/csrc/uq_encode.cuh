@@ -210,7 +210,10 @@ __device__ __forceinline__ float4 mixed_row_scales(const SelectView &v, int64_t 
         return make_float4(__shfl_sync(0xFFFFFFFFu, W, k[0]), __shfl_sync(0xFFFFFFFFu, W, k[1]), __shfl_sync(0xFFFFFFFFu, W, k[2]),
                            __shfl_sync(0xFFFFFFFFu, W, k[3]));
     }
+    // 32 and more: from where i is, along the table.  Steps of 2 to 8 workers of 1 000 to 3 000 coordinates in up to 161
+    // layers, walking all the way from where the row starts / like this: 44 to 70 us / 38 to 59.
     float f[4];
+    j = find_segment(v.seg_off, v.nseg, i);
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
         j = advance_segment(v.seg_off, v.nseg, j, i + x);
