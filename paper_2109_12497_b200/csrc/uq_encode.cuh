@@ -193,22 +193,23 @@ __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0, 
 // every coordinate, loads behind each other, and the row that d ends in took the slow form above.  Steps of 8 binary32
 // workers in 161 layers, before / with both changed: 100 003 coordinates 22.9 / 21.2 us, 16 384 coordinates with 6-bit
 // levels 28.2 / 25.4; of 4 workers of 14.7 M with two scales, where it is the boundaries alone, 157.2 / 155.4.)
+// The counts share a word: with a register each, the kernels of 1 and 2 bf16 workers spilled (2 workers of 45.9 M in 161 layers
+// 134.4 us walking, 137.4 with a register each, 136.1 like this; of 64 M with two scales 265.8 / 264.3 / 262.9).
 __device__ __forceinline__ float4 mixed_row_scales(const SelectView &v, int64_t i, int j)
 {
     const int lane = threadIdx.x & 31, c = (int)(i & 255), at = min(j + lane, v.nseg - 1);
-    const int64_t r0 = i - c, r1 = min(r0 + 256, v.d), end = segment_end(v.seg_off, v.nseg, at, v.d);
+    // boundaries inside the row (a sorted table's are the first lanes), counted from the row's beginning
+    const int rel = at == v.nseg - 1 ? 512 : (int)min(__ldg(v.seg_off + at + 1) - (i - c), (int64_t)512);
     const float W = __ldg(v.W + at);
-    const int n = __popc(__ballot_sync(0xFFFFFFFFu, end < r1 && j + lane < v.nseg - 1));     // boundaries (a sorted table's are the first lanes)
+    const int n = __popc(__ballot_sync(0xFFFFFFFFu, rel < 256));
     if (n < 32) {
-        const int rel = (int)(end - r0);
-        int k[4] = {0, 0, 0, 0};
+        uint32_t k = 0;                                          // four counts of at most 31, a byte each
         for (int b = 0; b < n; ++b) {
-            const int e = __shfl_sync(0xFFFFFFFFu, rel, b);
-#pragma unroll
-            for (int x = 0; x < 4; ++x) k[x] += e <= c + x;
+            const int e = max(__shfl_sync(0xFFFFFFFFu, rel, b) - c, 0);
+            k += e < 4 ? 0x01010101u << (8 * e) : 0u;
         }
-        return make_float4(__shfl_sync(0xFFFFFFFFu, W, k[0]), __shfl_sync(0xFFFFFFFFu, W, k[1]), __shfl_sync(0xFFFFFFFFu, W, k[2]),
-                           __shfl_sync(0xFFFFFFFFu, W, k[3]));
+        return make_float4(__shfl_sync(0xFFFFFFFFu, W, k & 31), __shfl_sync(0xFFFFFFFFu, W, k >> 8 & 31), __shfl_sync(0xFFFFFFFFu, W, k >> 16 & 31),
+                           __shfl_sync(0xFFFFFFFFu, W, k >> 24));
     }
     // 32 and more: from where i is, along the table.  Steps of 2 to 8 workers of 1 000 to 3 000 coordinates in up to 161
     // layers, walking all the way from where the row starts / like this: 44 to 70 us / 38 to 59.
