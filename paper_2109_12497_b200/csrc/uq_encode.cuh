@@ -688,8 +688,10 @@ encode_kernel(const __grid_constant__ EncodeParams p)
             }
 #pragma unroll
         for (int e = 0; e < 8; ++e) r[e] = __float_as_uint(__fmul_rn((float)(int)s[e], c[e]));
-        if (RAGGED && i + 8 > p.v.d) {                           // d ends in my unit
-            __shared__ uint32_t part[16];                         // (lanes of this unit hold the same values)
+        if (RAGGED) __syncwarp();                                 // what the lanes of the last unit store comes before its correction
+        if (RAGGED && i + 8 > p.v.d) {                           // d ends in my unit: the first of its lanes does the rest
+            if (((int)i & 255) >> 3 != (threadIdx.x & 31)) return;
+            __shared__ uint32_t part[16];
 #pragma unroll
             for (int e = 0; e < 8; ++e) { part[e] = r[e]; part[8 + e] = s[e]; }
             for (int e = 0; i + e < p.v.d; ++e) {

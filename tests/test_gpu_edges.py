@@ -186,14 +186,16 @@ def test_update_at_the_edges_of_its_vectors(d, fmt, s):
 
 
 # rows of 256 coordinates: the row that d ends in runs as the others do (binary32 steps of 2, 4 and 8 workers), whatever its
-# padding holds, and a row's boundaries are counted by its lanes (up to 31) or walked along the table (32 and more)
+# padding holds, and a row's boundaries are counted by its lanes (up to 31) or looked up (32 and more; any number of
+# them with 5 binary32 workers and no selection)
 @pytest.mark.parametrize("d", [1, 7, 255, 257, 2047, 2048, 4001, 4345, 6009])
 @pytest.mark.parametrize("dtype,fmt,s,N,idx_bits,rng_bits", [
     (torch.float32, "i8", 127, 1, 0, 32), (torch.float32, "i4x2", 7, 1, 0, 16), (torch.bfloat16, "i8", 127, 8, 4, 16),
     (torch.float32, "i6p", 31, 2, 1, 32), (torch.bfloat16, "i2x4", 1, 4, 2, 32), (torch.float32, "i8", 127, 3, 8, 32),
+    (torch.float32, "i2x4", 1, 1, 0, 32), (torch.float32, "i2x4", 1, 4, 2, 16), (torch.float32, "i4x2", 7, 8, 4, 32),
 ])
 @pytest.mark.parametrize("segments", [False, True])
-@pytest.mark.parametrize("M", [2, 4, 8])
+@pytest.mark.parametrize("M", [2, 4, 5, 8])
 def test_rows_that_end_early_or_hold_boundaries(M, d, dtype, fmt, s, N, idx_bits, rng_bits, segments):
     from paper_2109_12497_b200.pipeline import Quantizer
     cuts = [*range(3, 520, 7), 520, 520, 1024, 1500, 2000, 2001, 2009, d - 5, d - 1] if segments else []
@@ -205,6 +207,8 @@ def test_rows_that_end_early_or_hold_boundaries(M, d, dtype, fmt, s, N, idx_bits
     g = (torch.randn(M, q.stride, device="cuda", generator=gen) * torch.rand(q.stride, device="cuda", generator=gen) ** 6).to(dtype)
     g[:, d:] = torch.tensor([np.nan, np.inf, -np.inf, 3e38] * 8, device="cuda")[: q.stride - d].to(dtype)
     q.lev.fill_(0x55)
+    if q.multi:
+        q.idx.fill_(0x55)
     out = q.step(g, 11).cpu().numpy()
     W, lev = q.W.cpu().numpy(), q.lev.cpu().numpy().view(np.uint8)
     assert q.status_bits() == 0
@@ -213,7 +217,8 @@ def test_rows_that_end_early_or_hold_boundaries(M, d, dtype, fmt, s, N, idx_bits
     assert ulp_distance(W, o.agree_scale(g_np, table, o.NORM_L2)).max() <= 1
     if N > 1:
         idx = o.select_scale_multi(g_np, W, scales, seg_off=table)
-        want, packed = o.encode_multi(g_np, W, scales, idx, 11, rng_bits, seg_off=table), o.pack_index(idx, idx_bits)
+        want = o.encode_multi(g_np, W, scales, idx, 11, rng_bits, seg_off=table)
+        packed = o.pack_index(np.pad(idx, (0, -d % 8)), idx_bits)       # the last unit's padding: index 0
         assert np.array_equal(q.idx.cpu().numpy()[: len(packed)], packed)
         ref = o.decode(o.aggregate(want), M, W, scales=scales, idx=idx, seg_off=table)
     else:
