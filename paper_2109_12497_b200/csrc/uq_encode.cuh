@@ -61,6 +61,8 @@ constexpr int kGroup = 8;     // the number of workers that has kernels of its o
 // binary32, 2 and 4 workers: the kernels of 8 with fewer of them, no loop, nothing spilled.  Steps, general kernel / these:
 // 4 workers of 25 M coordinates 176 / 173 us, of 25 M in 161 layers with 4 scales 247 / 218, 4-bit levels 171 / 165; 14.7 M with
 // two scales and 6-bit levels 156.6 / 141.0; of 40 003, whose last row is no slow one now, 12.5 / 9.6 and with 4 scales 17.6 / 9.8.
+// Levels alone, 2 / 4 workers of 25 M: 16-bit draws 48.9 / 46.2, 81.5 / 77.1; 32-bit draws 62.4 / 59.7, 103 / 96; with the index
+// given 66.2 / 61.3, 108 / 102; selecting, without the average, 94.8 / 83.3, 149 / 131.  (Of 20 003 and of 1 M: 0.98 to 1.08 times.)
 //
 // Few workers (1 to 4 of bf16): what does not depend on the worker is then most of a lane's work, so all workers' blocks
 // go together straight-line, their rows are staged as the eight's are, and fewer registers let more warps hide the way
@@ -747,7 +749,11 @@ template <int DT, int FMT, int RNG> static cudaError_t dispatch_workers(const En
         if (p.v.M == 3) return dispatch_mode<DT, FMT, RNG, 3>(p, st);
         if (p.v.M == 4) return dispatch_mode<DT, FMT, RNG, 4>(p, st);
     } else {
-        if (p.v.M == 2) return dispatch_mode<DT, FMT, RNG, 2>(p, st);
+        // 2 workers, one scale, 32-bit draws, with the average: the general kernel is behind up to some 12 M coordinates (the
+        // row that d ends in) and ahead beyond.  Steps, general / own, us, int8 levels: 4 M 20.9 / 20.8, 8.4 M 36.9 / 37.5,
+        // 16 M 68.8 / 70.8, 60 M 241 / 249; 6-bit levels: 8.4 M 38.5 / 37.3, 16 M 70.4 / 71.2, 60 M 250.4 / 252.4.
+        const bool general = RNG == 32 && p.idx_bits == 0 && p.out != nullptr && p.v.d > 12000000;
+        if (p.v.M == 2 && !general) return dispatch_mode<DT, FMT, RNG, 2>(p, st);
         if (p.v.M == 4) return dispatch_mode<DT, FMT, RNG, 4>(p, st);
     }
     return p.v.M == kGroup ? dispatch_mode<DT, FMT, RNG, kGroup>(p, st) : dispatch_mode<DT, FMT, RNG, 0>(p, st);

@@ -185,6 +185,22 @@ def test_update_at_the_edges_of_its_vectors(d, fmt, s):
     assert (theta[:8] == 1).all() and (theta[8 + d:] == 1).all() and (mom[8 + d:] == 0.5).all()
 
 
+# 2 binary32 workers, one scale, 32-bit draws: another kernel from 12 000 001 coordinates on
+@pytest.mark.parametrize("d", [12_000_000, 12_000_001])
+def test_two_workers_on_both_sides_of_the_line(d):
+    from paper_2109_12497_b200.pipeline import Quantizer
+    q = Quantizer(2, d, torch.float32, [0, 1, 4_000_003, d - 300, d], keep_sums=True)
+    g = torch.randn((2, q.stride), device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    out = q.step(g, 7).cpu()
+    n, lev, S = -(-d // 8) * 8, q.lev.cpu(), q.S.cpu()
+    for t in (q.lev, q.out, q.S):
+        t.fill_(77)
+    q.encode(g, 7)                                                       # stage by stage: levels alone, then the sum
+    q.aggregate_decode()
+    assert q.status_bits() == 0 and torch.equal(lev[:, :n], q.lev.cpu()[:, :n])
+    assert torch.equal(S, q.S.cpu()) and torch.equal(out, q.out.cpu())
+
+
 # rows of 256 coordinates: the row that d ends in runs as the others do (binary32 steps of 2, 4 and 8 workers), whatever its
 # padding holds, and a row's boundaries are counted by its lanes (up to 31) or looked up (32 and more; any number of
 # them with 5 binary32 workers and no selection)
