@@ -10,21 +10,22 @@
 //            starts: the caller zeroes the scratch once, the last CTA to go zeroes it again).  Nothing is assumed
 //            about which CTAs are resident: a CTA marks its share as taken before it begins, and one that has
 //            waited for long takes a share that nobody has, so the grid gets on with whatever part of it runs (a
-//            CTA whose share was taken returns; W and the status flags are written by whoever holds share 0).  The wait is bounded all the same: a CTA that gives up sets
-//            UQ_STATUS_TIMEOUT and returns.  All warps add up the partials in the same fixed order, so all of
-//            them hold the same bits of W
+//            CTA whose share was taken returns; W and the status flags are written by whoever holds share 0).
+//            The wait is bounded all the same: a CTA that gives up sets UQ_STATUS_TIMEOUT and returns.  All
+//            warps add up the partials in the same fixed order, so all of them hold the same bits of W
 //   phase 2  [the shared indices from the maxima over the workers,] quantization of the workers' units, level
 //            rows, sums in packed lanes, average
-// Only a gradient with more units than the grid holds, and shares taken from others, are read again in phase 2.  Levels, indices, sums and the
-// reconstruction are bit for bit those of the separate calls given the same W; W itself is summed in another
-// fixed order (L2: within one unit in the last place of the regular kernel's).
+// Only a gradient with more units than the grid holds, and shares taken from others, are read again in phase 2.  Levels,
+// indices, sums and the reconstruction are bit for bit those of the separate calls given the same W; W itself is summed in
+// another fixed order (L2: within one unit in the last place of the regular kernel's).
 //
 // What bounds it is latency: one trip to memory, the barrier, the chains of the Philox rounds.  Measured on a
 // B200, launches back to back (a grid with a counter in memory, every value loaded twice -> this form):
 // 4 x 4099 bf16, 8 scales 8.8 -> 5.2 us, 8 x 10^4 fp32 10.1 -> 6.8 us (one cluster).  A step of 2 x 2^20 binary32 took
-// 12.3 us as a cooperative launch, which is what such launches take one after the other whatever the kernel does; as
-// an ordinary one, whose launch overlaps the kernel in front, 10.1, and with one fence at the barrier instead of three 9.7.  (The draws of the first units made while their
-// loads are on their way, kept in shared memory: no gain on the grid, one cluster 5.5 -> 6.0 us.)
+// 12.3 us as a cooperative launch, which is what such launches take one after the other in a stream whatever the kernel
+// does (11.0 in a replayed graph); as an ordinary one, whose launch overlaps the kernel in front, 10.1, and with one fence
+// at the barrier instead of three 9.8.  (The draws of the first units made while their loads are on their way, kept in
+// shared memory: no gain on the grid, one cluster 5.5 -> 6.0 us.)
 #pragma once
 #include "uq_device.cuh"
 #include "uq_norm.cuh"
@@ -401,8 +402,6 @@ small_step_kernel(const __grid_constant__ SmallParams p)
 // ---------------------------------------------------------------------------------------------
 // launch
 // ---------------------------------------------------------------------------------------------
-constexpr int kSmallMaxCtas = 148 * 8 * 2;            // bound used to size the scratch (far above today's largest part)
-
 // CTAs of one instantiation that fit the device at once (with more, shares would wait for one another); looked up once
 // per device and instantiation.
 template <typename K> static int resident_ctas(K kernel, int *cache)
@@ -452,8 +451,9 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
     // One cluster, a unit per thread, up to 4096 units: its few SMs then take no longer than a grid over all of them
-    // loses in its barrier (about 3 us; a unit-row is 8 coordinates at about 35 cycles per
-    // warp and scheduler, so 8 workers are 4.5 k cycles on 16 SMs).
+    // loses in its barrier.  Grid / cluster, replayed graph, us, 1, 2, 4 and 8 binary32 workers: 32 768 coordinates 5.7 / 4.2,
+    // 6.0 / 4.8, 6.6 / 5.6, 8.2 / 7.8; 40 000 5.8 / 4.8, 6.0 / 5.4, 6.6 / 6.6, 8.2 / 9.4; 50 000 5.8 / 5.5, 6.0 / 6.3,
+    // 6.7 / 7.9, 8.1 / 11.4.
     if (nunits <= 8 * kSmallThreads) {
         static int ccache[64] = {};
         // one warp per scheduler of 8 SMs is not worth spreading further
@@ -471,9 +471,9 @@ static cudaError_t launch_small_one(SmallParams p, cudaStream_t st)
     const int resident = min(resident_ctas(small_step_kernel<DT, NORM, RNG, MULTI, false, MW>, cache), kSmallShares);
     if (resident <= 0) return cudaErrorNotSupported;
     // As many CTAs as the GPU takes before any has more than kSmallMinThreads threads: with 512 threads in each, a
-    // gradient of 60 000 coordinates was left to a tenth of the SMs.  512 / 256 / 128 / 64 threads, launches without
-    // gaps, against an older kernel of 256: 1 binary32 worker of 60 000 coordinates 1.16 / 0.99 / 0.98 / 0.97, 8 workers
-    // 1.09 / 0.84 / 0.78 / 0.81, 8 bf16 workers of 151 552 1.07 / 0.84 / 0.86 / 0.86.
+    // gradient of 60 000 coordinates was left to a tenth of the SMs.  At least 256 / 128 / 64 threads, replayed graph, us: 1
+    // binary32 worker of 60 000 coordinates 5.9 / 5.8 / 5.8, 4 workers 7.2 / 6.8 / 7.1, 8 workers 8.9 / 8.4 / 8.8, 8 of 120 000
+    // 9.0 / 8.8 / 8.8, of 200 000 9.2 / 9.5 / 9.5.
     const int64_t threads = max((int64_t)kSmallMinThreads, min((int64_t)kSmallThreads, ((nunits + resident - 1) / resident + 31) / 32 * 32));
     const int64_t per = (nunits + threads - 1) / threads;                 // CTAs at one unit per thread
     p.rounds = (int)((per + (int64_t)resident * UPT - 1) / ((int64_t)resident * UPT));
