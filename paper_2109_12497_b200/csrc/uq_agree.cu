@@ -359,8 +359,10 @@ norm_staged_kernel(const void *__restrict__ g, int64_t d, int64_t stride, int ns
 // One CTA per segment, one warp per worker: lane l adds up the slots of the segment's tiles l, l + 32, .. one after
 // the other, and then the lanes' sums are added.  That order depends on the segment's tiles alone: a worker's sum has
 // the same bits whatever else is in the buffer.  What bounds it is the latency of the loads, of which a lane has K
-// in flight: 8 workers of 13.1 M coordinates in one segment 7.0 us with 8, 5.0 with 32.  (With 32 throughout, a CTA's
-// registers do not fit beside the kernel in front of it: a step of 64 workers of 114 688 coordinates 46.5 -> 48 us.)  (Several warps fetching a worker's slots into shared memory for the one that adds: 1 worker 14.9 -> 13.4
+// in flight: 8 workers of 13.1 M bf16 coordinates in one segment, the kernel 7.0 us with 8, 5.0 with 32, the step 132.2 and
+// 130.9; 2 such workers 46.3 and 44.9, one binary32 worker of 25 M 69.6 and 67.3; 16 of 67 M no difference.  (With 32
+// throughout, a CTA's registers do not fit beside the kernel in front of it: a step of 64 workers of 114 688 coordinates
+// 46.5 -> 48 us.)  (Several warps fetching a worker's slots into shared memory for the one that adds: 1 worker 14.9 -> 13.4
 // us, 2 to 4 workers no faster, and with 40 KB of it the kernel in front, beside whose CTAs these start, took 4 %
 // longer; norms of 25.6 M bf16 coordinates in one segment.)
 template <int NORM, int K>

@@ -13,14 +13,16 @@ cudaError_t launch_aggregate_decode(const uq_layout &L, const void *lev, int fmt
 
 // Whether selection, quantization, and sum with reconstruction run faster as kernels of their own.  In one kernel a warp
 // takes its row through all workers, so few rows of many workers leave most of the GPU idle, and the row that holds d, in
-// its slow form, is what the kernel ends up waiting for (0.55 to 0.7 us per worker); the kernels of their own deal the
+// its slow form, is what the kernel ends up waiting for (0.55 to 0.7 us per worker; steps of 2, 4 and 8 binary32 workers,
+// which no line below concerns, have no slow form there); the kernels of their own deal the
 // workers out in groups of eight and cost a launch each.  One kernel / separate ones, launches without gaps, binary32,
 // 4 scales, 32-bit draws (without selection; with it; selection and levels alone): 4 001 coordinates, M = 8: 0.84 / 1.00 /
 // 1.18, M = 16: 1.18 / 1.26 / 1.56, M = 64: 2.6 / 2.2 / 3.1 times; 399 999 coordinates, M = 16: 1.05 / 0.77 / 1.29, M = 32:
 // 1.51 / 1.04 / 1.25, M = 64: 1.59 / 1.35 / 1.70; 1 000 003, M = 32: 1.06 / 1.10 / 1.24.  Whole rows (d a multiple of 256),
 // 4 096 coordinates, M = 16: 1.00 / 0.78 / 1.10, M = 64: 1.88 / 1.45 / 2.10; 401 408, M = 32: 1.07 / 0.75 / 0.89.  With a
-// layer table the kernels of their own lose more in the rows that boundaries cross (M = 20, 60 001 coordinates in 161
-// layers: 0.80 / 0.75 / 1.07).  The lines below are straight ones through where the two are even, over both element types
+// layer table the kernels of their own lose more in the rows that boundaries cross, where they walk along the table (161
+// layers; 120 003 coordinates, M = 16: 0.91 / 0.81 / 1.08, M = 24: 1.12 / 0.90 / 1.25, M = 32: 1.29 / 0.91 / 1.54, M = 64: 1.74 /
+// 1.33 / 1.83; 400 001, M = 24: 0.91 / 0.80 / 0.99, M = 32: 1.20 / 0.84 / 1.11, M = 64: 1.51 / 1.19 / 1.48).  The lines below are straight ones through where the two are even, over both element types
 // and draw widths.
 static bool better_separate(const uq_layout &L, bool reconstruct)
 {

@@ -111,8 +111,9 @@ __device__ __forceinline__ void store_indices(uint8_t *idx, int64_t i, int ib, c
 
 // Everything for the coordinates [r0, min(r0 + 256, d)), looked up coordinate by coordinate, in plain
 // arithmetic: the row that d ends in, in the kernels that do not take it as the others, rows whose Philox
-// block numbers leave the launch's high word, and rows whose factors are too small or too large for the rescaled forms.  Workers m_first .. m_last - 1 (all of
-// them if the sums are wanted).  One warp; a lane takes a unit of 8 coordinates.
+// block numbers leave the launch's high word, and rows whose factors are too small or too large for the
+// rescaled forms.  Workers m_first .. m_last - 1 (all of them if the sums are wanted).  One warp; a lane
+// takes a unit of 8 coordinates.
 template <int DT, int FMT, int RNG, bool MULTI>
 __device__ __noinline__ void encode_row_slow(const EncodeParams &p, int64_t r0, int m_first, int m_last)
 {
@@ -611,7 +612,9 @@ encode_kernel(const __grid_constant__ EncodeParams p)
     lc.cap23 = __fmul_rn(p.v.s_hat, 8388608.0f);
     PhiloxBlockPart blk[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) blk[b] = philox_block_part(p.key, RAGGED ? (uint32_t)((uint64_t)(p.coord0 + i) >> BSH) + (uint32_t)b : (uint32_t)blk0 + (uint32_t)(lane * NB + b));
+    for (int b = 0; b < NB; ++b)
+        blk[b] = philox_block_part(p.key, RAGGED ? (uint32_t)((uint64_t)(p.coord0 + i) >> BSH) + (uint32_t)b
+                                                 : (uint32_t)blk0 + (uint32_t)(lane * NB + b));
 
     // The workers, straight-line.  The sums of two levels share a word: dp2a adds byte 0 and 2^14 times byte 1
     // (64 workers * 127 < 2^13, so the fields come apart again).

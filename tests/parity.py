@@ -24,7 +24,7 @@ def run_gpu(w, g_np, seed=None, mode="default"):
     """All stage outputs of the CUDA path as numpy arrays.  mode picks the form of the path:
     "default" (what the library picks: the one-kernel step for small gradients, else uq_step),
     "fused" (multi-scale: selection and encoding as one call, uq_select_encode_multi), "one" (the
-    whole step as one cooperative kernel), "separate" (never the one-kernel step), "nosums" (the step
+    whole step as one kernel), "separate" (never the one-kernel step), "nosums" (the step
     without the integer sums among its outputs: quantization, aggregation and reconstruction as one
     call, uq_encode_decode; the sums compared below then come from uq_aggregate over its levels),
     "fused_nosums" (multi-scale: everything behind the scale agreement as one call,

@@ -12,7 +12,7 @@ from parity import _check_parity, check_parity, ulp_distance
 pytestmark = pytest.mark.gpu
 
 
-# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 4096 units, a cooperative grid above: of 128
+# one-kernel step: 8 CTAs up to 1024 units of 8 coordinates, a cluster up to 4096 units, a grid above: of 128
 # threads per CTA up to 148 * 128 units, then more, and more than one pass per thread (values read again) beyond one unit
 # per register set
 @pytest.mark.parametrize("M,d", [(2, 8 * 1024), (2, 8 * 1024 + 1), (2, 8 * 4096), (2, 8 * 4096 + 1), (8, 8 * 4096 - 7), (3, 8 * 4097),

@@ -1,4 +1,4 @@
-"""uq_step_small: the whole step of either quantizer as one cooperative kernel, against the oracle
+"""uq_step_small: the whole step of either quantizer as one kernel, against the oracle
 and against the separate calls."""
 import ctypes as C
 import dataclasses
