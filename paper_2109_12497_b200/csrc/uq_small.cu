@@ -3,7 +3,7 @@
 
 namespace uq {
 
-size_t small_workspace_bytes() { return kSmallHeader + (size_t)kSmallShares * kSmallMaxWorkers * sizeof(double); }
+size_t small_workspace_bytes() { return kSmallHeader + (size_t)kSmallMaxCtas * kSmallMaxWorkers * sizeof(double); }
 
 bool small_step_supported(const uq_layout &L, int fmt)
 {

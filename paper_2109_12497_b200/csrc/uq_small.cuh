@@ -402,6 +402,9 @@ small_step_kernel(const __grid_constant__ SmallParams p)
 // ---------------------------------------------------------------------------------------------
 // launch
 // ---------------------------------------------------------------------------------------------
+constexpr int kSmallMaxCtas = 148 * 8 * 2;            // what callers size the scratch for; a grid has at most kSmallShares
+static_assert(kSmallShares <= kSmallMaxCtas, "the scratch holds a partial per share and worker");
+
 // CTAs of one instantiation that fit the device at once (with more, shares would wait for one another); looked up once
 // per device and instantiation.
 template <typename K> static int resident_ctas(K kernel, int *cache)
